@@ -157,10 +157,10 @@ int build(sht_batch_s *B) {
         const bool lo = g.lo[i] != 0;
         const sht_plan_s *P = B->plans[k];
         if (mixed)
-          leg_mixed_fill_args(P, polar, B->ptr_off[k], args.data() + i * rec);
+          leg_mixed_fill_args(P, polar, args.data() + i * rec);
         else
-          leg_fp64_fill_args(P, polar, B->ptr_off[k], args.data() + i * rec, lo);
-        if (tcrec) leg_tc_fill_args(P, polar, B->ptr_off[k], targs.data() + i * tc_args_size());
+          leg_fp64_fill_args(P, polar, args.data() + i * rec, lo);
+        if (tcrec) leg_tc_fill_args(P, polar, targs.data() + i * tc_args_size());
         for (auto &it : (lo ? P->syn_list_lo : P->syn_list)[polar])
           syn.push_back({it.first, make_int4(it.second.x, it.second.y, 0, (int)i)});
         for (auto &it : (lo ? P->ana_list_lo : P->ana_list)[polar])
@@ -272,8 +272,7 @@ extern "C" int sht_batch_execute(sht_batch_t B, int type, double *const *const *
   if (flags & ~(SHT_ADD_OUTPUT | SHT_NO_POLAR_OPT)) return set_error(SHT_ERR_INVALID_ARG, "unknown flags");
   if (!alm || !map) return set_error(SHT_ERR_INVALID_ARG, "pointer arrays are NULL");
   const int n = (int)B->plans.size();
-  PtrTable TA, TM;
-  memset(&TA, 0, sizeof(TA));
+  PtrTable TM;
   memset(&TM, 0, sizeof(TM));
   std::vector<DevPtrs> A(n), M(n);
   for (int k = 0; k < n; ++k) {
@@ -288,10 +287,7 @@ extern "C" int sht_batch_execute(sht_batch_t B, int type, double *const *const *
     }
     const int per = P->spin ? 2 : 1;
     for (int j = P->nmaps; j < P->nmaps_pad; ++j) A[k].p[j] = alm[k][j % per];
-    for (int j = 0; j < P->nmaps_pad; ++j) {
-      TA.p[B->ptr_off[k] + j] = A[k].p[j];
-      TM.p[B->ptr_off[k] + j] = M[k].p[j < P->nmaps ? j : 0];
-    }
+    for (int j = 0; j < P->nmaps_pad; ++j) TM.p[B->ptr_off[k] + j] = M[k].p[j < P->nmaps ? j : 0];
   }
   int cur = -1;
   cudaGetDevice(&cur);
@@ -318,8 +314,8 @@ extern "C" int sht_batch_execute(sht_batch_t B, int type, double *const *const *
         else if (stage == 1 && g.tca)
           r = launch_leg_tc_ana_batch(g.spin, g.nj, g.d_targs[polar], items, ni, s);
         else
-          r = mixed_groups ? launch_leg_mixed_batch(stage, g.spin, g.nj, g.ppt, g.d_args[polar], items, ni, TA, s)
-                           : launch_leg_fp64_batch(stage, g.spin, g.nj, g.ppt, g.d_args[polar], items, ni, TA, s);
+          r = mixed_groups ? launch_leg_mixed_batch(stage, g.spin, g.nj, g.ppt, g.d_args[polar], items, ni, s)
+                           : launch_leg_fp64_batch(stage, g.spin, g.nj, g.ppt, g.d_args[polar], items, ni, s);
       }
       return r;
     };

@@ -14,6 +14,12 @@
 // Blocks of the growth phase in which no lane has reached scale 0 run the
 // recursion alone.
 //
+// The recursion runs on p_l = Lambda_l / alpha_l (tables.cu), whose three-term form
+// has a unit coefficient: 2 FP64 instructions a step (4 at spin s) where the form with
+// three coefficients takes 3 (6).  The a_lm tables hold alpha_l a_lm, and the
+// reduction of an analysis multiplies by alpha_l.  The FP64 pipe issues one warp
+// instruction in 16 cycles per SM, so these kernels are bound by that count.
+//
 // Enhanced exponent range (Sect. 4.1): the recursion pair is held as
 // y * 2^(600 scale); while scale < 0 the terms are below ~2^-300 and are not
 // accumulated; every 8 steps values above 2^300 are scaled down by 2^-600.
@@ -26,21 +32,17 @@ struct LegArgs {
   const int *mval;
   const int64_t *mstart;
   const int64_t *coef_off;
-  const Coef *coef;
-  const double2 *pm;  // spin: P = E + iB, M = E - iB per (array, m, l), indexed like coef
-  int64_t ncoef;      // pm's entries per array
+  const double2 *coef;  // {a, b} of p_{l+1} = (a x + b) p_l - p_{l-1}
+  const double2 *pm;    // alpha_l times a_lm (spin: P = E + iB, M = E - iB) per (array, m, l), indexed like coef
+  int64_t ncoef;        // pm's entries per array
   const double2 *mpre;
   const PairDev *pairs;
-  DevPtrs alm;
   double2 *phase;  // [nmaps][nm][npairs][2]
   const int2 *syn_items;
   const int4 *ana_items;
   const int64_t *part_off;
   double *part;
-  int ppt, add;
-  int ptr_off;  // batch: first entry of this plan in the pointer table
-  int real;     // real-harmonic storage of the a_lm (spin-0 synthesis reads them directly)
-  int half;     // m > 0 coefficients count half (SHT_GRADIENT with the adjoint analysis)
+  int ppt;
 };
 
 __device__ __forceinline__ int warp_any(bool b) { return __any_sync(0xffffffffu, b); }
@@ -49,17 +51,15 @@ __device__ __forceinline__ int warp_any(bool b) { return __any_sync(0xffffffffu,
 // Synthesis, spin 0:  F_{m,y} = sum_l a_lm lambda_lm(theta_y)   (Eq. syn2)
 // ---------------------------------------------------------------------------
 template <int NJ>
-__device__ __forceinline__ void leg_syn_s0_body(const LegArgs &a, double *const *ptrs, const int2 item) {
+__device__ __forceinline__ void leg_syn_s0_body(const LegArgs &a, const int2 item) {
   const int mi = item.x;
   const int p = item.y + threadIdx.x;
   const bool valid = p < a.npairs;
   const int m = a.mval[mi];
   const int l0 = m, lmax = a.lmax;
-  const Coef *__restrict__ cf = a.coef + a.coef_off[mi] - l0;
-  const int64_t st = a.astride;
-  const double2 *al[NJ];
-#pragma unroll
-  for (int j = 0; j < NJ; ++j) al[j] = reinterpret_cast<const double2 *>(ptrs[j]) + a.mstart[mi];
+  const int64_t co = a.coef_off[mi] - l0;
+  const double2 *__restrict__ cf = a.coef + co;
+  const double2 *__restrict__ al = a.pm + co;  // array j at al + j ncoef
 
   const PairDev pd = a.pairs[valid ? p : 0];
   const double x = pd.x;
@@ -84,8 +84,7 @@ __device__ __forceinline__ void leg_syn_s0_body(const LegArgs &a, double *const 
 #pragma unroll
       for (int k = 0; k < 8; ++k) {
         if (l <= lmax) {
-          const Coef c = ldg_coef(cf + l);
-          const double ln = fma(c.a * x, lc, -c.c * lp);
+          const double ln = fma(__ldg(&cf[l].x) * x, lc, -lp);
           lp = lc;
           lc = ln;
           ++l;
@@ -106,12 +105,11 @@ __device__ __forceinline__ void leg_syn_s0_body(const LegArgs &a, double *const 
           const double w = (scale == 0) ? lc : 0.0;
 #pragma unroll
           for (int j = 0; j < NJ; ++j) {
-            const double2 av = __ldg(al[j] + l * st);
+            const double2 av = __ldg(al + j * a.ncoef + l);
             acc[par][j][0] = fma(av.x, w, acc[par][j][0]);
             acc[par][j][1] = fma(av.y, w, acc[par][j][1]);
           }
-          const Coef c = ldg_coef(cf + l);
-          const double ln = fma(c.a * x, lc, -c.c * lp);
+          const double ln = fma(__ldg(&cf[l].x) * x, lc, -lp);
           lp = lc;
           lc = ln;
           ++l;
@@ -131,12 +129,11 @@ __device__ __forceinline__ void leg_syn_s0_body(const LegArgs &a, double *const 
       const int ll = l + par;
 #pragma unroll
       for (int j = 0; j < NJ; ++j) {
-        const double2 av = __ldg(al[j] + ll * st);
+        const double2 av = __ldg(al + j * a.ncoef + ll);
         acc[par][j][0] = fma(av.x, lc, acc[par][j][0]);
         acc[par][j][1] = fma(av.y, lc, acc[par][j][1]);
       }
-      const Coef c = ldg_coef(cf + ll);
-      const double ln = fma(c.a * x, lc, -c.c * lp);
+      const double ln = fma(__ldg(&cf[ll].x) * x, lc, -lp);
       lp = lc;
       lc = ln;
     }
@@ -144,7 +141,7 @@ __device__ __forceinline__ void leg_syn_s0_body(const LegArgs &a, double *const 
   if (l <= lmax) {
 #pragma unroll
     for (int j = 0; j < NJ; ++j) {
-      const double2 av = __ldg(al[j] + l * st);
+      const double2 av = __ldg(al + j * a.ncoef + l);
       acc[0][j][0] = fma(av.x, lc, acc[0][j][0]);
       acc[0][j][1] = fma(av.y, lc, acc[0][j][1]);
     }
@@ -155,15 +152,6 @@ __device__ __forceinline__ void leg_syn_s0_body(const LegArgs &a, double *const 
     double2 fn = make_double2(acc[0][j][0] + acc[1][j][0], acc[0][j][1] + acc[1][j][1]);
     double2 fs = make_double2(acc[0][j][0] - acc[1][j][0], acc[0][j][1] - acc[1][j][1]);
     if (m == 0) fn.y = fs.y = 0.0;  // Im a_l0 is ignored: the field is real
-    if (a.real && m > 0) {  // stored [a_{l,m}, a_{l,-m}] = sqrt2 (Re a_lm, -Im a_lm): same factors for all l
-      const double r = 0.70710678118654752440;
-      fn = make_double2(fn.x * r, -fn.y * r);
-      fs = make_double2(fs.x * r, -fs.y * r);
-    }
-    if (a.half && m > 0) {  // the sum is linear in the a_lm: halving them halves F_m
-      fn = make_double2(0.5 * fn.x, 0.5 * fn.y);
-      fs = make_double2(0.5 * fs.x, 0.5 * fs.y);
-    }
     double2 *o = a.phase + (((size_t)j * a.nm + mi) * a.npairs + p) * 2;
     o[0] = fn;
     o[1] = fs;
@@ -171,14 +159,14 @@ __device__ __forceinline__ void leg_syn_s0_body(const LegArgs &a, double *const 
 }
 template <int NJ>
 __global__ void __launch_bounds__(kSynTile) leg_syn_s0(LegArgs a) {
-  leg_syn_s0_body<NJ>(a, a.alm.p, a.syn_items[blockIdx.x]);
+  leg_syn_s0_body<NJ>(a, a.syn_items[blockIdx.x]);
 }
 template <int NJ>
 __global__ void __launch_bounds__(kSynTile) leg_syn_s0_batch(const LegArgs *__restrict__ args,
-    const int4 *__restrict__ items, const PtrTable tbl) {
+    const int4 *__restrict__ items) {
   const int4 it = items[blockIdx.x];
   const LegArgs &a = args[it.w];
-  leg_syn_s0_body<NJ>(a, tbl.p + a.ptr_off, make_int2(it.x, it.y));
+  leg_syn_s0_body<NJ>(a, make_int2(it.x, it.y));
 }
 
 // ---------------------------------------------------------------------------
@@ -192,7 +180,7 @@ __global__ void __launch_bounds__(kSynTile) leg_syn_s0_batch(const LegArgs *__re
 // with sig = (-1)^s, from sLambda(pi - t) = (-1)^(l+m) (-s)Lambda(t).
 // ---------------------------------------------------------------------------
 template <int NJ>
-__device__ __forceinline__ void leg_syn_spin_body(const LegArgs &a, double *const *ptrs, const int2 item) {
+__device__ __forceinline__ void leg_syn_spin_body(const LegArgs &a, const int2 item) {
   const int mi = item.x;
   const int p = item.y + threadIdx.x;
   const bool valid = p < a.npairs;
@@ -200,7 +188,7 @@ __device__ __forceinline__ void leg_syn_spin_body(const LegArgs &a, double *cons
   const int s = a.spin, as = s < 0 ? -s : s;
   const int l0 = m > as ? m : as, lmax = a.lmax;
   const int64_t co = a.coef_off[mi] - l0;
-  const Coef *__restrict__ cf = a.coef + co;
+  const double2 *__restrict__ cf = a.coef + co;
   const PairDev pd = a.pairs[valid ? p : 0];
   const double x = pd.x;
   double m1, m2;
@@ -231,10 +219,10 @@ __device__ __forceinline__ void leg_syn_spin_body(const LegArgs &a, double *cons
       s4[j][0] = fma(M.x, sp, s4[j][0]);
       s4[j][1] = fma(M.y, sp, s4[j][1]);
     }
-    const Coef c = ldg_coef(cf + l);
-    const double u = fma(c.a, x, c.ak), v = fma(c.a, x, -c.ak);  // A x +- AK, one rounding each
-    const double np_ = fma(u, lpc, -c.c * lpp);
-    const double nm_ = fma(v, lmc, -c.c * lmp);
+    const double2 c = __ldg(cf + l);
+    const double u = fma(c.x, x, c.y), v = fma(c.x, x, -c.y);  // a x +- b, one rounding each
+    const double np_ = fma(u, lpc, -lpp);
+    const double nm_ = fma(v, lmc, -lmp);
     lpp = lpc;
     lpc = np_;
     lmp = lmc;
@@ -247,9 +235,9 @@ __device__ __forceinline__ void leg_syn_spin_body(const LegArgs &a, double *cons
 #pragma unroll
       for (int k = 0; k < 8; ++k) {
         if (l <= lmax) {
-          const Coef c = ldg_coef(cf + l);
-          const double np_ = fma(fma(c.a, x, c.ak), lpc, -c.c * lpp);
-          const double nm_ = fma(fma(c.a, x, -c.ak), lmc, -c.c * lmp);
+          const double2 c = __ldg(cf + l);
+          const double np_ = fma(fma(c.x, x, c.y), lpc, -lpp);
+          const double nm_ = fma(fma(c.x, x, -c.y), lmc, -lmp);
           lpp = lpc;
           lpc = np_;
           lmp = lmc;
@@ -311,14 +299,14 @@ __device__ __forceinline__ void leg_syn_spin_body(const LegArgs &a, double *cons
 }
 template <int NJ>
 __global__ void __launch_bounds__(kSynTile) leg_syn_spin(LegArgs a) {
-  leg_syn_spin_body<NJ>(a, a.alm.p, a.syn_items[blockIdx.x]);
+  leg_syn_spin_body<NJ>(a, a.syn_items[blockIdx.x]);
 }
 template <int NJ>
 __global__ void __launch_bounds__(kSynTile) leg_syn_spin_batch(const LegArgs *__restrict__ args,
-    const int4 *__restrict__ items, const PtrTable tbl) {
+    const int4 *__restrict__ items) {
   const int4 it = items[blockIdx.x];
   const LegArgs &a = args[it.w];
-  leg_syn_spin_body<NJ>(a, tbl.p + a.ptr_off, make_int2(it.x, it.y));
+  leg_syn_spin_body<NJ>(a, make_int2(it.x, it.y));
 }
 // ---------------------------------------------------------------------------
 // Analysis (Eq. ana1): a_lm = sum_y G_{m,y} lambda_lm(theta_y).
@@ -371,13 +359,13 @@ __device__ __forceinline__ double warp_reduce_scatter32(double (&v)[32]) {
 }
 
 template <int NJ, int PPT>
-__device__ __forceinline__ void leg_ana_s0_body(const LegArgs &a, double *const *ptrs, const int4 item) {
+__device__ __forceinline__ void leg_ana_s0_body(const LegArgs &a, const int4 item) {
   constexpr int V = 2 * NJ, LC = 32 / V;
   __shared__ double red[kAnaThreads / 32][32];
   const int mi = item.x, tile = item.y;
   const int m = a.mval[mi];
   const int l0 = m, lmax = a.lmax, nl = lmax - l0 + 1;
-  const Coef *__restrict__ cf = a.coef + a.coef_off[mi] - l0;
+  const double2 *__restrict__ cf = a.coef + a.coef_off[mi] - l0;
   double *outp = a.part + a.part_off[mi] + (int64_t)(item.z >> 8) * nl * V;  // this item's slot
 
   double x[PPT], lc[PPT], lp[PPT];
@@ -419,10 +407,10 @@ __device__ __forceinline__ void leg_ana_s0_body(const LegArgs &a, double *const 
       for (int q = 0; q < LC; ++q) {
         const int l = lb + q;
         if (l <= lmax) {
-          const Coef c = ldg_coef(cf + l);
+          const double ca = __ldg(&cf[l].x);
 #pragma unroll
           for (int k = 0; k < PPT; ++k) {
-            const double ln = fma(c.a * x[k], lc[k], -c.c * lp[k]);
+            const double ln = fma(ca * x[k], lc[k], -lp[k]);
             lp[k] = lc[k];
             lc[k] = ln;
           }
@@ -446,7 +434,7 @@ __device__ __forceinline__ void leg_ana_s0_body(const LegArgs &a, double *const 
     for (int q = 0; q < LC; ++q) {
       const int l = lb + q;
       if (l <= lmax) {
-        const Coef c = ldg_coef(cf + l);
+        const double ca = __ldg(&cf[l].x);
         const bool even = ((l - l0) & 1) == 0;
 #pragma unroll
         for (int k = 0; k < PPT; ++k) {
@@ -458,7 +446,7 @@ __device__ __forceinline__ void leg_ana_s0_body(const LegArgs &a, double *const 
             v[q * V + 2 * j] = fma(w, gr, v[q * V + 2 * j]);
             v[q * V + 2 * j + 1] = fma(w, gi, v[q * V + 2 * j + 1]);
           }
-          const double ln = fma(c.a * x[k], lc[k], -c.c * lp[k]);
+          const double ln = fma(ca * x[k], lc[k], -lp[k]);
           lp[k] = lc[k];
           lc[k] = ln;
         }
@@ -487,14 +475,14 @@ __device__ __forceinline__ void leg_ana_s0_body(const LegArgs &a, double *const 
 }
 template <int NJ, int PPT>
 __global__ void __launch_bounds__(kAnaThreads) leg_ana_s0(LegArgs a) {
-  leg_ana_s0_body<NJ, PPT>(a, a.alm.p, a.ana_items[blockIdx.x]);
+  leg_ana_s0_body<NJ, PPT>(a, a.ana_items[blockIdx.x]);
 }
 template <int NJ, int PPT>
 __global__ void __launch_bounds__(kAnaThreads) leg_ana_s0_batch(const LegArgs *__restrict__ args,
-    const int4 *__restrict__ items, const PtrTable tbl) {
+    const int4 *__restrict__ items) {
   const int4 it = items[blockIdx.x];
   const LegArgs &a = args[it.w];
-  leg_ana_s0_body<NJ, PPT>(a, tbl.p + a.ptr_off, make_int4(it.x, it.y, it.z, 0));
+  leg_ana_s0_body<NJ, PPT>(a, make_int4(it.x, it.y, it.z, 0));
 }
 
 // Spin analysis with separate +s / -s recursions.  Per ring W+ = GQ + i GU,
@@ -502,14 +490,14 @@ __global__ void __launch_bounds__(kAnaThreads) leg_ana_s0_batch(const LegArgs *_
 //   T1 = W+_N l+ + (-1)^(l+m) W+_S l-,   T2 = W-_N l- + (-1)^(l+m) W-_S l+,
 // and the reduction kernel forms E = -(T1 + sig T2)/2, B = -(i/2)(sig T2 - T1).
 template <int NJ, int PPT>
-__device__ __forceinline__ void leg_ana_spin_body(const LegArgs &a, double *const *ptrs, const int4 item) {
+__device__ __forceinline__ void leg_ana_spin_body(const LegArgs &a, const int4 item) {
   constexpr int V = 4 * NJ, LC = 32 / V;
   __shared__ double red[kAnaThreads / 32][32];
   const int mi = item.x, tile = item.y;
   const int m = a.mval[mi];
   const int s = a.spin, as = s < 0 ? -s : s;
   const int l0 = m > as ? m : as, lmax = a.lmax, nl = lmax - l0 + 1;
-  const Coef *__restrict__ cf = a.coef + a.coef_off[mi] - l0;
+  const double2 *__restrict__ cf = a.coef + a.coef_off[mi] - l0;
   double *outp = a.part + a.part_off[mi] + (int64_t)(item.z >> 8) * nl * V;  // this item's slot
   const double sg0 = ((l0 + m) & 1) ? -1.0 : 1.0;
 
@@ -564,11 +552,11 @@ __device__ __forceinline__ void leg_ana_spin_body(const LegArgs &a, double *cons
       for (int q = 0; q < LC; ++q) {
         const int l = lb + q;
         if (l <= lmax) {
-          const Coef c = ldg_coef(cf + l);
+          const double2 c = __ldg(cf + l);
 #pragma unroll
           for (int k = 0; k < PPT; ++k) {
-            const double np_ = fma(fma(c.a, x[k], c.ak), lpc[k], -c.c * lpp[k]);
-            const double nm_ = fma(fma(c.a, x[k], -c.ak), lmc[k], -c.c * lmp[k]);
+            const double np_ = fma(fma(c.x, x[k], c.y), lpc[k], -lpp[k]);
+            const double nm_ = fma(fma(c.x, x[k], -c.y), lmc[k], -lmp[k]);
             lpp[k] = lpc[k];
             lpc[k] = np_;
             lmp[k] = lmc[k];
@@ -599,7 +587,7 @@ __device__ __forceinline__ void leg_ana_spin_body(const LegArgs &a, double *cons
     for (int q = 0; q < LC; ++q) {
       const int l = lb + q;
       if (l <= lmax) {
-        const Coef c = ldg_coef(cf + l);
+        const double2 c = __ldg(cf + l);
         const bool even = ((l - l0) & 1) == 0;
 #pragma unroll
         for (int k = 0; k < PPT; ++k) {
@@ -614,9 +602,9 @@ __device__ __forceinline__ void leg_ana_spin_body(const LegArgs &a, double *cons
             v[o + 2] = fma(wm, wmn[k][j][0], fma(sp, wms[k][j][0], v[o + 2]));
             v[o + 3] = fma(wm, wmn[k][j][1], fma(sp, wms[k][j][1], v[o + 3]));
           }
-          const double u = fma(c.a, x[k], c.ak), w = fma(c.a, x[k], -c.ak);  // A x +- AK, one rounding each
-          const double np_ = fma(u, lpc[k], -c.c * lpp[k]);
-          const double nm_ = fma(w, lmc[k], -c.c * lmp[k]);
+          const double u = fma(c.x, x[k], c.y), w = fma(c.x, x[k], -c.y);  // a x +- b, one rounding each
+          const double np_ = fma(u, lpc[k], -lpp[k]);
+          const double nm_ = fma(w, lmc[k], -lmp[k]);
           lpp[k] = lpc[k];
           lpc[k] = np_;
           lmp[k] = lmc[k];
@@ -652,22 +640,24 @@ __device__ __forceinline__ void leg_ana_spin_body(const LegArgs &a, double *cons
 }
 template <int NJ, int PPT>
 __global__ void __launch_bounds__(kAnaThreads) leg_ana_spin(LegArgs a) {
-  leg_ana_spin_body<NJ, PPT>(a, a.alm.p, a.ana_items[blockIdx.x]);
+  leg_ana_spin_body<NJ, PPT>(a, a.ana_items[blockIdx.x]);
 }
 template <int NJ, int PPT>
 __global__ void __launch_bounds__(kAnaThreads) leg_ana_spin_batch(const LegArgs *__restrict__ args,
-    const int4 *__restrict__ items, const PtrTable tbl) {
+    const int4 *__restrict__ items) {
   const int4 it = items[blockIdx.x];
   const LegArgs &a = args[it.w];
-  leg_ana_spin_body<NJ, PPT>(a, tbl.p + a.ptr_off, make_int4(it.x, it.y, it.z, 0));
+  leg_ana_spin_body<NJ, PPT>(a, make_int4(it.x, it.y, it.z, 0));
 }
 
-// Adds the tiles of every (m, l) in tile order and writes a_lm.
+// Adds the tiles of every (m, l) in tile order, multiplies by alpha_l (the kernels
+// sum G_m p_l = G_m Lambda_lm / alpha_l) and writes a_lm.
 // spin 0: V = 2 njobs values (re, im per job).
 // spin s: V = 4 njobs values (T1, T2 per job): E = -(T1 + sig T2)/2, B = -(i/2)(sig T2 - T1).
 __global__ void ana_reduce(int lmax, int spin, int nm, int njobs_pad, int ncomp, int astride, int add,
                            int real, int grad,
                            const int *__restrict__ mval, const int64_t *__restrict__ mstart,
+                           const int64_t *__restrict__ coef_off, const double *__restrict__ alpha,
                            const int64_t *__restrict__ part_off, const int *__restrict__ nslot,
                            const double *__restrict__ part, DevPtrs alm) {
   const int mi = blockIdx.y;
@@ -679,6 +669,7 @@ __global__ void ana_reduce(int lmax, int spin, int nm, int njobs_pad, int ncomp,
   const int l = l0 + blockIdx.x * blockDim.x + threadIdx.x;
   if (l > lmax) return;
   const int nt = nslot[mi];
+  const double al = alpha[coef_off[mi] + (l - l0)];
   const double *pb = part + part_off[mi] + (int64_t)(l - l0) * V;
   const int64_t idx = mstart[mi] + (int64_t)l * astride;
   const int vper = spin ? 4 : 2;
@@ -686,6 +677,7 @@ __global__ void ana_reduce(int lmax, int spin, int nm, int njobs_pad, int ncomp,
     double t[4] = {0.0, 0.0, 0.0, 0.0};
     for (int tt = 0; tt < nt; ++tt)
       for (int k = 0; k < vper; ++k) t[k] += pb[(int64_t)tt * nl * V + vper * j + k];
+    for (int k = 0; k < vper; ++k) t[k] *= al;
     double2 out[2];
     int nout;
     if (spin == 0) {
@@ -720,44 +712,54 @@ __global__ void ana_reduce(int lmax, int spin, int nm, int njobs_pad, int ncomp,
   }
 }
 
-// P = E + iB, M = E - iB for every (m, l) of a spin plan, indexed like the coefficient table
+// alpha_l times the a_lm of every (m, l), indexed like the coefficient table: array j
+// at spin 0; P = E + iB and M = E - iB (arrays 2j, 2j + 1) at spin s
 __global__ void alm_to_pm(int lmax, int spin, int nm, int astride, const int *__restrict__ mval,
                           const int64_t *__restrict__ mstart, const int64_t *__restrict__ coef_off, int64_t ncoef,
-                          DevPtrs alm, double2 *__restrict__ out, int mode) {
+                          const double *__restrict__ alpha, DevPtrs alm, double2 *__restrict__ out, int mode) {
   const int mi = blockIdx.x, j = blockIdx.y;
-  if (coef_off[mi] >= ncoef) return;  // beyond the table (a mixed plan's m above its FP64 columns)
+  const int64_t co = coef_off[mi];
+  if (co >= ncoef) return;  // beyond the table (a mixed plan's m above its FP64 columns)
   const int deriv = mode & kAlmDeriv, real = (mode & kAlmReal) && mval[mi] > 0;
   const int m = mval[mi];
   const double hf = ((mode & kAlmHalf) && m > 0) ? 0.5 : 1.0;
   const int as = spin < 0 ? -spin : spin;
   const int l0 = m > as ? m : as;
+  if (spin == 0) {
+    const double2 *src = reinterpret_cast<const double2 *>(alm.p[j]) + mstart[mi];
+    for (int l = l0 + threadIdx.x; l <= lmax; l += blockDim.x) {
+      double2 v = src[(int64_t)l * astride];
+      if (real) v = real_to_complex(v);
+      const double f = hf * alpha[co + l - l0];
+      out[(int64_t)j * ncoef + co + l - l0] = make_double2(f * v.x, f * v.y);
+    }
+    return;
+  }
   // deriv (Sect. 4.3): E = sqrt(l(l+1)) a_lm of the spin-0 array j, B = 0
   const double2 *E = reinterpret_cast<const double2 *>(alm.p[deriv ? j : 2 * j]) + mstart[mi];
   const double2 *B = reinterpret_cast<const double2 *>(alm.p[deriv ? j : 2 * j + 1]) + mstart[mi];
-  double2 *P = out + (int64_t)(2 * j) * ncoef + coef_off[mi] - l0;
-  double2 *M = out + (int64_t)(2 * j + 1) * ncoef + coef_off[mi] - l0;
+  double2 *P = out + (int64_t)(2 * j) * ncoef + co - l0;
+  double2 *M = out + (int64_t)(2 * j + 1) * ncoef + co - l0;
   for (int l = l0 + threadIdx.x; l <= lmax; l += blockDim.x) {
     double2 e = E[(int64_t)l * astride], b = B[(int64_t)l * astride];
     if (real) {
       e = real_to_complex(e);
       b = real_to_complex(b);
     }
+    double f = hf * alpha[co + l - l0];
     if (deriv) {
-      const double f = sqrt((double)l * (double)(l + 1));
-      e = make_double2(e.x * f, e.y * f);
+      f *= sqrt((double)l * (double)(l + 1));
       b = make_double2(0.0, 0.0);
     }
     if (m == 0) e.y = b.y = 0.0;  // Im of m = 0 coefficients is ignored
-    e = make_double2(hf * e.x, hf * e.y);
-    b = make_double2(hf * b.x, hf * b.y);
-    P[l] = make_double2(e.x - b.y, e.y + b.x);
-    M[l] = make_double2(e.x + b.y, e.y - b.x);
+    P[l] = make_double2(f * (e.x - b.y), f * (e.y + b.x));
+    M[l] = make_double2(f * (e.x + b.y), f * (e.y - b.x));
   }
 }
 // ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
-static LegArgs make_args(const sht_plan_s *P, const DevPtrs &alm, int polar, bool lo = false) {
+static LegArgs make_args(const sht_plan_s *P, int polar, bool lo = false) {
   LegArgs a;
   a.lmax = P->lmax;
   a.spin = P->spin;
@@ -772,27 +774,21 @@ static LegArgs make_args(const sht_plan_s *P, const DevPtrs &alm, int polar, boo
   a.ncoef = P->ncoef64;  // the P/M table's stride between arrays
   a.mpre = P->d_mpre;
   a.pairs = P->d_pairs;
-  a.alm = alm;
   a.phase = P->d_phase;
   a.syn_items = lo ? P->d_syn_lo[polar] : P->d_syn_items[polar];
   a.ana_items = lo ? P->d_ana_lo[polar] : P->d_ana_items[polar];
   a.part_off = P->d_ana_part_off[polar];
   a.part = P->d_part;
   a.ppt = P->ana_ppt;
-  a.add = 0;
-  a.real = 0;
-  a.half = 0;
   return a;
 }
 
 // Legendre stage over an explicit work list (stage 0: synthesis items int2, 1:
 // analysis items int4); no a_lm conversion (launch_alm_prepare_fp64 does it)
-cudaError_t launch_leg_fp64_items(const sht_plan_s *P, int stage, const DevPtrs &alm, int polar, const void *items,
-                                  int n, cudaStream_t st, int amode) {
+cudaError_t launch_leg_fp64_items(const sht_plan_s *P, int stage, int polar, const void *items, int n,
+                                  cudaStream_t st) {
   if (n == 0) return cudaSuccess;
-  LegArgs a = make_args(P, alm, polar);
-  a.real = (amode & kAlmReal) ? 1 : 0;
-  a.half = (amode & kAlmHalf) ? 1 : 0;
+  LegArgs a = make_args(P, polar);
   const int nj = P->njobs_pad;
   if (stage == 0) {
     a.syn_items = static_cast<const int2 *>(items);
@@ -832,14 +828,12 @@ cudaError_t launch_leg_syn_fp64(const sht_plan_s *P, const DevPtrs &alm, int pol
   if (n == 0) return cudaSuccess;
   cudaError_t e = launch_alm_prepare_fp64(P, alm, st, mode);
   if (e != cudaSuccess) return e;
-  return launch_leg_fp64_items(P, 0, alm, polar, lo ? (const void *)P->d_syn_lo[polar] : P->d_syn_items[polar], n,
-                               st, mode);
+  return launch_leg_fp64_items(P, 0, polar, lo ? (const void *)P->d_syn_lo[polar] : P->d_syn_items[polar], n, st);
 }
 
-cudaError_t launch_leg_ana_fp64(const sht_plan_s *P, const DevPtrs &alm, int polar, cudaStream_t st, bool lo) {
+cudaError_t launch_leg_ana_fp64(const sht_plan_s *P, int polar, cudaStream_t st, bool lo) {
   const int n = lo ? P->nana_lo[polar] : P->nana_items[polar];
-  return launch_leg_fp64_items(P, 1, alm, polar, lo ? (const void *)P->d_ana_lo[polar] : P->d_ana_items[polar], n,
-                               st);
+  return launch_leg_fp64_items(P, 1, polar, lo ? (const void *)P->d_ana_lo[polar] : P->d_ana_items[polar], n, st);
 }
 
 cudaError_t launch_ana_reduce(const sht_plan_s *P, const DevPtrs &alm, int polar, int add, cudaStream_t st,
@@ -847,7 +841,8 @@ cudaError_t launch_ana_reduce(const sht_plan_s *P, const DevPtrs &alm, int polar
   dim3 grid((P->lmax + 1 + 127) / 128, P->nm);
   ana_reduce<<<grid, 128, 0, st>>>(P->lmax, P->spin, P->nm, P->njobs_pad, P->ncomp, P->astride, add,
                                    real ? 1 : 0, grad ? 1 : 0,
-                                   P->d_mval, P->d_mstart, P->d_ana_part_off[polar], P->d_ana_nslot[polar],
+                                   P->d_mval, P->d_mstart, P->d_coef_off, P->d_alpha, P->d_ana_part_off[polar],
+                                   P->d_ana_nslot[polar],
                                    P->d_part, alm);
   return cudaGetLastError();
 }
@@ -861,52 +856,49 @@ namespace sht {
 
 size_t leg_fp64_args_size() { return sizeof(LegArgs); }
 
-void leg_fp64_fill_args(const sht_plan_s *P, int polar, int ptr_off, void *out, bool lo) {
-  DevPtrs none;
-  memset(&none, 0, sizeof(none));
-  LegArgs a = make_args(P, none, polar, lo);
-  a.ptr_off = ptr_off;
+void leg_fp64_fill_args(const sht_plan_s *P, int polar, void *out, bool lo) {
+  LegArgs a = make_args(P, polar, lo);
   memcpy(out, &a, sizeof(a));
 }
 
 cudaError_t launch_alm_prepare_fp64(const sht_plan_s *P, const DevPtrs &alm, cudaStream_t st, int mode) {
-  if (P->spin == 0 || P->nm == 0) return cudaSuccess;
+  if (P->nm == 0) return cudaSuccess;
   dim3 g(P->nm, P->njobs_pad);
   alm_to_pm<<<g, 256, 0, st>>>(P->lmax, P->spin, P->nm, P->astride, P->d_mval, P->d_mstart, P->d_coef_off,
-                               P->ncoef64, alm, P->d_pm64, mode);
+                               P->ncoef64, P->d_alpha, alm, P->d_pm64, mode);
   return cudaGetLastError();
 }
 
 // stage 0: synthesis, 1: analysis; all plans of the launch share spin class, njobs_pad and tiling
 cudaError_t launch_leg_fp64_batch(int stage, int spin, int nj, int ppt, const void *args, const int4 *items,
-                                  int n, const PtrTable &tbl, cudaStream_t st) {
+                                  int n, cudaStream_t st) {
   if (n == 0) return cudaSuccess;
   const LegArgs *a = static_cast<const LegArgs *>(args);
   if (stage == 0) {
     if (spin == 0) {
       switch (nj) {
-        case 1: leg_syn_s0_batch<1><<<n, kSynTile, 0, st>>>(a, items, tbl); break;
-        case 2: leg_syn_s0_batch<2><<<n, kSynTile, 0, st>>>(a, items, tbl); break;
-        case 4: leg_syn_s0_batch<4><<<n, kSynTile, 0, st>>>(a, items, tbl); break;
-        case 8: leg_syn_s0_batch<8><<<n, kSynTile, 0, st>>>(a, items, tbl); break;
-        default: leg_syn_s0_batch<16><<<n, kSynTile, 0, st>>>(a, items, tbl); break;
+        case 1: leg_syn_s0_batch<1><<<n, kSynTile, 0, st>>>(a, items); break;
+        case 2: leg_syn_s0_batch<2><<<n, kSynTile, 0, st>>>(a, items); break;
+        case 4: leg_syn_s0_batch<4><<<n, kSynTile, 0, st>>>(a, items); break;
+        case 8: leg_syn_s0_batch<8><<<n, kSynTile, 0, st>>>(a, items); break;
+        default: leg_syn_s0_batch<16><<<n, kSynTile, 0, st>>>(a, items); break;
       }
     } else {
       switch (nj) {
-        case 1: leg_syn_spin_batch<1><<<n, kSynTile, 0, st>>>(a, items, tbl); break;
-        case 2: leg_syn_spin_batch<2><<<n, kSynTile, 0, st>>>(a, items, tbl); break;
-        case 4: leg_syn_spin_batch<4><<<n, kSynTile, 0, st>>>(a, items, tbl); break;
-        default: leg_syn_spin_batch<8><<<n, kSynTile, 0, st>>>(a, items, tbl); break;
+        case 1: leg_syn_spin_batch<1><<<n, kSynTile, 0, st>>>(a, items); break;
+        case 2: leg_syn_spin_batch<2><<<n, kSynTile, 0, st>>>(a, items); break;
+        case 4: leg_syn_spin_batch<4><<<n, kSynTile, 0, st>>>(a, items); break;
+        default: leg_syn_spin_batch<8><<<n, kSynTile, 0, st>>>(a, items); break;
       }
     }
   } else {
     if (spin == 0)
       ana_shape_s0(nj, ppt, [&](auto sh) {
-        leg_ana_s0_batch<decltype(sh)::nj, decltype(sh)::ppt><<<n, kAnaThreads, 0, st>>>(a, items, tbl);
+        leg_ana_s0_batch<decltype(sh)::nj, decltype(sh)::ppt><<<n, kAnaThreads, 0, st>>>(a, items);
       });
     else
       ana_shape_spin(nj, ppt, [&](auto sh) {
-        leg_ana_spin_batch<decltype(sh)::nj, decltype(sh)::ppt><<<n, kAnaThreads, 0, st>>>(a, items, tbl);
+        leg_ana_spin_batch<decltype(sh)::nj, decltype(sh)::ppt><<<n, kAnaThreads, 0, st>>>(a, items);
       });
   }
   return cudaGetLastError();

@@ -21,11 +21,11 @@
 namespace sht {
 
 // ---------------------------------------------------------------------------
-// a_lm (FP64, user layout) -> double-float table indexed like the coefficients
+// alpha_l a_lm (a_lm: FP64, user layout) -> double-float table indexed like the coefficients
 // ---------------------------------------------------------------------------
 __global__ void alm_to_f2(int lmax, int spin, int nm, int narr, int astride, const int *__restrict__ mval,
                           const int64_t *__restrict__ mstart, const int64_t *__restrict__ coef_off, int64_t ncoef,
-                          DevPtrs alm, float4 *__restrict__ out, int mode) {
+                          const double *__restrict__ alpha, DevPtrs alm, float4 *__restrict__ out, int mode) {
   const int mi = blockIdx.x;
   const int deriv = mode & kAlmDeriv, real = (mode & kAlmReal) && mval[mi] > 0;
   const int j = blockIdx.y;
@@ -33,13 +33,15 @@ __global__ void alm_to_f2(int lmax, int spin, int nm, int narr, int astride, con
   const double hf = ((mode & kAlmHalf) && m > 0) ? 0.5 : 1.0;
   const int as = spin < 0 ? -spin : spin;
   const int l0 = m > as ? m : as;
+  const double *__restrict__ al = alpha + coef_off[mi] - l0;
   if (spin == 0) {
     const double2 *src = reinterpret_cast<const double2 *>(alm.p[j]) + mstart[mi];
     float4 *dst = out + (int64_t)j * ncoef + coef_off[mi] - l0;
     for (int l = l0 + threadIdx.x; l <= lmax; l += blockDim.x) {
       double2 v = src[(int64_t)l * astride];
       if (real) v = real_to_complex(v);
-      const f2 re = f2_of(hf * v.x), im = f2_of(hf * v.y);
+      const double f = hf * al[l];
+      const f2 re = f2_of(f * v.x), im = f2_of(f * v.y);
       dst[l] = make_float4(re.h, re.l, im.h, im.l);
     }
     return;
@@ -56,15 +58,14 @@ __global__ void alm_to_f2(int lmax, int spin, int nm, int narr, int astride, con
       e = real_to_complex(e);
       b = real_to_complex(b);
     }
+    double f = hf * al[l];
     if (deriv) {
-      const double f = sqrt((double)l * (double)(l + 1));
-      e = make_double2(e.x * f, e.y * f);
+      f *= sqrt((double)l * (double)(l + 1));
       b = make_double2(0.0, 0.0);
     }
     if (m == 0) e.y = b.y = 0.0;
-    e = make_double2(hf * e.x, hf * e.y);
-    b = make_double2(hf * b.x, hf * b.y);
-    const f2 pr = f2_of(e.x - b.y), pi = f2_of(e.y + b.x), mr = f2_of(e.x + b.y), mi_ = f2_of(e.y - b.x);
+    const f2 pr = f2_of(f * (e.x - b.y)), pi = f2_of(f * (e.y + b.x));
+    const f2 mr = f2_of(f * (e.x + b.y)), mi_ = f2_of(f * (e.y - b.x));
     P[l] = make_float4(pr.h, pr.l, pi.h, pi.l);
     M[l] = make_float4(mr.h, mr.l, mi_.h, mi_.l);
   }
@@ -78,16 +79,17 @@ __global__ void alm_to_f2(int lmax, int spin, int nm, int narr, int astride, con
 // bodies stalled the issue on instruction fetch.
 // ---------------------------------------------------------------------------
 template <int NJ>
-__device__ __forceinline__ void mix_syn_s0_body(const MixArgs &a, double *const *ptrs, const int2 item) {
+__device__ __forceinline__ void mix_syn_s0_body(const MixArgs &a, const int2 item) {
   const int mi = item.x;
   const int p = item.y + threadIdx.x;
   const bool valid = p < a.npairs;
   const int m = a.mval[mi];
   const int l0 = m, lmax = a.lmax;
   const int64_t co = a.coef_off[mi] - l0;
-  const float4 *__restrict__ cf = a.coef32 + 2 * co;
+  const float4 *__restrict__ cf = a.coef32 + co;
   const PairDev pd = a.pairs[valid ? p : 0];
-  const f3 x = f3_of(pd.x);
+  const bool polar = polar_warp(pd.x, valid);
+  const f3 x = node_of(pd.x, polar);
   // zero until the pair joins at its join record's block (no terms, a recursion of zeros)
   f2 lc = {0.f, 0.f}, lp = {0.f, 0.f};
   int scale = 0;
@@ -99,7 +101,7 @@ __device__ __forceinline__ void mix_syn_s0_body(const MixArgs &a, double *const 
 #pragma unroll
     for (int j = 0; j < NJ; ++j) acc[q][j][0] = acc[q][j][1] = f2{0.f, 0.f};
 
-  auto step = [&](int l, int par, bool act) {
+  auto step = [&](const bool pol, int l, int par, bool act) {
     const f2 w = act ? lc : weight(lc, scale);
 #pragma unroll
     for (int j = 0; j < NJ; ++j) {
@@ -107,18 +109,10 @@ __device__ __forceinline__ void mix_syn_s0_body(const MixArgs &a, double *const 
       acc_mul(acc[par][j][0], w, v.x, v.y);
       acc_mul(acc[par][j][1], w, v.z, v.w);
     }
-    const Coef32 c = ld_coef32(cf + 2 * l);
-    const f2 t = mul(c.a, x);
-    const f2 ln = dot2(t, lc, neg(c.c), lp);
-    lp = lc;
-    lc = ln;
+    step_s0(ld_coef32(cf + l), x, pol, lc, lp);
   };
-  auto recur = [&](int l) {  // recursion only (every lane's term negligible)
-    const Coef32 c = ld_coef32(cf + 2 * l);
-    const f2 t = mul(c.a, x);
-    const f2 ln = dot2(t, lc, neg(c.c), lp);
-    lp = lc;
-    lc = ln;
+  auto recur = [&](const bool pol, int l) {  // recursion only (every lane's term negligible)
+    step_s0(ld_coef32(cf + l), x, pol, lc, lp);
   };
   auto renorm_all = [&]() {
 #pragma unroll
@@ -132,42 +126,46 @@ __device__ __forceinline__ void mix_syn_s0_body(const MixArgs &a, double *const 
 
   // the warp starts at its lanes' earliest join block and walks carefully (scale
   // checks, negligible terms skipped) while a lane is below scale 0 or yet to join
-  int l = __reduce_min_sync(0xffffffffu, lj);
-  while (l <= lmax && __any_sync(0xffffffffu, scale < 0 || (lj <= lmax && lj >= l))) {
-    if (lj == l) {
-      const JoinRec r = ld_join(jrec);
-      lc = r.lpc;
-      lp = r.lpp;
-      scale = r.scp;
-    }
+  auto walk = [&](const bool pol) __attribute__((always_inline)) {
+    int l = __reduce_min_sync(0xffffffffu, lj);
+    while (l <= lmax && __any_sync(0xffffffffu, scale < 0 || (lj <= lmax && lj >= l))) {
+      if (lj == l) {
+        const JoinRec r = ld_join(jrec, polar);
+        lc = r.lpc;
+        lp = r.lpp;
+        scale = r.scp;
+      }
 #pragma unroll 1
-    for (int k = 0; k < 4 && l <= lmax; ++k, l += 2) {
-      if (__all_sync(0xffffffffu, negligible(lc, scale))) {
-        recur(l);
-        if (l + 1 <= lmax) recur(l + 1);
-      } else {
-        step(l, 0, false);
-        if (l + 1 <= lmax) step(l + 1, 1, false);
+      for (int k = 0; k < 4 && l <= lmax; ++k, l += 2) {
+        if (__all_sync(0xffffffffu, negligible(lc, scale))) {
+          recur(pol, l);
+          if (l + 1 <= lmax) recur(pol, l + 1);
+        } else {
+          step(pol, l, 0, false);
+          if (l + 1 <= lmax) step(pol, l + 1, 1, false);
+        }
+      }
+      if (scale < 0 && fabsf(lc.h) > kScaleUp32) {
+        lc = {lc.h * kScaleFactor32, lc.l * kScaleFactor32};
+        lp = {lp.h * kScaleFactor32, lp.l * kScaleFactor32};
+        ++scale;
+      }
+      renorm_all();
+    }
+    int since = 0;
+#pragma unroll 1
+    for (; l + 1 <= lmax; l += 2) {
+      step(pol, l, 0, true);
+      step(pol, l + 1, 1, true);
+      if (++since == 8) {
+        renorm_all();
+        since = 0;
       }
     }
-    if (scale < 0 && fabsf(lc.h) > kScaleUp32) {
-      lc = {lc.h * kScaleFactor32, lc.l * kScaleFactor32};
-      lp = {lp.h * kScaleFactor32, lp.l * kScaleFactor32};
-      ++scale;
-    }
-    renorm_all();
-  }
-  int since = 0;
-#pragma unroll 1
-  for (; l + 1 <= lmax; l += 2) {
-    step(l, 0, true);
-    step(l + 1, 1, true);
-    if (++since == 8) {
-      renorm_all();
-      since = 0;
-    }
-  }
-  if (l <= lmax) step(l, 0, true);
+    if (l <= lmax) step(pol, l, 0, true);
+  };
+  if (polar) walk(true);
+  else walk(false);
   if (!valid) return;
 #pragma unroll
   for (int j = 0; j < NJ; ++j) {
@@ -182,21 +180,21 @@ __device__ __forceinline__ void mix_syn_s0_body(const MixArgs &a, double *const 
 }
 template <int NJ>
 __global__ void __launch_bounds__(kSynTile) mix_syn_s0(MixArgs a) {
-  mix_syn_s0_body<NJ>(a, nullptr, a.syn_items[blockIdx.x]);
+  mix_syn_s0_body<NJ>(a, a.syn_items[blockIdx.x]);
 }
 template <int NJ>
 __global__ void __launch_bounds__(kSynTile) mix_syn_s0_batch(const MixArgs *__restrict__ args,
-    const int4 *__restrict__ items, const PtrTable tbl) {
+    const int4 *__restrict__ items) {
   const int4 it = items[blockIdx.x];
   const MixArgs &a = args[it.w];
-  mix_syn_s0_body<NJ>(a, tbl.p + a.ptr_off, make_int2(it.x, it.y));
+  mix_syn_s0_body<NJ>(a, make_int2(it.x, it.y));
 }
 
 // ---------------------------------------------------------------------------
 // synthesis, spin s: separate +s / -s recursions (see legendre_fp64.cu)
 // ---------------------------------------------------------------------------
 template <int NJ>
-__device__ __forceinline__ void mix_syn_spin_body(const MixArgs &a, double *const *ptrs, const int2 item) {
+__device__ __forceinline__ void mix_syn_spin_body(const MixArgs &a, const int2 item) {
   const int mi = item.x;
   const int p = item.y + threadIdx.x;
   const bool valid = p < a.npairs;
@@ -204,9 +202,10 @@ __device__ __forceinline__ void mix_syn_spin_body(const MixArgs &a, double *cons
   const int s = a.spin, as = s < 0 ? -s : s;
   const int l0 = m > as ? m : as, lmax = a.lmax;
   const int64_t co = a.coef_off[mi] - l0;
-  const float4 *__restrict__ cf = a.coef32 + 2 * co;
+  const float4 *__restrict__ cf = a.coef32 + co;
   const PairDev pd = a.pairs[valid ? p : 0];
-  const f3 x = f3_of(pd.x);
+  const bool polar = polar_warp(pd.x, valid);
+  const f3 x = node_of(pd.x, polar);
   // zero until the pair joins at its join record's block (no terms, a recursion of zeros)
   f2 lpc = {0.f, 0.f}, lmc = {0.f, 0.f}, lpp = {0.f, 0.f}, lmp = {0.f, 0.f};
   int scp = 0, scm = 0;
@@ -219,7 +218,7 @@ __device__ __forceinline__ void mix_syn_spin_body(const MixArgs &a, double *cons
 #pragma unroll
     for (int k = 0; k < 4; ++k) r[j][k][0] = r[j][k][1] = f2{0.f, 0.f};
 
-  auto step = [&](int l, int par, bool act) {
+  auto step = [&](const bool pol, int l, int par, bool act) {
     const f2 wp = act ? lpc : weight(lpc, scp), wm = act ? lmc : weight(lmc, scm);
     const f2 sp = par ? neg(wp) : wp, sm = par ? neg(wm) : wm;
 #pragma unroll
@@ -235,26 +234,10 @@ __device__ __forceinline__ void mix_syn_spin_body(const MixArgs &a, double *cons
       acc_mul(r[j][3][0], sp, M.x, M.y);
       acc_mul(r[j][3][1], sp, M.z, M.w);
     }
-    const Coef32 c = ld_coef32(cf + 2 * l);
-    const f2 t = mul(c.a, x);
-    const f2 nc = neg(c.c);
-    const f2 np_ = dot3(t, lpc, c.ak, lpc, nc, lpp);
-    const f2 nm_ = dot3(t, lmc, neg(c.ak), lmc, nc, lmp);
-    lpp = lpc;
-    lpc = np_;
-    lmp = lmc;
-    lmc = nm_;
+    step_spin(ld_coef32(cf + l), x, pol, lpc, lpp, lmc, lmp);
   };
-  auto recur = [&](int l) {  // recursion only (every lane's terms negligible)
-    const Coef32 c = ld_coef32(cf + 2 * l);
-    const f2 t = mul(c.a, x);
-    const f2 nc = neg(c.c);
-    const f2 np_ = dot3(t, lpc, c.ak, lpc, nc, lpp);
-    const f2 nm_ = dot3(t, lmc, neg(c.ak), lmc, nc, lmp);
-    lpp = lpc;
-    lpc = np_;
-    lmp = lmc;
-    lmc = nm_;
+  auto recur = [&](const bool pol, int l) {  // recursion only (every lane's terms negligible)
+    step_spin(ld_coef32(cf + l), x, pol, lpc, lpp, lmc, lmp);
   };
   auto renorm_all = [&]() {
 #pragma unroll
@@ -268,50 +251,54 @@ __device__ __forceinline__ void mix_syn_spin_body(const MixArgs &a, double *cons
 
   // the warp starts at its lanes' earliest join block and walks carefully (scale
   // checks, negligible terms skipped) while a lane is below scale 0 or yet to join
-  int l = __reduce_min_sync(0xffffffffu, lj);
-  while (l <= lmax && __any_sync(0xffffffffu, scp < 0 || scm < 0 || (lj <= lmax && lj >= l))) {
-    if (lj == l) {
-      const JoinRec r = ld_join(jrec);
-      lpc = r.lpc;
-      lpp = r.lpp;
-      lmc = r.lmc;
-      lmp = r.lmp;
-      scp = r.scp;
-      scm = r.scm;
-    }
+  auto walk = [&](const bool pol) __attribute__((always_inline)) {
+    int l = __reduce_min_sync(0xffffffffu, lj);
+    while (l <= lmax && __any_sync(0xffffffffu, scp < 0 || scm < 0 || (lj <= lmax && lj >= l))) {
+      if (lj == l) {
+        const JoinRec r = ld_join(jrec, polar);
+        lpc = r.lpc;
+        lpp = r.lpp;
+        lmc = r.lmc;
+        lmp = r.lmp;
+        scp = r.scp;
+        scm = r.scm;
+      }
 #pragma unroll 1
-    for (int k = 0; k < 4 && l <= lmax; ++k, l += 2) {
-      if (__all_sync(0xffffffffu, negligible(lpc, scp) && negligible(lmc, scm))) {
-        recur(l);
-        if (l + 1 <= lmax) recur(l + 1);
-      } else {
-        step(l, 0, false);
-        if (l + 1 <= lmax) step(l + 1, 1, false);
+      for (int k = 0; k < 4 && l <= lmax; ++k, l += 2) {
+        if (__all_sync(0xffffffffu, negligible(lpc, scp) && negligible(lmc, scm))) {
+          recur(pol, l);
+          if (l + 1 <= lmax) recur(pol, l + 1);
+        } else {
+          step(pol, l, 0, false);
+          if (l + 1 <= lmax) step(pol, l + 1, 1, false);
+        }
+      }
+      if (scp < 0 && fabsf(lpc.h) > kScaleUp32) {
+        lpc = {lpc.h * kScaleFactor32, lpc.l * kScaleFactor32};
+        lpp = {lpp.h * kScaleFactor32, lpp.l * kScaleFactor32};
+        ++scp;
+      }
+      if (scm < 0 && fabsf(lmc.h) > kScaleUp32) {
+        lmc = {lmc.h * kScaleFactor32, lmc.l * kScaleFactor32};
+        lmp = {lmp.h * kScaleFactor32, lmp.l * kScaleFactor32};
+        ++scm;
+      }
+      renorm_all();
+    }
+    int since = 0;
+#pragma unroll 1
+    for (; l + 1 <= lmax; l += 2) {
+      step(pol, l, 0, true);
+      step(pol, l + 1, 1, true);
+      if (++since == 8) {
+        renorm_all();
+        since = 0;
       }
     }
-    if (scp < 0 && fabsf(lpc.h) > kScaleUp32) {
-      lpc = {lpc.h * kScaleFactor32, lpc.l * kScaleFactor32};
-      lpp = {lpp.h * kScaleFactor32, lpp.l * kScaleFactor32};
-      ++scp;
-    }
-    if (scm < 0 && fabsf(lmc.h) > kScaleUp32) {
-      lmc = {lmc.h * kScaleFactor32, lmc.l * kScaleFactor32};
-      lmp = {lmp.h * kScaleFactor32, lmp.l * kScaleFactor32};
-      ++scm;
-    }
-    renorm_all();
-  }
-  int since = 0;
-#pragma unroll 1
-  for (; l + 1 <= lmax; l += 2) {
-    step(l, 0, true);
-    step(l + 1, 1, true);
-    if (++since == 8) {
-      renorm_all();
-      since = 0;
-    }
-  }
-  if (l <= lmax) step(l, 0, true);
+    if (l <= lmax) step(pol, l, 0, true);
+  };
+  if (polar) walk(true);
+  else walk(false);
   if (!valid) return;
 
   const double sig = (as & 1) ? -1.0 : 1.0;
@@ -341,14 +328,14 @@ __device__ __forceinline__ void mix_syn_spin_body(const MixArgs &a, double *cons
 }
 template <int NJ>
 __global__ void __launch_bounds__(kSynTile) mix_syn_spin(MixArgs a) {
-  mix_syn_spin_body<NJ>(a, nullptr, a.syn_items[blockIdx.x]);
+  mix_syn_spin_body<NJ>(a, a.syn_items[blockIdx.x]);
 }
 template <int NJ>
 __global__ void __launch_bounds__(kSynTile) mix_syn_spin_batch(const MixArgs *__restrict__ args,
-    const int4 *__restrict__ items, const PtrTable tbl) {
+    const int4 *__restrict__ items) {
   const int4 it = items[blockIdx.x];
   const MixArgs &a = args[it.w];
-  mix_syn_spin_body<NJ>(a, tbl.p + a.ptr_off, make_int2(it.x, it.y));
+  mix_syn_spin_body<NJ>(a, make_int2(it.x, it.y));
 }
 
 // ---------------------------------------------------------------------------
@@ -366,7 +353,7 @@ __global__ void __launch_bounds__(kSynTile) mix_syn_spin_batch(const MixArgs *__
 // Degrees are walked two at a time so the even/odd parity is static.
 // ---------------------------------------------------------------------------
 template <int NJ, int PPT, bool SPIN>
-__device__ __forceinline__ void mix_ana_body(const MixArgs &a, double *const *ptrs, const int4 item) {
+__device__ __forceinline__ void mix_ana_body(const MixArgs &a, const int4 item) {
   constexpr int V = (SPIN ? 4 : 2) * NJ, LC = 32 / V;
   static_assert(V * LC == 32, "32 slots per chunk");
   __shared__ f2 slot[32][kAnaThreads + 1];
@@ -376,7 +363,7 @@ __device__ __forceinline__ void mix_ana_body(const MixArgs &a, double *const *pt
   const int m = a.mval[mi];
   const int s = a.spin, as = s < 0 ? -s : s;
   const int l0 = m > as ? m : as, lmax = a.lmax, nl = lmax - l0 + 1;
-  const float4 *__restrict__ cf = a.coef32 + 2 * (a.coef_off[mi] - l0);
+  const float4 *__restrict__ cf = a.coef32 + (a.coef_off[mi] - l0);
   double *outp = a.part + a.part_off[mi] + (int64_t)(item.z >> 8) * nl * V;
   const double sg0 = ((l0 + m) & 1) ? -1.0 : 1.0;
   const int tid = threadIdx.x;
@@ -395,12 +382,15 @@ __device__ __forceinline__ void mix_ana_body(const MixArgs &a, double *const *pt
     // spin:   g[k][j][0..3] = W+_N, W-_N, (-1)^(l0+m) W+_S, (-1)^(l0+m) W-_S (complex)
     f2 g[PPT][NJ][SPIN ? 4 : 2][2];
     int jmin = lmax + 1;
+    double xd[PPT];
+    bool near = false;
   #pragma unroll
     for (int k = 0; k < PPT; ++k) {
       const int p = tile * (kAnaThreads * PPT) + tid + k * kAnaThreads;
       const bool valid = p < a.npairs;
       const PairDev pd = a.pairs[valid ? p : 0];
-      x[k] = f3_of(pd.x);
+      xd[k] = pd.x;
+      near = near || (valid && 1.0 - pd.x < 0.5 * kPolarTheta * kPolarTheta);
       lj[k] = valid ? __float_as_int(__ldg(a.join + ((size_t)mi * a.npairs + p) * 3 + 2).z) : lmax + 1;
       jmin = min(jmin, lj[k]);
       lpc[k] = lmc[k] = lpp[k] = lmp[k] = f2{0.f, 0.f};
@@ -442,6 +432,10 @@ __device__ __forceinline__ void mix_ana_body(const MixArgs &a, double *const *pt
       }
     }
 
+    const bool polar = __any_sync(0xffffffffu, near);
+  #pragma unroll
+    for (int k = 0; k < PPT; ++k) x[k] = node_of(xd[k], polar);
+
     // the tile starts at its pairs' earliest join block; the first tile of the group
     // zeroes the slot's degrees before it (the others leave their sums there)
     {
@@ -457,12 +451,11 @@ __device__ __forceinline__ void mix_ana_body(const MixArgs &a, double *const *pt
 
     // one degree: this thread's V contributions (summed over its pairs) into c[];
     // the first term of each output is its exact product (no sum with zero)
-    auto step = [&](int l, bool odd, bool act, f2 (&c)[V]) {
+    auto step = [&](const bool pol, int l, bool odd, bool act, f2 (&c)[V]) {
       // past lmax (second half of the last pair of degrees) the coefficients of
       // lmax stand in: the values are finite, never stored, and no table entry
       // outside this m is read
-      const Coef32 cc = ld_coef32(cf + 2 * (l <= lmax ? l : lmax));
-      const f2 nc = neg(cc.c);
+      const Coef32 cc = ld_coef32(cf + (l <= lmax ? l : lmax));
   #pragma unroll
       for (int k = 0; k < PPT; ++k) {
         const f2 wp = act ? lpc[k] : weight(lpc[k], scp[k]);
@@ -479,10 +472,7 @@ __device__ __forceinline__ void mix_ana_body(const MixArgs &a, double *const *pt
               acc_mul(c[2 * j + 1], wp, gi.h, gi.l);
             }
           }
-          const f2 t = mul(cc.a, x[k]);
-          const f2 ln = dot2(t, lpc[k], nc, lpp[k]);
-          lpp[k] = lpc[k];
-          lpc[k] = ln;
+          step_s0(cc, x[k], pol, lpc[k], lpp[k]);
         } else {
           const f2 wm = act ? lmc[k] : weight(lmc[k], scm[k]);
           const f2 sp = odd ? neg(wp) : wp, sm = odd ? neg(wm) : wm;
@@ -505,13 +495,7 @@ __device__ __forceinline__ void mix_ana_body(const MixArgs &a, double *const *pt
             acc_mul(c[4 * j + 2], sp, g[k][j][3][0].h, g[k][j][3][0].l);
             acc_mul(c[4 * j + 3], sp, g[k][j][3][1].h, g[k][j][3][1].l);
           }
-          const f2 t = mul(cc.a, x[k]);
-          const f2 np_ = dot3(t, lpc[k], cc.ak, lpc[k], nc, lpp[k]);
-          const f2 nm_ = dot3(t, lmc[k], neg(cc.ak), lmc[k], nc, lmp[k]);
-          lpp[k] = lpc[k];
-          lpc[k] = np_;
-          lmp[k] = lmc[k];
-          lmc[k] = nm_;
+          step_spin(cc, x[k], pol, lpc[k], lpp[k], lmc[k], lmp[k]);
         }
       }
     };
@@ -535,24 +519,12 @@ __device__ __forceinline__ void mix_ana_body(const MixArgs &a, double *const *pt
       for (int v = 0; v < V; ++v) slot[q * V + v][tid] = c[v];
     };
 
-    auto recur = [&](int l) {  // recursion only
-      const Coef32 cc = ld_coef32(cf + 2 * (l <= lmax ? l : lmax));
-      const f2 nc = neg(cc.c);
+    auto recur = [&](const bool pol, int l) {  // recursion only
+      const Coef32 cc = ld_coef32(cf + (l <= lmax ? l : lmax));
   #pragma unroll
       for (int k = 0; k < PPT; ++k) {
-        const f2 t = mul(cc.a, x[k]);
-        if (!SPIN) {
-          const f2 ln = dot2(t, lpc[k], nc, lpp[k]);
-          lpp[k] = lpc[k];
-          lpc[k] = ln;
-        } else {
-          const f2 np_ = dot3(t, lpc[k], cc.ak, lpc[k], nc, lpp[k]);
-          const f2 nm_ = dot3(t, lmc[k], neg(cc.ak), lmc[k], nc, lmp[k]);
-          lpp[k] = lpc[k];
-          lpc[k] = np_;
-          lmp[k] = lmc[k];
-          lmc[k] = nm_;
-        }
+        if (!SPIN) step_s0(cc, x[k], pol, lpc[k], lpp[k]);
+        else step_spin(cc, x[k], pol, lpc[k], lpp[k], lmc[k], lmp[k]);
       }
     };
     auto mode = [&]() {  // 0: all terms at scale 0, 2: all negligible, 1: weighted
@@ -576,7 +548,7 @@ __device__ __forceinline__ void mix_ana_body(const MixArgs &a, double *const *pt
       for (int k = 0; k < PPT; ++k)
         if (lj[k] == lb) {
           const int p = tile * (kAnaThreads * PPT) + tid + k * kAnaThreads;
-          const JoinRec r = ld_join(a.join + ((size_t)mi * a.npairs + p) * 3);
+          const JoinRec r = ld_join(a.join + ((size_t)mi * a.npairs + p) * 3, polar);
           lpc[k] = r.lpc;
           lpp[k] = r.lpp;
           lmc[k] = r.lmc;
@@ -593,47 +565,52 @@ __device__ __forceinline__ void mix_ana_body(const MixArgs &a, double *const *pt
       const bool mine = tid < 32 && lb + tid / V <= lmax;
       double *const o = outp + (int64_t)(lb - l0) * V + tid;
       const double prev = (gi > 0 && mine) ? *o : 0.0;
-      if (!wlive) {
-      } else if (LC >= 2) {
+      auto chunk = [&](const bool pol) __attribute__((always_inline)) {
+        if (LC >= 2) {
   #pragma unroll 1
-        for (int q = 0; q < LC; q += 2) {
-          const int l = lb + q;
-          if (l > lmax) break;
-          const int md = settled ? 0 : mode();
-          settled = md == 0;
-          if (md == 2) {
-            recur(l);
-            recur(l + 1);
-            put(q, zero);
-            put(q + 1, zero);
-          } else {
-            f2 c0[V], c1[V];
-            if (md == 0) {
-              step(l, false, true, c0);
-              step(l + 1, true, true, c1);
+          for (int q = 0; q < LC; q += 2) {
+            const int l = lb + q;
+            if (l > lmax) break;
+            const int md = settled ? 0 : mode();
+            settled = md == 0;
+            if (md == 2) {
+              recur(pol, l);
+              recur(pol, l + 1);
+              put(q, zero);
+              put(q + 1, zero);
             } else {
-              step(l, false, false, c0);
-              step(l + 1, true, false, c1);
+              f2 c0[V], c1[V];
+              if (md == 0) {
+                step(pol, l, false, true, c0);
+                step(pol, l + 1, true, true, c1);
+              } else {
+                step(pol, l, false, false, c0);
+                step(pol, l + 1, true, false, c1);
+              }
+              put(q, c0);
+              put(q + 1, c1);
             }
-            put(q, c0);
-            put(q + 1, c1);
+            since += 2;
+            if (!settled && since >= 8) {
+              rescale_all();
+              since = 0;
+            }
           }
-          since += 2;
-          if (!settled && since >= 8) {
+        } else {  // one degree per chunk: parity alternates between chunks
+          f2 c0[V];
+          const bool odd = ((lb - l0) & 1) != 0;
+          settled = settled || mode() == 0;
+          if (settled) step(pol, lb, odd, true, c0); else step(pol, lb, odd, false, c0);
+          put(0, c0);
+          if (!settled && ++since >= 8) {
             rescale_all();
             since = 0;
           }
         }
-      } else {  // one degree per chunk: parity alternates between chunks
-        f2 c0[V];
-        const bool odd = ((lb - l0) & 1) != 0;
-        settled = settled || mode() == 0;
-        if (settled) step(lb, odd, true, c0); else step(lb, odd, false, c0);
-        put(0, c0);
-        if (!settled && ++since >= 8) {
-          rescale_all();
-          since = 0;
-        }
+      };
+      if (wlive) {
+        if (polar) chunk(true);
+        else chunk(false);
       }
       // a warp's slot columns are written and read by that warp only: warp-level sync
       __syncwarp();
@@ -672,14 +649,14 @@ constexpr int mix_ana_min_blocks() {
 }
 template <int NJ, int PPT, bool SPIN>
 __global__ void __launch_bounds__(kAnaThreads, (mix_ana_min_blocks<NJ, PPT, SPIN>())) mix_ana(MixArgs a) {
-  mix_ana_body<NJ, PPT, SPIN>(a, nullptr, a.ana_items[blockIdx.x]);
+  mix_ana_body<NJ, PPT, SPIN>(a, a.ana_items[blockIdx.x]);
 }
 template <int NJ, int PPT, bool SPIN>
 __global__ void __launch_bounds__(kAnaThreads, (mix_ana_min_blocks<NJ, PPT, SPIN>())) mix_ana_batch(const MixArgs *__restrict__ args,
-    const int4 *__restrict__ items, const PtrTable tbl) {
+    const int4 *__restrict__ items) {
   const int4 it = items[blockIdx.x];
   const MixArgs &a = args[it.w];
-  mix_ana_body<NJ, PPT, SPIN>(a, tbl.p + a.ptr_off, make_int4(it.x, it.y, it.z, 0));
+  mix_ana_body<NJ, PPT, SPIN>(a, make_int4(it.x, it.y, it.z, 0));
 }
 
 // ---------------------------------------------------------------------------
@@ -702,7 +679,6 @@ static MixArgs make_mix(const sht_plan_s *P, int polar) {
   a.part_off = P->d_ana_part_off[polar];
   a.part = P->d_part;
   a.join = P->d_join;
-  a.ptr_off = 0;
   return a;
 }
 
@@ -720,7 +696,7 @@ __global__ void __launch_bounds__(128) join_kernel(MixArgs a, float4 *__restrict
   const int m = a.mval[mi];
   const int s = a.spin, as = s < 0 ? -s : s;
   const int l0 = m > as ? m : as, lmax = a.lmax;
-  const float4 *__restrict__ cf = a.coef32 + 2 * (a.coef_off[mi] - l0);
+  const float4 *__restrict__ cf = a.coef32 + (a.coef_off[mi] - l0);
   const PairDev pd = a.pairs[p];
   const f3 x = f3_of(pd.x);
   f2 lpc, lmc = {0.f, 0.f}, lpp = {0.f, 0.f}, lmp = {0.f, 0.f};
@@ -733,21 +709,9 @@ __global__ void __launch_bounds__(128) join_kernel(MixArgs a, float4 *__restrict
   }
   // one recursion step at degree l (its row's coefficients; lmax's past lmax)
   auto step = [&](int l) {
-    const Coef32 cc = ld_coef32(cf + 2 * (l <= lmax ? l : lmax));
-    const f2 t = mul(cc.a, x);
-    const f2 nc = neg(cc.c);
-    if (SPIN) {
-      const f2 np_ = dot3(t, lpc, cc.ak, lpc, nc, lpp);
-      const f2 nm_ = dot3(t, lmc, neg(cc.ak), lmc, nc, lmp);
-      lpp = lpc;
-      lpc = np_;
-      lmp = lmc;
-      lmc = nm_;
-    } else {
-      const f2 ln = dot2(t, lpc, nc, lpp);
-      lpp = lpc;
-      lpc = ln;
-    }
+    const Coef32 cc = ld_coef32(cf + (l <= lmax ? l : lmax));
+    if (SPIN) step_spin(cc, x, false, lpc, lpp, lmc, lmp);
+    else step_s0(cc, x, false, lpc, lpp);
   };
   // the kernels' exponent check, made after every eight degrees from l0
   auto rescale = [&]() {
@@ -869,7 +833,7 @@ cudaError_t launch_leg_syn_mixed(const sht_plan_s *P, const DevPtrs &alm, int po
   return launch_leg_mixed_items(P, 0, polar, P->d_syn_items[polar], P->nsyn_items[polar], st);
 }
 
-cudaError_t launch_leg_ana_mixed(const sht_plan_s *P, const DevPtrs &, int polar, cudaStream_t st) {
+cudaError_t launch_leg_ana_mixed(const sht_plan_s *P, int polar, cudaStream_t st) {
   return launch_leg_mixed_items(P, 1, polar, P->d_ana_items[polar], P->nana_items[polar], st);
 }
 
@@ -882,9 +846,8 @@ namespace sht {
 
 size_t leg_mixed_args_size() { return sizeof(MixArgs); }
 
-void leg_mixed_fill_args(const sht_plan_s *P, int polar, int ptr_off, void *out) {
+void leg_mixed_fill_args(const sht_plan_s *P, int polar, void *out) {
   MixArgs a = make_mix(P, polar);
-  a.ptr_off = ptr_off;
   memcpy(out, &a, sizeof(a));
 }
 
@@ -892,39 +855,39 @@ cudaError_t launch_alm_prepare_mixed(const sht_plan_s *P, const DevPtrs &alm, cu
   if (P->nm == 0) return cudaSuccess;
   dim3 g(P->nm, P->spin ? P->njobs_pad : P->nmaps_pad);
   alm_to_f2<<<g, 256, 0, st>>>(P->lmax, P->spin, P->nm, P->nmaps_pad, P->astride, P->d_mval, P->d_mstart,
-                               P->d_coef_off, P->ncoef, alm, P->d_alm32, mode);
+                               P->d_coef_off, P->ncoef, P->d_alpha, alm, P->d_alm32, mode);
   return cudaGetLastError();
 }
 
 cudaError_t launch_leg_mixed_batch(int stage, int spin, int nj, int ppt, const void *args, const int4 *items,
-                                   int n, const PtrTable &tbl, cudaStream_t st) {
+                                   int n, cudaStream_t st) {
   if (n == 0) return cudaSuccess;
   const MixArgs *a = static_cast<const MixArgs *>(args);
   if (stage == 0) {
     if (spin == 0) {
       switch (nj) {
-        case 1: mix_syn_s0_batch<1><<<n, kSynTile, 0, st>>>(a, items, tbl); break;
-        case 2: mix_syn_s0_batch<2><<<n, kSynTile, 0, st>>>(a, items, tbl); break;
-        case 4: mix_syn_s0_batch<4><<<n, kSynTile, 0, st>>>(a, items, tbl); break;
-        case 8: mix_syn_s0_batch<8><<<n, kSynTile, 0, st>>>(a, items, tbl); break;
-        default: mix_syn_s0_batch<16><<<n, kSynTile, 0, st>>>(a, items, tbl); break;
+        case 1: mix_syn_s0_batch<1><<<n, kSynTile, 0, st>>>(a, items); break;
+        case 2: mix_syn_s0_batch<2><<<n, kSynTile, 0, st>>>(a, items); break;
+        case 4: mix_syn_s0_batch<4><<<n, kSynTile, 0, st>>>(a, items); break;
+        case 8: mix_syn_s0_batch<8><<<n, kSynTile, 0, st>>>(a, items); break;
+        default: mix_syn_s0_batch<16><<<n, kSynTile, 0, st>>>(a, items); break;
       }
     } else {
       switch (nj) {
-        case 1: mix_syn_spin_batch<1><<<n, kSynTile, 0, st>>>(a, items, tbl); break;
-        case 2: mix_syn_spin_batch<2><<<n, kSynTile, 0, st>>>(a, items, tbl); break;
-        case 4: mix_syn_spin_batch<4><<<n, kSynTile, 0, st>>>(a, items, tbl); break;
-        default: mix_syn_spin_batch<8><<<n, kSynTile, 0, st>>>(a, items, tbl); break;
+        case 1: mix_syn_spin_batch<1><<<n, kSynTile, 0, st>>>(a, items); break;
+        case 2: mix_syn_spin_batch<2><<<n, kSynTile, 0, st>>>(a, items); break;
+        case 4: mix_syn_spin_batch<4><<<n, kSynTile, 0, st>>>(a, items); break;
+        default: mix_syn_spin_batch<8><<<n, kSynTile, 0, st>>>(a, items); break;
       }
     }
   } else {
     if (spin == 0)
       ana_shape_s0(nj, ppt, [&](auto sh) {
-        mix_ana_batch<decltype(sh)::nj, decltype(sh)::ppt, false><<<n, kAnaThreads, 0, st>>>(a, items, tbl);
+        mix_ana_batch<decltype(sh)::nj, decltype(sh)::ppt, false><<<n, kAnaThreads, 0, st>>>(a, items);
       });
     else
       ana_shape_spin(nj, ppt, [&](auto sh) {
-        mix_ana_batch<decltype(sh)::nj, decltype(sh)::ppt, true><<<n, kAnaThreads, 0, st>>>(a, items, tbl);
+        mix_ana_batch<decltype(sh)::nj, decltype(sh)::ppt, true><<<n, kAnaThreads, 0, st>>>(a, items);
       });
   }
   return cudaGetLastError();

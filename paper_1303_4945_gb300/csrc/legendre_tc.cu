@@ -79,10 +79,10 @@ struct Shape {
   static constexpr int DTILE = NCW * kK * 2;  // bytes of one a_lm digit tile
   static constexpr int A_BYTES = NL * kLamDigits * kATile;
   static constexpr int B_BYTES = NL * NDT * DTILE;
-  // per degree of a K-step, staged in shared memory one K-step ahead: the two
-  // float4 of its recursion coefficients and one float4 per a_lm table row read
+  // per degree of a K-step, staged in shared memory one K-step ahead: the float4
+  // of its recursion coefficients and one float4 per a_lm table row read
   static constexpr int NARR = SPIN ? 2 * NJ : NJ;
-  static constexpr int ROW = 2 + NARR;
+  static constexpr int ROW = 1 + NARR;
   static constexpr int STG = kK * ROW;                 // float4 per K-step
   static constexpr int PF = (STG + kRows - 1) / kRows;  // of them per thread
   static constexpr int ST_BYTES = 2 * STG * 16;        // two buffers
@@ -117,7 +117,7 @@ __device__ __forceinline__ f2 alm_value(const MixArgs &a, int64_t ci, int v) {
 // the double-float a_lm value v from a staged degree row (coefficients, then the tables)
 template <int NJ, bool SPIN>
 __device__ __forceinline__ f2 staged_value(const float4 *row, int v) {
-  const float4 q = SPIN ? row[2 + 2 * (v / 4) + ((v & 2) ? 1 : 0)] : row[2 + v / 2];
+  const float4 q = SPIN ? row[1 + 2 * (v / 4) + ((v & 2) ? 1 : 0)] : row[1 + v / 2];
   return (v & 1) ? f2{q.z, q.w} : f2{q.x, q.y};
 }
 
@@ -221,7 +221,7 @@ __device__ __forceinline__ void tc_syn_body(const TcArgs &ta, const int2 item, u
   const int l0 = m > as ? m : as, lmax = a.lmax;
   const int nks = (lmax - l0 + tc::kK) / tc::kK;
   const int64_t co = a.coef_off[mi] - l0;
-  const float4 *__restrict__ cf = a.coef32 + 2 * co;
+  const float4 *__restrict__ cf = a.coef32 + co;
   unsigned char *const Abuf = smem;
   float4 *const stage = reinterpret_cast<float4 *>(smem + S::A_BYTES);
   unsigned char *const Bt = smem + S::A_BYTES + S::ST_BYTES;
@@ -238,7 +238,7 @@ __device__ __forceinline__ void tc_syn_body(const TcArgs &ta, const int2 item, u
       pf[i] = make_float4(0.f, 0.f, 0.f, 0.f);
       if (e < S::STG) {
         const int k = e / S::ROW, c = e % S::ROW, l = lb + k;
-        if (l <= lmax) pf[i] = c < 2 ? __ldg(cf + 2 * l + c) : __ldg(a.alm32 + (int64_t)(c - 2) * a.ncoef + co + l);
+        if (l <= lmax) pf[i] = c < 1 ? __ldg(cf + l) : __ldg(a.alm32 + (int64_t)(c - 1) * a.ncoef + co + l);
       }
     }
   };
@@ -282,7 +282,8 @@ __device__ __forceinline__ void tc_syn_body(const TcArgs &ta, const int2 item, u
   // recursion state (as in the double-float synthesis): +s values lpc/lpp, -s lmc/lmp,
   // zero until the pair joins (no terms, and a recursion of zeros)
   const PairDev pd = a.pairs[valid ? p : 0];
-  const f3 x = f3_of(pd.x);
+  const bool polar = polar_warp(pd.x, valid);
+  const f3 x = node_of(pd.x, polar);
   f2 lpc = {0.f, 0.f}, lmc = {0.f, 0.f}, lpp = {0.f, 0.f}, lmp = {0.f, 0.f};
   int scp = 0, scm = 0;
   // digit grid of Lambda: magic constants of the quanta u 2^-7, u 2^-15, u 2^-23,
@@ -303,7 +304,7 @@ __device__ __forceinline__ void tc_syn_body(const TcArgs &ta, const int2 item, u
   // Every second degree the warp votes: if every lane's values are negligible for
   // the next two steps (as in the double-float kernels) the digits are zero and
   // only the recursion runs.
-  auto part = [&](const float4 *rows, uint32_t (&pk)[NL][tc::kLamDigits][tc::kPack / 2]) {
+  auto part = [&](const bool pol, const float4 *rows, uint32_t (&pk)[NL][tc::kLamDigits][tc::kPack / 2]) {
     float dlo[NL][tc::kLamDigits];
     bool dead = false;
 #pragma unroll
@@ -340,8 +341,8 @@ __device__ __forceinline__ void tc_syn_body(const TcArgs &ta, const int2 item, u
 #pragma unroll
         for (int j = 0; j < NJ; ++j) {
           if (SPIN) {
-            const float4 P = row[2 + 2 * j];
-            const float4 M = row[3 + 2 * j];
+            const float4 P = row[1 + 2 * j];
+            const float4 M = row[2 + 2 * j];
             const float rp = rr[0], rm = rr[1], sp = odd ? -rr[0] : rr[0], sm = odd ? -rr[1] : rr[1];
             racc[8 * j + 0] = __fmaf_rn(rp, P.x, racc[8 * j + 0]);
             racc[8 * j + 1] = __fmaf_rn(rp, P.z, racc[8 * j + 1]);
@@ -352,7 +353,7 @@ __device__ __forceinline__ void tc_syn_body(const TcArgs &ta, const int2 item, u
             racc[8 * j + 6] = __fmaf_rn(sm, P.x, racc[8 * j + 6]);
             racc[8 * j + 7] = __fmaf_rn(sm, P.z, racc[8 * j + 7]);
           } else {
-            const float4 v = row[2 + j];
+            const float4 v = row[1 + j];
             const int c = 4 * j + (odd ? 2 : 0);
             racc[c] = __fmaf_rn(rr[0], v.x, racc[c]);
             racc[c + 1] = __fmaf_rn(rr[0], v.z, racc[c + 1]);
@@ -371,22 +372,10 @@ __device__ __forceinline__ void tc_syn_body(const TcArgs &ta, const int2 item, u
         }
       }
       {
-        const float4 u = row[0], v = row[1];
-        const Coef32 cc = {{u.x, u.y}, {u.z, u.w}, {v.x, v.y}};
-        const f2 t = mul(cc.a, x);
-        const f2 nc = neg(cc.c);
-        if (SPIN) {
-          const f2 np_ = dot3(t, lpc, cc.ak, lpc, nc, lpp);
-          const f2 nm_ = dot3(t, lmc, neg(cc.ak), lmc, nc, lmp);
-          lpp = lpc;
-          lpc = np_;
-          lmp = lmc;
-          lmc = nm_;
-        } else {
-          const f2 ln = dot2(t, lpc, nc, lpp);
-          lpp = lpc;
-          lpc = ln;
-        }
+        const float4 u = row[0];
+        const Coef32 cc = {{u.x, u.y}, {u.z, u.w}};
+        if (SPIN) step_spin(cc, x, pol, lpc, lpp, lmc, lmp);
+        else step_s0(cc, x, pol, lpc, lpp);
       }
     }
   };
@@ -482,7 +471,7 @@ __device__ __forceinline__ void tc_syn_body(const TcArgs &ta, const int2 item, u
       __syncthreads();
     }
     if (lj == lb) {  // this pair joins: the recursion state where its terms start
-      const JoinRec r = ld_join(jrec);
+      const JoinRec r = ld_join(jrec, polar);
       lpc = r.lpc;
       lpp = r.lpp;
       lmc = r.lmc;
@@ -505,7 +494,8 @@ __device__ __forceinline__ void tc_syn_body(const TcArgs &ta, const int2 item, u
     for (int q0 = 0; q0 < tc::kK; q0 += tc::kPack) {
       uint32_t pk[NL][tc::kLamDigits][tc::kPack / 2];
       if (wlive) {
-        part(rows + q0 * S::ROW, pk);
+        if (polar) part(true, rows + q0 * S::ROW, pk);
+        else part(false, rows + q0 * S::ROW, pk);
       } else {  // no lane of the warp has joined: zero digits, and nothing to advance
 #pragma unroll
         for (int t = 0; t < NL; ++t)
@@ -656,9 +646,9 @@ float tc_lambda_bound(int lmax) {
 
 size_t tc_args_size() { return sizeof(TcArgs); }
 
-void leg_tc_fill_args(const sht_plan_s *P, int polar, int ptr_off, void *out) {
+void leg_tc_fill_args(const sht_plan_s *P, int polar, void *out) {
   TcArgs ta;
-  leg_mixed_fill_args(P, polar, ptr_off, &ta.m);
+  leg_mixed_fill_args(P, polar, &ta.m);
   ta.lam_bound = P->tc_lam_bound;
   ta.err = P->d_err;
   memcpy(out, &ta, sizeof(ta));

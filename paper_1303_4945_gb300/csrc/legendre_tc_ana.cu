@@ -139,7 +139,7 @@ __device__ __forceinline__ void tc_ana_body(const TcArgs &ta, const int4 item, u
   const int m = a.mval[mi];
   const int s = a.spin, as = s < 0 ? -s : s;
   const int l0 = m > as ? m : as, lmax = a.lmax, nl = lmax - l0 + 1;
-  const float4 *__restrict__ cf = a.coef32 + 2 * (a.coef_off[mi] - l0);
+  const float4 *__restrict__ cf = a.coef32 + (a.coef_off[mi] - l0);
   double *const outp = a.part + a.part_off[mi] + (int64_t)(item.z >> 8) * nl * V;
   const double sg0 = ((l0 + m) & 1) ? -1.0 : 1.0;
   unsigned char *const Abuf = tca_smem;
@@ -287,7 +287,9 @@ __device__ __forceinline__ void tc_ana_body(const TcArgs &ta, const int4 item, u
     if (lstart > lmax) continue;
 
     // the walk over the tile's blocks of 8 degrees (from its pairs' earliest join)
-    const f3 x = f3_of(valid ? a.pairs[p].x : 0.0);
+    const double xd = valid ? a.pairs[p].x : 0.0;
+    const bool polar = polar_warp(xd, valid);
+    const f3 x = node_of(xd, polar);
     f2 lpc = {0.f, 0.f}, lmc = {0.f, 0.f}, lpp = {0.f, 0.f}, lmp = {0.f, 0.f};
     int scp = 0, scm = 0;
     const float ulx = __int_as_float((127 - lexp) << 23);  // 1 / u_p
@@ -299,7 +301,7 @@ __device__ __forceinline__ void tc_ana_body(const TcArgs &ta, const int4 item, u
     // joined pair are not tested for negligibility: the join record already skips
     // the stretch before its first non-negligible degree pair, and later values
     // below the digits' grid give zero digits.)
-    auto part = [&](int lb4, uint32_t (&pk)[NSET][kDig][2]) {
+    auto part = [&](const bool pol, int lb4, uint32_t (&pk)[NSET][kDig][2]) {
       float hold[NSET][kDig];
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
@@ -320,21 +322,9 @@ __device__ __forceinline__ void tc_ana_body(const TcArgs &ta, const int4 item, u
           }
         // recursion to l + 1 (past lmax the coefficients of lmax stand in: finite
         // values no output reads)
-        const Coef32 cc = ld_coef32(cf + 2 * (l <= lmax ? l : lmax));
-        const f2 t = mul(cc.a, x);
-        const f2 nc = neg(cc.c);
-        if (SPIN) {
-          const f2 np_ = dot3(t, lpc, cc.ak, lpc, nc, lpp);
-          const f2 nm_ = dot3(t, lmc, neg(cc.ak), lmc, nc, lmp);
-          lpp = lpc;
-          lpc = np_;
-          lmp = lmc;
-          lmc = nm_;
-        } else {
-          const f2 ln = dot2(t, lpc, nc, lpp);
-          lpp = lpc;
-          lpc = ln;
-        }
+        const Coef32 cc = ld_coef32(cf + (l <= lmax ? l : lmax));
+        if (SPIN) step_spin(cc, x, pol, lpc, lpp, lmc, lmp);
+        else step_s0(cc, x, pol, lpc, lpp);
       }
     };
     // the enhanced exponent's check after every block of 8 degrees (see mixed_common.cuh)
@@ -465,7 +455,7 @@ __device__ __forceinline__ void tc_ana_body(const TcArgs &ta, const int4 item, u
       double prev = 0.0;
       if (o_prev && gi > 0) asm volatile("ld.global.f64 %0, [%1];" : "=d"(prev) : "l"(o_prev));
       if (lj == lb) {  // this pair joins: the recursion state where its terms start
-        const JoinRec r = ld_join(jrec);
+        const JoinRec r = ld_join(jrec, polar);
         lpc = r.lpc;
         lpp = r.lpp;
         lmc = r.lmc;
@@ -485,7 +475,8 @@ __device__ __forceinline__ void tc_ana_body(const TcArgs &ta, const int4 item, u
 #pragma unroll 1
         for (int h = 0; h < 2; ++h) {
           uint32_t pk[NSET][kDig][2];
-          part(lb + 4 * h, pk);
+          if (polar) part(true, lb + 4 * h, pk);
+          else part(false, lb + 4 * h, pk);
           // this warp's products of its previous block read the tiles: wait for them
           // before the first write (they have long finished by now)
           if (h == 0 && nmine > nmine_done) {

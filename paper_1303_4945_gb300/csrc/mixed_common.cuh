@@ -35,12 +35,16 @@ __device__ __forceinline__ f2 mul(f2 a, f3 x) {
   e = __fmaf_rn(a.h, x.m, e);
   return {p, e};
 }
-// a b + c d + e f, normalised (see dot2)
-__device__ __forceinline__ f2 dot3(f2 a, f2 b, f2 c, f2 d, f2 e, f2 f) {
-  const f2 p = mul(a, b), q = mul(c, d), r = mul(e, f);
-  const f2 s1 = two_sum(p.h, q.h);
-  const f2 s2 = two_sum(s1.h, r.h);
-  return fast_two_sum(s2.h, __fadd_rn(__fadd_rn(__fadd_rn(p.l, q.l), r.l), __fadd_rn(s1.l, s2.l)));
+// a b - c, normalised (see dot2): a recursion step p_{l+1} = u p_l - p_{l-1}
+__device__ __forceinline__ f2 mul_sub(f2 a, f2 b, f2 c) {
+  const f2 p = mul(a, b);
+  const f2 s = two_sum(p.h, -c.h);
+  return fast_two_sum(s.h, __fadd_rn(__fsub_rn(p.l, c.l), s.l));
+}
+// a + b as an unevaluated pair
+__device__ __forceinline__ f2 sum2(f2 a, f2 b) {
+  const f2 s = two_sum(a.h, b.h);
+  return {s.h, __fadd_rn(__fadd_rn(a.l, b.l), s.l)};
 }
 // acc += w * a with a lazily carried low word (renormalised every few steps)
 __device__ __forceinline__ void acc_mul(f2 &acc, f2 w, float ah, float al) {
@@ -107,14 +111,23 @@ __device__ __forceinline__ JoinRec ld_join(const float4 *p) {
   r.lexp = __float_as_int(c.w);
   return r;
 }
+// the record as a polar warp's state (see step_polar)
+__device__ __forceinline__ JoinRec ld_join(const float4 *p, bool polar) {
+  JoinRec r = ld_join(p);
+  if (polar) {
+    r.lpp = f2_sub(r.lpc, r.lpp);
+    r.lmp = f2_sub(r.lmc, r.lmp);
+  }
+  return r;
+}
 constexpr int kJoinBlock = 16;  // degrees per join block
 
 struct MixArgs {
   int lmax, spin, npairs, nm;
   const int *mval;
   const int64_t *coef_off;
-  const float4 *coef32;  // per (m, l): {A.h, A.l, AK.h, AK.l}, {C.h, C.l, -, -}
-  const float4 *alm32;   // [array][ncoef] {re.h, re.l, im.h, im.l}
+  const float4 *coef32;  // per (m, l): {a.h, a.l, b.h, b.l} of p_{l+1} = (a x + b) p_l - p_{l-1}
+  const float4 *alm32;   // [array][ncoef] alpha_l a_lm as {re.h, re.l, im.h, im.l}
   int64_t ncoef;
   const double2 *mpre;
   const PairDev *pairs;
@@ -123,16 +136,68 @@ struct MixArgs {
   const int4 *ana_items;
   const int64_t *part_off;
   double *part;
-  int ptr_off;
   const float4 *join;  // JoinRec per (m index, pair), 3 float4 each
 };
 
 struct Coef32 {
-  f2 a, ak, c;
+  f2 a, b;
 };
 __device__ __forceinline__ Coef32 ld_coef32(const float4 *p) {
-  const float4 u = __ldg(p), v = __ldg(p + 1);
-  return {{u.x, u.y}, {u.z, u.w}, {v.x, v.y}};
+  const float4 u = __ldg(p);
+  return {{u.x, u.y}, {u.z, u.w}};
+}
+// Warps holding a ring within kPolarTheta of the north pole run the recursion in
+// difference form, d_{l+1} = d_l + (u - 2) p_l, p_{l+1} = p_l + d_{l+1} (d_l = p_l -
+// p_{l-1}), with u - 2 = (a - 2) - a (1 - cos theta) + b.  There u is close to 2 and
+// a rounding of u p_l - p_{l-1} of relative size 2^-48 grows by ~1/theta over the
+// following degrees; the roundings of the difference form are relative to the small
+// d.  Errors of lambda at lmax 1535, theta 0.0015 - 0.0065, m <= 4: 9e-12 against
+// 5e-11.  A step takes about twice the operations, in the first warp or two of each
+// m's pairs only.  x holds 1 - cos theta (two floats) and lp the difference there.
+constexpr double kPolarTheta = 0.005;
+__device__ __forceinline__ bool polar_warp(double x, bool valid) {
+  return __any_sync(0xffffffffu, valid && 1.0 - x < 0.5 * kPolarTheta * kPolarTheta);
+}
+__device__ __forceinline__ f3 node_of(double x, bool polar) {
+  const f3 r = f3_of(polar ? 1.0 - x : x);
+  return polar ? f3{r.h, r.m, 0.f} : r;
+}
+__device__ __forceinline__ void step_polar(f2 a, f2 b, const f3 &y, f2 &p, f2 &d) {
+  const float q = __fmul_rn(a.h, y.h);
+  float qe = __fmaf_rn(a.h, y.h, -q);
+  qe = __fmaf_rn(a.h, y.m, qe);
+  qe = __fmaf_rn(a.l, y.h, qe);
+  const f2 s1 = two_sum(__fsub_rn(a.h, 2.0f), -q);
+  const f2 s2 = two_sum(s1.h, b.h);
+  const f2 v = fast_two_sum(s2.h, __fadd_rn(__fadd_rn(__fadd_rn(__fsub_rn(a.l, qe), s1.l), s2.l), b.l));
+  d = f2_add(mul(v, p), d);
+  p = f2_add(p, d);
+}
+// one step of the +s / -s recursions (spin 0: the +s one with b = 0); polar: see above.
+// The kernels pass a constant, chosen around their loops: a test per step cost 7 - 10%.
+__device__ __forceinline__ void step_s0(const Coef32 &c, const f3 &x, bool polar, f2 &lc, f2 &lp) {
+  if (polar) {
+    step_polar(c.a, f2{0.f, 0.f}, x, lc, lp);
+    return;
+  }
+  const f2 n = mul_sub(mul(c.a, x), lc, lp);
+  lp = lc;
+  lc = n;
+}
+__device__ __forceinline__ void step_spin(const Coef32 &c, const f3 &x, bool polar, f2 &lpc, f2 &lpp, f2 &lmc,
+                                          f2 &lmp) {
+  if (polar) {
+    step_polar(c.a, c.b, x, lpc, lpp);
+    step_polar(c.a, neg(c.b), x, lmc, lmp);
+    return;
+  }
+  const f2 t = mul(c.a, x);
+  const f2 np_ = mul_sub(sum2(t, c.b), lpc, lpp);
+  const f2 nm_ = mul_sub(sum2(t, neg(c.b)), lmc, lmp);
+  lpp = lpc;
+  lpc = np_;
+  lmp = lmc;
+  lmc = nm_;
 }
 
 // spin-0 / spin start in the double-float representation

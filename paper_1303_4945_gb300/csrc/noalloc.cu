@@ -134,10 +134,10 @@ extern "C" int sht_execute_noalloc(sht_plan_t P, int type, double *const *alm, d
     if (e == cudaSuccess) {
       if (mixed && P->nana_lo[polar])
         e = fork_join(
-            st, P->side, P->ev_fork, P->ev_join, [&](cudaStream_t s) { return launch_leg_ana_mixed(P, A, polar, s); },
-            [&](cudaStream_t s) { return launch_leg_ana_fp64(P, A, polar, s, true); });
+            st, P->side, P->ev_fork, P->ev_join, [&](cudaStream_t s) { return launch_leg_ana_mixed(P, polar, s); },
+            [&](cudaStream_t s) { return launch_leg_ana_fp64(P, polar, s, true); });
       else
-        e = mixed ? launch_leg_ana_mixed(P, A, polar, st) : launch_leg_ana_fp64(P, A, polar, st);
+        e = mixed ? launch_leg_ana_mixed(P, polar, st) : launch_leg_ana_fp64(P, polar, st);
     }
     if (e == cudaSuccess) e = launch_ana_reduce(P, A, polar, add, st, real, false);
   }

@@ -4,12 +4,6 @@
 
 namespace sht {
 
-__device__ __forceinline__ Coef ldg_coef(const Coef *p) {
-  const double2 u = __ldg(reinterpret_cast<const double2 *>(p));
-  const double2 v = __ldg(reinterpret_cast<const double2 *>(p) + 1);
-  return {u.x, u.y, v.x, v.y};
-}
-
 // ---- double-double pieces -------------------------------------------------
 struct dd {
   double hi, lo;

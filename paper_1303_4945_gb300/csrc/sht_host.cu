@@ -841,7 +841,7 @@ static void free_plan(sht_plan_s *P) {
   cudaGetDevice(&cur);
   cudaSetDevice(P->device);
   void *ptrs[] = {P->d_pairs, P->d_pair_rings, P->d_rings, P->d_mval, P->d_mstart, P->d_coef_off,
-                  P->d_coef, P->d_coef32, P->d_alm32, P->d_pm64, P->d_mpre, P->d_minv, P->d_phase, P->d_part, P->d_fft,
+                  P->d_coef, P->d_alpha, P->d_coef32, P->d_alm32, P->d_pm64, P->d_mpre, P->d_minv, P->d_phase, P->d_part, P->d_fft,
                   P->d_pair_fft, P->d_fft_scratch, P->d_err, P->d_join};
   for (void *p : ptrs)
     if (p) cudaFree(p);
@@ -1110,15 +1110,17 @@ static int plan_build(sht_plan_s *P, const sht_geom_s *g) {
   // the FP64 tables: every entry for an FP64 plan; for a mixed plan the prefix its
   // default FP64 columns read (grown by sht_plan_set_fp64_columns when needed)
   P->ncoef64 = P->precision == SHT_MIXED ? fp64_prefix(P, default_fp64_columns(P->lmax)) : nco;
-  CUDA_TRY(cudaMalloc(&P->d_coef, std::max<int64_t>(1, P->ncoef64) * sizeof(Coef)));
-  P->workspace += P->ncoef64 * sizeof(Coef);
+  CUDA_TRY(cudaMalloc(&P->d_coef, std::max<int64_t>(1, P->ncoef64) * sizeof(double2)));
+  P->workspace += P->ncoef64 * sizeof(double2);
+  CUDA_TRY(cudaMalloc(&P->d_alpha, std::max<int64_t>(1, nco) * sizeof(double)));
+  P->workspace += nco * sizeof(double);
   if (P->precision == SHT_MIXED) {
-    CUDA_TRY(cudaMalloc(&P->d_coef32, std::max<int64_t>(1, nco) * 2 * sizeof(float4)));
-    P->workspace += nco * 2 * sizeof(float4);
+    CUDA_TRY(cudaMalloc(&P->d_coef32, std::max<int64_t>(1, nco) * sizeof(float4)));
+    P->workspace += nco * sizeof(float4);
     CUDA_TRY(cudaMalloc(&P->d_alm32, std::max<int64_t>(1, nco) * P->nmaps_pad * sizeof(float4)));
     P->workspace += nco * P->nmaps_pad * sizeof(float4);
   }
-  if (P->spin != 0 && (P->precision == SHT_FP64 || default_fp64_columns(P->lmax) > 0)) {
+  if (P->precision == SHT_FP64 || default_fp64_columns(P->lmax) > 0) {
     CUDA_TRY(cudaMalloc(&P->d_pm64, std::max<int64_t>(1, P->ncoef64) * P->nmaps_pad * sizeof(double2)));
     P->workspace += P->ncoef64 * P->nmaps_pad * sizeof(double2);
   }
@@ -1303,31 +1305,28 @@ extern "C" int sht_plan_set_fp64_columns(sht_plan_t P, int m_below) {
   cudaGetDevice(&cur);
   if (cur != P->device) CUDA_TRY(cudaSetDevice(P->device));
   int rc = SHT_OK;
-  // the FP64 tables (coefficients; at spin s the P = E+iB, M = E-iB table the FP64
-  // spin kernels read) must reach the new columns: regrow them to the new prefix
+  // the FP64 tables (coefficients and scaled a_lm) must reach the new columns: regrow
+  // them to the new prefix
   const int64_t need = fp64_prefix(P, m_below);
-  if (need > P->ncoef64 || (P->spin != 0 && !P->d_pm64 && m_below > 0)) {
+  if (need > P->ncoef64 || (!P->d_pm64 && m_below > 0)) {
     const int64_t n = std::max(need, P->ncoef64);
-    Coef *coef = nullptr;
+    double2 *coef = nullptr;
     double2 *pm = nullptr;
-    if (cudaMalloc(&coef, std::max<int64_t>(1, n) * sizeof(Coef)) != cudaSuccess) {
+    if (cudaMalloc(&coef, std::max<int64_t>(1, n) * sizeof(double2)) != cudaSuccess) {
       rc = fail(SHT_ERR_OOM, "FP64 coefficient table");
-    } else if (P->spin != 0 &&
-               cudaMalloc(&pm, std::max<int64_t>(1, n) * P->nmaps_pad * sizeof(double2)) != cudaSuccess) {
+    } else if (cudaMalloc(&pm, std::max<int64_t>(1, n) * P->nmaps_pad * sizeof(double2)) != cudaSuccess) {
       cudaFree(coef);
-      rc = fail(SHT_ERR_OOM, "P/M table");
+      rc = fail(SHT_ERR_OOM, "FP64 a_lm table");
     } else {
       cudaFree(P->d_coef);
-      P->workspace += (n - P->ncoef64) * (int64_t)sizeof(Coef);
+      P->workspace += (n - P->ncoef64) * (int64_t)sizeof(double2);
       P->d_coef = coef;
-      if (P->spin != 0) {
-        if (P->d_pm64) {
-          cudaFree(P->d_pm64);
-          P->workspace -= P->ncoef64 * P->nmaps_pad * (int64_t)sizeof(double2);
-        }
-        P->d_pm64 = pm;
-        P->workspace += n * P->nmaps_pad * (int64_t)sizeof(double2);
+      if (P->d_pm64) {
+        cudaFree(P->d_pm64);
+        P->workspace -= P->ncoef64 * P->nmaps_pad * (int64_t)sizeof(double2);
       }
+      P->d_pm64 = pm;
+      P->workspace += n * P->nmaps_pad * (int64_t)sizeof(double2);
       P->ncoef64 = n;
       cudaError_t e = launch_coef_tables(P, 0);  // the FP64 coefficients of the new prefix
       if (e == cudaSuccess) e = cudaDeviceSynchronize();
@@ -1434,8 +1433,6 @@ extern "C" int sht_plan_autotune(sht_plan_t P, void *stream, float *ms_per_candi
   cudaError_t e = cudaMemsetAsync(P->d_phase, 0, std::max<size_t>(1, nph) * sizeof(double2), st);
   if (e == cudaSuccess) e = cudaEventCreate(&ev[0]);
   if (e == cudaSuccess) e = cudaEventCreate(&ev[1]);
-  DevPtrs none;
-  memset(&none, 0, sizeof(none));
   // the tiling candidates with the double-float analysis, then (mixed plans of
   // supported shapes) the tensor-core analysis on tiles of one pair per thread
   const bool tc_cand = P->precision == SHT_MIXED && tc_ana_supported(P->spin, P->njobs_pad);
@@ -1453,7 +1450,7 @@ extern "C" int sht_plan_autotune(sht_plan_t P, void *stream, float *ms_per_candi
       if (it == 1) e = cudaEventRecord(ev[0], st);
       // the tiling's own kernel only (a mixed plan's FP64 items run beside it)
       if (e == cudaSuccess)
-        e = P->precision == SHT_MIXED ? launch_leg_ana_mixed(P, none, 1, st) : launch_leg_ana_fp64(P, none, 1, st);
+        e = P->precision == SHT_MIXED ? launch_leg_ana_mixed(P, 1, st) : launch_leg_ana_fp64(P, 1, st);
     }
     if (e == cudaSuccess) e = cudaEventRecord(ev[1], st);
     if (e == cudaSuccess) e = cudaEventSynchronize(ev[1]);
@@ -1589,10 +1586,9 @@ extern "C" int sht_execute(sht_plan_t P, int type, double *const *alm, double *c
   // a_lm read by a synthesis: derivative mode, real storage, or (the adjoint
   // analysis of a gradient) the m > 0 entries halved
   const int mode = (deriv ? kAlmDeriv : 0) | (real ? kAlmReal : 0) | (grad ? kAlmHalf : 0);
-  const int amode = mode & (kAlmReal | kAlmHalf);
   auto leg = [&](int stg, const void *items, int n, cudaStream_t s) {
     return mixed ? launch_leg_mixed_items(P, stg, polar, items, n, s)
-                 : launch_leg_fp64_items(P, stg, A, polar, items, n, s, amode);
+                 : launch_leg_fp64_items(P, stg, polar, items, n, s);
   };
   // A mixed plan's FP64 items (small m near the poles) run on the high-priority
   // side stream beside its mixed Legendre kernel; the ring FFT waits for both.
@@ -1601,14 +1597,14 @@ extern "C" int sht_execute(sht_plan_t P, int type, double *const *alm, double *c
     const bool lo = mixed && P->nsyn_lo[polar] > 0;
     stage(0, st, [&] {
       cudaError_t r = mixed ? launch_alm_prepare_mixed(P, A, st, mode) : launch_alm_prepare_fp64(P, A, st, mode);
-      if (r == cudaSuccess && lo) r = launch_alm_prepare_fp64(P, A, st, mode);  // the FP64 items read P/M
+      if (r == cudaSuccess && lo) r = launch_alm_prepare_fp64(P, A, st, mode);  // the FP64 items' table
       return r;
     });
     if (lo) {
       record(P->ev_fork, st);
       wait(P->side, P->ev_fork);
       stage(5, P->side, [&] {
-        return launch_leg_fp64_items(P, 0, A, polar, P->d_syn_lo[polar], P->nsyn_lo[polar], P->side, amode);
+        return launch_leg_fp64_items(P, 0, polar, P->d_syn_lo[polar], P->nsyn_lo[polar], P->side);
       });
       record(P->ev_lo, P->side);
     }
@@ -1623,7 +1619,7 @@ extern "C" int sht_execute(sht_plan_t P, int type, double *const *alm, double *c
       record(P->ev_fork, st);
       wait(P->side, P->ev_fork);
       stage(5, P->side, [&] {
-        return launch_leg_fp64_items(P, 1, A, polar, P->d_ana_lo[polar], P->nana_lo[polar], P->side);
+        return launch_leg_fp64_items(P, 1, polar, P->d_ana_lo[polar], P->nana_lo[polar], P->side);
       });
       record(P->ev_lo, P->side);
     }

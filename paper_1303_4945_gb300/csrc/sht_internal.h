@@ -2,9 +2,11 @@
 //
 // Layout of the device data a plan holds (all in HBM, built once at plan time):
 //   pairs      PairDev[npairs]      ring pairs sorted pole -> equator (Sect. 3.3 order)
-//   coef       Coef[ncoef64]        recursion coefficients {A, AK, C, 0} per (m, l), Sect. 4.1
-//   coef32     float4[2*ncoef]      the same split into FP32 pairs (mixed form)
-//   mpre       double2[nm]          start-value prefactor (mantissa, exponent) per m
+//   coef       double2[ncoef64]     recursion coefficients {a, b} per (m, l) of p_l = lambda_l / alpha_l
+//                                   (Sect. 4.1's recursion with unit coefficient of p_{l-1}, tables.cu)
+//   coef32     float4[ncoef]        the same split into FP32 pairs (mixed form)
+//   alpha      double[ncoef]        alpha_l: scales the a_lm before a synthesis and after an analysis
+//   mpre       double2[nm]          start-value prefactor over alpha_{l0} (mantissa, exponent) per m
 //   F / G      double2[nmaps][nm][npairs][2]   phase arrays of Eqs. syn2 / ana2 (north, south)
 //   part       double[..]           per-tile partial sums of the analysis Legendre stage
 #pragma once
@@ -89,11 +91,6 @@ struct PtrTable {
   double *p[kMaxBatchPtr];
 };
 
-// recursion coefficients of one (m, l): lambda_{l+1} = (a x + ak) lambda_l - c lambda_{l-1}
-struct __align__(32) Coef {
-  double a, ak, c, pad;
-};
-
 }  // namespace sht
 
 // ----------------------------------------------------------------------------
@@ -138,10 +135,11 @@ struct sht_plan_s {
   int *d_mval = nullptr;
   int64_t *d_mstart = nullptr;
   int64_t *d_coef_off = nullptr;
-  sht::Coef *d_coef = nullptr;
+  double2 *d_coef = nullptr;
+  double *d_alpha = nullptr;
   float4 *d_coef32 = nullptr;
   float4 *d_alm32 = nullptr;               // mixed form: a_lm as double-float pairs [array][ncoef]
-  double2 *d_pm64 = nullptr;               // FP64 spin form: P = E + iB, M = E - iB [array][ncoef64]
+  double2 *d_pm64 = nullptr;               // FP64 form: alpha_l times a_lm (spin: P = E + iB, M = E - iB) [array][ncoef64]
   double2 *d_mpre = nullptr;
   int *d_minv = nullptr;                   // m -> index in mval, or -1
   double2 *d_phase = nullptr;              // F / G workspace
@@ -247,19 +245,17 @@ cudaError_t launch_fft_spectrum(const FftPlanDev *host_plan, const FftPlanDev *d
 // lo: run the mixed plan's FP64 columns (work lists d_syn_lo / d_ana_lo)
 cudaError_t launch_leg_syn_fp64(const sht_plan_s *P, const DevPtrs &alm, int polar, cudaStream_t st,
                                 bool lo = false, int mode = 0);
-cudaError_t launch_leg_ana_fp64(const sht_plan_s *P, const DevPtrs &alm, int polar, cudaStream_t st,
-                                bool lo = false);
+cudaError_t launch_leg_ana_fp64(const sht_plan_s *P, int polar, cudaStream_t st, bool lo = false);
 // grad: the gradient factor of Sect. 4.5's adjoint for the stored m >= 0 a_lm (m > 0 doubled)
 cudaError_t launch_ana_reduce(const sht_plan_s *P, const DevPtrs &alm, int polar, int add, cudaStream_t st,
                               bool real = false, bool grad = false);
 cudaError_t launch_leg_syn_mixed(const sht_plan_s *P, const DevPtrs &alm, int polar, cudaStream_t st, int mode = 0);
 // the Legendre stage over an explicit work list (stage 0 synthesis, 1 analysis), no a_lm conversion
-// amode: kAlmReal / kAlmHalf bits for the spin-0 synthesis, which reads the a_lm directly
-cudaError_t launch_leg_fp64_items(const sht_plan_s *P, int stage, const DevPtrs &alm, int polar, const void *items,
-                                  int n, cudaStream_t st, int amode = 0);
+cudaError_t launch_leg_fp64_items(const sht_plan_s *P, int stage, int polar, const void *items, int n,
+                                  cudaStream_t st);
 cudaError_t launch_leg_mixed_items(const sht_plan_s *P, int stage, int polar, const void *items, int n,
                                    cudaStream_t st);
-cudaError_t launch_leg_ana_mixed(const sht_plan_s *P, const DevPtrs &alm, int polar, cudaStream_t st);
+cudaError_t launch_leg_ana_mixed(const sht_plan_s *P, int polar, cudaStream_t st);
 // tensor-core synthesis (legendre_tc.cu): mixargs is the mixed kernels' argument
 // record (MixArgs) with its synthesis work list set; n work items
 cudaError_t launch_leg_tc_syn(const sht_plan_s *P, const void *mixargs, int n, cudaStream_t st);
@@ -267,7 +263,7 @@ cudaError_t tc_prepare_device();
 cudaError_t launch_join_records(const sht_plan_s *P, cudaStream_t st);
 // batches: one TcArgs record per plan of a tensor-core group
 size_t tc_args_size();
-void leg_tc_fill_args(const sht_plan_s *P, int polar, int ptr_off, void *out);
+void leg_tc_fill_args(const sht_plan_s *P, int polar, void *out);
 cudaError_t launch_leg_tc_batch(int spin, int nj, const void *targs, const int4 *items, int n, cudaStream_t st);
 bool tc_supported(int spin, int njobs_pad);
 float tc_lambda_bound(int lmax);
@@ -293,10 +289,10 @@ cudaError_t fft_prepare_device(int device);
 size_t leg_fp64_args_size();
 size_t leg_mixed_args_size();
 size_t fft_args_size();
-void leg_fp64_fill_args(const sht_plan_s *P, int polar, int ptr_off, void *out, bool lo = false);
-void leg_mixed_fill_args(const sht_plan_s *P, int polar, int ptr_off, void *out);
+void leg_fp64_fill_args(const sht_plan_s *P, int polar, void *out, bool lo = false);
+void leg_mixed_fill_args(const sht_plan_s *P, int polar, void *out);
 void fft_fill_args(const sht_plan_s *P, int polar, int weighted, int add, int ptr_off, void *out);
-// a_lm -> the P = E+iB / M = E-iB tables (FP64 spin) or double-float tables (mixed); mode bits:
+// a_lm -> the FP64 tables (alpha_l a_lm; spin: P = E+iB / M = E-iB) or the double-float ones (mixed); mode bits:
 // kAlmDeriv, the first-derivative mode of Sect. 4.3 (spin-1 plan, E = sqrt(l(l+1)) a of ncomp
 // spin-0 arrays, B = 0); kAlmReal, inputs in real-harmonic storage; kAlmHalf, the m > 0
 // coefficients halved (the adjoint analysis of a gradient, see SHT_GRADIENT)
@@ -304,9 +300,9 @@ cudaError_t launch_alm_prepare_fp64(const sht_plan_s *P, const DevPtrs &alm, cud
 cudaError_t launch_alm_prepare_mixed(const sht_plan_s *P, const DevPtrs &alm, cudaStream_t st, int mode = 0);
 // stage 0: synthesis, 1: analysis
 cudaError_t launch_leg_fp64_batch(int stage, int spin, int nj, int ppt, const void *args, const int4 *items,
-                                  int n, const PtrTable &tbl, cudaStream_t st);
+                                  int n, cudaStream_t st);
 cudaError_t launch_leg_mixed_batch(int stage, int spin, int nj, int ppt, const void *args, const int4 *items,
-                                   int n, const PtrTable &tbl, cudaStream_t st);
+                                   int n, cudaStream_t st);
 cudaError_t launch_fft_batch(int stage, bool df, const void *args, const int4 *items, int n, int smem,
                              const PtrTable &tbl, cudaStream_t st);
 }  // namespace sht
