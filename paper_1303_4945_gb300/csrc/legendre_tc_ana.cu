@@ -19,37 +19,42 @@
 //    power of two above column c's largest |G'| over the tile.
 //  * Every product Gj Li is a multiple of v_c 2^(-14-8(i+j)); a digit is at most
 //    128 of its quanta (192 for digit 3, which takes the low word), so a sum over
-//    the tile's K = 128 or 256 pair entries stays below 256 * 192^2 < 2^24 quanta
-//    and the FP32 accumulation is exact whatever its order.
+//    K = 512 entries stays below 512 * 192 * 128 < 2^24 quanta (of 512 * 192^2 for the
+//    product of two digits 3, level 6, only its rounding below 2^-70 could depend on
+//    the order) and the FP32 accumulation is exact whatever its order.
 //
-// One MMA per 16 pair entries: M = 64 rows (column c's six G digits and two zero
-// rows at rows 8c .. 8c + 7), N = 48 (the six Lambda digits of 8 degrees), so D
-// holds every digit product G_j L_i of a column and degree, each an exact sum; the
-// products with i + j <= 2 are added in double-float, those with 3 <= i + j <= 6 in
-// FP32 (below 2^-24 of the sum), the rest dropped (below 2^-56).  Measured at spin
-// 2, lmax 4095 on GB300 (double-float analysis 76.5 ms): three MMAs of N = 16 per 16
-// entries whose A row shifts summed the levels on the tensor cores, 92 ms (each
-// read 4 KB of A from shared memory); one MMA of N = 48 at M = 128, 86 ms; M = 64
-// and waits that suspend the waiting warp, 80 ms; no per-degree negligibility vote
-// (the join records cover it), 73.8 ms.
+// One MMA per 16 entries: M = 64 rows (a column's six G digits and two zero rows
+// together), N = 48 (the six Lambda digits of 8 degrees), so D holds every digit
+// product G_j L_i of a column and degree, each an exact sum; the products with i + j
+// <= 2 are added in double-float, those with 3 <= i + j <= 6 in FP32 (below 2^-24 of
+// the sum), the rest dropped (below 2^-56).
 //
-// Each warp owns the K entries of its 32 pairs: it writes their Lambda digits and
-// issues their MMAs itself (lane 0), with no CTA barrier per block.  Two TMEM
-// accumulators of 48 columns alternate between blocks of 8 degrees; mbarriers
-// order the steps: a warp's own commits free its Lambda tiles, every warp's
-// commit (or plain arrival for a warp with no joined pair) fills an accumulator,
-// and the warps holding its rows (M = 64 puts D row r in TMEM lane 32 (r / 16) +
-// r % 16: warp w holds columns 2w and 2w + 1) release it after reading and zeroing
-// it.  Every
-// wait is bounded; a wait that gives up flags the plan's status word and stops the
-// CTA.
+// Each warp owns the K entries of its 32 threads: it writes their Lambda digits and
+// issues their MMAs itself, with no CTA barrier per block.  TMEM accumulators of 48
+// columns rotate between blocks of 8 degrees; mbarriers order the steps: a warp's own
+// commits free its Lambda tiles, every warp's commit (or plain arrival for a warp with
+// no joined pair) fills an accumulator, and the warps whose turn it is read its rows,
+// zero and release it.  Every wait is bounded; a wait that gives up flags the plan's
+// status word and stops the CTA.
+//
+// What bounds it (GB300, spin 2, lmax 4095): issue slots and dependency latency on the
+// CUDA cores (59% issue, FP32 pipe 48%, tensor pipe 25% at 16 warps per SM).  With
+// parts left out: recursion and digits 37 ms, MMA issue 3.5, accumulator reads 7.5 (of
+// which 6 are warps waiting for one another, 1.2 the TMEM loads), level sums 3.2.
+// History: scalar recursions with three coefficients, 128 threads per CTA, every wait
+// reading the clock, MMAs issued through a divergent lane 73.9 ms; unit-coefficient
+// recursion 65; both recursions as packed lanes 55.7; 256 threads, four accumulators
+// read in turn by two groups 57.0; waits that try once before reading the clock and
+// MMAs from an elected lane with uniform descriptors 53.5; the block's two halves
+// unrolled 51.4.  Coefficients staged in shared memory (56.7 against 55.7) and pairs
+// interleaved over the warps (54.4 against 51.4) were slower.
+#include "dual.cuh"
 #include "tcgen05.cuh"
 
 namespace sht {
 namespace tca {
 
-constexpr int kPairs = 128;      // ring pairs per CTA = threads
-constexpr int kWarps = kPairs / 32;
+constexpr int kTile = 128;       // ring pairs per tile of the work lists
 constexpr int kBlk = 8;          // degrees per block
 constexpr int kDig = 6;          // digits of Lambda / u_p and of G'
 constexpr int kN = kDig * kBlk;  // MMA N: every Lambda digit of the block's degrees
@@ -57,42 +62,61 @@ constexpr int kColRows = 8;      // A rows per column: its six G digits, two zer
 constexpr int kDCols = 64;       // TMEM columns per accumulator (kN used)
 constexpr int kM = 64;           // MMA M: the columns' digit rows
 constexpr int kEStride = kN + 4; // floats per staged D row (rows 16 bytes off the banks of the next)
-constexpr int kKStride = 144;    // bytes between 8-pair K-groups of the Lambda tiles (stores without bank conflicts)
+constexpr int kKStride = 144;    // bytes between 8-pair K-groups of the Lambda tiles
 
 // Columns per job j: 4j + {0, 1} and 4j + {2, 3} (re, im of the two sums the
-// kernel below describes); K entries 0..127 hold the pairs' +s (or spin-0) values,
-// 128..255 the -s values times (-1)^(l - l0).  Column c's six G digit rows and
-// two zero rows make 8 rows of A and of D.
+// kernel below describes).  A thread runs the two recursions of Dual; its value of
+// lane t is K entry t TH + tid.  Column c's six G digit rows and two zero rows make 8
+// rows of A and of D.
+//
+// One job: 256 threads, four accumulators, one column in each TMEM quarter.  Reading
+// an accumulator back (waits, loads, zeroing, the sum over the digit products) costs a
+// warp about 75 instructions for 8 degrees whatever K is, so twice the pairs per CTA
+// halve it, and each group of four warps reads every second block, one column a warp,
+// two blocks after its products were issued.  (128 threads, two accumulators, both
+// columns of a quarter read by warps 0 and 1, which share their SM quarters with those
+// of the other CTAs: 55.7 ms at spin 2, lmax 4095.)  Two jobs take twice the A digits:
+// 128 threads, two columns a quarter, every warp reads every block.
 template <int NJ, bool SPIN>
 struct AnaShape {
-  static constexpr int NSET = SPIN ? 2 : 1;
+  static constexpr int TH = NJ == 1 ? 256 : 128;
+  static constexpr int WARPS = TH / 32;
+  static constexpr int NP = SPIN ? 1 : 2;                // ring pairs per thread
+  static constexpr int TILES = NP * TH / kTile;          // tiles walked at a time
+  static constexpr int NACC = NJ == 1 ? 4 : 2;           // accumulators
+  static constexpr int GROUPS = WARPS / 4;               // groups of reading warps (block ib: group ib % GROUPS)
+  static constexpr int LAG = NJ == 1 ? 2 : 1;            // blocks between issuing and reading (a multiple of GROUPS)
+  static constexpr int NSET = 2;
   static constexpr int NC = 4 * NJ;
-  static constexpr int KG = NSET * kPairs / 8;  // 8-entry K-groups
-  // MMA M = 64: D row r lands in TMEM lane 32 (r / 16) + r % 16 (measured).
-  // Column c's rows are A and D rows 8c .. 8c + 7, so warp w holds columns 2w and
-  // 2w + 1 in lanes 0 .. 15; the rows of one K-group are contiguous (SBO = 128,
-  // LBO = the rows' bytes).
-  static constexpr int NREAD = NC / 2;        // warps holding D rows
+  static constexpr int CPW = NC / 4;                     // columns per TMEM quarter
+  static constexpr int KG = NSET * TH / 8;               // 8-entry K-groups
+  // MMA M = 64: D row r lands in TMEM lane 32 (r / 16) + r % 16 (measured): warp w
+  // reads quarter w % 4, its columns' rows in lanes 0 .. 8 CPW - 1.  The rows of one
+  // K-group are contiguous.  One column a quarter: 8-row groups 64 bytes apart put
+  // column c in row group 2c (the odd groups overlap two columns; no one reads them).
   static constexpr int A_LBO = NC * kColRows * 16;  // bytes between K-groups
-  static constexpr int A_SBO = 128;                 // bytes between 8-row groups
+  static constexpr int A_SBO = CPW == 1 ? 64 : 128; // bytes between 8-row groups
   static constexpr int A_BYTES = KG * A_LBO;
   // byte offset of (column c, digit row j, K-group h)
   __host__ __device__ static constexpr int a_at(int c, int j, int h) { return h * A_LBO + (kColRows * c + j) * 16; }
   static constexpr int B_SBO = KG * kKStride;  // bytes between the 8-degree N-groups (one per digit)
   static constexpr int B_BYTES = kDig * B_SBO;
-  static constexpr int EROWS = 2 * kColRows;  // staged D rows per reading warp: lanes 0 .. 15
-  static constexpr int E_BYTES = NREAD * EROWS * kEStride * 4;
+  static constexpr int EROWS = CPW * kColRows;  // staged D rows per warp: lanes 0 .. EROWS - 1
+  static constexpr int E_BYTES = WARPS * EROWS * kEStride * 4;
   static constexpr int SMEM = A_BYTES + B_BYTES + E_BYTES;
-  // at most 512 / 128 CTAs per SM, so that their TMEM allocations never wait
-  static constexpr int SMEM_FLOOR = (228 * 1024) / 5 - 1024 + 1;
+  static constexpr int TCOLS = NACC * kDCols;
+  // at most 512 / TCOLS CTAs per SM, so that their TMEM allocations never wait
+  static constexpr int SMEM_FLOOR = (228 * 1024) / (512 / TCOLS + 1) - 1024 + 1;
   static constexpr int SMEM_LAUNCH = SMEM > SMEM_FLOOR ? SMEM : SMEM_FLOOR;
   static constexpr int V = (SPIN ? 4 : 2) * NJ;  // partial sums per degree
-  static constexpr int MINB = SMEM_LAUNCH <= 57 * 1024 ? 4 : (SMEM_LAUNCH <= 75 * 1024 ? 3 : 2);
-  static_assert(kColRows * NC <= kM && NREAD <= kWarps, "columns within the MMA's rows");
-  // the MMA reads kM rows of two K-groups from a K-step's base: from the last
+  static constexpr int MINB = NJ == 1 ? 2 : 3;
+  static_assert(kColRows * NC <= kM && CPW <= 2, "columns within the MMA's rows");
+  static_assert(LAG % GROUPS == 0 && LAG < NACC, "a group reads the blocks it holds the turn of");
+  // the MMA reads 8 row groups of two K-groups from a K-step's base: from the last
   // one's, inside A and the B tiles that follow it
-  static_assert((KG - 1) * A_LBO + kM * 16 <= A_BYTES + B_BYTES, "A operand inside shared memory");
+  static_assert((KG - 1) * A_LBO + 7 * A_SBO + 128 <= A_BYTES + B_BYTES, "A operand inside shared memory");
   static_assert(A_BYTES % 16 == 0 && B_SBO % 16 == 0, "descriptor alignment");
+  static_assert(MINB * (SMEM_LAUNCH + 2048) <= 228 * 1024, "CTAs per SM");
 };
 
 // six digits of x on the grid whose first quantum has the magic constant s0
@@ -114,27 +138,48 @@ __device__ __forceinline__ void split6(f2 x, float s0, float (&d)[kDig]) {
   d[5] = tc::round_to(r, s0 * 0x1p-40f);
 }
 
+// the same of two values (quanta 2^-7, 2^-15, ...)
+__device__ __forceinline__ void split6(float2 h, float2 l, float2 (&d)[kDig]) {
+  constexpr float s0 = 98304.0f;  // 1.5 * 2^23 * 2^-7
+  auto round2 = [](float2 r, float s) { return add2(add2(r, both(s)), both(-s)); };
+  float2 r = h;
+  d[0] = round2(r, s0);
+  r = sub2(r, d[0]);
+  d[1] = round2(r, s0 * 0x1p-8f);
+  r = sub2(r, d[1]);
+  d[2] = round2(r, s0 * 0x1p-16f);
+  r = add2(sub2(r, d[2]), l);
+  d[3] = round2(r, s0 * 0x1p-24f);
+  r = sub2(r, d[3]);
+  d[4] = round2(r, s0 * 0x1p-32f);
+  r = sub2(r, d[4]);
+  d[5] = round2(r, s0 * 0x1p-40f);
+}
+
 }  // namespace tca
 
 // ---------------------------------------------------------------------------
-// Columns' K entries per ring pair (mixed analysis naming: W+_N, W-_N the north
-// ring's spin combinations, W+_S', W-_S' the south ring's times (-1)^(l0 + m)):
-// spin, T1 = sum l+ W+_N + s l- W+_S' and s T2 = sum l+ W-_S' + s l- W-_N with
-// s = (-1)^(l - l0), so the K entries are the +s values and the -s values times s,
-// and T2 is s times its row; spin 0, the even-l sum over G_N + G_S and the odd-l
-// sum over G_N - G_S.
+// Columns' K entries (mixed analysis naming: W+_N, W-_N the north ring's spin
+// combinations, W+_S', W-_S' the south ring's times (-1)^(l0 + m)): spin, T1 = sum l+
+// W+_N + s l- W+_S' and s T2 = sum l+ W-_S' + s l- W-_N with s = (-1)^(l - l0), so the K
+// entries are the +s values and the -s values times s (the two lanes of Dual), and T2
+// is s times its row; spin 0, the even-l sum over G_N + G_S and the odd-l sum over
+// G_N - G_S, the two lanes two neighbouring pairs.
 // ---------------------------------------------------------------------------
 template <int NJ, bool SPIN>
 __device__ __forceinline__ void tc_ana_body(const TcArgs &ta, const int4 item, unsigned char *tca_smem) {
   using S = tca::AnaShape<NJ, SPIN>;
-  constexpr int NSET = S::NSET, NC = S::NC, V = S::V, kDig = tca::kDig;
-  __shared__ __align__(8) uint64_t full[2], freeb[2], mine[tca::kWarps];
+  constexpr int NSET = S::NSET, NC = S::NC, V = S::V, kDig = tca::kDig, TH = S::TH, NP = S::NP;
+  constexpr int NACC = S::NACC, GROUPS = S::GROUPS, LAG = S::LAG;
+  __shared__ __align__(8) uint64_t full[NACC], freeb[NACC], mine[S::WARPS];
   __shared__ uint32_t tslot;
   __shared__ unsigned vmax[NC];
-  __shared__ int tstart[tca::kWarps];
+  __shared__ int tstart[S::WARPS];
   __shared__ volatile int stop;
   const MixArgs &a = ta.m;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  // the warp's number from a shuffle: the compiler sees it uniform, and so the MMAs'
+  // descriptors, which then live in uniform registers
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   const int mi = item.x, ng = item.z & 255;
   const int m = a.mval[mi];
   const int s = a.spin, as = s < 0 ? -s : s;
@@ -144,31 +189,33 @@ __device__ __forceinline__ void tc_ana_body(const TcArgs &ta, const int4 item, u
   const double sg0 = ((l0 + m) & 1) ? -1.0 : 1.0;
   unsigned char *const Abuf = tca_smem;
   unsigned char *const Bbuf = tca_smem + S::A_BYTES;
-  // a reading warp's staged D rows (kN columns each; the other warps never use theirs)
-  float *const Ebuf =
-      reinterpret_cast<float *>(tca_smem + S::A_BYTES + S::B_BYTES) + (warp % S::NREAD) * S::EROWS * tca::kEStride;
+  // this warp's staged D rows (kN columns each)
+  float *const Ebuf = reinterpret_cast<float *>(tca_smem + S::A_BYTES + S::B_BYTES) + warp * S::EROWS * tca::kEStride;
 
-  if (warp == 0) tc::tmem_alloc(&tslot, 2 * tca::kDCols);
+  if (warp == 0) tc::tmem_alloc(&tslot, S::TCOLS);
   if (tid == 0) {
-    tc::bar_init(&full[0], tca::kWarps);
-    tc::bar_init(&full[1], tca::kWarps);
-    tc::bar_init(&freeb[0], S::NREAD);  // the warps holding D rows read and release it
-    tc::bar_init(&freeb[1], S::NREAD);
 #pragma unroll
-    for (int w = 0; w < tca::kWarps; ++w) tc::bar_init(&mine[w], 1);
+    for (int x = 0; x < NACC; ++x) {
+      tc::bar_init(&full[x], S::WARPS);
+      tc::bar_init(&freeb[x], 4);  // the warps of one group read and release it
+    }
+#pragma unroll
+    for (int w = 0; w < S::WARPS; ++w) tc::bar_init(&mine[w], 1);
     stop = 0;
   }
   // A starts at zero: rows 6 and 7 of each column (below its six digits) stay so
-  for (int i = tid; i < S::A_BYTES / 16; i += tca::kPairs) reinterpret_cast<uint4 *>(Abuf)[i] = make_uint4(0, 0, 0, 0);
+  for (int i = tid; i < S::A_BYTES / 16; i += TH) reinterpret_cast<uint4 *>(Abuf)[i] = make_uint4(0, 0, 0, 0);
   tc::fence_before();
   __syncthreads();
   tc::fence_after();
   const uint32_t tbase = tslot;
-  const uint32_t tlane = tbase + ((uint32_t)(warp * 32) << 16);
-  // both accumulators start at zero (ordered before any MMA by the tile's barriers)
-  if (warp < S::NREAD) {
+  const uint32_t tlane = tbase + ((uint32_t)((warp & 3) * 32) << 16);
+  // the accumulators start at zero (ordered before any MMA by the tile's barriers)
+  if (warp < 4) {
 #pragma unroll
-    for (int q = 0; q < 2 * tca::kN / 16; ++q) tc::tmem_zero16(tlane + (q / 3) * tca::kDCols + (q % 3) * 16);
+    for (int x = 0; x < NACC; ++x)
+#pragma unroll
+      for (int q = 0; q < tca::kN / 16; ++q) tc::tmem_zero16(tlane + x * tca::kDCols + q * 16);
     tc::tmem_wait_st();
   }
   tc::fence_before();
@@ -177,11 +224,12 @@ __device__ __forceinline__ void tc_ana_body(const TcArgs &ta, const int4 item, u
   const uint64_t bdesc0 = tc::mat_desc(tc::smem_u32(Bbuf), tca::kKStride, S::B_SBO);
   constexpr uint32_t idesc = tc::instr_desc(tca::kM, tca::kN, true);
 
-  int ib = 0;                    // blocks walked by the CTA over all its tiles: accumulator ib & 1
+  int ib = 0;                    // blocks walked by the CTA over all its tiles: accumulator ib % NACC
   int nmine = 0, nmine_done = 0;  // this warp's commits to mine[warp], and those waited for
   bool ok = true;
   // a bounded wait of the whole warp (false for every lane if any lane gave up)
-  auto wait_warp = [&](uint64_t *bar, uint32_t parity) {
+  auto wait_warp = [&](uint64_t *bar, uint32_t parity) -> bool {
+    if (__all_sync(0xffffffffu, tc::bar_try(bar, parity))) return true;  // mostly: no clock read
     const bool r = tc::bar_wait_or(bar, parity, &stop);
     return __all_sync(0xffffffffu, r);
   };
@@ -189,39 +237,50 @@ __device__ __forceinline__ void tc_ana_body(const TcArgs &ta, const int4 item, u
     if (lane == 0) stop = 1;
     ok = false;
   };
-  auto wfac = [](int sc) { return sc == 0 ? 1.f : (sc == -1 ? kScaleFactor32 : 0.f); };
 
+  // a thread's ring pairs: one (spin), or two neighbours (spin 0: they join at about
+  // the same degree; pairs TH apart took 28.6 ms at lmax 4095, neighbours 27.2)
 #pragma unroll 1
-  for (int gi = 0; gi < ng; ++gi) {
-    const int tile = item.y + gi;
-    const int p = tile * tca::kPairs + tid;
-    const bool valid = p < a.npairs;
-    const float4 *jrec = a.join + ((size_t)mi * a.npairs + (valid ? p : 0)) * 3;
-    int lj = lmax + 1, lexp = 0;
-    if (valid) {
-      const float4 c = __ldg(jrec + 2);
-      lj = __float_as_int(c.z);
-      lexp = __float_as_int(c.w);
+  for (int gi = 0; gi < ng; gi += S::TILES) {
+    int pr[NP], lj[NP], lexp[NP];
+    bool valid[NP];
+    const float4 *jrec[NP];
+#pragma unroll
+    for (int t = 0; t < NP; ++t) {
+      pr[t] = (item.y + gi) * tca::kTile + NP * tid + t;
+      valid[t] = pr[t] < min(a.npairs, (item.y + ng) * tca::kTile);
+      jrec[t] = a.join + ((size_t)mi * a.npairs + (valid[t] ? pr[t] : 0)) * 3;
+      lj[t] = lmax + 1;
+      lexp[t] = 0;
+      if (valid[t]) {
+        const float4 c = __ldg(jrec[t] + 2);
+        lj[t] = __float_as_int(c.z);
+        lexp[t] = __float_as_int(c.w);
+      }
     }
-    // this pair's K entries of every column, times its Lambda bound u_p = 2^lexp
+    const int jmin = min(lj[0], lj[NP - 1]);
+    // the K entries of every column, times the pairs' Lambda bounds u_p = 2^lexp
     // (zero for a pair that never joins)
     double gv[NSET][NC];
 #pragma unroll
     for (int t = 0; t < NSET; ++t)
 #pragma unroll
       for (int c = 0; c < NC; ++c) gv[t][c] = 0.0;
-    if (valid && lj <= lmax) {
-      const double u = ldexp(1.0, lexp);
+#pragma unroll
+    for (int t = 0; t < NP; ++t) {
+      if (!valid[t] || lj[t] > lmax) continue;
+      const int p = pr[t];
+      const double u = ldexp(1.0, lexp[t]);
       const bool south = a.pairs[p].south;
 #pragma unroll
       for (int j = 0; j < NJ; ++j) {
         if (!SPIN) {
           const double2 *gp = a.phase + (((size_t)j * a.nm + mi) * a.npairs + p) * 2;
           const double2 gn = gp[0], gs = south ? gp[1] : make_double2(0.0, 0.0);
-          gv[0][4 * j + 0] = u * (gn.x + gs.x);
-          gv[0][4 * j + 1] = u * (gn.y + gs.y);
-          gv[0][4 * j + 2] = u * (gn.x - gs.x);
-          gv[0][4 * j + 3] = u * (gn.y - gs.y);
+          gv[t][4 * j + 0] = u * (gn.x + gs.x);
+          gv[t][4 * j + 1] = u * (gn.y + gs.y);
+          gv[t][4 * j + 2] = u * (gn.x - gs.x);
+          gv[t][4 * j + 3] = u * (gn.y - gs.y);
         } else {
           const double2 *gq = a.phase + (((size_t)(2 * j) * a.nm + mi) * a.npairs + p) * 2;
           const double2 *gu = a.phase + (((size_t)(2 * j + 1) * a.nm + mi) * a.npairs + p) * 2;
@@ -250,7 +309,7 @@ __device__ __forceinline__ void tc_ana_body(const TcArgs &ta, const int4 item, u
     }
     if (tid < NC) vmax[tid] = 0u;
     {
-      const int wmin = __reduce_min_sync(0xffffffffu, lj);
+      const int wmin = __reduce_min_sync(0xffffffffu, jmin);
       if (lane == 0) tstart[warp] = wmin;
     }
     __syncthreads();
@@ -265,7 +324,7 @@ __device__ __forceinline__ void tc_ana_body(const TcArgs &ta, const int4 item, u
     __syncthreads();
     int lstart = tstart[0];
 #pragma unroll
-    for (int w = 1; w < tca::kWarps; ++w) lstart = min(lstart, tstart[w]);
+    for (int w = 1; w < S::WARPS; ++w) lstart = min(lstart, tstart[w]);
     // the G' digits of this pair into A: column c's digit j at its row j of the
     // pair's K-group, entry tid % 8 (rows 6 and 7 stay zero)
 #pragma unroll
@@ -275,76 +334,77 @@ __device__ __forceinline__ void tc_ana_body(const TcArgs &ta, const int4 item, u
       for (int t = 0; t < NSET; ++t) {
         float d[kDig];
         tca::split6(f2_of(gv[t][c]), s0, d);
-        unsigned char *dst = Abuf + S::a_at(c, 0, t * (tca::kPairs / 8) + tid / 8) + (tid % 8) * 2;
+        unsigned char *dst = Abuf + S::a_at(c, 0, t * (TH / 8) + tid / 8) + (tid % 8) * 2;
 #pragma unroll
         for (int j = 0; j < kDig; ++j) *reinterpret_cast<uint16_t *>(dst + j * 16) = tc::bf16_of(d[j]);
       }
     }
     if (gi == 0)  // the slot's degrees before the tile's first block (later tiles add to them)
-      for (int i = tid; i < (min(lstart, lmax + 1) - l0) * V; i += tca::kPairs) outp[i] = 0.0;
+      for (int i = tid; i < (min(lstart, lmax + 1) - l0) * V; i += TH) outp[i] = 0.0;
     tc::fence_async_smem();
     __syncthreads();
     if (lstart > lmax) continue;
 
-    // the walk over the tile's blocks of 8 degrees (from its pairs' earliest join)
-    const double xd = valid ? a.pairs[p].x : 0.0;
-    const bool polar = polar_warp(xd, valid);
-    const f3 x = node_of(xd, polar);
-    f2 lpc = {0.f, 0.f}, lmc = {0.f, 0.f}, lpp = {0.f, 0.f}, lmp = {0.f, 0.f};
-    int scp = 0, scm = 0;
-    const float ulx = __int_as_float((127 - lexp) << 23);  // 1 / u_p
-    float wfp = 0.f, wfm = 0.f;  // weight of the +s / -s values over u_p (zero until the pair joins)
-    bool settled = false;        // every lane of the warp at scale 0 (warp-uniform)
+    // the walk over the tile's blocks of 8 degrees (from its pairs' earliest join):
+    // the recursions run on Lambda / u_p
+    Dual<SPIN> rec;
+    rec.p = rec.q = d2{both(0.f), both(0.f)};
+    int sc0 = 0, sc1 = 0;
+    double xd[NP];
+    bool near = false;
+#pragma unroll
+    for (int t = 0; t < NP; ++t) {
+      xd[t] = valid[t] ? a.pairs[pr[t]].x : 0.0;
+      near = near || (valid[t] && 1.0 - xd[t] < 0.5 * kPolarTheta * kPolarTheta);
+    }
+    const bool polar = __any_sync(0xffffffffu, near);
+#pragma unroll
+    for (int t = 0; t < NP; ++t) rec.x[t] = node_of(xd[t], polar);
+    const int lfast = SPIN ? fast_from(as, rec.x[0].h, valid[0], lmax) : 0;
+    float2 wf = both(0.f);  // weights of the two lanes' values (zero until they join)
+    bool settled = false;   // every lane of the warp at scale 0 (warp-uniform)
 
-    // 4 degrees from lb4 (lb4 - l0 even): digits of l+ / u_p and s l- / u_p packed per
-    // pair of degrees into pk[set][digit][q / 2]; recursion advanced.  (Values of a
-    // joined pair are not tested for negligibility: the join record already skips
-    // the stretch before its first non-negligible degree pair, and later values
-    // below the digits' grid give zero digits.)
-    auto part = [&](const bool pol, int lb4, uint32_t (&pk)[NSET][kDig][2]) {
-      float hold[NSET][kDig];
+    // 4 degrees from lb4 (lb4 - l0 even): the digits packed per pair of degrees into
+    // pk[set][digit][q / 2]; recursion advanced.  (Values of a joined pair are not
+    // tested for negligibility: the join record already skips the stretch before its
+    // first non-negligible degree pair, and later values below the digits' grid give
+    // zero digits.)  kFast: settled, weights 1.
+    auto part = [&](const StepMode mode, int lb4, uint32_t (&pk)[NSET][kDig][2]) __attribute__((always_inline)) {
+      float2 hold[kDig];
+      float4 cv[4];
+      // past lmax the entries of the next m (or the table's zero tail) give finite
+      // values no output reads
+#pragma unroll
+      for (int q = 0; q < 4; ++q) cv[q] = __ldg(cf + lb4 + q);
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        const int l = lb4 + q;
         const bool odd = q & 1;
-        float d[NSET][kDig];
-        tca::split6(f2{lpc.h * wfp, lpc.l * wfp}, 98304.0f, d[0]);
-        if (SPIN) {
-          const float f = odd ? -wfm : wfm;
-          tca::split6(f2{lmc.h * f, lmc.l * f}, 98304.0f, d[NSET - 1]);
+        float2 d[kDig];
+        if (mode == kFast) {
+          tca::split6(rec.p.h, rec.p.l, d);
+        } else {
+          const float2 f = make_float2(wf.x, (SPIN && mode == kPolar && odd) ? -wf.y : wf.y);
+          tca::split6(mul2(rec.p.h, f), mul2(rec.p.l, f), d);
         }
 #pragma unroll
-        for (int t = 0; t < NSET; ++t)
-#pragma unroll
-          for (int i = 0; i < kDig; ++i) {
-            if (!odd) hold[t][i] = d[t][i];
-            else pk[t][i][q >> 1] = tc::pack_bf16(hold[t][i], d[t][i]);
+        for (int i = 0; i < kDig; ++i) {
+          if (!odd) {
+            hold[i] = d[i];
+          } else {
+            pk[0][i][q >> 1] = tc::pack_bf16(hold[i].x, d[i].x);
+            pk[1][i][q >> 1] = tc::pack_bf16(hold[i].y, d[i].y);
           }
-        // recursion to l + 1 (past lmax the coefficients of lmax stand in: finite
-        // values no output reads)
-        const Coef32 cc = ld_coef32(cf + (l <= lmax ? l : lmax));
-        if (SPIN) step_spin(cc, x, pol, lpc, lpp, lmc, lmp);
-        else step_s0(cc, x, pol, lpc, lpp);
+        }
+        rec.step(mode, cv[q]);
       }
     };
     // the enhanced exponent's check after every block of 8 degrees (see mixed_common.cuh)
     auto rescale = [&]() {
       if (settled) return;
-      if (scp < 0 && fabsf(lpc.h) > kScaleUp32) {
-        lpc = {lpc.h * kScaleFactor32, lpc.l * kScaleFactor32};
-        lpp = {lpp.h * kScaleFactor32, lpp.l * kScaleFactor32};
-        ++scp;
-      }
-      if (SPIN && scm < 0 && fabsf(lmc.h) > kScaleUp32) {
-        lmc = {lmc.h * kScaleFactor32, lmc.l * kScaleFactor32};
-        lmp = {lmp.h * kScaleFactor32, lmp.l * kScaleFactor32};
-        ++scm;
-      }
-      if (lj <= lmax) {
-        wfp = wfac(scp) * ulx;
-        wfm = wfac(scm) * ulx;
-      }
-      settled = __all_sync(0xffffffffu, scp == 0 && scm == 0);
+      rec.rescale(sc0, sc1);
+      if (lj[0] <= lmax) wf.x = scale_weight(sc0);
+      if (lj[NP - 1] <= lmax) wf.y = scale_weight(sc1);
+      settled = __all_sync(0xffffffffu, sc0 == 0 && sc1 == 0);
     };
     // this warp's digits of degrees 4h .. 4h + 3 of the block: entry tid % 8 of K-group
     // (set, tid / 8), N-group = digit, bytes 8h .. 8h + 7 of the 16-byte row
@@ -353,7 +413,7 @@ __device__ __forceinline__ void tc_ana_body(const TcArgs &ta, const int4 item, u
       for (int t = 0; t < NSET; ++t)
 #pragma unroll
         for (int i = 0; i < kDig; ++i) {
-          unsigned char *dst = Bbuf + i * S::B_SBO + (t * (tca::kPairs / 8) + tid / 8) * tca::kKStride + (tid % 8) * 16 + h * 8;
+          unsigned char *dst = Bbuf + i * S::B_SBO + (t * (TH / 8) + tid / 8) * tca::kKStride + (tid % 8) * 16 + h * 8;
           *reinterpret_cast<uint2 *>(dst) = make_uint2(pk[t][i][0], pk[t][i][1]);
         }
     };
@@ -365,7 +425,7 @@ __device__ __forceinline__ void tc_ana_body(const TcArgs &ta, const int4 item, u
       for (int t = 0; t < NSET; ++t)
 #pragma unroll
         for (int hh = 0; hh < 2; ++hh) {
-          const int kk = t * (tca::kPairs / 16) + 2 * warp + hh;
+          const int kk = t * (TH / 16) + 2 * warp + hh;
           const uint64_t ad = adesc0 + (uint64_t)((2 * kk * S::A_LBO) >> 4);
           const uint64_t bd = bdesc0 + (uint64_t)((2 * kk * tca::kKStride) >> 4);
           tc::mma_bf16(tbase + xb * tca::kDCols, ad, bd, idesc, 1u);
@@ -373,11 +433,11 @@ __device__ __forceinline__ void tc_ana_body(const TcArgs &ta, const int4 item, u
       tc::mma_commit(&mine[warp]);
       tc::mma_commit(&full[xb]);
     };
-    // reading warps: block ibp's D rows from accumulator ibp & 1 into shared memory;
-    // the accumulator zeroed and released
+    // block ibp's D rows of this warp's quarter into shared memory; the accumulator
+    // zeroed and released
     auto epi_read = [&](int ibp) {
-      const int xb = ibp & 1;
-      if (!wait_warp(&full[xb], (uint32_t)(ibp >> 1) & 1u)) {
+      const int xb = ibp % NACC;
+      if (!wait_warp(&full[xb], (uint32_t)(ibp / NACC) & 1u)) {
         give_up();
         return;
       }
@@ -403,11 +463,12 @@ __device__ __forceinline__ void tc_ana_body(const TcArgs &ta, const int4 item, u
       __syncwarp();
       if (lane == 0) tc::bar_arrive(&freeb[xb]);
     };
-    // the column and degree a lane sums: lanes 0 .. 15 of the reading warps, column
-    // 2 warp + lane / 8, degree lane % 8; the slot entry it writes for block lbp
-    // (nullptr: none; neg: add the negation)
-    const int ocol = 2 * warp + (lane >> 3), odeg = lane & 7;
-    const bool oact = warp < S::NREAD && lane < S::EROWS;
+    // the column and degree a lane sums (one column a quarter: four lanes share a
+    // degree, epart 0 .. 3, and lane epart 0 writes it); the slot entry written for
+    // block lbp (nullptr: none; neg: add the negation)
+    const int odeg = lane & 7, epart = lane >> 3;
+    const int ocol = S::CPW == 1 ? (warp & 3) : 2 * (warp & 3) + (epart & 1);
+    const bool oact = S::CPW == 1 ? epart == 0 : lane < S::EROWS;
     auto out_at = [&](int lbp, bool &neg) -> double * {
       const int l = lbp + odeg, j = ocol >> 2, cc = ocol & 3;
       neg = false;
@@ -419,23 +480,46 @@ __device__ __forceinline__ void tc_ana_body(const TcArgs &ta, const int4 item, u
       // spin 0: the even-l columns at even l - l0, the odd ones at odd
       return (cc >> 1) == (odeg & 1) ? outp + (int64_t)(l - l0) * V + 2 * j + (cc & 1) : nullptr;
     };
-    // the staged digit products of the lane's column and degree, by level: levels
-    // 0 to 2 exact in FP32 (at most three sums of 2^22 quanta), added in
-    // double-float; levels 3 to 6 in FP32; the slot entry written (prev: its value
-    // from the group's earlier tiles)
+    // the staged digit products by level: levels 0 to 2 exact in FP32 (at most three
+    // sums of 2^22 quanta), added in double-float; levels 3 to 6 in FP32; the slot
+    // entry written (prev: its value from the group's earlier tiles).  D(i, j) = sum of
+    // G_j L_i.
     auto epi_sum = [&](double *o, bool neg, double prev) {
-      if (o) {
-        const float *e = Ebuf + (lane >> 3) * tca::kColRows * tca::kEStride + odeg;
-        auto D = [&](int i, int j) { return e[j * tca::kEStride + i * 8]; };  // sum of G_j L_i
-        const float L1 = __fadd_rn(D(1, 0), D(0, 1));
-        const float L2 = __fadd_rn(__fadd_rn(D(2, 0), D(1, 1)), D(0, 2));
-        float lo = 0.f;
+      float L0, L1, L2, lo = 0.f;
+      if (S::CPW == 1) {
+        // lane epart q takes row j = q, and of rows 4 and 5 lane 2 + (j - 4) takes one
+        const float *e = Ebuf + epart * tca::kEStride + odeg;
+        float v[kDig];
+#pragma unroll
+        for (int i = 0; i < kDig; ++i) v[i] = e[i * 8];
+        const float *e2 = e + 2 * tca::kEStride;  // parts 2, 3: rows 4, 5 (others': not used)
+        const float w0 = e2[0], w1 = e2[8], w2 = e2[16];
+        lo = __fadd_rn(epart < 2 ? v[5] : w1, epart < 3 ? v[4] : 0.f);
+        lo = __fadd_rn(lo, epart == 2 ? w2 : 0.f);
+        lo = __fadd_rn(lo, v[3]);
+        lo = __fadd_rn(lo, epart < 2 ? 0.f : w0);
+        lo = __fadd_rn(lo, epart < 1 ? 0.f : v[2]);
+        lo = __fadd_rn(lo, epart < 2 ? 0.f : v[1]);
+        lo = __fadd_rn(lo, epart < 3 ? 0.f : v[0]);
+        lo = __fadd_rn(lo, __shfl_xor_sync(0xffffffffu, lo, 16));
+        lo = __fadd_rn(lo, __shfl_xor_sync(0xffffffffu, lo, 8));
+        L0 = v[0];
+        L1 = __fadd_rn(v[1], __shfl_down_sync(0xffffffffu, v[0], 8));
+        L2 = __fadd_rn(__fadd_rn(v[2], __shfl_down_sync(0xffffffffu, v[1], 8)), __shfl_down_sync(0xffffffffu, v[0], 16));
+      } else {
+        const float *e = Ebuf + (epart & 1) * tca::kColRows * tca::kEStride + odeg;
+        auto D = [&](int i, int j) { return e[j * tca::kEStride + i * 8]; };
+        L0 = D(0, 0);
+        L1 = __fadd_rn(D(1, 0), D(0, 1));
+        L2 = __fadd_rn(__fadd_rn(D(2, 0), D(1, 1)), D(0, 2));
 #pragma unroll
         for (int k = 6; k >= 3; --k)
 #pragma unroll
           for (int i = 0; i < kDig; ++i)
             if (k - i >= 0 && k - i < kDig) lo = __fadd_rn(lo, D(i, k - i));
-        f2 t = two_sum(D(0, 0), L1);
+      }
+      if (o) {
+        f2 t = two_sum(L0, L1);
         t = f2_add_lazy(t, f2{L2, 0.f});
         t = fast_two_sum(t.h, __fadd_rn(t.l, lo));
         const double val = f2_val(t);
@@ -445,38 +529,53 @@ __device__ __forceinline__ void tc_ana_body(const TcArgs &ta, const int4 item, u
     };
 
     int lb = lstart;
+    const int ib0 = ib;
 #pragma unroll 1
     for (; lb <= lmax; lb += tca::kBlk, ++ib) {
-      const int xb = ib & 1;
-      // the slot entry this lane adds the previous block to: read now, its latency
-      // hidden behind this block's recursion
-      bool neg_prev;
-      double *const o_prev = lb > lstart ? out_at(lb - tca::kBlk, neg_prev) : nullptr;
+      const int xb = ib % NACC;
+      // this warp's turn to read: block ib - LAG.  The slot entry its lanes add that
+      // block to is read now, its latency hidden behind this block's recursion.
+      const bool turn = ib - LAG >= ib0 && (GROUPS == 1 || (ib & 1) == (warp >> 2));
+      bool neg_prev = false;
+      double *const o_prev = turn ? out_at(lb - LAG * tca::kBlk, neg_prev) : nullptr;
       double prev = 0.0;
       if (o_prev && gi > 0) asm volatile("ld.global.f64 %0, [%1];" : "=d"(prev) : "l"(o_prev));
-      if (lj == lb) {  // this pair joins: the recursion state where its terms start
-        const JoinRec r = ld_join(jrec, polar);
-        lpc = r.lpc;
-        lpp = r.lpp;
-        lmc = r.lmc;
-        lmp = r.lmp;
-        scp = r.scp;
-        scm = r.scm;
-        wfp = wfac(scp) * ulx;
-        wfm = wfac(scm) * ulx;
-      }
-      if (__any_sync(0xffffffffu, lj == lb)) settled = __all_sync(0xffffffffu, scp == 0 && scm == 0);
+      // pairs joining here take the recursion state where their terms start, over u_p
+      bool joins = false;
+#pragma unroll
+      for (int t = 0; t < NP; ++t)
+        if (lj[t] == lb) {
+          const JoinRec r = ld_join(jrec[t], polar);
+          const float ulx = __int_as_float((127 - lexp[t]) << 23);
+          if (t == 0) {
+            rec.start(0, r.lpc, r.lpp, ulx);
+            sc0 = r.scp;
+            wf.x = scale_weight(sc0);
+          } else {
+            rec.start(1, r.lpc, r.lpp, ulx);
+            sc1 = r.scp;
+            wf.y = scale_weight(sc1);
+          }
+          if (SPIN) {  // lane 1 holds s l- (l- itself in a polar warp): the previous degree's sign is -1
+            rec.start(1, r.lmc, polar ? r.lmp : neg(r.lmp), ulx);
+            sc1 = r.scm;
+            wf.y = scale_weight(sc1);
+          }
+          joins = true;
+        }
+      if (__any_sync(0xffffffffu, joins)) settled = __all_sync(0xffffffffu, sc0 == 0 && sc1 == 0);
       // a warp none of whose pairs has joined adds nothing: no digits, no products,
-      // a plain arrival.  Every warp first waits until the reading warps have
-      // released the accumulator's previous block, so that no arrival (or commit)
-      // of this block can fall into the phase of the block two before.
-      const bool live = __any_sync(0xffffffffu, lj <= lb);
+      // a plain arrival.  Every warp first waits until the reading warps have released
+      // the accumulator's previous block, so that no arrival (or commit) of this block
+      // can fall into the phase of the block NACC before.
+      const bool live = __any_sync(0xffffffffu, jmin <= lb);
       if (live) {
-#pragma unroll 1
+#pragma unroll
         for (int h = 0; h < 2; ++h) {
           uint32_t pk[NSET][kDig][2];
-          if (polar) part(true, lb + 4 * h, pk);
-          else part(false, lb + 4 * h, pk);
+          if (polar) part(kPolar, lb + 4 * h, pk);
+          else if (settled && lb >= lfast) part(kFast, lb + 4 * h, pk);
+          else part(kCareful, lb + 4 * h, pk);
           // this warp's products of its previous block read the tiles: wait for them
           // before the first write (they have long finished by now)
           if (h == 0 && nmine > nmine_done) {
@@ -493,30 +592,33 @@ __device__ __forceinline__ void tc_ana_body(const TcArgs &ta, const int4 item, u
         tc::fence_async_smem();
         __syncwarp();
       }
-      if (ib >= 2 && !wait_warp(&freeb[xb], (uint32_t)((ib - 2) >> 1) & 1u)) {
+      if (ib >= NACC && !wait_warp(&freeb[xb], (uint32_t)(ib / NACC - 1) & 1u)) {
         give_up();
         break;
       }
       if (live) {
-        if (lane == 0) issue(xb);
+        if (tc::elect_one()) issue(xb);
         __syncwarp();
         ++nmine;
       } else if (lane == 0) {
         tc::bar_arrive(&full[xb]);
       }
-      if (warp < S::NREAD && lb > lstart) {
-        epi_read(ib - 1);
+      if (turn) {
+        epi_read(ib - LAG);
         if (!ok) break;
         epi_sum(o_prev, neg_prev, prev);
       }
     }
     if (!ok) continue;  // to the next tile's barrier, where the CTA stops
-    if (warp < S::NREAD) {  // the tile's last block
+    // the tile's last blocks
+#pragma unroll 1
+    for (int k = ib - LAG > ib0 ? ib - LAG : ib0; k < ib; ++k) {
+      if (GROUPS > 1 && (k & 1) != (warp >> 2)) continue;
       bool neg;
-      double *o = out_at(lb - tca::kBlk, neg);
+      double *o = out_at(lb - (ib - k) * tca::kBlk, neg);
       const double prev = (o && gi > 0) ? *o : 0.0;
-      epi_read(ib - 1);
-      if (!ok) continue;
+      epi_read(k);
+      if (!ok) break;
       epi_sum(o, neg, prev);
     }
   }
@@ -528,18 +630,18 @@ __device__ __forceinline__ void tc_ana_body(const TcArgs &ta, const int4 item, u
   tc::fence_before();
   __syncthreads();
   tc::fence_after();
-  if (warp == 0) tc::tmem_dealloc(tbase, 2 * tca::kDCols);
+  if (warp == 0) tc::tmem_dealloc(tbase, S::TCOLS);
 }
 
 template <int NJ, bool SPIN>
-__global__ void __launch_bounds__(tca::kPairs, (tca::AnaShape<NJ, SPIN>::MINB)) tc_ana(TcArgs ta) {
+__global__ void __launch_bounds__((tca::AnaShape<NJ, SPIN>::TH), (tca::AnaShape<NJ, SPIN>::MINB)) tc_ana(TcArgs ta) {
   extern __shared__ __align__(128) unsigned char tca_smem[];
   tc_ana_body<NJ, SPIN>(ta, ta.m.ana_items[blockIdx.x], tca_smem);
 }
 
 // batches: item (mi, first tile, slot << 8 | tiles, record); the record holds the plan's arguments
 template <int NJ, bool SPIN>
-__global__ void __launch_bounds__(tca::kPairs, (tca::AnaShape<NJ, SPIN>::MINB))
+__global__ void __launch_bounds__((tca::AnaShape<NJ, SPIN>::TH), (tca::AnaShape<NJ, SPIN>::MINB))
     tc_ana_batch(const TcArgs *__restrict__ args, const int4 *__restrict__ items) {
   extern __shared__ __align__(128) unsigned char tca_smem[];
   const int4 it = items[blockIdx.x];
@@ -571,19 +673,24 @@ bool tc_ana_supported(int spin, int njobs_pad) {
   return njobs_pad <= 2;
 }
 
+int tc_ana_tiles(int spin, int njobs_pad) {
+  if (spin == 0) return njobs_pad == 1 ? tca::AnaShape<1, false>::TILES : tca::AnaShape<2, false>::TILES;
+  return njobs_pad == 1 ? tca::AnaShape<1, true>::TILES : tca::AnaShape<2, true>::TILES;
+}
+
 cudaError_t launch_leg_tc_ana_batch(int spin, int nj, const void *targs, const int4 *items, int n, cudaStream_t st) {
   if (n == 0) return cudaSuccess;
   const TcArgs *a = static_cast<const TcArgs *>(targs);
   if (spin == 0) {
     switch (nj) {
-      case 1: tc_ana_batch<1, false><<<n, tca::kPairs, tca::AnaShape<1, false>::SMEM_LAUNCH, st>>>(a, items); break;
-      case 2: tc_ana_batch<2, false><<<n, tca::kPairs, tca::AnaShape<2, false>::SMEM_LAUNCH, st>>>(a, items); break;
+      case 1: tc_ana_batch<1, false><<<n, tca::AnaShape<1, false>::TH, tca::AnaShape<1, false>::SMEM_LAUNCH, st>>>(a, items); break;
+      case 2: tc_ana_batch<2, false><<<n, tca::AnaShape<2, false>::TH, tca::AnaShape<2, false>::SMEM_LAUNCH, st>>>(a, items); break;
       default: return cudaErrorInvalidValue;
     }
   } else {
     switch (nj) {
-      case 1: tc_ana_batch<1, true><<<n, tca::kPairs, tca::AnaShape<1, true>::SMEM_LAUNCH, st>>>(a, items); break;
-      case 2: tc_ana_batch<2, true><<<n, tca::kPairs, tca::AnaShape<2, true>::SMEM_LAUNCH, st>>>(a, items); break;
+      case 1: tc_ana_batch<1, true><<<n, tca::AnaShape<1, true>::TH, tca::AnaShape<1, true>::SMEM_LAUNCH, st>>>(a, items); break;
+      case 2: tc_ana_batch<2, true><<<n, tca::AnaShape<2, true>::TH, tca::AnaShape<2, true>::SMEM_LAUNCH, st>>>(a, items); break;
       default: return cudaErrorInvalidValue;
     }
   }
@@ -599,14 +706,14 @@ cudaError_t launch_leg_tc_ana(const sht_plan_s *P, const void *mixargs, int n, c
   const int nj = P->njobs_pad;
   if (P->spin == 0) {
     switch (nj) {
-      case 1: tc_ana<1, false><<<n, tca::kPairs, tca::AnaShape<1, false>::SMEM_LAUNCH, st>>>(ta); break;
-      case 2: tc_ana<2, false><<<n, tca::kPairs, tca::AnaShape<2, false>::SMEM_LAUNCH, st>>>(ta); break;
+      case 1: tc_ana<1, false><<<n, tca::AnaShape<1, false>::TH, tca::AnaShape<1, false>::SMEM_LAUNCH, st>>>(ta); break;
+      case 2: tc_ana<2, false><<<n, tca::AnaShape<2, false>::TH, tca::AnaShape<2, false>::SMEM_LAUNCH, st>>>(ta); break;
       default: return cudaErrorInvalidValue;
     }
   } else {
     switch (nj) {
-      case 1: tc_ana<1, true><<<n, tca::kPairs, tca::AnaShape<1, true>::SMEM_LAUNCH, st>>>(ta); break;
-      case 2: tc_ana<2, true><<<n, tca::kPairs, tca::AnaShape<2, true>::SMEM_LAUNCH, st>>>(ta); break;
+      case 1: tc_ana<1, true><<<n, tca::AnaShape<1, true>::TH, tca::AnaShape<1, true>::SMEM_LAUNCH, st>>>(ta); break;
+      case 2: tc_ana<2, true><<<n, tca::AnaShape<2, true>::TH, tca::AnaShape<2, true>::SMEM_LAUNCH, st>>>(ta); break;
       default: return cudaErrorInvalidValue;
     }
   }

@@ -995,6 +995,11 @@ static int build_ana_lists(sht_plan_s *P, int ppt) {
     for (int i = 0; i < P->nm; ++i)
       if (P->lmax >= std::max(P->mval[i], as)) ntile += tiles - P->first_pair[i] / TA;
     group = (int)std::max<int64_t>(1, std::min<int64_t>(kAnaGroupTiles, ntile / ((int64_t)kAnaItemsPerSm * P->sms)));
+    // whole passes of the tensor-core analysis, which walks several tiles at a time
+    if (P->tc_ana) {
+      const int nt = tc_ana_tiles(P->spin, P->njobs_pad);
+      group = (group + nt - 1) / nt * nt;
+    }
   }
   int64_t need = 0;
   for (int polar = 0; polar < 2; ++polar) {
@@ -1115,8 +1120,10 @@ static int plan_build(sht_plan_s *P, const sht_geom_s *g) {
   CUDA_TRY(cudaMalloc(&P->d_alpha, std::max<int64_t>(1, nco) * sizeof(double)));
   P->workspace += nco * sizeof(double);
   if (P->precision == SHT_MIXED) {
-    CUDA_TRY(cudaMalloc(&P->d_coef32, std::max<int64_t>(1, nco) * sizeof(float4)));
-    P->workspace += nco * sizeof(float4);
+    // (a tail of zeros: the kernels read up to a block of degrees past lmax)
+    CUDA_TRY(cudaMalloc(&P->d_coef32, (nco + kCoefTail) * sizeof(float4)));
+    CUDA_TRY(cudaMemset(P->d_coef32 + nco, 0, kCoefTail * sizeof(float4)));
+    P->workspace += (nco + kCoefTail) * sizeof(float4);
     CUDA_TRY(cudaMalloc(&P->d_alm32, std::max<int64_t>(1, nco) * P->nmaps_pad * sizeof(float4)));
     P->workspace += nco * P->nmaps_pad * sizeof(float4);
   }
@@ -1383,9 +1390,11 @@ extern "C" int sht_plan_set_tensor_core_analysis(sht_plan_t P, int on) {
     return fail(SHT_ERR_UNSUPPORTED, "tensor-core analysis holds at most two jobs (ncomp <= 2)");
   if (P->batch_refs)
     return fail(SHT_ERR_INVALID_ARG, "the plan belongs to %d batch(es); destroy them first", P->batch_refs);
-  if (on && P->ana_ppt != 1) {  // its tiles: one ring pair per thread
+  if (on && !P->tc_ana) {  // its tiles: one ring pair per thread
+    P->tc_ana = 1;
     const int rc = retile(P, 1);
-    if (rc != SHT_OK) return rc;
+    if (rc != SHT_OK) P->tc_ana = 0;
+    return rc;
   }
   P->tc_ana = on ? 1 : 0;
   return SHT_OK;

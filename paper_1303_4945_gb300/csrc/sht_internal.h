@@ -25,6 +25,7 @@ constexpr int kMaxPtr = 32;       // max device pointers per execute (maps or a_
 constexpr int kMaxJobs = 16;      // ncomp limit
 constexpr int kSynTile = 128;     // ring pairs per synthesis Legendre CTA (one per thread)
 constexpr int kAnaThreads = 128;  // threads per analysis Legendre CTA
+constexpr int kCoefTail = 8;      // entries past the end of the double-float coefficient table
 constexpr int kAnaGroupTiles = 16;  // most tiles a mixed analysis item walks, one after another
 constexpr int kAnaItemsPerSm = 24;  // fewest mixed analysis items per SM the grouping leaves
 constexpr int kMaxRadix = 8 * 4;  // odd radices with register butterflies and constant cos/sin tables (primes <= 31)
@@ -273,6 +274,7 @@ cudaError_t launch_leg_tc_ana(const sht_plan_s *P, const void *mixargs, int n, c
 cudaError_t launch_leg_tc_ana_batch(int spin, int nj, const void *targs, const int4 *items, int n, cudaStream_t st);
 cudaError_t tc_ana_prepare_device();
 bool tc_ana_supported(int spin, int njobs_pad);
+int tc_ana_tiles(int spin, int njobs_pad);  // tiles of kAnaThreads pairs it walks at a time
 // ring FFTs
 // ring pairs [p0, p1) (p1 < 0: to the last pair)
 cudaError_t launch_fft_syn(const sht_plan_s *P, const DevPtrs &map, int polar, int weighted, int add,
