@@ -41,6 +41,17 @@
 // first ones of a window overwrite every level read later); the recursion's
 // digits of K-step s + 1 are written once the MMAs of s have completed, and B is
 // rebuilt then too.
+//
+// What bounds it (GB300, spin 2, one E/B pair, lmax 4095; lmax 2047 under ncu): the
+// FP32 pipe (58% busy) and issue (67%), with the K-step's barrier the largest stall;
+// 20 warps per SM.  A step takes about 73 FP32 lane operations (recursions 45, digits
+// 20, remainders 8), so at the pipe's measured rate the kernel needs 29 ms.  History:
+// 54.3 ms with scalar recursions of three coefficients, 49.6 with the unit-coefficient
+// recursion, 39.9 with both recursions packed, on Lambda / u_p and with the signs in
+// the recursion, 38.7 with 16-byte digit stores and B built between the halves (8
+// spin-0 maps at lmax 2047: 10.2 -> 8.7).  The B build split evenly over the threads
+// was slower (40.5 against 39.9), four CTAs per SM with more registers too (42.9).
+#include "dual.cuh"
 #include "tcgen05.cuh"
 
 namespace sht {
@@ -53,11 +64,11 @@ constexpr int kLamDigits = 3;       // bf16 digits of Lambda (plus an FP32 remai
 constexpr int kAlmDigits = 6;       // bf16 digits of the a_lm columns
 constexpr int kLevels = 6;          // TMEM levels read: digit products with i + j <= 5
 constexpr int kATile = kRows * kK * 2;  // bytes of one 128 x 16 bf16 tile
-constexpr int kPack = 4;            // degrees of digits held in registers before a shared-memory store
-// the thread issuing the MMAs: lane 0 of the last warp, whose threads neither load
+constexpr int kPack = 8;            // degrees of digits held in registers before a 16-byte shared-memory store
+// the warp issuing the MMAs (an elected lane): the last, whose threads neither load
 // the staged rows nor build B (threads 0-63 at one E/B pair), so that the warps
 // reach the K-step's barrier together (152.4 -> 151.8 ms per headline pair)
-constexpr int kIssuerThread = 96;
+constexpr int kIssuerWarp = 3;
 // Shapes: NCOL output columns per pair (spin: N1, S4, N2, S3 as re/im per job;
 // spin 0: even-l and odd-l sums as re/im per job), NCW = max(NCOL, 8) TMEM columns
 // per level and rows per a_lm digit tile, MMA width N = 2 NCW (two digit tiles, two
@@ -137,10 +148,10 @@ __device__ __forceinline__ void window_bounds(const MixArgs &a, int64_t co, int 
   if ((threadIdx.x & 31) < S::NV) atomicMax(reinterpret_cast<int *>(umax) + v, __float_as_int(mx));
 }
 
-// The a_lm digit stacks of a K-step from its staged rows (zero past lmax): value v
-// of degree lb + k split into kAlmDigits digits on its window's grid and written,
-// with the parity sign s = (-1)^(l - l0) where the column needs it, into the rows
-// of the columns that read it (see the column layout in tc_syn_body).  Set t's
+// The a_lm digit stacks of a K-step from its staged rows (zero past lmax; M times s =
+// (-1)^(l - l0)): value v of degree lb + k split into kAlmDigits digits on its window's
+// grid and written into the rows of the columns that read it (see the column layout
+// in tc_syn_body).  Set t's
 // stack holds NDT digit tiles of NCW rows, digit j at rows (j + 1) NCW ..; rows no
 // value writes (the other set's columns, padding columns, the tile of digit -1)
 // stay zero from the kernel's start.
@@ -166,18 +177,16 @@ __device__ __forceinline__ void build_b(const float4 *stg, const float *umax, un
     d[4] = round_to(r, s0 * 0x1p-32f);
     r = __fsub_rn(r, d[4]);
     d[5] = round_to(r, s0 * 0x1p-40f);
-    const bool odd = k & 1;
-    // (set, column) pairs of this value; spin: P.re -> (+, 8j) and (-, 8j+6) signed,
-    // P.im -> (+, 8j+1) and (-, 8j+7) signed, M.re -> (+, 8j+2) signed and (-, 8j+4),
-    // M.im -> (+, 8j+3) signed and (-, 8j+5); spin 0: the even- or odd-l column of its job
-    int col0, col1 = 0, neg0 = 0, neg1 = 0, zcol = 0;
+    // (set, column) pairs of this value; spin: P.re -> (+, 8j) and (-, 8j+6), P.im ->
+    // (+, 8j+1) and (-, 8j+7), s M.re -> (+, 8j+2) and (-, 8j+4), s M.im -> (+, 8j+3) and
+    // (-, 8j+5); spin 0: the even- or odd-l column of its job
+    int col0, col1 = 0, zcol = 0;
     if (SPIN) {
       const int j = v / 4, c = v % 4;
       col0 = 8 * j + c;
       col1 = 8 * j + (c < 2 ? 6 + c : 2 + c);
-      neg0 = (c >= 2) && odd;
-      neg1 = (c < 2) && odd;
     } else {
+      const bool odd = k & 1;
       const int j = v / 2, c = v % 2;
       col0 = 4 * j + (odd ? 2 : 0) + c;
       zcol = 4 * j + (odd ? 0 : 2) + c;
@@ -185,9 +194,9 @@ __device__ __forceinline__ void build_b(const float4 *stg, const float *umax, un
 #pragma unroll
     for (int dj = 0; dj < kAlmDigits; ++dj) {
       const int r = (dj + 1) * S::NCW;
-      *reinterpret_cast<uint16_t *>(Bt + at(r + col0, k)) = bf16_of(neg0 ? -d[dj] : d[dj]);
+      *reinterpret_cast<uint16_t *>(Bt + at(r + col0, k)) = bf16_of(d[dj]);
       if (SPIN)
-        *reinterpret_cast<uint16_t *>(Bt + S::NDT * S::DTILE + at(r + col1, k)) = bf16_of(neg1 ? -d[dj] : d[dj]);
+        *reinterpret_cast<uint16_t *>(Bt + S::NDT * S::DTILE + at(r + col1, k)) = bf16_of(d[dj]);
       else
         *reinterpret_cast<uint16_t *>(Bt + at(r + zcol, k)) = 0;
     }
@@ -202,8 +211,9 @@ __device__ __forceinline__ void build_b(const float4 *stg, const float *umax, un
 // Columns of the product (per job j): spin, 8j + {0,1} N1 = sum P l+, {2,3}
 // S4 = sum s M l+, {4,5} N2 = sum M l-, {6,7} S3 = sum s P l- (re, im; s =
 // (-1)^(l - l0), P = E + iB, M = E - iB); spin 0, 4j + {0,1} the even-l and
-// 4j + {2,3} the odd-l sums of a_lm lambda.  The +s digits (A set 0) meet B rows
-// holding P, s M; the -s digits (A set 1) rows holding M, s P.
+// 4j + {2,3} the odd-l sums of a_lm lambda.  A set 0 holds the digits of l+, set 1
+// those of s l-, so both meet B rows holding P and s M.  All sums run on Lambda / u_p
+// (u_p the pair's bound) and are multiplied by u_p at the end.
 // ---------------------------------------------------------------------------
 template <int NJ, bool SPIN>
 __device__ __forceinline__ void tc_syn_body(const TcArgs &ta, const int2 item, unsigned char *smem) {
@@ -211,8 +221,10 @@ __device__ __forceinline__ void tc_syn_body(const TcArgs &ta, const int2 item, u
   constexpr int NL = S::NL, NCOL = S::NCOL;
   __shared__ __align__(8) uint64_t mbar;
   __shared__ uint32_t tslot;
+  __shared__ volatile int stop;
   const MixArgs &a = ta.m;
-  const int tid = threadIdx.x, warp = tid >> 5;
+  // the warp's number from a shuffle, so that the compiler sees it uniform
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
   const int mi = item.x;
   const int p = item.y + tid;
   const bool valid = p < a.npairs;
@@ -239,6 +251,7 @@ __device__ __forceinline__ void tc_syn_body(const TcArgs &ta, const int2 item, u
       if (e < S::STG) {
         const int k = e / S::ROW, c = e % S::ROW, l = lb + k;
         if (l <= lmax) pf[i] = c < 1 ? __ldg(cf + l) : __ldg(a.alm32 + (int64_t)(c - 1) * a.ncoef + co + l);
+        if (SPIN && c > 0 && !(c & 1) && (k & 1)) pf[i] = make_float4(-pf[i].x, -pf[i].y, -pf[i].z, -pf[i].w);  // s M
       }
     }
   };
@@ -261,7 +274,10 @@ __device__ __forceinline__ void tc_syn_body(const TcArgs &ta, const int2 item, u
     if ((tid & 31) == 0) kstart[warp] = wmin;
   }
   if (warp == 0) tc::tmem_alloc(&tslot, S::TCOLS);
-  if (tid == 0) tc::bar_init(&mbar);
+  if (tid == 0) {
+    tc::bar_init(&mbar);
+    stop = 0;
+  }
   for (int i = tid; i < S::B_BYTES / 16; i += tc::kRows) reinterpret_cast<uint4 *>(Bt)[i] = make_uint4(0, 0, 0, 0);
   if (tid < 2 * S::NV) umax[tid] = 0.f;
   tc::fence_before();
@@ -279,122 +295,115 @@ __device__ __forceinline__ void tc_syn_body(const TcArgs &ta, const int2 item, u
 #pragma unroll
   for (int c = 0; c < NCOL; ++c) accs[c * tc::kRows + tid] = f2{0.f, 0.f};
 
-  // recursion state (as in the double-float synthesis): +s values lpc/lpp, -s lmc/lmp,
-  // zero until the pair joins (no terms, and a recursion of zeros)
+  // the recursions, on Lambda / u_p: zero until the pair joins (no terms, and a
+  // recursion of zeros).  Spin 0 runs one lane.
   const PairDev pd = a.pairs[valid ? p : 0];
   const bool polar = polar_warp(pd.x, valid);
-  const f3 x = node_of(pd.x, polar);
-  f2 lpc = {0.f, 0.f}, lmc = {0.f, 0.f}, lpp = {0.f, 0.f}, lmp = {0.f, 0.f};
-  int scp = 0, scm = 0;
-  // digit grid of Lambda: magic constants of the quanta u 2^-7, u 2^-15, u 2^-23,
-  // u the pair's own bound from its join record (the plan-wide bound until it joins)
-  float ls0 = ta.lam_bound * 98304.0f, ls1 = ls0 * 0x1p-8f, ls2 = ls0 * 0x1p-16f;
+  Dual<true> rec;
+  rec.p = rec.q = d2{both(0.f), both(0.f)};
+  rec.x[0] = node_of(pd.x, polar);
+  int sc0 = 0, sc1 = 0;
+  const int lfast = SPIN ? fast_from(as, rec.x[0].h, valid, lmax) : 0;
   float racc[NCOL];
 #pragma unroll
   for (int c = 0; c < NCOL; ++c) racc[c] = 0.f;
+  float2 wf = both(1.f);  // weights of the two lanes' values; scales change only at the rescale checks
+  bool settled = false;   // every lane of the warp at scale 0 (warp-uniform; scales only rise)
 
-  // accumulation weight of the +s / -s values (see weight() in mixed_common.cuh): 1 at
-  // scale 0, 2^-104 at scale -1, 0 below; scales change only at the rescale checks
-  auto wfac = [](int sc) { return sc == 0 ? 1.f : (sc == -1 ? kScaleFactor32 : 0.f); };
-  float wfp = wfac(scp), wfm = wfac(scm);
-  bool settled = false;  // every lane of the warp at scale 0 (warp-uniform; scales only rise)
-
-  // kPack degrees from rows (lb - l0 even): digits packed per pair of degrees into
-  // pk[set][digit][q / 2], remainders contracted into racc, recursion advanced.
-  // Every second degree the warp votes: if every lane's values are negligible for
-  // the next two steps (as in the double-float kernels) the digits are zero and
-  // only the recursion runs.
-  auto part = [&](const bool pol, const float4 *rows, uint32_t (&pk)[NL][tc::kLamDigits][tc::kPack / 2]) {
-    float dlo[NL][tc::kLamDigits];
+  // one step of the recursions with a row's coefficients
+  auto advance = [&](const StepMode mode, const float4 &c) {
+    if (SPIN) {
+      rec.step(mode, c);
+    } else {
+      f2 lc = lane0(rec.p), lp = lane0(rec.q);
+      step_s0(Coef32{{c.x, c.y}, {0.f, 0.f}}, rec.x[0], mode == kPolar, lc, lp);
+      rec.start(0, lc, lp, 1.f);
+    }
+  };
+  // kPack degrees from rows (lb - l0 even): digits (quanta 2^-7, 2^-15, 2^-23) packed
+  // per pair of degrees into pk[set][digit][q / 2], remainders contracted into racc,
+  // recursion advanced.  Unless every lane is at scale 0 (kFast; a polar warp tests
+  // too) the values take their weights, and every second degree the warp votes: if
+  // every lane's values are negligible for the next two steps (as in the double-float
+  // kernels) the digits are zero and only the recursion runs.
+  auto part = [&](const StepMode mode, const float4 *rows,
+                  uint32_t (&pk)[NL][tc::kLamDigits][tc::kPack / 2]) __attribute__((always_inline)) {
+    constexpr float s0 = 98304.0f, s1 = s0 * 0x1p-8f, s2 = s0 * 0x1p-16f;  // 1.5 * 2^23 * quantum
+    float2 dlo[tc::kLamDigits];
     bool dead = false;
 #pragma unroll
     for (int q = 0; q < tc::kPack; ++q) {
       // past lmax the staged rows are zero: the recursion runs on zero coefficients
-      // (its values become zero one degree later) and meets zero a_lm, so those
-      // degrees add nothing and need no test
+      // (values of one degree's size, alternating) and meets zero a_lm, so those degrees
+      // add nothing and need no test
       const bool odd = q & 1;
-      if (!odd) dead = !settled && __all_sync(0xffffffffu, negligible(lpc, scp) && (!SPIN || negligible(lmc, scm)));
+      if (!odd && mode != kFast)
+        dead = !settled && __all_sync(0xffffffffu, negligible(lane0(rec.p), sc0) && (!SPIN || negligible(lane1(rec.p), sc1)));
       const float4 *row = rows + q * S::ROW;  // this degree's staged coefficients and a_lm
-      if (!dead) {
-        f2 w[NL];
-        w[0] = f2{lpc.h * wfp, lpc.l * wfp};
-        if (SPIN) w[1] = f2{lmc.h * wfm, lmc.l * wfm};
-        float rr[NL];
-#pragma unroll
-        for (int t = 0; t < NL; ++t) {
-          const float d0 = tc::round_to(w[t].h, ls0);
-          float r = __fsub_rn(w[t].h, d0);
-          const float d1 = tc::round_to(r, ls1);
-          r = __fsub_rn(r, d1);
-          const float d2 = tc::round_to(r, ls2);
-          rr[t] = __fadd_rn(__fsub_rn(r, d2), w[t].l);
-          if (!odd) {
-            dlo[t][0] = d0;
-            dlo[t][1] = d1;
-            dlo[t][2] = d2;
-          } else {
-            pk[t][0][q / 2] = tc::pack_bf16(dlo[t][0], d0);
-            pk[t][1][q / 2] = tc::pack_bf16(dlo[t][1], d1);
-            pk[t][2][q / 2] = tc::pack_bf16(dlo[t][2], d2);
-          }
+      float2 d[tc::kLamDigits] = {both(0.f), both(0.f), both(0.f)};
+      if (mode == kFast || !dead) {
+        float2 h = rec.p.h, lo = rec.p.l;
+        if (mode != kFast) {
+          const float2 f = make_float2(wf.x, (mode == kPolar && odd) ? -wf.y : wf.y);
+          h = mul2(h, f);
+          lo = mul2(lo, f);
+        }
+        float2 rr;
+        if (SPIN) {
+          auto round2 = [](float2 r, float c) { return add2(add2(r, both(c)), both(-c)); };
+          d[0] = round2(h, s0);
+          rr = sub2(h, d[0]);
+          d[1] = round2(rr, s1);
+          rr = sub2(rr, d[1]);
+          d[2] = round2(rr, s2);
+          rr = add2(sub2(rr, d[2]), lo);
+        } else {
+          d[0].x = tc::round_to(h.x, s0);
+          float r = __fsub_rn(h.x, d[0].x);
+          d[1].x = tc::round_to(r, s1);
+          r = __fsub_rn(r, d[1].x);
+          d[2].x = tc::round_to(r, s2);
+          rr.x = __fadd_rn(__fsub_rn(r, d[2].x), lo.x);
         }
 #pragma unroll
         for (int j = 0; j < NJ; ++j) {
           if (SPIN) {
             const float4 P = row[1 + 2 * j];
-            const float4 M = row[2 + 2 * j];
-            const float rp = rr[0], rm = rr[1], sp = odd ? -rr[0] : rr[0], sm = odd ? -rr[1] : rr[1];
-            racc[8 * j + 0] = __fmaf_rn(rp, P.x, racc[8 * j + 0]);
-            racc[8 * j + 1] = __fmaf_rn(rp, P.z, racc[8 * j + 1]);
-            racc[8 * j + 2] = __fmaf_rn(sp, M.x, racc[8 * j + 2]);
-            racc[8 * j + 3] = __fmaf_rn(sp, M.z, racc[8 * j + 3]);
-            racc[8 * j + 4] = __fmaf_rn(rm, M.x, racc[8 * j + 4]);
-            racc[8 * j + 5] = __fmaf_rn(rm, M.z, racc[8 * j + 5]);
-            racc[8 * j + 6] = __fmaf_rn(sm, P.x, racc[8 * j + 6]);
-            racc[8 * j + 7] = __fmaf_rn(sm, P.z, racc[8 * j + 7]);
+            const float4 M = row[2 + 2 * j];  // s M
+            racc[8 * j + 0] = __fmaf_rn(rr.x, P.x, racc[8 * j + 0]);
+            racc[8 * j + 1] = __fmaf_rn(rr.x, P.z, racc[8 * j + 1]);
+            racc[8 * j + 2] = __fmaf_rn(rr.x, M.x, racc[8 * j + 2]);
+            racc[8 * j + 3] = __fmaf_rn(rr.x, M.z, racc[8 * j + 3]);
+            racc[8 * j + 4] = __fmaf_rn(rr.y, M.x, racc[8 * j + 4]);
+            racc[8 * j + 5] = __fmaf_rn(rr.y, M.z, racc[8 * j + 5]);
+            racc[8 * j + 6] = __fmaf_rn(rr.y, P.x, racc[8 * j + 6]);
+            racc[8 * j + 7] = __fmaf_rn(rr.y, P.z, racc[8 * j + 7]);
           } else {
             const float4 v = row[1 + j];
             const int c = 4 * j + (odd ? 2 : 0);
-            racc[c] = __fmaf_rn(rr[0], v.x, racc[c]);
-            racc[c + 1] = __fmaf_rn(rr[0], v.z, racc[c + 1]);
+            racc[c] = __fmaf_rn(rr.x, v.x, racc[c]);
+            racc[c + 1] = __fmaf_rn(rr.x, v.z, racc[c + 1]);
           }
         }
-      } else {  // zero digits (negligible values)
+      }
 #pragma unroll
-        for (int t = 0; t < NL; ++t) {
-          if (!odd) {
-            dlo[t][0] = dlo[t][1] = dlo[t][2] = 0.f;
-          } else {
-            pk[t][0][q / 2] = tc::pack_bf16(dlo[t][0], 0.f);
-            pk[t][1][q / 2] = tc::pack_bf16(dlo[t][1], 0.f);
-            pk[t][2][q / 2] = tc::pack_bf16(dlo[t][2], 0.f);
-          }
+      for (int i = 0; i < tc::kLamDigits; ++i) {
+        if (!odd) {
+          dlo[i] = d[i];
+        } else {
+          pk[0][i][q / 2] = tc::pack_bf16(dlo[i].x, d[i].x);
+          if (SPIN) pk[NL - 1][i][q / 2] = tc::pack_bf16(dlo[i].y, d[i].y);
         }
       }
-      {
-        const float4 u = row[0];
-        const Coef32 cc = {{u.x, u.y}, {u.z, u.w}};
-        if (SPIN) step_spin(cc, x, pol, lpc, lpp, lmc, lmp);
-        else step_s0(cc, x, pol, lpc, lpp);
-      }
+      advance(mode, row[0]);
     }
   };
   // enhanced exponent: rescale every eight degrees (see mixed_common.cuh)
   auto rescale = [&]() {
     if (settled) return;
-    if (scp < 0 && fabsf(lpc.h) > kScaleUp32) {
-      lpc = {lpc.h * kScaleFactor32, lpc.l * kScaleFactor32};
-      lpp = {lpp.h * kScaleFactor32, lpp.l * kScaleFactor32};
-      ++scp;
-    }
-    if (SPIN && scm < 0 && fabsf(lmc.h) > kScaleUp32) {
-      lmc = {lmc.h * kScaleFactor32, lmc.l * kScaleFactor32};
-      lmp = {lmp.h * kScaleFactor32, lmp.l * kScaleFactor32};
-      ++scm;
-    }
-    wfp = wfac(scp);
-    wfm = wfac(scm);
-    settled = __all_sync(0xffffffffu, scp == 0 && scm == 0);
+    rec.rescale(sc0, sc1);
+    wf = make_float2(scale_weight(sc0), scale_weight(sc1));
+    settled = __all_sync(0xffffffffu, sc0 == 0 && sc1 == 0);
   };
   // this thread's digits of degrees q0 .. q0 + kPack - 1 of the K-step into the A tiles
   auto store_a = [&](int q0, const uint32_t (&pk)[NL][tc::kLamDigits][tc::kPack / 2]) {
@@ -404,10 +413,7 @@ __device__ __forceinline__ void tc_syn_body(const TcArgs &ta, const int2 item, u
       for (int i = 0; i < tc::kLamDigits; ++i) {
         unsigned char *dst = Abuf + (t * tc::kLamDigits + i) * tc::kATile + (tid / 8) * 256 + (q0 / 8) * 128 +
                              (tid % 8) * 16 + (q0 % 8) * 2;
-        if (tc::kPack == 8)
-          *reinterpret_cast<uint4 *>(dst) = *reinterpret_cast<const uint4 *>(pk[t][i]);
-        else
-          *reinterpret_cast<uint2 *>(dst) = *reinterpret_cast<const uint2 *>(pk[t][i]);
+        *reinterpret_cast<uint4 *>(dst) = make_uint4(pk[t][i][0], pk[t][i][1], pk[t][i][2], pk[t][i][3]);
       }
   };
 
@@ -461,6 +467,12 @@ __device__ __forceinline__ void tc_syn_body(const TcArgs &ta, const int2 item, u
 
   int ncommit = 0, nwaited = 0;
   bool ok = true;
+  // waits for the last commit (mostly done: no clock read); a wait that gives up sets
+  // `stop`, which ends the later ones at once, and the CTA leaves at its window's end
+  auto wait_mma = [&]() -> bool {
+    const uint32_t par = (uint32_t)(ncommit - 1) & 1u;
+    return tc::bar_try(&mbar, par) || tc::bar_wait_or(&mbar, par, &stop);
+  };
   for (int ks = ks0; ks < nks; ++ks) {
     const int lb = l0 + ks * tc::kK;
     if (ks % tc::kWin == 0 || ks == ks0) {  // column bounds of this window's a_lm (from lb on)
@@ -470,21 +482,18 @@ __device__ __forceinline__ void tc_syn_body(const TcArgs &ta, const int2 item, u
       tc::window_bounds<NJ, SPIN>(a, co, lb, lw1 < lmax ? lw1 : lmax, um);
       __syncthreads();
     }
-    if (lj == lb) {  // this pair joins: the recursion state where its terms start
+    if (lj == lb) {  // this pair joins: the recursion state where its terms start, over u_p
       const JoinRec r = ld_join(jrec, polar);
-      lpc = r.lpc;
-      lpp = r.lpp;
-      lmc = r.lmc;
-      lmp = r.lmp;
-      scp = r.scp;
-      scm = r.scm;
-      wfp = wfac(scp);
-      wfm = wfac(scm);
-      ls0 = __int_as_float((127 + r.lexp) << 23) * 98304.0f;
-      ls1 = ls0 * 0x1p-8f;
-      ls2 = ls0 * 0x1p-16f;
+      const float ulx = __int_as_float((127 - r.lexp) << 23);
+      rec.start(0, r.lpc, r.lpp, ulx);
+      sc0 = r.scp;
+      if (SPIN) {  // lane 1 holds s l- (l- itself in a polar warp): the previous degree's sign is -1
+        rec.start(1, r.lmc, polar ? r.lmp : neg(r.lmp), ulx);
+        sc1 = r.scm;
+      }
+      wf = make_float2(scale_weight(sc0), scale_weight(sc1));
     }
-    if (__any_sync(0xffffffffu, lj == lb)) settled = __all_sync(0xffffffffu, scp == 0 && scm == 0);
+    if (__any_sync(0xffffffffu, lj == lb)) settled = __all_sync(0xffffffffu, sc0 == 0 && sc1 == 0);
     // a warp none of whose lanes has joined holds zeros: it skips the recursion
     const bool wlive = __any_sync(0xffffffffu, lj <= lb);
     const float4 *rows = stage + (ks & 1) * S::STG;
@@ -494,8 +503,9 @@ __device__ __forceinline__ void tc_syn_body(const TcArgs &ta, const int2 item, u
     for (int q0 = 0; q0 < tc::kK; q0 += tc::kPack) {
       uint32_t pk[NL][tc::kLamDigits][tc::kPack / 2];
       if (wlive) {
-        if (polar) part(true, rows + q0 * S::ROW, pk);
-        else part(false, rows + q0 * S::ROW, pk);
+        if (polar) part(kPolar, rows + q0 * S::ROW, pk);
+        else if (settled && lb >= lfast) part(kFast, rows + q0 * S::ROW, pk);
+        else part(kCareful, rows + q0 * S::ROW, pk);
       } else {  // no lane of the warp has joined: zero digits, and nothing to advance
 #pragma unroll
         for (int t = 0; t < NL; ++t)
@@ -504,28 +514,27 @@ __device__ __forceinline__ void tc_syn_body(const TcArgs &ta, const int2 item, u
 #pragma unroll
             for (int q = 0; q < tc::kPack / 2; ++q) pk[t][i][q] = 0u;
       }
-      if (q0 % 8 == tc::kPack % 8) rescale();  // after every eight degrees
+      rescale();  // after every eight degrees
       // the previous K-step's MMAs read the A and B tiles: wait for them before
       // the first write (they have long finished by now)
       if (q0 == 0 && ncommit > nwaited) {
-        fail = !tc::bar_wait(&mbar, (uint32_t)(ncommit - 1) & 1u);
+        fail = !wait_mma();
         nwaited = ncommit;
       }
       if (!fail) store_a(q0, pk);
+      // (between the halves: the warps that build B reach the barrier later by less)
+      if (q0 == 0 && !fail) tc::build_b<NJ, SPIN>(rows, umax + ((ks / tc::kWin) & 1) * S::NV, Bt);
     }
-    if (!fail) tc::build_b<NJ, SPIN>(rows, umax + ((ks / tc::kWin) & 1) * S::NV, Bt);
     if (ks + 1 < nks) stage_store(ks + 1);  // its buffer's last readers finished before the previous barrier
     tc::fence_async_smem();
-    if (__syncthreads_or(fail)) {
-      ok = false;
-      break;
-    }
-    if (tid == tc::kIssuerThread) issue(ks);
+    if (fail) stop = 1;
+    __syncthreads();
+    if (warp == tc::kIssuerWarp && tc::elect_one()) issue(ks);
     ++ncommit;
     if (ks % tc::kWin == tc::kWin - 1 || ks == nks - 1) {
-      fail = !tc::bar_wait(&mbar, (uint32_t)(ncommit - 1) & 1u);
+      fail = !wait_mma();
       nwaited = ncommit;
-      if (__syncthreads_or(fail)) {
+      if (__syncthreads_or(fail || stop)) {
         ok = false;
         break;
       }
@@ -543,7 +552,9 @@ __device__ __forceinline__ void tc_syn_body(const TcArgs &ta, const int2 item, u
   tc::fence_after();
   if (warp == 0) tc::tmem_dealloc(tbase, S::TCOLS);
   if (!ok || !valid) return;
-  auto colsum = [&](int c) { return f2_val(accs[c * tc::kRows + tid]); };
+  const int lexp = __float_as_int(__ldg(jrec + 2).w);
+  const double u = __hiloint2double((1023 + lexp) << 20, 0);  // u_p
+  auto colsum = [&](int c) { return u * f2_val(accs[c * tc::kRows + tid]); };
 
   if (SPIN) {
     const double sig = (as & 1) ? -1.0 : 1.0;
@@ -649,7 +660,6 @@ size_t tc_args_size() { return sizeof(TcArgs); }
 void leg_tc_fill_args(const sht_plan_s *P, int polar, void *out) {
   TcArgs ta;
   leg_mixed_fill_args(P, polar, &ta.m);
-  ta.lam_bound = P->tc_lam_bound;
   ta.err = P->d_err;
   memcpy(out, &ta, sizeof(ta));
 }
@@ -680,7 +690,6 @@ cudaError_t launch_leg_tc_syn(const sht_plan_s *P, const void *mixargs, int n, c
   if (n == 0) return cudaSuccess;
   TcArgs ta;
   memcpy(&ta.m, mixargs, sizeof(MixArgs));
-  ta.lam_bound = P->tc_lam_bound;
   ta.err = P->d_err;
   const int nj = P->njobs_pad;
   if (P->spin == 0) {

@@ -701,7 +701,6 @@ cudaError_t launch_leg_tc_ana(const sht_plan_s *P, const void *mixargs, int n, c
   if (n == 0) return cudaSuccess;
   TcArgs ta;
   memcpy(&ta.m, mixargs, sizeof(MixArgs));
-  ta.lam_bound = P->tc_lam_bound;
   ta.err = P->d_err;
   const int nj = P->njobs_pad;
   if (P->spin == 0) {

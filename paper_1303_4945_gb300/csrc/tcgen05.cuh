@@ -157,7 +157,6 @@ __device__ __forceinline__ float pow2_above(float x) {
 
 struct TcArgs {
   MixArgs m;        // tables, work items and phase array of the mixed form
-  float lam_bound;  // power of two bounding |Lambda_lm| over the plan
   int *err;         // device status word: bit 0 set when a bounded wait gave up
 };
 
