@@ -117,8 +117,8 @@ int build(sht_batch_s *B) {
   auto join = [&](int k, int precision, bool lo) {
     const sht_plan_s *P = B->plans[k];
     const int spin_class = P->spin ? 1 : 0;
-    const bool tc = precision == SHT_MIXED && P->tc_syn;
-    const bool tca = precision == SHT_MIXED && P->tc_ana;
+    const bool tc = precision == SHT_MIXED ? P->tc_syn != 0 : (!lo && P->tc64_syn);
+    const bool tca = precision == SHT_MIXED ? P->tc_ana != 0 : (!lo && P->tc64_ana);
     Group *g = nullptr;
     for (auto &c : B->groups)
       if (c.precision == precision && c.spin == spin_class && c.nj == P->njobs_pad && c.ppt == P->ana_ppt &&
@@ -149,7 +149,7 @@ int build(sht_batch_s *B) {
     const size_t rec = mixed ? leg_mixed_args_size() : leg_fp64_args_size();
     for (int polar = 0; polar < 2; ++polar) {
       std::vector<unsigned char> args(rec * g.plans.size());
-      const bool tcrec = g.tc || g.tca;
+      const bool tcrec = mixed && (g.tc || g.tca);
       std::vector<unsigned char> targs(tcrec ? tc_args_size() * g.plans.size() : 0);
       std::vector<std::pair<int64_t, int4>> syn, ana;
       for (size_t i = 0; i < g.plans.size(); ++i) {
@@ -309,7 +309,9 @@ extern "C" int sht_batch_execute(sht_batch_t B, int type, double *const *const *
         if ((g.precision == SHT_MIXED) != mixed_groups || r != cudaSuccess) continue;
         const int4 *items = stage ? g.d_ana[polar] : g.d_syn[polar];
         const int ni = stage ? g.nana[polar] : g.nsyn[polar];
-        if (stage == 0 && g.tc)
+        if (!mixed_groups && (stage ? g.tca : g.tc))
+          r = launch_leg_tc64_batch(stage, g.spin, g.nj, g.d_args[polar], items, ni, s);
+        else if (stage == 0 && g.tc)
           r = launch_leg_tc_batch(g.spin, g.nj, g.d_targs[polar], items, ni, s);
         else if (stage == 1 && g.tca)
           r = launch_leg_tc_ana_batch(g.spin, g.nj, g.d_targs[polar], items, ni, s);

@@ -23,27 +23,9 @@
 // Enhanced exponent range (Sect. 4.1): the recursion pair is held as
 // y * 2^(600 scale); while scale < 0 the terms are below ~2^-300 and are not
 // accumulated; every 8 steps values above 2^300 are scaled down by 2^-600.
-#include "sht_device.cuh"
+#include "leg64.cuh"
 
 namespace sht {
-
-struct LegArgs {
-  int lmax, spin, npairs, nm, astride;
-  const int *mval;
-  const int64_t *mstart;
-  const int64_t *coef_off;
-  const double2 *coef;  // {a, b} of p_{l+1} = (a x + b) p_l - p_{l-1}
-  const double2 *pm;    // alpha_l times a_lm (spin: P = E + iB, M = E - iB) per (array, m, l), indexed like coef
-  int64_t ncoef;        // pm's entries per array
-  const double2 *mpre;
-  const PairDev *pairs;
-  double2 *phase;  // [nmaps][nm][npairs][2]
-  const int2 *syn_items;
-  const int4 *ana_items;
-  const int64_t *part_off;
-  double *part;
-  int ppt;
-};
 
 __device__ __forceinline__ int warp_any(bool b) { return __any_sync(0xffffffffu, b); }
 
@@ -780,6 +762,8 @@ static LegArgs make_args(const sht_plan_s *P, int polar, bool lo = false) {
   a.part_off = P->d_ana_part_off[polar];
   a.part = P->d_part;
   a.ppt = P->ana_ppt;
+  a.lexp = P->d_lexp;
+  a.err = P->d_err;
   return a;
 }
 
@@ -789,6 +773,7 @@ cudaError_t launch_leg_fp64_items(const sht_plan_s *P, int stage, int polar, con
                                   cudaStream_t st) {
   if (n == 0) return cudaSuccess;
   LegArgs a = make_args(P, polar);
+  if (stage == 0 ? P->tc64_syn : P->tc64_ana) return launch_leg_tc64_items(P, stage, &a, items, n, st);
   const int nj = P->njobs_pad;
   if (stage == 0) {
     a.syn_items = static_cast<const int2 *>(items);

@@ -841,7 +841,7 @@ static void free_plan(sht_plan_s *P) {
   cudaGetDevice(&cur);
   cudaSetDevice(P->device);
   void *ptrs[] = {P->d_pairs, P->d_pair_rings, P->d_rings, P->d_mval, P->d_mstart, P->d_coef_off,
-                  P->d_coef, P->d_alpha, P->d_coef32, P->d_alm32, P->d_pm64, P->d_mpre, P->d_minv, P->d_phase, P->d_part, P->d_fft,
+                  P->d_coef, P->d_alpha, P->d_lexp, P->d_coef32, P->d_alm32, P->d_pm64, P->d_mpre, P->d_minv, P->d_phase, P->d_part, P->d_fft,
                   P->d_pair_fft, P->d_fft_scratch, P->d_err, P->d_join};
   for (void *p : ptrs)
     if (p) cudaFree(p);
@@ -986,18 +986,18 @@ static int build_ana_lists(sht_plan_s *P, int ppt) {
   int rc;
   const int as = abs(P->spin);
   const int V = (P->spin ? 4 : 2) * P->njobs_pad;  // doubles per l in the analysis partials
-  const int TA = kAnaThreads * ppt;
+  const int TA = kAnaThreads * (P->tc64_ana ? 1 : ppt);
   const int tiles = (P->npairs + TA - 1) / TA;
   const bool mixed = P->precision == SHT_MIXED;
   int group = 1;
-  if (mixed) {  // tiles of the polar-cut variant (the default) over items per SM wanted
+  if (mixed || P->tc64_ana) {  // tiles of the polar-cut variant (the default) over items per SM wanted
     int64_t ntile = 0;
     for (int i = 0; i < P->nm; ++i)
       if (P->lmax >= std::max(P->mval[i], as)) ntile += tiles - P->first_pair[i] / TA;
     group = (int)std::max<int64_t>(1, std::min<int64_t>(kAnaGroupTiles, ntile / ((int64_t)kAnaItemsPerSm * P->sms)));
     // whole passes of the tensor-core analysis, which walks several tiles at a time
-    if (P->tc_ana) {
-      const int nt = tc_ana_tiles(P->spin, P->njobs_pad);
+    if (P->tc_ana || P->tc64_ana) {
+      const int nt = P->tc_ana ? tc_ana_tiles(P->spin, P->njobs_pad) : tc64_ana_tiles(P->spin, P->njobs_pad);
       group = (group + nt - 1) / nt * nt;
     }
   }
@@ -1054,6 +1054,20 @@ static int build_ana_lists(sht_plan_s *P, int ppt) {
   }
   P->ana_ppt = ppt;
   return SHT_OK;
+}
+
+// Where the FP64 form contracts on the tensor cores (legendre_tc64.cu): it leaves only
+// the recursions on the FP64 pipe but adds a fixed cost per block of degrees, so the
+// line lies where the longest column covers that, earlier the more arrays share a
+// recursion.  Measured on GB300 (Gauss-Legendre nlat = lmax + 1; FP64 contraction ->
+// tensor cores, us): synthesis, one array lmax 191 54 -> 64, 255 70 -> 59, 1023 1735 ->
+// 1194; two 127 70 -> 74, 191 114 -> 108, 767 2250 -> 1080; four 31 41 -> 39, 63 41 -> 37,
+// 767 3569 -> 1324; analysis, one 191 117 -> 119, 255 164 -> 158, 1023 2350 -> 1560; two
+// 31 36 -> 30, 767 3826 -> 1228; four 31 53 -> 31, 767 6277 -> 1506.
+static void tc64_choose(sht_plan_s *P) {
+  const int n = P->nmaps_pad;  // arrays per side
+  P->tc64_syn = tc64_syn_supported(P->spin, P->njobs_pad) && P->lmax >= (n == 1 ? 224 : (n == 2 ? 192 : 48));
+  P->tc64_ana = tc64_ana_supported(P->spin, P->njobs_pad) && P->lmax >= (n == 1 ? 208 : 24);
 }
 
 static int plan_build(sht_plan_s *P, const sht_geom_s *g) {
@@ -1143,6 +1157,16 @@ static int plan_build(sht_plan_s *P, const sht_geom_s *g) {
     P->tc_syn = tc_supported(P->spin, P->njobs_pad) && !(P->spin == 0 && P->njobs_pad == 1);
   }
   CUDA_TRY(launch_coef_tables(P, 0));
+  if (P->precision == SHT_FP64) {
+    tc64_choose(P);
+    if ((P->tc64_syn || P->tc64_ana) && P->nm > 0 && P->npairs > 0) {
+      CUDA_TRY(tc64_prepare_device());
+      const size_t bytes = (size_t)P->nm * P->npairs;
+      CUDA_TRY(cudaMalloc(&P->d_lexp, bytes));
+      P->workspace += bytes;
+      CUDA_TRY(launch_bounds64(P, 0));
+    }
+  }
   if (P->precision == SHT_MIXED && P->nm > 0 && P->npairs > 0) {
     // where each ring pair's terms start, per m (the mixed Legendre kernels skip
     // the recursion over the negligible stretch before it)
@@ -1286,7 +1310,8 @@ extern "C" int sht_plan_set_tiling(sht_plan_t P, int pairs_per_thread) {
   if (std::find(c.begin(), c.end(), pairs_per_thread) == c.end())
     return fail(SHT_ERR_UNSUPPORTED, "no analysis kernel with %d ring pairs per thread for this plan",
                 pairs_per_thread);
-  if (pairs_per_thread == P->ana_ppt) return SHT_OK;
+  if (pairs_per_thread == P->ana_ppt && !P->tc64_ana) return SHT_OK;
+  if (P->tc64_ana && !P->batch_refs) P->tc64_ana = 0;  // a tiling asked for is one of the FP64 kernel
   if (P->tc_ana)
     return fail(SHT_ERR_UNSUPPORTED, "the tensor-core analysis takes one ring pair per thread");
   return retile(P, pairs_per_thread);
@@ -1447,12 +1472,17 @@ extern "C" int sht_plan_autotune(sht_plan_t P, void *stream, float *ms_per_candi
   const bool tc_cand = P->precision == SHT_MIXED && tc_ana_supported(P->spin, P->njobs_pad);
   const size_t ncand = cands.size() + (tc_cand ? 1 : 0);
   int best_tc = P->tc_ana;
+  // an FP64 plan's tensor-core analysis is timed too, last, without a time of its own
+  const bool t64 = P->precision == SHT_FP64 && P->tc64_ana;
+  const size_t ncand64 = ncand + (t64 ? 1 : 0);
+  P->tc64_ana = 0;
   if (ms_per_candidate)
     for (size_t i = 0; i <= cands.size(); ++i) ms_per_candidate[i] = 0.f;
-  for (size_t i = 0; i < ncand && e == cudaSuccess && rc == SHT_OK; ++i) {
-    const bool tc = i == cands.size();
-    const int ppt = tc ? 1 : cands[i];
+  for (size_t i = 0; i < ncand64 && e == cudaSuccess && rc == SHT_OK; ++i) {
+    const bool tc = !t64 && i == cands.size();
+    const int ppt = tc ? 1 : (i < cands.size() ? cands[i] : best);
     P->tc_ana = tc ? 1 : 0;
+    P->tc64_ana = t64 && i == cands.size();
     if ((rc = build_ana_lists(P, ppt)) != SHT_OK) break;
     // one untimed and two timed runs of the analysis Legendre stage (polar cut on)
     for (int it = 0; it < 3 && e == cudaSuccess; ++it) {
@@ -1465,6 +1495,13 @@ extern "C" int sht_plan_autotune(sht_plan_t P, void *stream, float *ms_per_candi
     if (e == cudaSuccess) e = cudaEventSynchronize(ev[1]);
     float ms = 0.f;
     if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, ev[0], ev[1]);
+    if (P->tc64_ana) {  // keep it, or return to the fastest tiling
+      if (ms >= best_ms) {
+        P->tc64_ana = 0;
+        rc = build_ana_lists(P, best);
+      }
+      break;
+    }
     if (ms_per_candidate) ms_per_candidate[i] = ms / 2;
     if (e == cudaSuccess && (i == 0 || ms < best_ms)) {
       best_ms = ms;

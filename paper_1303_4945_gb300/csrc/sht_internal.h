@@ -172,6 +172,11 @@ struct sht_plan_s {
   // tiles of kAnaThreads ring pairs, one per thread)
   int tc_ana = 0;
   float tc_lam_bound = 0.f;  // power of two bounding |Lambda_lm| for lmax
+  // FP64 plans: the contractions on the tensor cores (legendre_tc64.cu), for shapes and
+  // sizes where they are faster (tc64_choose in sht_host.cu); d_lexp: per (m index, pair)
+  // the exponent of a power of two bounding the recursion's values
+  int tc64_syn = 0, tc64_ana = 0;
+  signed char *d_lexp = nullptr;
   int *d_err = nullptr;      // device status word written by kernels with bounded waits
   float4 *d_join = nullptr;  // mixed plans: join record per (m index, pair), 3 float4 each
   int64_t triples_joined = 0;  // steps from each kept pair's join block on (polar cut applied)
@@ -250,6 +255,16 @@ cudaError_t launch_leg_ana_fp64(const sht_plan_s *P, int polar, cudaStream_t st,
 // grad: the gradient factor of Sect. 4.5's adjoint for the stored m >= 0 a_lm (m > 0 doubled)
 cudaError_t launch_ana_reduce(const sht_plan_s *P, const DevPtrs &alm, int polar, int add, cudaStream_t st,
                               bool real = false, bool grad = false);
+// FP64 form with the contraction on the tensor cores (legendre_tc64.cu); legargs: LegArgs
+cudaError_t launch_leg_tc64_items(const sht_plan_s *P, int stage, const void *legargs, const void *items, int n,
+                                  cudaStream_t st);
+cudaError_t launch_leg_tc64_batch(int stage, int spin, int nj, const void *args, const int4 *items, int n,
+                                  cudaStream_t st);
+cudaError_t launch_bounds64(const sht_plan_s *P, cudaStream_t st);
+cudaError_t tc64_prepare_device();
+bool tc64_syn_supported(int spin, int njobs_pad);
+bool tc64_ana_supported(int spin, int njobs_pad);
+int tc64_ana_tiles(int spin, int njobs_pad);
 cudaError_t launch_leg_syn_mixed(const sht_plan_s *P, const DevPtrs &alm, int polar, cudaStream_t st, int mode = 0);
 // the Legendre stage over an explicit work list (stage 0 synthesis, 1 analysis), no a_lm conversion
 cudaError_t launch_leg_fp64_items(const sht_plan_s *P, int stage, int polar, const void *items, int n,
