@@ -42,6 +42,14 @@ struct Group {
   int nana[2] = {0, 0};
 };
 
+// plans whose ring FFTs run the same engine with the same CTA size (as in their own calls)
+struct FftGroup {
+  bool df = false;
+  int threads = 0, smem = 0, n = 0;
+  int4 *d_items = nullptr;  // (pair, map, -, plan)
+  std::vector<std::pair<int64_t, int4>> items;
+};
+
 }  // namespace
 
 struct sht_batch_s {
@@ -51,9 +59,7 @@ struct sht_batch_s {
   std::vector<Group> groups;
   void *d_fft_syn[2][2][2] = {};  // [polar][weighted][add]: FFT argument records
   void *d_fft_ana[2] = {};        // [weighted]
-  int4 *d_fft_items[2] = {};      // (pair, map, -, plan) by FFT engine: FP64 [0], double-float [1]
-  int nfft_items[2] = {};
-  int fft_smem = 0;
+  std::vector<FftGroup> fft;      // ring FFTs, one launch per group and stage
   std::vector<void *> allocs;
   // FP64 groups run beside mixed groups: a side stream forked and joined by events
   cudaStream_t side = nullptr;
@@ -191,20 +197,30 @@ int build(sht_batch_s *B) {
     for (int k = 0; k < n; ++k) fft_fill_args(B->plans[k], 1, w, 0, B->ptr_off[k], args.data() + k * rec);
     if (e == cudaSuccess) e = upload_bytes(B, args, &B->d_fft_ana[w]);
   }
-  std::vector<std::pair<int64_t, int4>> fi[2];  // by engine: FP64, double-float
   for (int k = 0; k < n; ++k) {
     const sht_plan_s *P = B->plans[k];
-    B->fft_smem = std::max(B->fft_smem, P->fft_smem);
-    const int df = P->fft_df ? 1 : 0;
+    FftGroup *g = nullptr;
+    for (auto &c : B->fft)
+      if (c.df == P->fft_df && c.threads == P->fft_threads) g = &c;
+    if (!g) {
+      B->fft.emplace_back();
+      g = &B->fft.back();
+      g->df = P->fft_df;
+      g->threads = P->fft_threads;
+    }
+    g->smem = std::max(g->smem, P->fft_smem);
     for (int p = 0; p < P->npairs; ++p)
-      for (int j = 0; j < P->nmaps; ++j) fi[df].push_back({(int64_t)P->pair_len[p], make_int4(p, j, 0, k)});
+      for (int j = 0; j < P->nmaps; ++j) g->items.push_back({(int64_t)P->pair_len[p], make_int4(p, j, 0, k)});
   }
-  for (int df = 0; df < 2; ++df) {
-    sort_by_cost(fi[df]);
-    auto fv = strip(fi[df]);
-    B->nfft_items[df] = (int)fv.size();
-    if (e == cudaSuccess && !fv.empty()) e = upload(B, fv.data(), fv.size(), &B->d_fft_items[df]);
+  for (auto &g : B->fft) {
+    sort_by_cost(g.items);
+    auto fv = strip(g.items);
+    g.items.clear();
+    g.n = (int)fv.size();
+    if (e == cudaSuccess && !fv.empty()) e = upload(B, fv.data(), fv.size(), &g.d_items);
   }
+  // the groups of the longest rings first
+  std::stable_sort(B->fft.begin(), B->fft.end(), [](const FftGroup &a, const FftGroup &b) { return a.smem > b.smem; });
   int least = 0, greatest = 0;
   if (e == cudaSuccess) e = cudaDeviceGetStreamPriorityRange(&least, &greatest);
   if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&B->side, cudaStreamNonBlocking, greatest);
@@ -336,13 +352,14 @@ extern "C" int sht_batch_execute(sht_batch_t B, int type, double *const *const *
         e = launch_alm_prepare_fp64(P, A[k], st);
     }
     if (e == cudaSuccess) e = legendre(0);
-    for (int df = 0; df < 2 && e == cudaSuccess; ++df)
-      e = launch_fft_batch(0, df, B->d_fft_syn[polar][weighted][add], B->d_fft_items[df], B->nfft_items[df],
-                           B->fft_smem, TM, st);
+    for (auto &g : B->fft)
+      if (e == cudaSuccess)
+        e = launch_fft_batch(0, g.df, B->d_fft_syn[polar][weighted][add], g.d_items, g.n, g.threads, g.smem, TM, st);
   } else {
     const int weighted = type == SHT_ANALYSIS;
-    for (int df = 0; df < 2 && e == cudaSuccess; ++df)
-      e = launch_fft_batch(1, df, B->d_fft_ana[weighted], B->d_fft_items[df], B->nfft_items[df], B->fft_smem, TM, st);
+    for (auto &g : B->fft)
+      if (e == cudaSuccess)
+        e = launch_fft_batch(1, g.df, B->d_fft_ana[weighted], g.d_items, g.n, g.threads, g.smem, TM, st);
     if (e == cudaSuccess) e = legendre(1);
     for (int k = 0; k < n && e == cudaSuccess; ++k) e = launch_ana_reduce(B->plans[k], A[k], polar, add, st);
   }

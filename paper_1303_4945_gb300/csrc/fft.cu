@@ -766,6 +766,18 @@ __global__ void __launch_bounds__(kFftThreads) fft_ana_kernel_global(FftArgs a, 
   }
 }
 
+// A ring transform is a chain of passes with a barrier each, and the kernels use 128
+// registers a thread: 512 threads leave room for one CTA per SM, which idles at every
+// barrier.  Smaller CTAs let two or four rings share an SM wherever their buffers fit
+// (16 bytes a point).  Measured (synthesis + analysis, us, 512 / 256 / 128 threads): 612
+// points (Rader 613) 133 / 114 / 88; 1024 FP64 384 / 308 / 295; 2047 FP64 881 / 764 / 769; 2048
+// (HEALPix Nside 512) 667 / 581 / 690; 4095, eight maps 4306 / 3655 / 3967; 6006 1027 / 1004 /
+// 1479.
+int fft_cta_threads(int len) {
+  if (len <= 1024) return kFftThreads / 4;
+  return 2 * (len * (int)sizeof(double2) + 2048) <= 227 * 1024 ? kFftThreads / 2 : kFftThreads;
+}
+
 static FftArgs make_fft_args(const sht_plan_s *P, const DevPtrs &map, int polar) {
   FftArgs a;
   a.nm = P->nm;
@@ -810,9 +822,9 @@ cudaError_t launch_fft_syn(const sht_plan_s *P, const DevPtrs &map, int polar, i
   }
   dim3 grid(a.npairs_run, P->nmaps);
   if (df)
-    fft_syn_kernel<DF><<<grid, kFftThreads, P->fft_smem, st>>>(a);
+    fft_syn_kernel<DF><<<grid, P->fft_threads, P->fft_smem, st>>>(a);
   else
-    fft_syn_kernel<F64><<<grid, kFftThreads, P->fft_smem, st>>>(a);
+    fft_syn_kernel<F64><<<grid, P->fft_threads, P->fft_smem, st>>>(a);
   return cudaGetLastError();
 }
 
@@ -835,9 +847,9 @@ cudaError_t launch_fft_ana(const sht_plan_s *P, const DevPtrs &map, int weighted
   }
   dim3 grid(a.npairs_run, P->nmaps);
   if (df)
-    fft_ana_kernel<DF><<<grid, kFftThreads, P->fft_smem, st>>>(a);
+    fft_ana_kernel<DF><<<grid, P->fft_threads, P->fft_smem, st>>>(a);
   else
-    fft_ana_kernel<F64><<<grid, kFftThreads, P->fft_smem, st>>>(a);
+    fft_ana_kernel<F64><<<grid, P->fft_threads, P->fft_smem, st>>>(a);
   return cudaGetLastError();
 }
 
@@ -902,20 +914,20 @@ cudaError_t fft_prepare_device(int device) {
 
 // synthesis (stage 0) or analysis (stage 1) ring FFTs of every item (pair, map, -, args index),
 // in double-float (df: items of mixed plans) or FP64
-cudaError_t launch_fft_batch(int stage, bool df, const void *args, const int4 *items, int n, int smem,
+cudaError_t launch_fft_batch(int stage, bool df, const void *args, const int4 *items, int n, int threads, int smem,
                              const PtrTable &tbl, cudaStream_t st) {
   if (n == 0) return cudaSuccess;
   const FftArgs *a = static_cast<const FftArgs *>(args);
   if (stage == 0) {
     if (df)
-      fft_syn_kernel_batch<DF><<<n, kFftThreads, smem, st>>>(a, items, tbl);
+      fft_syn_kernel_batch<DF><<<n, threads, smem, st>>>(a, items, tbl);
     else
-      fft_syn_kernel_batch<F64><<<n, kFftThreads, smem, st>>>(a, items, tbl);
+      fft_syn_kernel_batch<F64><<<n, threads, smem, st>>>(a, items, tbl);
   } else {
     if (df)
-      fft_ana_kernel_batch<DF><<<n, kFftThreads, smem, st>>>(a, items, tbl);
+      fft_ana_kernel_batch<DF><<<n, threads, smem, st>>>(a, items, tbl);
     else
-      fft_ana_kernel_batch<F64><<<n, kFftThreads, smem, st>>>(a, items, tbl);
+      fft_ana_kernel_batch<F64><<<n, threads, smem, st>>>(a, items, tbl);
   }
   return cudaGetLastError();
 }

@@ -1235,6 +1235,7 @@ static int plan_build(sht_plan_s *P, const sht_geom_s *g) {
   if ((rc = upload(P, pf, &P->d_pair_fft)) != SHT_OK) return rc;
   if (maxlen <= kFftMaxLen) {
     P->fft_smem = maxlen * (int)sizeof(double2);
+    P->fft_threads = fft_cta_threads(maxlen);
   } else {  // rings beyond shared memory: one L2-resident scratch slot per SM (one CTA each)
     int sms = 0;
     CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, P->device));
