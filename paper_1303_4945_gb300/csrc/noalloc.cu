@@ -10,10 +10,11 @@
 // the analysis tile sums and the converted a_lm tables (both, for a mixed plan
 // with FP64 columns) -- from one fixed area compiled into the library
 // (kNoallocBytes below), so the call itself makes no allocation of any kind.
-// Two things still come from the plan, both allocated once when the plan was
-// made: its read-only tables (recursion coefficients, ring pairs, work lists,
-// FFT twiddles) and, for rings longer than the in-shared-memory limit
-// (kFftMaxLen points), its FFT scratch slots.  The plan's workspace pointers
+// What still comes from the plan was allocated when the plan was made: its read-only
+// tables (recursion coefficients, ring pairs, work lists, FFT twiddles), the scaled
+// spin-0 a_lm of FP64 kernels, tile sums too large for the rest of the area and, for
+// rings longer than the in-shared-memory limit (kFftMaxLen points), its FFT scratch
+// slots.  The plan's workspace pointers
 // are swapped to the area for the length of the call and restored on return,
 // so no other call on the same plan (sht_execute included) may run
 // concurrently from another thread.  Every GPU that loads the library holds
@@ -80,7 +81,9 @@ extern "C" int sht_execute_noalloc(sht_plan_t P, int type, double *const *alm, d
   const bool lo = mixed && (P->nsyn_lo[0] || P->nsyn_lo[1]);  // mixed plan with FP64 columns
   const int64_t b_pm64 =
       (synth && P->spin && (!mixed || lo)) ? align256(P->ncoef64 * P->nmaps_pad * (int64_t)sizeof(double2)) : 0;
-  const int64_t need = b_phase + b_part + b_alm32 + b_pm64;
+  // the limit is one of the transform, not of the tiling that its kernel takes: partial
+  // sums beyond the area are the plan's own
+  const int64_t need = b_phase + (synth ? 0 : align256(P->part_limit * (int64_t)sizeof(double))) + b_alm32 + b_pm64;
   if (need > kNoallocBytes)
     return set_error(SHT_ERR_UNSUPPORTED, "this transform needs %lld bytes of working memory; the static area holds %lld",
                      (long long)need, (long long)kNoallocBytes);
@@ -114,7 +117,7 @@ extern "C" int sht_execute_noalloc(sht_plan_t P, int type, double *const *alm, d
   float4 *alm320 = P->d_alm32;
   double2 *pm640 = P->d_pm64;
   P->d_phase = reinterpret_cast<double2 *>(base);
-  if (b_part) P->d_part = reinterpret_cast<double *>(base + b_phase);
+  if (b_part && b_phase + b_part <= kNoallocBytes) P->d_part = reinterpret_cast<double *>(base + b_phase);
   if (b_alm32) P->d_alm32 = reinterpret_cast<float4 *>(base + b_phase);
   if (b_pm64) P->d_pm64 = reinterpret_cast<double2 *>(base + b_phase + b_alm32);
   cudaStream_t st = (cudaStream_t)stream;

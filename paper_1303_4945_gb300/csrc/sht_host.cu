@@ -876,10 +876,12 @@ static int upload(sht_plan_s *P, const std::vector<T> &h, T **d) {
 }
 
 // Tilings of the analysis Legendre kernels (ring pairs per thread) built for a
-// spin class and padded job count; the first is the default.
-static std::vector<int> ana_ppt_candidates(int spin, int nj) {
+// spin class and padded job count; the first is the default.  One spin-0 map: two pairs a
+// thread in the mixed form (lmax 4095 22.6 ms against 24.7 at four, lmax 1535 on HEALPix
+// 1.89 against 2.53: four spill), four in FP64.
+static std::vector<int> ana_ppt_candidates(int spin, int nj, int precision) {
   if (spin == 0) {
-    if (nj == 1) return {4, 8, 2};
+    if (nj == 1) return precision == SHT_MIXED ? std::vector<int>{2, 4, 8} : std::vector<int>{4, 8, 2};
     if (nj == 2) return {4, 2};
     return {2};
   }
@@ -979,6 +981,39 @@ static int build_syn_lists(sht_plan_s *P) {
 // GB300 at lmax 4095 is as fast as one CTA per tile (152.5 against 153.0 ms per
 // pair) with a sixteenth of the partials; an 8-map plan's analysis kernel is 4.4
 // ms slower grouped, its slot reduction 6.6 ms faster (lmax 4095: 157.3 + 1.1
+// items of consecutive tiles of TA ring pairs: the tiles per item, whole passes of nt
+static int ana_group(const sht_plan_s *P, int TA, int nt) {
+  const int tiles = (P->npairs + TA - 1) / TA, as = abs(P->spin);
+  int64_t ntile = 0;  // tiles of the polar-cut variant (the default) over items per SM wanted
+  for (int i = 0; i < P->nm; ++i)
+    if (P->lmax >= std::max(P->mval[i], as)) ntile += tiles - P->first_pair[i] / TA;
+  const int group =
+      (int)std::max<int64_t>(1, std::min<int64_t>(kAnaGroupTiles, ntile / ((int64_t)kAnaItemsPerSm * P->sms)));
+  return (group + nt - 1) / nt * nt;
+}
+
+// the tiles of m index i's item that starts at tile t, and whether it runs in FP64
+static int ana_item_tiles(const sht_plan_s *P, int i, int t, int TA, int group, bool *lo) {
+  const int tiles = (P->npairs + TA - 1) / TA;
+  *lo = lo_item(P, i, t * TA, (t + 1) * TA);
+  int n = 1;
+  if (!*lo)
+    while (n < group && t + n < tiles && !lo_item(P, i, (t + n) * TA, (t + n + 1) * TA)) ++n;
+  return n;
+}
+
+// doubles of partial sums that a tiling takes
+static int64_t ana_part_need(const sht_plan_s *P, int TA, int group) {
+  const int tiles = (P->npairs + TA - 1) / TA, V = (P->spin ? 4 : 2) * P->njobs_pad;
+  int64_t off = 0;  // without the polar cut every m takes as many slots or more
+  for (int i = 0; i < P->nm; ++i) {
+    const int nl = P->lmax - std::max(P->mval[i], abs(P->spin)) + 1;
+    bool lo;
+    for (int t = 0; nl > 0 && t < tiles; t += ana_item_tiles(P, i, t, TA, group, &lo)) off += (int64_t)nl * V;
+  }
+  return off;
+}
+
 // against 152.9 + 7.7 ms).  FP64 items (the FP64 form, and a mixed plan's tiles
 // next to the poles) take one tile each.  Item (m index, first tile,
 // slot << 8 | tiles, -); the slots of m are summed by the reduction kernel.
@@ -989,18 +1024,11 @@ static int build_ana_lists(sht_plan_s *P, int ppt) {
   const int TA = kAnaThreads * (P->tc64_ana ? 1 : ppt);
   const int tiles = (P->npairs + TA - 1) / TA;
   const bool mixed = P->precision == SHT_MIXED;
-  int group = 1;
-  if (mixed || P->tc64_ana) {  // tiles of the polar-cut variant (the default) over items per SM wanted
-    int64_t ntile = 0;
-    for (int i = 0; i < P->nm; ++i)
-      if (P->lmax >= std::max(P->mval[i], as)) ntile += tiles - P->first_pair[i] / TA;
-    group = (int)std::max<int64_t>(1, std::min<int64_t>(kAnaGroupTiles, ntile / ((int64_t)kAnaItemsPerSm * P->sms)));
-    // whole passes of the tensor-core analysis, which walks several tiles at a time
-    if (P->tc_ana || P->tc64_ana) {
-      const int nt = P->tc_ana ? tc_ana_tiles(P->spin, P->njobs_pad) : tc64_ana_tiles(P->spin, P->njobs_pad);
-      group = (group + nt - 1) / nt * nt;
-    }
-  }
+  // whole passes of a tensor-core analysis, which walks several tiles at a time
+  const int nt = P->tc_ana     ? tc_ana_tiles(P->spin, P->njobs_pad)
+                 : P->tc64_ana ? tc64_ana_tiles(P->spin, P->njobs_pad)
+                               : 1;
+  const int group = mixed || P->tc64_ana ? ana_group(P, TA, nt) : 1;
   int64_t need = 0;
   for (int polar = 0; polar < 2; ++polar) {
     std::vector<std::pair<int64_t, int4>> ana, lo;
@@ -1015,17 +1043,10 @@ static int build_ana_lists(sht_plan_s *P, int ppt) {
       int fp = polar ? P->first_pair[i] : 0;
       int slot = 0;
       for (int t = fp / TA; t < tiles;) {
-        const auto cost = [&](int tt) { return (int64_t)nl * std::min(TA, P->npairs - tt * TA); };
-        if (lo_item(P, i, t * TA, (t + 1) * TA)) {
-          lo.push_back({cost(t), make_int4(i, t, (slot << 8) | 1, 0)});
-          ++t;
-        } else {
-          int n = 0;
-          int64_t c = 0;
-          while (n < group && t + n < tiles && !lo_item(P, i, (t + n) * TA, (t + n + 1) * TA)) c += cost(t + n++);
-          ana.push_back({c, make_int4(i, t, (slot << 8) | n, 0)});
-          t += n;
-        }
+        bool l;
+        const int n = ana_item_tiles(P, i, t, TA, group, &l);
+        (l ? lo : ana).push_back({(int64_t)nl * (std::min(P->npairs, (t + n) * TA) - t * TA), make_int4(i, t, (slot << 8) | n, 0)});
+        t += n;
         ++slot;
       }
       nslot[i] = slot;
@@ -1063,6 +1084,13 @@ static int build_ana_lists(sht_plan_s *P, int ppt) {
 // tensor cores, us): synthesis, one array lmax 191 54 -> 64, 255 70 -> 59, 1023 1735 ->
 // 1194; two 127 70 -> 74, 191 114 -> 108, 767 2250 -> 1080; four 31 41 -> 39, 63 41 -> 37,
 // 767 3569 -> 1324; analysis, one 191 117 -> 119, 255 164 -> 158, 1023 2350 -> 1560; two
+  // What the call that allocates nothing counts against its area: of the FP64 form the
+  // FP64 kernel's tiling, of one spin-0 map in the mixed form four pairs a thread until a
+  // tiling is chosen, whichever tiles run
+  P->part_limit = need;
+  if (P->tc64_ana) P->part_limit = ana_part_need(P, kAnaThreads * ppt, 1);
+  else if (mixed && P->spin == 0 && P->njobs_pad == 1 && !P->tc_ana && !P->tiling_chosen)
+    P->part_limit = ana_part_need(P, kAnaThreads * 4, ana_group(P, kAnaThreads * 4, 1));
 // 31 36 -> 30, 767 3826 -> 1228; four 31 53 -> 31, 767 6277 -> 1506.
 static void tc64_choose(sht_plan_s *P) {
   const int n = P->nmaps_pad;  // arrays per side
@@ -1203,7 +1231,7 @@ static int plan_build(sht_plan_s *P, const sht_geom_s *g) {
       CUDA_TRY(cudaEventCreateWithFlags(ev, cudaEventDisableTiming));
   }
   if ((rc = build_syn_lists(P)) != SHT_OK) return rc;
-  if ((rc = build_ana_lists(P, ana_ppt_candidates(P->spin, P->njobs_pad)[0])) != SHT_OK) return rc;
+  if ((rc = build_ana_lists(P, ana_ppt_candidates(P->spin, P->njobs_pad, P->precision)[0])) != SHT_OK) return rc;
 
   // ---- phase-array workspace F/G [nmaps][nm][npairs][2] ----
   size_t nph = (size_t)P->nmaps_pad * P->nm * P->npairs * 2;
@@ -1307,11 +1335,18 @@ static int retile(sht_plan_s *P, int ppt) {
 
 extern "C" int sht_plan_set_tiling(sht_plan_t P, int pairs_per_thread) {
   if (!P) return fail(SHT_ERR_INVALID_ARG, "plan is NULL");
-  const auto c = ana_ppt_candidates(P->spin, P->njobs_pad);
+  const auto c = ana_ppt_candidates(P->spin, P->njobs_pad, P->precision);
   if (std::find(c.begin(), c.end(), pairs_per_thread) == c.end())
     return fail(SHT_ERR_UNSUPPORTED, "no analysis kernel with %d ring pairs per thread for this plan",
                 pairs_per_thread);
-  if (pairs_per_thread == P->ana_ppt && !P->tc64_ana) return SHT_OK;
+  if (pairs_per_thread == P->ana_ppt && !P->tc64_ana) {
+    if (!P->batch_refs) {
+      P->tiling_chosen = 1;
+      P->part_limit = P->part_doubles;
+    }
+    return SHT_OK;
+  }
+  if (!P->batch_refs) P->tiling_chosen = 1;
   if (P->tc64_ana && !P->batch_refs) P->tc64_ana = 0;  // a tiling asked for is one of the FP64 kernel
   if (P->tc_ana)
     return fail(SHT_ERR_UNSUPPORTED, "the tensor-core analysis takes one ring pair per thread");
@@ -1321,7 +1356,7 @@ extern "C" int sht_plan_set_tiling(sht_plan_t P, int pairs_per_thread) {
 extern "C" int sht_plan_get_tiling(sht_plan_t P, int *pairs_per_thread, int *ncandidates, int *candidates) {
   if (!P || !pairs_per_thread) return fail(SHT_ERR_INVALID_ARG, "NULL argument");
   *pairs_per_thread = P->ana_ppt;
-  const auto c = ana_ppt_candidates(P->spin, P->njobs_pad);
+  const auto c = ana_ppt_candidates(P->spin, P->njobs_pad, P->precision);
   if (ncandidates) *ncandidates = (int)c.size();
   if (candidates)
     for (size_t i = 0; i < c.size(); ++i) candidates[i] = c[i];
@@ -1459,7 +1494,8 @@ extern "C" int sht_plan_autotune(sht_plan_t P, void *stream, float *ms_per_candi
   cudaGetDevice(&cur);
   if (cur != P->device) CUDA_TRY(cudaSetDevice(P->device));
   cudaStream_t st = (cudaStream_t)stream;
-  const auto cands = ana_ppt_candidates(P->spin, P->njobs_pad);
+  const auto cands = ana_ppt_candidates(P->spin, P->njobs_pad, P->precision);
+  P->tiling_chosen = 1;
   // the analysis kernels read the phase array: give it defined contents
   const size_t nph = (size_t)P->nmaps_pad * P->nm * P->npairs * 2;
   cudaEvent_t ev[2] = {nullptr, nullptr};

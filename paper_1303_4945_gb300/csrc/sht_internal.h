@@ -147,6 +147,8 @@ struct sht_plan_s {
   double *d_part = nullptr;                // analysis partials
   int64_t part_doubles = 0;
 
+  int64_t part_limit = 0;  // of them, what sht_execute_noalloc counts (sht_host.cu)
+  int tiling_chosen = 0;   // a call chose the analysis tiling
   // work lists (polar-cut / uncut): synthesis (mi, first pair) and analysis (mi, tile, part offset)
   int2 *d_syn_items[2] = {nullptr, nullptr};
   int nsyn_items[2] = {0, 0};
