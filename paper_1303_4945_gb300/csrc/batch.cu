@@ -31,6 +31,7 @@ namespace {
 struct Group {
   int precision = 0, spin = 0, nj = 1, ppt = 2;
   bool tc = false;                   // mixed plans whose synthesis runs on the tensor cores
+  bool two = false;                  // tensor-core synthesis items of up to two tiles
   bool tca = false;                  // mixed plans whose analysis runs on the tensor cores
   void *d_targs[2] = {nullptr, nullptr};  // per polar: their TcArgs records (tensor-core kernels)
   std::vector<int> plans;            // batch indices; item.w is the position in this list
@@ -124,11 +125,12 @@ int build(sht_batch_s *B) {
     const sht_plan_s *P = B->plans[k];
     const int spin_class = P->spin ? 1 : 0;
     const bool tc = precision == SHT_MIXED ? P->tc_syn != 0 : (!lo && P->tc64_syn);
+    const bool two = precision == SHT_MIXED && P->syn_two;
     const bool tca = precision == SHT_MIXED ? P->tc_ana != 0 : (!lo && P->tc64_ana);
     Group *g = nullptr;
     for (auto &c : B->groups)
       if (c.precision == precision && c.spin == spin_class && c.nj == P->njobs_pad && c.ppt == P->ana_ppt &&
-          c.tc == tc && c.tca == tca)
+          c.tc == tc && c.tca == tca && c.two == two)
         g = &c;
     if (!g) {
       B->groups.emplace_back();
@@ -139,6 +141,7 @@ int build(sht_batch_s *B) {
       g->ppt = P->ana_ppt;
       g->tc = tc;
       g->tca = tca;
+      g->two = two;
     }
     g->plans.push_back(k);
     g->lo.push_back(lo ? 1 : 0);
@@ -328,7 +331,7 @@ extern "C" int sht_batch_execute(sht_batch_t B, int type, double *const *const *
         if (!mixed_groups && (stage ? g.tca : g.tc))
           r = launch_leg_tc64_batch(stage, g.spin, g.nj, g.d_args[polar], items, ni, s);
         else if (stage == 0 && g.tc)
-          r = launch_leg_tc_batch(g.spin, g.nj, g.d_targs[polar], items, ni, s);
+          r = launch_leg_tc_batch(g.spin, g.nj, g.two, g.d_targs[polar], items, ni, s);
         else if (stage == 1 && g.tca)
           r = launch_leg_tc_ana_batch(g.spin, g.nj, g.d_targs[polar], items, ni, s);
         else

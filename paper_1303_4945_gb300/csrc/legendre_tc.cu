@@ -77,19 +77,26 @@ constexpr int kIssuerWarp = 3;
 // digit -1 zero: Lambda digit i meets the windows of digits
 // (j0, j0 + 1) with j0 = -(i mod 2), j0 + 2, ..., which start on even levels i + j0,
 // so every MMA writes the 2 NCW columns of a level pair at a multiple of N.
-template <int NJ, bool SPIN>
+//
+// TWO (spin 0, one or two maps): a thread runs two neighbouring pairs as the two lanes
+// of Dual, whose digits are two A sets meeting the same B in accumulators of their own.
+template <int NJ, bool SPIN, bool TWO>
 struct Shape {
-  static constexpr int NL = SPIN ? 2 : 1;
+  static constexpr bool DUAL = TWO;
+  static constexpr int NP = DUAL ? 2 : 1;         // ring pairs per thread
+  static constexpr int NL = SPIN || DUAL ? 2 : 1; // A sets
+  static constexpr int NB = SPIN ? 2 : 1;         // B stacks
   static constexpr int NCOL = SPIN ? 8 * NJ : 4 * NJ;
   static constexpr int NCW = NCOL < 8 ? 8 : NCOL;
   static constexpr int N = 2 * NCW;
   static constexpr int NDT = kAlmDigits + 1;  // digit tiles per Lambda set: -1 .. 5
-  static constexpr int COLS = kLevels * NCW;  // TMEM: levels 0 .. 5
+  static constexpr int COLS1 = kLevels * NCW; // TMEM: levels 0 .. 5
+  static constexpr int COLS = NP * COLS1;
   static constexpr int TCOLS = COLS <= 32 ? 32 : (COLS <= 64 ? 64 : (COLS <= 128 ? 128 : 256));
   static constexpr int NV = SPIN ? 4 * NJ : 2 * NJ;
   static constexpr int DTILE = NCW * kK * 2;  // bytes of one a_lm digit tile
   static constexpr int A_BYTES = NL * kLamDigits * kATile;
-  static constexpr int B_BYTES = NL * NDT * DTILE;
+  static constexpr int B_BYTES = NB * NDT * DTILE;
   // per degree of a K-step, staged in shared memory one K-step ahead: the float4
   // of its recursion coefficients and one float4 per a_lm table row read
   static constexpr int NARR = SPIN ? 2 * NJ : NJ;
@@ -97,7 +104,7 @@ struct Shape {
   static constexpr int STG = kK * ROW;                 // float4 per K-step
   static constexpr int PF = (STG + kRows - 1) / kRows;  // of them per thread
   static constexpr int ST_BYTES = 2 * STG * 16;        // two buffers
-  static constexpr int ACC_BYTES = NCOL * kRows * 8;  // the double-float column sums [col][pair]
+  static constexpr int ACC_BYTES = NP * NCOL * kRows * 8;  // the double-float column sums [pair of the thread][col][thread]
   static constexpr int SMEM = A_BYTES + ST_BYTES + B_BYTES + ACC_BYTES + 2 * NV * 4;
   // CTAs per SM the kernel is compiled for, and the dynamic shared memory
   // requested: at least enough that no more than 512 / TCOLS CTAs fit on an SM,
@@ -107,7 +114,8 @@ struct Shape {
   static constexpr int SMEM_LAUNCH = SMEM > SMEM_FLOOR ? SMEM : SMEM_FLOOR;
   static_assert(N % 16 == 0 && N <= 256 && NCW % 8 == 0, "MMA width; digit tiles of whole core-matrix rows");
   static_assert(kLevels % 2 == 0 && kLamDigits <= 3, "level pairs");
-  static_assert(COLS <= TCOLS, "TMEM allocation");
+  static_assert(COLS <= TCOLS && COLS1 % 2 == 0, "TMEM allocation");
+  static_assert(!TWO || (!SPIN && NJ <= 2), "two pairs a thread: spin 0, one or two maps");
   static_assert(NCOL <= 32, "tensor-core synthesis: at most 32 output columns");
   static_assert(128 % NV == 0, "a_lm values per degree must divide the CTA");
 };
@@ -137,7 +145,7 @@ __device__ __forceinline__ f2 staged_value(const float4 *row, int v) {
 // caller synchronises before the bounds are read.
 template <int NJ, bool SPIN>
 __device__ __forceinline__ void window_bounds(const MixArgs &a, int64_t co, int lw0, int lw1, float *umax) {
-  using S = Shape<NJ, SPIN>;
+  using S = Shape<NJ, SPIN, false>;
   const int v = threadIdx.x % S::NV;
   float mx = 0.f;
   for (int l = lw0 + (int)threadIdx.x / S::NV; l <= lw1; l += kRows / S::NV)
@@ -157,7 +165,7 @@ __device__ __forceinline__ void window_bounds(const MixArgs &a, int64_t co, int 
 // stay zero from the kernel's start.
 template <int NJ, bool SPIN>
 __device__ __forceinline__ void build_b(const float4 *stg, const float *umax, unsigned char *Bt) {
-  using S = Shape<NJ, SPIN>;
+  using S = Shape<NJ, SPIN, false>;
   // byte offset of (row r of the stack, degree k) in the K-major core-matrix layout
   auto at = [](int r, int k) { return (r / 8) * 256 + (r % 8) * 16 + (k / 8) * 128 + (k % 8) * 2; };
   for (int t = threadIdx.x; t < kK * S::NV; t += kRows) {
@@ -215,9 +223,9 @@ __device__ __forceinline__ void build_b(const float4 *stg, const float *umax, un
 // those of s l-, so both meet B rows holding P and s M.  All sums run on Lambda / u_p
 // (u_p the pair's bound) and are multiplied by u_p at the end.
 // ---------------------------------------------------------------------------
-template <int NJ, bool SPIN>
+template <int NJ, bool SPIN, bool TWO>
 __device__ __forceinline__ void tc_syn_body(const TcArgs &ta, const int2 item, unsigned char *smem) {
-  using S = tc::Shape<NJ, SPIN>;
+  using S = tc::Shape<NJ, SPIN, TWO>;
   constexpr int NL = S::NL, NCOL = S::NCOL;
   __shared__ __align__(8) uint64_t mbar;
   __shared__ uint32_t tslot;
@@ -226,8 +234,17 @@ __device__ __forceinline__ void tc_syn_body(const TcArgs &ta, const int2 item, u
   // the warp's number from a shuffle, so that the compiler sees it uniform
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
   const int mi = item.x;
-  const int p = item.y + tid;
-  const bool valid = p < a.npairs;
+  constexpr int NP = S::NP;
+  // the pairs of the item: one tile of kRows, or (DUAL) as many as kSynTwoTiles says
+  const int p0 = item.y & ~kSynTwoTiles, np = S::DUAL && (item.y & kSynTwoTiles) ? 2 * tc::kRows : tc::kRows;
+  int pr[NP], lj[NP];
+  bool valid[NP];
+  const float4 *jrec[NP];
+#pragma unroll
+  for (int t = 0; t < NP; ++t) {
+    pr[t] = p0 + NP * tid + t;
+    valid[t] = pr[t] < min(a.npairs, p0 + np);
+  }
   const int m = a.mval[mi];
   const int s = a.spin, as = s < 0 ? -s : s;
   const int l0 = m > as ? m : as, lmax = a.lmax;
@@ -237,7 +254,8 @@ __device__ __forceinline__ void tc_syn_body(const TcArgs &ta, const int2 item, u
   unsigned char *const Abuf = smem;
   float4 *const stage = reinterpret_cast<float4 *>(smem + S::A_BYTES);
   unsigned char *const Bt = smem + S::A_BYTES + S::ST_BYTES;
-  f2 *const accs = reinterpret_cast<f2 *>(Bt + S::B_BYTES);  // column c of this pair at accs[c * 128 + tid]
+  // column c of pair t of this thread at accs[(t NCOL + c) * 128 + tid]
+  f2 *const accs = reinterpret_cast<f2 *>(Bt + S::B_BYTES);
   float *const umax = reinterpret_cast<float *>(Bt + S::B_BYTES + S::ACC_BYTES);
 
   // the staged rows of K-step ks: thread t loads entries t, t + 128, ... (zero past lmax)
@@ -266,10 +284,14 @@ __device__ __forceinline__ void tc_syn_body(const TcArgs &ta, const int2 item, u
   __shared__ int kstart[tc::kRows / 32];
   // the K-step (block of 16 degrees) at which this pair's terms start (join record);
   // the CTA starts at its pairs' earliest
-  const float4 *jrec = a.join + ((size_t)mi * a.npairs + (valid ? p : 0)) * 3;
-  const int lj = valid ? __float_as_int(__ldg(jrec + 2).z) : lmax + 1;
+#pragma unroll
+  for (int t = 0; t < NP; ++t) {
+    jrec[t] = a.join + ((size_t)mi * a.npairs + (valid[t] ? pr[t] : 0)) * 3;
+    lj[t] = valid[t] ? __float_as_int(__ldg(jrec[t] + 2).z) : lmax + 1;
+  }
+  const int jmin = min(lj[0], lj[NP - 1]);
   {
-    const int kj = lj <= lmax ? (lj - l0) / tc::kK : nks;
+    const int kj = jmin <= lmax ? (jmin - l0) / tc::kK : nks;
     const int wmin = __reduce_min_sync(0xffffffffu, kj);
     if ((tid & 31) == 0) kstart[warp] = wmin;
   }
@@ -293,26 +315,35 @@ __device__ __forceinline__ void tc_syn_body(const TcArgs &ta, const int2 item, u
     stage_store(ks0);
   }
 #pragma unroll
-  for (int c = 0; c < NCOL; ++c) accs[c * tc::kRows + tid] = f2{0.f, 0.f};
+  for (int c = 0; c < NP * NCOL; ++c) accs[c * tc::kRows + tid] = f2{0.f, 0.f};
 
   // the recursions, on Lambda / u_p: zero until the pair joins (no terms, and a
-  // recursion of zeros).  Spin 0 runs one lane.
-  const PairDev pd = a.pairs[valid ? p : 0];
-  const bool polar = polar_warp(pd.x, valid);
-  Dual<true> rec;
-  rec.p = rec.q = d2{both(0.f), both(0.f)};
-  rec.x[0] = node_of(pd.x, polar);
-  int sc0 = 0, sc1 = 0;
-  const int lfast = SPIN ? fast_from(as, rec.x[0].h, valid, lmax) : 0;
-  float racc[NCOL];
+  // recursion of zeros).  Spin 0 without DUAL runs one lane.
+  double xd[NP];
+  bool near = false;
 #pragma unroll
-  for (int c = 0; c < NCOL; ++c) racc[c] = 0.f;
+  for (int t = 0; t < NP; ++t) {
+    xd[t] = a.pairs[valid[t] ? pr[t] : 0].x;
+    near = near || (valid[t] && 1.0 - xd[t] < 0.5 * kPolarTheta * kPolarTheta);
+  }
+  const bool polar = __any_sync(0xffffffffu, near);
+  Dual<!S::DUAL> rec;
+  rec.p = rec.q = d2{both(0.f), both(0.f)};
+#pragma unroll
+  for (int t = 0; t < NP; ++t) rec.x[t] = node_of(xd[t], polar);
+  int sc0 = 0, sc1 = 0;
+  const int lfast = SPIN ? fast_from(as, rec.x[0].h, valid[0], lmax) : 0;
+  float racc[NP][NCOL];
+#pragma unroll
+  for (int t = 0; t < NP; ++t)
+#pragma unroll
+    for (int c = 0; c < NCOL; ++c) racc[t][c] = 0.f;
   float2 wf = both(1.f);  // weights of the two lanes' values; scales change only at the rescale checks
   bool settled = false;   // every lane of the warp at scale 0 (warp-uniform; scales only rise)
 
   // one step of the recursions with a row's coefficients
   auto advance = [&](const StepMode mode, const float4 &c) {
-    if (SPIN) {
+    if (SPIN || S::DUAL) {
       rec.step(mode, c);
     } else {
       f2 lc = lane0(rec.p), lp = lane0(rec.q);
@@ -338,18 +369,18 @@ __device__ __forceinline__ void tc_syn_body(const TcArgs &ta, const int2 item, u
       // add nothing and need no test
       const bool odd = q & 1;
       if (!odd && mode != kFast)
-        dead = !settled && __all_sync(0xffffffffu, negligible(lane0(rec.p), sc0) && (!SPIN || negligible(lane1(rec.p), sc1)));
+        dead = !settled && __all_sync(0xffffffffu, negligible(lane0(rec.p), sc0) && (NL == 1 || negligible(lane1(rec.p), sc1)));
       const float4 *row = rows + q * S::ROW;  // this degree's staged coefficients and a_lm
       float2 d[tc::kLamDigits] = {both(0.f), both(0.f), both(0.f)};
       if (mode == kFast || !dead) {
         float2 h = rec.p.h, lo = rec.p.l;
         if (mode != kFast) {
-          const float2 f = make_float2(wf.x, (mode == kPolar && odd) ? -wf.y : wf.y);
+          const float2 f = make_float2(wf.x, (SPIN && mode == kPolar && odd) ? -wf.y : wf.y);
           h = mul2(h, f);
           lo = mul2(lo, f);
         }
         float2 rr;
-        if (SPIN) {
+        if (NL == 2) {
           auto round2 = [](float2 r, float c) { return add2(add2(r, both(c)), both(-c)); };
           d[0] = round2(h, s0);
           rr = sub2(h, d[0]);
@@ -370,19 +401,23 @@ __device__ __forceinline__ void tc_syn_body(const TcArgs &ta, const int2 item, u
           if (SPIN) {
             const float4 P = row[1 + 2 * j];
             const float4 M = row[2 + 2 * j];  // s M
-            racc[8 * j + 0] = __fmaf_rn(rr.x, P.x, racc[8 * j + 0]);
-            racc[8 * j + 1] = __fmaf_rn(rr.x, P.z, racc[8 * j + 1]);
-            racc[8 * j + 2] = __fmaf_rn(rr.x, M.x, racc[8 * j + 2]);
-            racc[8 * j + 3] = __fmaf_rn(rr.x, M.z, racc[8 * j + 3]);
-            racc[8 * j + 4] = __fmaf_rn(rr.y, M.x, racc[8 * j + 4]);
-            racc[8 * j + 5] = __fmaf_rn(rr.y, M.z, racc[8 * j + 5]);
-            racc[8 * j + 6] = __fmaf_rn(rr.y, P.x, racc[8 * j + 6]);
-            racc[8 * j + 7] = __fmaf_rn(rr.y, P.z, racc[8 * j + 7]);
+            racc[0][8 * j + 0] = __fmaf_rn(rr.x, P.x, racc[0][8 * j + 0]);
+            racc[0][8 * j + 1] = __fmaf_rn(rr.x, P.z, racc[0][8 * j + 1]);
+            racc[0][8 * j + 2] = __fmaf_rn(rr.x, M.x, racc[0][8 * j + 2]);
+            racc[0][8 * j + 3] = __fmaf_rn(rr.x, M.z, racc[0][8 * j + 3]);
+            racc[0][8 * j + 4] = __fmaf_rn(rr.y, M.x, racc[0][8 * j + 4]);
+            racc[0][8 * j + 5] = __fmaf_rn(rr.y, M.z, racc[0][8 * j + 5]);
+            racc[0][8 * j + 6] = __fmaf_rn(rr.y, P.x, racc[0][8 * j + 6]);
+            racc[0][8 * j + 7] = __fmaf_rn(rr.y, P.z, racc[0][8 * j + 7]);
           } else {
             const float4 v = row[1 + j];
             const int c = 4 * j + (odd ? 2 : 0);
-            racc[c] = __fmaf_rn(rr.x, v.x, racc[c]);
-            racc[c + 1] = __fmaf_rn(rr.x, v.z, racc[c + 1]);
+            racc[0][c] = __fmaf_rn(rr.x, v.x, racc[0][c]);
+            racc[0][c + 1] = __fmaf_rn(rr.x, v.z, racc[0][c + 1]);
+            if (S::DUAL) {
+              racc[NP - 1][c] = __fmaf_rn(rr.y, v.x, racc[NP - 1][c]);
+              racc[NP - 1][c + 1] = __fmaf_rn(rr.y, v.z, racc[NP - 1][c + 1]);
+            }
           }
         }
       }
@@ -392,7 +427,7 @@ __device__ __forceinline__ void tc_syn_body(const TcArgs &ta, const int2 item, u
           dlo[i] = d[i];
         } else {
           pk[0][i][q / 2] = tc::pack_bf16(dlo[i].x, d[i].x);
-          if (SPIN) pk[NL - 1][i][q / 2] = tc::pack_bf16(dlo[i].y, d[i].y);
+          if (NL == 2) pk[NL - 1][i][q / 2] = tc::pack_bf16(dlo[i].y, d[i].y);
         }
       }
       advance(mode, row[0]);
@@ -436,8 +471,10 @@ __device__ __forceinline__ void tc_syn_body(const TcArgs &ta, const int2 item, u
 #pragma unroll
         for (int j0 = -(i & 1); j0 <= tc::kAlmDigits - 1 && i + j0 < tc::kLevels; j0 += 2) {
           const uint64_t ad = adesc0 + (uint64_t)(((t * tc::kLamDigits + i) * tc::kATile) >> 4);
-          const uint64_t bd = bdesc0 + (uint64_t)((t * S::NDT * S::DTILE + (j0 + 1) * S::DTILE) >> 4);
-          tc::mma_bf16(tbase + (i + j0) * S::NCW, ad, bd, idesc, (first && t == 0 && i == 0) ? 0u : 1u);
+          const int tb = SPIN ? t : 0, td = S::DUAL ? t : 0;  // B stack, accumulators
+          const uint64_t bd = bdesc0 + (uint64_t)((tb * S::NDT * S::DTILE + (j0 + 1) * S::DTILE) >> 4);
+          tc::mma_bf16(tbase + td * S::COLS1 + (i + j0) * S::NCW, ad, bd, idesc,
+                       (first && t == td && i == 0) ? 0u : 1u);
         }
     tc::mma_commit(&mbar);
   };
@@ -446,10 +483,11 @@ __device__ __forceinline__ void tc_syn_body(const TcArgs &ta, const int2 item, u
   // added to the double-float column sums
   auto readout = [&]() {
 #pragma unroll
-    for (int c0 = 0; c0 < NCOL; c0 += 8) {
+    for (int cc = 0; cc < NP * NCOL; cc += NCOL < 8 ? NCOL : 8) {
+      const int pt = cc / NCOL, c0 = cc % NCOL;
       uint32_t dv[tc::kLevels][8];
 #pragma unroll
-      for (int k = 0; k < tc::kLevels; ++k) tc::tmem_ld8(lane + k * S::NCW + c0, dv[k]);
+      for (int k = 0; k < tc::kLevels; ++k) tc::tmem_ld8(lane + pt * S::COLS1 + k * S::NCW + c0, dv[k]);
       tc::tmem_wait_ld();
 #pragma unroll
       for (int c = 0; c < 8; ++c) {
@@ -457,9 +495,9 @@ __device__ __forceinline__ void tc_syn_body(const TcArgs &ta, const int2 item, u
         f2 t = {__uint_as_float(dv[0][c]), 0.f};
 #pragma unroll
         for (int k = 1; k < tc::kLevels; ++k) t = f2_add_lazy(t, f2{__uint_as_float(dv[k][c]), 0.f});
-        t = f2_add_lazy(t, f2{racc[c0 + c], 0.f});
-        racc[c0 + c] = 0.f;
-        f2 &acc = accs[(c0 + c) * tc::kRows + tid];
+        t = f2_add_lazy(t, f2{racc[pt][c0 + c], 0.f});
+        racc[pt][c0 + c] = 0.f;
+        f2 &acc = accs[(pt * NCOL + c0 + c) * tc::kRows + tid];
         acc = f2_add(acc, t);
       }
     }
@@ -482,20 +520,25 @@ __device__ __forceinline__ void tc_syn_body(const TcArgs &ta, const int2 item, u
       tc::window_bounds<NJ, SPIN>(a, co, lb, lw1 < lmax ? lw1 : lmax, um);
       __syncthreads();
     }
-    if (lj == lb) {  // this pair joins: the recursion state where its terms start, over u_p
-      const JoinRec r = ld_join(jrec, polar);
-      const float ulx = __int_as_float((127 - r.lexp) << 23);
-      rec.start(0, r.lpc, r.lpp, ulx);
-      sc0 = r.scp;
-      if (SPIN) {  // lane 1 holds s l- (l- itself in a polar warp): the previous degree's sign is -1
-        rec.start(1, r.lmc, polar ? r.lmp : neg(r.lmp), ulx);
-        sc1 = r.scm;
+    // pairs joining here take the recursion state where their terms start, over u_p
+    bool joins = false;
+#pragma unroll
+    for (int t = 0; t < NP; ++t)
+      if (lj[t] == lb) {
+        const JoinRec r = ld_join(jrec[t], polar);
+        const float ulx = __int_as_float((127 - r.lexp) << 23);
+        rec.start(t, r.lpc, r.lpp, ulx);
+        (t ? sc1 : sc0) = r.scp;
+        if (SPIN) {  // lane 1 holds s l- (l- itself in a polar warp): the previous degree's sign is -1
+          rec.start(1, r.lmc, polar ? r.lmp : neg(r.lmp), ulx);
+          sc1 = r.scm;
+        }
+        wf = make_float2(scale_weight(sc0), scale_weight(sc1));
+        joins = true;
       }
-      wf = make_float2(scale_weight(sc0), scale_weight(sc1));
-    }
-    if (__any_sync(0xffffffffu, lj == lb)) settled = __all_sync(0xffffffffu, sc0 == 0 && sc1 == 0);
+    if (__any_sync(0xffffffffu, joins)) settled = __all_sync(0xffffffffu, sc0 == 0 && sc1 == 0);
     // a warp none of whose lanes has joined holds zeros: it skips the recursion
-    const bool wlive = __any_sync(0xffffffffu, lj <= lb);
+    const bool wlive = __any_sync(0xffffffffu, jmin <= lb);
     const float4 *rows = stage + (ks & 1) * S::STG;
     if (ks + 1 < nks) prefetch(ks + 1);  // its latency hides behind this K-step's work
     bool fail = false;
@@ -551,46 +594,49 @@ __device__ __forceinline__ void tc_syn_body(const TcArgs &ta, const int2 item, u
   __syncthreads();
   tc::fence_after();
   if (warp == 0) tc::tmem_dealloc(tbase, S::TCOLS);
-  if (!ok || !valid) return;
-  const int lexp = __float_as_int(__ldg(jrec + 2).w);
-  const double u = __hiloint2double((1023 + lexp) << 20, 0);  // u_p
-  auto colsum = [&](int c) { return u * f2_val(accs[c * tc::kRows + tid]); };
-
-  if (SPIN) {
-    const double sig = (as & 1) ? -1.0 : 1.0;
-    const double h0 = ((l0 + m) & 1) ? -0.5 : 0.5;
+  if (!ok) return;
 #pragma unroll
-    for (int j = 0; j < NJ; ++j) {
-      const double n1r = colsum(8 * j + 0), n1i = colsum(8 * j + 1);
-      const double s4r = colsum(8 * j + 2), s4i = colsum(8 * j + 3);
-      const double n2r = colsum(8 * j + 4), n2i = colsum(8 * j + 5);
-      const double s3r = colsum(8 * j + 6), s3i = colsum(8 * j + 7);
-      const double ar = n1r + sig * n2r, ai = n1i + sig * n2i;
-      const double br = sig * n2r - n1r, bi = sig * n2i - n1i;
-      const double cr = s3r + sig * s4r, ci = s3i + sig * s4i;
-      const double dr = sig * s4r - s3r, di = sig * s4i - s3i;
-      double2 qn = make_double2(-0.5 * ar, -0.5 * ai);
-      double2 un = make_double2(0.5 * bi, -0.5 * br);
-      double2 qs = make_double2(-h0 * cr, -h0 * ci);
-      double2 us = make_double2(h0 * di, -h0 * dr);
-      if (m == 0) qn.y = qs.y = un.y = us.y = 0.0;
-      double2 *oq = a.phase + (((size_t)(2 * j) * a.nm + mi) * a.npairs + p) * 2;
-      double2 *ou = a.phase + (((size_t)(2 * j + 1) * a.nm + mi) * a.npairs + p) * 2;
-      oq[0] = qn;
-      oq[1] = qs;
-      ou[0] = un;
-      ou[1] = us;
-    }
-  } else {
+  for (int t = 0; t < NP; ++t) {
+    if (!valid[t]) continue;
+    const int p = pr[t], lexp = __float_as_int(__ldg(jrec[t] + 2).w);
+    const double u = __hiloint2double((1023 + lexp) << 20, 0);  // u_p
+    auto colsum = [&](int c) { return u * f2_val(accs[(t * NCOL + c) * tc::kRows + tid]); };
+    if (SPIN) {
+      const double sig = (as & 1) ? -1.0 : 1.0;
+      const double h0 = ((l0 + m) & 1) ? -0.5 : 0.5;
 #pragma unroll
-    for (int j = 0; j < NJ; ++j) {
-      const double e0 = colsum(4 * j + 0), e1 = colsum(4 * j + 1);
-      const double o0 = colsum(4 * j + 2), o1 = colsum(4 * j + 3);
-      double2 fn = make_double2(e0 + o0, e1 + o1), fs = make_double2(e0 - o0, e1 - o1);
-      if (m == 0) fn.y = fs.y = 0.0;
-      double2 *o = a.phase + (((size_t)j * a.nm + mi) * a.npairs + p) * 2;
-      o[0] = fn;
-      o[1] = fs;
+      for (int j = 0; j < NJ; ++j) {
+        const double n1r = colsum(8 * j + 0), n1i = colsum(8 * j + 1);
+        const double s4r = colsum(8 * j + 2), s4i = colsum(8 * j + 3);
+        const double n2r = colsum(8 * j + 4), n2i = colsum(8 * j + 5);
+        const double s3r = colsum(8 * j + 6), s3i = colsum(8 * j + 7);
+        const double ar = n1r + sig * n2r, ai = n1i + sig * n2i;
+        const double br = sig * n2r - n1r, bi = sig * n2i - n1i;
+        const double cr = s3r + sig * s4r, ci = s3i + sig * s4i;
+        const double dr = sig * s4r - s3r, di = sig * s4i - s3i;
+        double2 qn = make_double2(-0.5 * ar, -0.5 * ai);
+        double2 un = make_double2(0.5 * bi, -0.5 * br);
+        double2 qs = make_double2(-h0 * cr, -h0 * ci);
+        double2 us = make_double2(h0 * di, -h0 * dr);
+        if (m == 0) qn.y = qs.y = un.y = us.y = 0.0;
+        double2 *oq = a.phase + (((size_t)(2 * j) * a.nm + mi) * a.npairs + p) * 2;
+        double2 *ou = a.phase + (((size_t)(2 * j + 1) * a.nm + mi) * a.npairs + p) * 2;
+        oq[0] = qn;
+        oq[1] = qs;
+        ou[0] = un;
+        ou[1] = us;
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < NJ; ++j) {
+        const double e0 = colsum(4 * j + 0), e1 = colsum(4 * j + 1);
+        const double o0 = colsum(4 * j + 2), o1 = colsum(4 * j + 3);
+        double2 fn = make_double2(e0 + o0, e1 + o1), fs = make_double2(e0 - o0, e1 - o1);
+        if (m == 0) fn.y = fs.y = 0.0;
+        double2 *o = a.phase + (((size_t)j * a.nm + mi) * a.npairs + p) * 2;
+        o[0] = fn;
+        o[1] = fs;
+      }
     }
   }
 }
@@ -599,53 +645,94 @@ __device__ __forceinline__ void tc_syn_body(const TcArgs &ta, const int2 item, u
 
 namespace sht {
 
-template <int NJ, bool SPIN>
-__global__ void __launch_bounds__(tc::kRows, tc::Shape<NJ, SPIN>::MINB) tc_syn(TcArgs ta) {
+template <int NJ, bool SPIN, bool TWO>
+__global__ void __launch_bounds__(tc::kRows, tc::Shape<NJ, SPIN, TWO>::MINB) tc_syn(TcArgs ta) {
   extern __shared__ __align__(128) unsigned char tc_smem[];
-  tc_syn_body<NJ, SPIN>(ta, ta.m.syn_items[blockIdx.x], tc_smem);
+  tc_syn_body<NJ, SPIN, TWO>(ta, ta.m.syn_items[blockIdx.x], tc_smem);
 }
 
 // batches: item (mi, first pair, -, record); the record holds the plan's arguments
-template <int NJ, bool SPIN>
-__global__ void __launch_bounds__(tc::kRows, tc::Shape<NJ, SPIN>::MINB)
+template <int NJ, bool SPIN, bool TWO>
+__global__ void __launch_bounds__(tc::kRows, tc::Shape<NJ, SPIN, TWO>::MINB)
     tc_syn_batch(const TcArgs *__restrict__ args, const int4 *__restrict__ items) {
   extern __shared__ __align__(128) unsigned char tc_smem[];
   const int4 it = items[blockIdx.x];
-  tc_syn_body<NJ, SPIN>(args[it.w], make_int2(it.x, it.y), tc_smem);
+  tc_syn_body<NJ, SPIN, TWO>(args[it.w], make_int2(it.x, it.y), tc_smem);
 }
 
-template <int NJ, bool SPIN>
+template <int NJ, bool SPIN, bool TWO>
 static cudaError_t tc_set_smem() {
   // the request, and a shared-memory carveout that lets the compiled number of CTAs fit
-  cudaError_t e = cudaFuncSetAttribute(tc_syn_batch<NJ, SPIN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       tc::Shape<NJ, SPIN>::SMEM_LAUNCH);
+  cudaError_t e = cudaFuncSetAttribute(tc_syn_batch<NJ, SPIN, TWO>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       tc::Shape<NJ, SPIN, TWO>::SMEM_LAUNCH);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(tc_syn<NJ, SPIN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             tc::Shape<NJ, SPIN>::SMEM_LAUNCH);
+    e = cudaFuncSetAttribute(tc_syn<NJ, SPIN, TWO>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             tc::Shape<NJ, SPIN, TWO>::SMEM_LAUNCH);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(tc_syn_batch<NJ, SPIN>, cudaFuncAttributePreferredSharedMemoryCarveout,
+    e = cudaFuncSetAttribute(tc_syn_batch<NJ, SPIN, TWO>, cudaFuncAttributePreferredSharedMemoryCarveout,
                              cudaSharedmemCarveoutMaxShared);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(tc_syn<NJ, SPIN>, cudaFuncAttributePreferredSharedMemoryCarveout,
+    e = cudaFuncSetAttribute(tc_syn<NJ, SPIN, TWO>, cudaFuncAttributePreferredSharedMemoryCarveout,
                              cudaSharedmemCarveoutMaxShared);
   return e;
 }
 
 // shared-memory attributes of every instance (once per device, at plan time)
 cudaError_t tc_prepare_device() {
-  cudaError_t e = tc_set_smem<1, false>();
-  if (e == cudaSuccess) e = tc_set_smem<2, false>();
-  if (e == cudaSuccess) e = tc_set_smem<4, false>();
-  if (e == cudaSuccess) e = tc_set_smem<8, false>();
-  if (e == cudaSuccess) e = tc_set_smem<1, true>();
-  if (e == cudaSuccess) e = tc_set_smem<2, true>();
-  if (e == cudaSuccess) e = tc_set_smem<4, true>();
+  cudaError_t e = tc_set_smem<1, false, false>();
+  if (e == cudaSuccess) e = tc_set_smem<1, false, true>();
+  if (e == cudaSuccess) e = tc_set_smem<2, false, false>();
+  if (e == cudaSuccess) e = tc_set_smem<2, false, true>();
+  if (e == cudaSuccess) e = tc_set_smem<4, false, false>();
+  if (e == cudaSuccess) e = tc_set_smem<8, false, false>();
+  if (e == cudaSuccess) e = tc_set_smem<1, true, false>();
+  if (e == cudaSuccess) e = tc_set_smem<2, true, false>();
+  if (e == cudaSuccess) e = tc_set_smem<4, true, false>();
   return e;
 }
 
 bool tc_supported(int spin, int njobs_pad) {
   return spin == 0 ? njobs_pad <= 8 : njobs_pad <= 4;
 }
+
+// One or two spin-0 maps: two pairs a thread where the 128-pair tiles fill the chip at
+// least kTwoPerSm times over.  It saves issue slots (the two lanes' recursions and
+// digits are packed) but halves the CTAs, whose fixed cost per block of degrees is then
+// longer: two maps on Gauss-Legendre rings, one pair a thread against two, lmax 511
+// 132 / 156 us, 1023 (27 tiles per SM) 567 / 583, HEALPix 1535 (81) 2128 / 1846, 2047
+// (108) 3600 / 3130, 4095 25.6 / 20.9 ms.
+bool tc_syn_two_tiles(const sht_plan_s *P, int64_t tiles) {
+  constexpr int kTwoPerSm = 40;
+  return P->spin == 0 && P->njobs_pad <= 2 && tiles >= (int64_t)kTwoPerSm * P->sms;
+}
+
+namespace {
+// calls f with the shape of a spin class, padded job count and pairs per thread; false: none
+template <int NJ, bool SPIN, bool TWO>
+struct SynShape {
+  static constexpr int nj = NJ;
+  static constexpr bool spin = SPIN, two = TWO;
+  static constexpr int smem = tc::Shape<NJ, SPIN, TWO>::SMEM_LAUNCH;
+};
+template <class F>
+bool syn_shape(int spin, int nj, bool two, F &&f) {
+  if (spin == 0) {
+    switch (nj) {
+      case 1: two ? f(SynShape<1, false, true>()) : f(SynShape<1, false, false>()); return true;
+      case 2: two ? f(SynShape<2, false, true>()) : f(SynShape<2, false, false>()); return true;
+      case 4: f(SynShape<4, false, false>()); return true;
+      case 8: f(SynShape<8, false, false>()); return true;
+    }
+  } else {
+    switch (nj) {
+      case 1: f(SynShape<1, true, false>()); return true;
+      case 2: f(SynShape<2, true, false>()); return true;
+      case 4: f(SynShape<4, true, false>()); return true;
+    }
+  }
+  return false;
+}
+}  // namespace
 
 float tc_lambda_bound(int lmax) {
   // |sLambda_lm| <= sqrt((2l + 1) / (4 pi)) (|d^l| <= 1) up to l = lmax + 1 (the
@@ -664,26 +751,15 @@ void leg_tc_fill_args(const sht_plan_s *P, int polar, void *out) {
   memcpy(out, &ta, sizeof(ta));
 }
 
-cudaError_t launch_leg_tc_batch(int spin, int nj, const void *targs, const int4 *items, int n, cudaStream_t st) {
+cudaError_t launch_leg_tc_batch(int spin, int nj, bool two, const void *targs, const int4 *items, int n,
+                                cudaStream_t st) {
   if (n == 0) return cudaSuccess;
   const TcArgs *a = static_cast<const TcArgs *>(targs);
-  if (spin == 0) {
-    switch (nj) {
-      case 1: tc_syn_batch<1, false><<<n, tc::kRows, tc::Shape<1, false>::SMEM_LAUNCH, st>>>(a, items); break;
-      case 2: tc_syn_batch<2, false><<<n, tc::kRows, tc::Shape<2, false>::SMEM_LAUNCH, st>>>(a, items); break;
-      case 4: tc_syn_batch<4, false><<<n, tc::kRows, tc::Shape<4, false>::SMEM_LAUNCH, st>>>(a, items); break;
-      case 8: tc_syn_batch<8, false><<<n, tc::kRows, tc::Shape<8, false>::SMEM_LAUNCH, st>>>(a, items); break;
-      default: return cudaErrorInvalidValue;
-    }
-  } else {
-    switch (nj) {
-      case 1: tc_syn_batch<1, true><<<n, tc::kRows, tc::Shape<1, true>::SMEM_LAUNCH, st>>>(a, items); break;
-      case 2: tc_syn_batch<2, true><<<n, tc::kRows, tc::Shape<2, true>::SMEM_LAUNCH, st>>>(a, items); break;
-      case 4: tc_syn_batch<4, true><<<n, tc::kRows, tc::Shape<4, true>::SMEM_LAUNCH, st>>>(a, items); break;
-      default: return cudaErrorInvalidValue;
-    }
-  }
-  return cudaGetLastError();
+  const bool ok = syn_shape(spin, nj, two, [&](auto sh) {
+    using H = decltype(sh);
+    tc_syn_batch<H::nj, H::spin, H::two><<<n, tc::kRows, H::smem, st>>>(a, items);
+  });
+  return ok ? cudaGetLastError() : cudaErrorInvalidValue;
 }
 
 cudaError_t launch_leg_tc_syn(const sht_plan_s *P, const void *mixargs, int n, cudaStream_t st) {
@@ -691,24 +767,11 @@ cudaError_t launch_leg_tc_syn(const sht_plan_s *P, const void *mixargs, int n, c
   TcArgs ta;
   memcpy(&ta.m, mixargs, sizeof(MixArgs));
   ta.err = P->d_err;
-  const int nj = P->njobs_pad;
-  if (P->spin == 0) {
-    switch (nj) {
-      case 1: tc_syn<1, false><<<n, tc::kRows, tc::Shape<1, false>::SMEM_LAUNCH, st>>>(ta); break;
-      case 2: tc_syn<2, false><<<n, tc::kRows, tc::Shape<2, false>::SMEM_LAUNCH, st>>>(ta); break;
-      case 4: tc_syn<4, false><<<n, tc::kRows, tc::Shape<4, false>::SMEM_LAUNCH, st>>>(ta); break;
-      case 8: tc_syn<8, false><<<n, tc::kRows, tc::Shape<8, false>::SMEM_LAUNCH, st>>>(ta); break;
-      default: return cudaErrorInvalidValue;
-    }
-  } else {
-    switch (nj) {
-      case 1: tc_syn<1, true><<<n, tc::kRows, tc::Shape<1, true>::SMEM_LAUNCH, st>>>(ta); break;
-      case 2: tc_syn<2, true><<<n, tc::kRows, tc::Shape<2, true>::SMEM_LAUNCH, st>>>(ta); break;
-      case 4: tc_syn<4, true><<<n, tc::kRows, tc::Shape<4, true>::SMEM_LAUNCH, st>>>(ta); break;
-      default: return cudaErrorInvalidValue;
-    }
-  }
-  return cudaGetLastError();
+  const bool ok = syn_shape(P->spin, P->njobs_pad, P->syn_two != 0, [&](auto sh) {
+    using H = decltype(sh);
+    tc_syn<H::nj, H::spin, H::two><<<n, tc::kRows, H::smem, st>>>(ta);
+  });
+  return ok ? cudaGetLastError() : cudaErrorInvalidValue;
 }
 
 }  // namespace sht

@@ -938,6 +938,10 @@ static int upload_list(sht_plan_s *P, const std::vector<std::pair<int64_t, T>> &
 static int build_syn_lists(sht_plan_s *P) {
   int rc;
   const int as = abs(P->spin);
+  int64_t ntile = 0;  // of the polar-cut variant
+  for (int i = 0; i < P->nm; ++i)
+    if (P->lmax >= std::max(P->mval[i], as)) ntile += (P->npairs + kSynTile - 1) / kSynTile - P->first_pair[i] / kSynTile;
+  P->syn_two = P->tc_syn && tc_syn_two_tiles(P, ntile);
   for (int polar = 0; polar < 2; ++polar) {
     std::vector<std::pair<int64_t, int2>> syn, lo;
     std::vector<int> sfirst(P->nm);
@@ -953,9 +957,15 @@ static int build_syn_lists(sht_plan_s *P) {
       trip += (int64_t)(P->npairs - fp) * nl;
       int sf = (fp / kSynTile) * kSynTile;
       sfirst[i] = sf;
-      for (int p = sf; p < P->npairs; p += kSynTile)
-        (lo_item(P, i, p, p + kSynTile) ? lo : syn)
-            .push_back({(int64_t)nl * std::min(kSynTile, P->npairs - p), make_int2(i, p)});
+      for (int p = sf; p < P->npairs; p += kSynTile) {
+        const bool l = lo_item(P, i, p, p + kSynTile);
+        if (P->syn_two && !l && p + kSynTile < P->npairs && !lo_item(P, i, p + kSynTile, p + 2 * kSynTile)) {
+          syn.push_back({(int64_t)nl * std::min(2 * kSynTile, P->npairs - p), make_int2(i, p | kSynTwoTiles)});
+          p += kSynTile;
+          continue;
+        }
+        (l ? lo : syn).push_back({(int64_t)nl * std::min(kSynTile, P->npairs - p), make_int2(i, p)});
+      }
     }
     P->triples[polar] = trip;
     std::stable_sort(syn.begin(), syn.end(), [](auto &a, auto &b) { return a.first > b.first; });
@@ -971,16 +981,6 @@ static int build_syn_lists(sht_plan_s *P) {
   return SHT_OK;
 }
 
-// Analysis work lists: per polar variant the cost-sorted items and, per m, where
-// their partial sums go.  A tile is kAnaThreads * ppt ring pairs; a mixed-form item
-// walks a group of consecutive tiles of one m one after another and sums them into
-// one slot of partial sums, so the partials' size shrinks by the group size (their
-// DRAM traffic only while the slots of the resident CTAs fit in L2).  Groups are
-// as large as keeps at least kAnaItemsPerSm items per SM (and at most
-// kAnaGroupTiles tiles): the same work in fewer, longer CTAs, which on
-// GB300 at lmax 4095 is as fast as one CTA per tile (152.5 against 153.0 ms per
-// pair) with a sixteenth of the partials; an 8-map plan's analysis kernel is 4.4
-// ms slower grouped, its slot reduction 6.6 ms faster (lmax 4095: 157.3 + 1.1
 // items of consecutive tiles of TA ring pairs: the tiles per item, whole passes of nt
 static int ana_group(const sht_plan_s *P, int TA, int nt) {
   const int tiles = (P->npairs + TA - 1) / TA, as = abs(P->spin);
@@ -1014,6 +1014,16 @@ static int64_t ana_part_need(const sht_plan_s *P, int TA, int group) {
   return off;
 }
 
+// Analysis work lists: per polar variant the cost-sorted items and, per m, where
+// their partial sums go.  A tile is kAnaThreads * ppt ring pairs; a mixed-form item
+// walks a group of consecutive tiles of one m one after another and sums them into
+// one slot of partial sums, so the partials' size shrinks by the group size (their
+// DRAM traffic only while the slots of the resident CTAs fit in L2).  Groups are
+// as large as keeps at least kAnaItemsPerSm items per SM (and at most
+// kAnaGroupTiles tiles): the same work in fewer, longer CTAs, which on
+// GB300 at lmax 4095 is as fast as one CTA per tile (152.5 against 153.0 ms per
+// pair) with a sixteenth of the partials; an 8-map plan's analysis kernel is 4.4
+// ms slower grouped, its slot reduction 6.6 ms faster (lmax 4095: 157.3 + 1.1
 // against 152.9 + 7.7 ms).  FP64 items (the FP64 form, and a mixed plan's tiles
 // next to the poles) take one tile each.  Item (m index, first tile,
 // slot << 8 | tiles, -); the slots of m are summed by the reduction kernel.
@@ -1074,6 +1084,13 @@ static int build_ana_lists(sht_plan_s *P, int ppt) {
     CUDA_TRY(cudaMalloc(&P->d_part, std::max<int64_t>(1, P->part_doubles) * sizeof(double)));
   }
   P->ana_ppt = ppt;
+  // What the call that allocates nothing counts against its area: of the FP64 form the
+  // FP64 kernel's tiling, of one spin-0 map in the mixed form four pairs a thread until a
+  // tiling is chosen, whichever tiles run
+  P->part_limit = need;
+  if (P->tc64_ana) P->part_limit = ana_part_need(P, kAnaThreads * ppt, 1);
+  else if (mixed && P->spin == 0 && P->njobs_pad == 1 && !P->tc_ana && !P->tiling_chosen)
+    P->part_limit = ana_part_need(P, kAnaThreads * 4, ana_group(P, kAnaThreads * 4, 1));
   return SHT_OK;
 }
 
@@ -1084,13 +1101,6 @@ static int build_ana_lists(sht_plan_s *P, int ppt) {
 // tensor cores, us): synthesis, one array lmax 191 54 -> 64, 255 70 -> 59, 1023 1735 ->
 // 1194; two 127 70 -> 74, 191 114 -> 108, 767 2250 -> 1080; four 31 41 -> 39, 63 41 -> 37,
 // 767 3569 -> 1324; analysis, one 191 117 -> 119, 255 164 -> 158, 1023 2350 -> 1560; two
-  // What the call that allocates nothing counts against its area: of the FP64 form the
-  // FP64 kernel's tiling, of one spin-0 map in the mixed form four pairs a thread until a
-  // tiling is chosen, whichever tiles run
-  P->part_limit = need;
-  if (P->tc64_ana) P->part_limit = ana_part_need(P, kAnaThreads * ppt, 1);
-  else if (mixed && P->spin == 0 && P->njobs_pad == 1 && !P->tc_ana && !P->tiling_chosen)
-    P->part_limit = ana_part_need(P, kAnaThreads * 4, ana_group(P, kAnaThreads * 4, 1));
 // 31 36 -> 30, 767 3826 -> 1228; four 31 53 -> 31, 767 6277 -> 1506.
 static void tc64_choose(sht_plan_s *P) {
   const int n = P->nmaps_pad;  // arrays per side
@@ -1440,8 +1450,15 @@ extern "C" int sht_plan_set_tensor_cores(sht_plan_t P, int on) {
     return fail(SHT_ERR_UNSUPPORTED, "tensor-core synthesis holds at most 32 columns (spin 0: ncomp <= 8, spin: ncomp <= 4)");
   if (P->batch_refs)
     return fail(SHT_ERR_INVALID_ARG, "the plan belongs to %d batch(es); destroy them first", P->batch_refs);
+  if ((on != 0) == (P->tc_syn != 0)) return SHT_OK;
   P->tc_syn = on ? 1 : 0;
-  return SHT_OK;
+  if (P->spin || P->njobs_pad > 2) return SHT_OK;
+  int cur = -1;  // its items may take two tiles
+  cudaGetDevice(&cur);
+  if (cur != P->device) CUDA_TRY(cudaSetDevice(P->device));
+  const int rc = build_syn_lists(P);
+  if (cur != P->device) cudaSetDevice(cur);
+  return rc;
 }
 
 extern "C" int sht_plan_set_tensor_core_analysis(sht_plan_t P, int on) {

@@ -24,6 +24,7 @@ namespace sht {
 constexpr int kMaxPtr = 32;       // max device pointers per execute (maps or a_lm arrays)
 constexpr int kMaxJobs = 16;      // ncomp limit
 constexpr int kSynTile = 128;     // ring pairs per synthesis Legendre CTA (one per thread)
+constexpr int kSynTwoTiles = 1 << 30;  // in a synthesis item's first pair: two tiles (tensor-core kernel, spin 0)
 constexpr int kAnaThreads = 128;  // threads per analysis Legendre CTA
 constexpr int kCoefTail = 8;      // entries past the end of the double-float coefficient table
 constexpr int kAnaGroupTiles = 16;  // most tiles a mixed analysis item walks, one after another
@@ -146,9 +147,9 @@ struct sht_plan_s {
   double2 *d_phase = nullptr;              // F / G workspace
   double *d_part = nullptr;                // analysis partials
   int64_t part_doubles = 0;
-
   int64_t part_limit = 0;  // of them, what sht_execute_noalloc counts (sht_host.cu)
   int tiling_chosen = 0;   // a call chose the analysis tiling
+
   // work lists (polar-cut / uncut): synthesis (mi, first pair) and analysis (mi, tile, part offset)
   int2 *d_syn_items[2] = {nullptr, nullptr};
   int nsyn_items[2] = {0, 0};
@@ -170,6 +171,7 @@ struct sht_plan_s {
   bool fft_df = false;  // ring FFTs in double-float (mixed plans, by default)
   // mixed plans: the synthesis contraction on the tensor cores (legendre_tc.cu)
   int tc_syn = 0;
+  int syn_two = 0;  // its items are up to two tiles (spin 0, one or two maps)
   // mixed plans: the analysis contraction on the tensor cores (legendre_tc_ana.cu;
   // tiles of kAnaThreads ring pairs, one per thread)
   int tc_ana = 0;
@@ -283,8 +285,10 @@ cudaError_t launch_join_records(const sht_plan_s *P, cudaStream_t st);
 // batches: one TcArgs record per plan of a tensor-core group
 size_t tc_args_size();
 void leg_tc_fill_args(const sht_plan_s *P, int polar, void *out);
-cudaError_t launch_leg_tc_batch(int spin, int nj, const void *targs, const int4 *items, int n, cudaStream_t st);
+cudaError_t launch_leg_tc_batch(int spin, int nj, bool two, const void *targs, const int4 *items, int n,
+                                cudaStream_t st);
 bool tc_supported(int spin, int njobs_pad);
+bool tc_syn_two_tiles(const sht_plan_s *P, int64_t tiles);  // its items are up to two of the tiles
 float tc_lambda_bound(int lmax);
 // tensor-core analysis (legendre_tc_ana.cu): mixargs with its analysis work list set
 cudaError_t launch_leg_tc_ana(const sht_plan_s *P, const void *mixargs, int n, cudaStream_t st);

@@ -1,9 +1,13 @@
-"""The limit of the call that allocates nothing is one of the transform, not of the
-tiling that serves it."""
+"""Work items whose size follows from the plan's: synthesis items of up to two tiles of
+ring pairs (spin 0, one or two maps, tensor-core form) at ring counts around whole tiles,
+with FP64 columns between them, and the limit of the call that allocates nothing, which
+is one of the transform and not of the tiling that serves it."""
 import pytest
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
+
+MIX_L2 = 1e-10  # the mixed form's bound, relative L2 against the FP64 form
 
 
 @pytest.fixture(scope="module")
@@ -25,6 +29,36 @@ def random_alm(lay, lmax, n):
         a[: lmax + 1].imag.zero_()  # m = 0
         out.append(a)
     return out
+
+
+def rel(a, b):
+    return float(torch.linalg.vector_norm(a - b) / torch.linalg.vector_norm(b))
+
+
+@pytest.mark.parametrize("nlat", [256, 257, 511, 514, 770])
+@pytest.mark.parametrize("ncomp", [1, 2])
+def test_two_tile_items(sht, nlat, ncomp):
+    lmax = 4800  # columns enough that one or two tiles each reach the rule's work per SM
+    geom = sht.sht_geom_gauss(nlat, 96)
+    lay = sht.sht_alm_create(lmax, lmax)
+    mixed = sht.sht_plan_create(geom, lay, 0, ncomp, sht.SHT_MIXED)
+    ref = sht.sht_plan_create(geom, lay, 0, ncomp, sht.SHT_FP64)
+    alm = random_alm(lay, lmax, ncomp)
+    maps = [torch.empty(geom.npix, dtype=torch.float64, device="cuda") for _ in range(ncomp)]
+    want = [torch.empty_like(x) for x in maps]
+    mixed.tensor_cores = True
+    for flags in (0, sht.SHT_NO_POLAR_OPT):
+        for x in maps:
+            x.fill_(float("nan"))
+        sht.sht_execute(mixed, sht.SHT_SYNTHESIS, alm, maps, flags)
+        sht.sht_execute(ref, sht.SHT_SYNTHESIS, alm, want, flags)
+        assert mixed.device_status() == 0
+        for x, y in zip(maps, want):
+            assert rel(x, y) <= MIX_L2
+    mixed.tensor_cores = False  # the lists go back to single tiles
+    sht.sht_execute(mixed, sht.SHT_SYNTHESIS, alm, maps, sht.SHT_NO_POLAR_OPT)
+    for x, y in zip(maps, want):
+        assert rel(x, y) <= MIX_L2
 
 
 @pytest.mark.parametrize("precision", [0, 1])
