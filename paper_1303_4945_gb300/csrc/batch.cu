@@ -126,7 +126,7 @@ int build(sht_batch_s *B) {
     const int spin_class = P->spin ? 1 : 0;
     const bool tc = precision == SHT_MIXED ? P->tc_syn != 0 : (!lo && P->tc64_syn);
     const bool two = precision == SHT_MIXED && P->syn_two;
-    const bool tca = precision == SHT_MIXED ? P->tc_ana != 0 : (!lo && P->tc64_ana);
+    const bool tca = precision == SHT_MIXED ? P->tc_ana || tc_ana_quad(P) : (!lo && P->tc64_ana);
     Group *g = nullptr;
     for (auto &c : B->groups)
       if (c.precision == precision && c.spin == spin_class && c.nj == P->njobs_pad && c.ppt == P->ana_ppt &&

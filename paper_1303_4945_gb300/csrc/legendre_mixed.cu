@@ -666,6 +666,7 @@ static MixArgs make_mix(const sht_plan_s *P, int polar) {
   a.spin = P->spin;
   a.npairs = P->npairs;
   a.nm = P->nm;
+  a.nj = P->njobs_pad;
   a.mval = P->d_mval;
   a.coef_off = P->d_coef_off;
   a.coef32 = P->d_coef32;
@@ -814,10 +815,12 @@ cudaError_t launch_leg_mixed_items(const sht_plan_s *P, int stage, int polar, co
     }
   } else {
     a.ana_items = static_cast<const int4 *>(items);
-    if (P->tc_ana) return launch_leg_tc_ana(P, &a, n, st);
+    if (P->tc_ana || tc_ana_quad(P)) return launch_leg_tc_ana(P, &a, n, st);
     if (P->spin == 0)
       ana_shape_s0(nj, P->ana_ppt, [&](auto sh) {
-        mix_ana<decltype(sh)::nj, decltype(sh)::ppt, false><<<n, kAnaThreads, 0, st>>>(a);
+        // (more maps: tc_ana_quad)
+        if constexpr (decltype(sh)::nj <= 2)
+          mix_ana<decltype(sh)::nj, decltype(sh)::ppt, false><<<n, kAnaThreads, 0, st>>>(a);
       });
     else
       ana_shape_spin(nj, P->ana_ppt, [&](auto sh) {
@@ -883,7 +886,9 @@ cudaError_t launch_leg_mixed_batch(int stage, int spin, int nj, int ppt, const v
   } else {
     if (spin == 0)
       ana_shape_s0(nj, ppt, [&](auto sh) {
-        mix_ana_batch<decltype(sh)::nj, decltype(sh)::ppt, false><<<n, kAnaThreads, 0, st>>>(a, items);
+        // (more maps: tc_ana_quad)
+        if constexpr (decltype(sh)::nj <= 2)
+          mix_ana_batch<decltype(sh)::nj, decltype(sh)::ppt, false><<<n, kAnaThreads, 0, st>>>(a, items);
       });
     else
       ana_shape_spin(nj, ppt, [&](auto sh) {

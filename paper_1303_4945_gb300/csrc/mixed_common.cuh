@@ -124,6 +124,7 @@ constexpr int kJoinBlock = 16;  // degrees per join block
 
 struct MixArgs {
   int lmax, spin, npairs, nm;
+  int nj;  // the plan's padded job count
   const int *mval;
   const int64_t *coef_off;
   const float4 *coef32;  // per (m, l): {a.h, a.l, b.h, b.l} of p_{l+1} = (a x + b) p_l - p_{l-1}

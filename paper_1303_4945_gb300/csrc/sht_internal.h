@@ -295,6 +295,7 @@ cudaError_t launch_leg_tc_ana(const sht_plan_s *P, const void *mixargs, int n, c
 // batches: one TcArgs record per plan of a tensor-core analysis group
 cudaError_t launch_leg_tc_ana_batch(int spin, int nj, const void *targs, const int4 *items, int n, cudaStream_t st);
 cudaError_t tc_ana_prepare_device();
+bool tc_ana_quad(const sht_plan_s *P);  // plans that always take it, four jobs at a time on tiles of 256 pairs
 bool tc_ana_supported(int spin, int njobs_pad);
 int tc_ana_tiles(int spin, int njobs_pad);  // tiles of kAnaThreads pairs it walks at a time
 // ring FFTs

@@ -81,3 +81,46 @@ def test_noalloc_limit_is_the_transforms(sht, precision):
     except sht.ShtError as e:
         code = e.code
     assert code == sht.SHT_ERR_UNSUPPORTED
+
+
+@pytest.mark.parametrize("nlat,lmax,ncomp", [(1, 0, 3), (2, 1, 4), (31, 33, 5), (254, 200, 16), (257, 260, 4), (511, 515, 8),
+                                             (513, 518, 3), (1026, 600, 9), (700, 2100, 4)])
+def test_analysis_of_more_than_two_maps(sht, nlat, lmax, ncomp):
+    """Four maps at a time on the tensor cores: rings around whole tiles of 256 pairs,
+    padded maps, FP64 columns (lmax >= 2000), no polar cut, added outputs."""
+    geom = sht.sht_geom_gauss(nlat, 64)
+    lay = sht.sht_alm_create(lmax, lmax)
+    mixed = sht.sht_plan_create(geom, lay, 0, ncomp, sht.SHT_MIXED)
+    ref = sht.sht_plan_create(geom, lay, 0, ncomp, sht.SHT_FP64)
+    g = torch.Generator(device="cuda").manual_seed(4945)
+    maps = [10.0 ** (2 * k) * torch.randn(geom.npix, dtype=torch.float64, device="cuda", generator=g) for k in range(-1, ncomp - 1)]
+    got, want = ([torch.ones(lay.size(), dtype=torch.complex128, device="cuda") for _ in range(ncomp)] for _ in range(2))
+    for flags in (0, sht.SHT_NO_POLAR_OPT, sht.SHT_ADD_OUTPUT):
+        for type_ in (sht.SHT_ANALYSIS, sht.SHT_ADJOINT_SYNTHESIS):
+            sht.sht_execute(mixed, type_, got, maps, flags)
+            sht.sht_execute(ref, type_, want, maps, flags)
+            assert mixed.device_status() == 0
+            for x, y in zip(got, want):
+                assert rel(x, y) <= MIX_L2
+
+
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+@pytest.mark.parametrize("ncomp,tca", [(1, True), (2, True), (4, False), (8, False)])
+def test_analysis_keeps_nan(sht, bad, ncomp, tca):
+    """A pixel that is not finite, on the first ring (most columns' recursions never reach
+    it) or the equator, leaves no finite coefficient of its map and every one of the others."""
+    lmax = 299
+    geom = sht.sht_geom_gauss(300, 601)
+    lay = sht.sht_alm_create(lmax, lmax)
+    plan = sht.sht_plan_create(geom, lay, 0, ncomp, sht.SHT_MIXED)
+    plan.tensor_core_analysis = tca
+    g = torch.Generator(device="cuda").manual_seed(7)
+    for pos in (100, geom.npix // 2):
+        maps = [torch.randn(geom.npix, dtype=torch.float64, device="cuda", generator=g) for _ in range(ncomp)]
+        alm = [torch.zeros(lay.size(), dtype=torch.complex128, device="cuda") for _ in range(ncomp)]
+        maps[0][pos] = bad
+        sht.sht_execute(plan, sht.SHT_ANALYSIS, alm, maps)
+        assert plan.device_status() == 0
+        assert not torch.isfinite(torch.view_as_real(alm[0])[lmax + 1:]).any()
+        assert not torch.isfinite(alm[0][: lmax + 1].real).any()
+        assert all(torch.isfinite(torch.view_as_real(a)).all() for a in alm[1:])
