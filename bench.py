@@ -349,6 +349,8 @@ def paper_rule_times(sht, torch, plan, alm_d, maps_d, out_d, stream, budget_s=2.
 # three-term one 31.
 #   spin s: two recursions (5 + 2 x 31) + 8 ncomp multiply-adds = 67 + 96 ncomp
 #   spin 0: one recursion (5 + 19)       + 2 ncomp multiply-adds = 24 + 24 ncomp
+# (the method's recursion with its three coefficients; the kernels' form with a unit
+# coefficient issues 51 and 20 for the recursions)
 def f32_ops_per_triple(spin, ncomp):
     return (67 + 96 * ncomp) if spin else (24 + 24 * ncomp)
 
@@ -370,8 +372,9 @@ MEASURED_TRAFFIC = {
 
 KERNEL_HEADERS = {"legendre_fp64.cu": ("sht_device.cuh",),
                   "legendre_mixed.cu": ("df.cuh", "sht_device.cuh", "mixed_common.cuh", "sht_internal.h"),
-                  "legendre_tc.cu": ("df.cuh", "sht_device.cuh", "mixed_common.cuh", "tcgen05.cuh"),
-                  "legendre_tc_ana.cu": ("df.cuh", "sht_device.cuh", "mixed_common.cuh", "tcgen05.cuh", "sht_internal.h")}
+                  "legendre_tc.cu": ("df.cuh", "sht_device.cuh", "mixed_common.cuh", "dual.cuh", "tcgen05.cuh"),
+                  "legendre_tc_ana.cu": ("df.cuh", "sht_device.cuh", "mixed_common.cuh", "dual.cuh", "tcgen05.cuh",
+                                         "sht_internal.h")}
 
 
 def _kernel_digest(kernel_file):
@@ -396,7 +399,8 @@ def launches_per_step(spin, form, fp64_items=False):
     """Kernels one synthesis + analysis launches: Legendre, FFT each way, the tile
     reduction, the a_lm conversion (spin, or the mixed form), and for a mixed plan
     with FP64 items near the poles their two Legendre kernels (plus the P/M
-    conversion they read when the spin is not 0)."""
+    conversion they read when the spin is not 0).  At spin 0 the FP64 kernels'
+    a_lm scaling is one launch more, which this count leaves out."""
     n = 5 + (1 if (spin != 0 or form == "mixed") else 0)
     if form == "mixed" and fp64_items:
         n += 2 + (1 if spin != 0 else 0)

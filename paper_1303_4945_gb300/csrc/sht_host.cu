@@ -1191,7 +1191,9 @@ static int plan_build(sht_plan_s *P, const sht_geom_s *g) {
     CUDA_TRY(tc_prepare_device());
     CUDA_TRY(tc_ana_prepare_device());
     // the tensor-core synthesis by default wherever it was measured faster: every
-    // supported shape except a single spin-0 map (lmax 4095: 32.1 ms against 25.6)
+    // supported shape except a single spin-0 map (lmax 511 137 us against 106, 2047 2.77
+    // ms against 2.78, 4095 18.7 against 20.4: ahead only at the largest sizes, where a
+    // caller sets it)
     P->tc_syn = tc_supported(P->spin, P->njobs_pad) && !(P->spin == 0 && P->njobs_pad == 1);
   }
   CUDA_TRY(launch_coef_tables(P, 0));
