@@ -125,7 +125,7 @@ int build(sht_batch_s *B) {
     const sht_plan_s *P = B->plans[k];
     const int spin_class = P->spin ? 1 : 0;
     const bool tc = precision == SHT_MIXED ? P->tc_syn != 0 : (!lo && P->tc64_syn);
-    const bool two = precision == SHT_MIXED && P->syn_two;
+    const bool two = precision == SHT_MIXED && syn_two_on(P);
     const bool tca = precision == SHT_MIXED ? P->tc_ana || tc_ana_quad(P) : (!lo && P->tc64_ana);
     Group *g = nullptr;
     for (auto &c : B->groups)
@@ -170,7 +170,7 @@ int build(sht_batch_s *B) {
         else
           leg_fp64_fill_args(P, polar, args.data() + i * rec, lo);
         if (tcrec) leg_tc_fill_args(P, polar, targs.data() + i * tc_args_size());
-        for (auto &it : (lo ? P->syn_list_lo : P->syn_list)[polar])
+        for (auto &it : (lo ? P->syn_list_lo : mixed && syn_two_on(P) ? P->syn_list_two : P->syn_list)[polar])
           syn.push_back({it.first, make_int4(it.second.x, it.second.y, 0, (int)i)});
         for (auto &it : (lo ? P->ana_list_lo : P->ana_list)[polar])
           ana.push_back({it.first, make_int4(it.second.x, it.second.y, it.second.z, (int)i)});

@@ -675,7 +675,7 @@ static MixArgs make_mix(const sht_plan_s *P, int polar) {
   a.mpre = P->d_mpre;
   a.pairs = P->d_pairs;
   a.phase = P->d_phase;
-  a.syn_items = P->d_syn_items[polar];
+  a.syn_items = syn_items(P, polar);
   a.ana_items = P->d_ana_items[polar];
   a.part_off = P->d_ana_part_off[polar];
   a.part = P->d_part;
@@ -833,7 +833,7 @@ cudaError_t launch_leg_mixed_items(const sht_plan_s *P, int stage, int polar, co
 cudaError_t launch_leg_syn_mixed(const sht_plan_s *P, const DevPtrs &alm, int polar, cudaStream_t st, int mode) {
   cudaError_t e = launch_alm_prepare_mixed(P, alm, st, mode);
   if (e != cudaSuccess) return e;
-  return launch_leg_mixed_items(P, 0, polar, P->d_syn_items[polar], P->nsyn_items[polar], st);
+  return launch_leg_mixed_items(P, 0, polar, syn_items(P, polar), nsyn_items(P, polar), st);
 }
 
 cudaError_t launch_leg_ana_mixed(const sht_plan_s *P, int polar, cudaStream_t st) {

@@ -703,7 +703,7 @@ bool tc_supported(int spin, int njobs_pad) {
 // (108) 3600 / 3130, 4095 25.6 / 20.9 ms.
 bool tc_syn_two_tiles(const sht_plan_s *P, int64_t tiles) {
   constexpr int kTwoPerSm = 40;
-  return P->spin == 0 && P->njobs_pad <= 2 && tiles >= (int64_t)kTwoPerSm * P->sms;
+  return P->precision == SHT_MIXED && P->spin == 0 && P->njobs_pad <= 2 && tiles >= (int64_t)kTwoPerSm * P->sms;
 }
 
 namespace {

@@ -847,6 +847,7 @@ static void free_plan(sht_plan_s *P) {
     if (p) cudaFree(p);
   for (int k = 0; k < 2; ++k) {
     if (P->d_syn_items[k]) cudaFree(P->d_syn_items[k]);
+    if (P->d_syn_two[k]) cudaFree(P->d_syn_two[k]);
     if (P->d_syn_first[k]) cudaFree(P->d_syn_first[k]);
     if (P->d_ana_items[k]) cudaFree(P->d_ana_items[k]);
     if (P->d_ana_part_off[k]) cudaFree(P->d_ana_part_off[k]);
@@ -941,9 +942,9 @@ static int build_syn_lists(sht_plan_s *P) {
   int64_t ntile = 0;  // of the polar-cut variant
   for (int i = 0; i < P->nm; ++i)
     if (P->lmax >= std::max(P->mval[i], as)) ntile += (P->npairs + kSynTile - 1) / kSynTile - P->first_pair[i] / kSynTile;
-  P->syn_two = P->tc_syn && tc_syn_two_tiles(P, ntile);
+  P->syn_two = tc_syn_two_tiles(P, ntile);
   for (int polar = 0; polar < 2; ++polar) {
-    std::vector<std::pair<int64_t, int2>> syn, lo;
+    std::vector<std::pair<int64_t, int2>> syn, two, lo;
     std::vector<int> sfirst(P->nm);
     int64_t trip = 0;
     for (int i = 0; i < P->nm; ++i) {
@@ -957,22 +958,26 @@ static int build_syn_lists(sht_plan_s *P) {
       trip += (int64_t)(P->npairs - fp) * nl;
       int sf = (fp / kSynTile) * kSynTile;
       sfirst[i] = sf;
-      for (int p = sf; p < P->npairs; p += kSynTile) {
-        const bool l = lo_item(P, i, p, p + kSynTile);
-        if (P->syn_two && !l && p + kSynTile < P->npairs && !lo_item(P, i, p + kSynTile, p + 2 * kSynTile)) {
-          syn.push_back({(int64_t)nl * std::min(2 * kSynTile, P->npairs - p), make_int2(i, p | kSynTwoTiles)});
-          p += kSynTile;
-          continue;
-        }
-        (l ? lo : syn).push_back({(int64_t)nl * std::min(kSynTile, P->npairs - p), make_int2(i, p)});
+      for (int p = sf; p < P->npairs; p += kSynTile)
+        (lo_item(P, i, p, p + kSynTile) ? lo : syn)
+            .push_back({(int64_t)nl * std::min(kSynTile, P->npairs - p), make_int2(i, p)});
+      // the same tiles for the kernel that takes two neighbours where both are its own
+      for (int p = sf; P->syn_two && p < P->npairs; p += kSynTile) {
+        if (lo_item(P, i, p, p + kSynTile)) continue;
+        const bool pair = p + kSynTile < P->npairs && !lo_item(P, i, p + kSynTile, p + 2 * kSynTile);
+        two.push_back({(int64_t)nl * std::min((pair ? 2 : 1) * kSynTile, P->npairs - p), make_int2(i, pair ? p | kSynTwoTiles : p)});
+        if (pair) p += kSynTile;
       }
     }
     P->triples[polar] = trip;
     std::stable_sort(syn.begin(), syn.end(), [](auto &a, auto &b) { return a.first > b.first; });
+    std::stable_sort(two.begin(), two.end(), [](auto &a, auto &b) { return a.first > b.first; });
     std::stable_sort(lo.begin(), lo.end(), [](auto &a, auto &b) { return a.first > b.first; });
     P->syn_list[polar] = syn;
+    P->syn_list_two[polar] = two;
     P->syn_list_lo[polar] = lo;
     if ((rc = upload_list(P, syn, &P->d_syn_items[polar], &P->nsyn_items[polar])) != SHT_OK) return rc;
+    if ((rc = upload_list(P, two, &P->d_syn_two[polar], &P->nsyn_two[polar])) != SHT_OK) return rc;
     if ((rc = upload_list(P, lo, &P->d_syn_lo[polar], &P->nsyn_lo[polar])) != SHT_OK) return rc;
     if (P->d_syn_first[polar]) cudaFree(P->d_syn_first[polar]);
     P->d_syn_first[polar] = nullptr;
@@ -1452,15 +1457,8 @@ extern "C" int sht_plan_set_tensor_cores(sht_plan_t P, int on) {
     return fail(SHT_ERR_UNSUPPORTED, "tensor-core synthesis holds at most 32 columns (spin 0: ncomp <= 8, spin: ncomp <= 4)");
   if (P->batch_refs)
     return fail(SHT_ERR_INVALID_ARG, "the plan belongs to %d batch(es); destroy them first", P->batch_refs);
-  if ((on != 0) == (P->tc_syn != 0)) return SHT_OK;
   P->tc_syn = on ? 1 : 0;
-  if (P->spin || P->njobs_pad > 2) return SHT_OK;
-  int cur = -1;  // its items may take two tiles
-  cudaGetDevice(&cur);
-  if (cur != P->device) CUDA_TRY(cudaSetDevice(P->device));
-  const int rc = build_syn_lists(P);
-  if (cur != P->device) cudaSetDevice(cur);
-  return rc;
+  return SHT_OK;
 }
 
 extern "C" int sht_plan_set_tensor_core_analysis(sht_plan_t P, int on) {
@@ -1710,7 +1708,7 @@ extern "C" int sht_execute(sht_plan_t P, int type, double *const *alm, double *c
       });
       record(P->ev_lo, P->side);
     }
-    stage(0, st, [&] { return leg(0, P->d_syn_items[polar], P->nsyn_items[polar], st); });
+    stage(0, st, [&] { return leg(0, syn_items(P, polar), nsyn_items(P, polar), st); });
     if (lo) wait(st, P->ev_lo);
     stage(1, st, [&] { return launch_fft_syn(P, M, polar, weighted, add, st); });
   } else {

@@ -153,6 +153,8 @@ struct sht_plan_s {
   // work lists (polar-cut / uncut): synthesis (mi, first pair) and analysis (mi, tile, part offset)
   int2 *d_syn_items[2] = {nullptr, nullptr};
   int nsyn_items[2] = {0, 0};
+  int2 *d_syn_two[2] = {nullptr, nullptr};  // the items of the tensor-core kernel that takes two tiles (syn_two)
+  int nsyn_two[2] = {0, 0};
   int *d_syn_first[2] = {nullptr, nullptr};  // per m: first pair the synthesis wrote (FFT reads 0 below)
   int4 *d_ana_items[2] = {nullptr, nullptr};
   int nana_items[2] = {0, 0};
@@ -161,7 +163,7 @@ struct sht_plan_s {
   int ana_ppt = 4;                                  // ring pairs per analysis thread (tiling)
   int batch_refs = 0;                               // batches built on this plan's work lists
   // host copies of the work lists with their costs (l count x pairs), for merging into batches
-  std::vector<std::pair<int64_t, int2>> syn_list[2];
+  std::vector<std::pair<int64_t, int2>> syn_list[2], syn_list_two[2];
   std::vector<std::pair<int64_t, int4>> ana_list[2];
   // mixed form: the work items of columns m < fp64_m_below that touch a ring within
   // kFp64PolarCap of a pole run in the FP64 kernels (work lists of their own): there
@@ -171,7 +173,7 @@ struct sht_plan_s {
   bool fft_df = false;  // ring FFTs in double-float (mixed plans, by default)
   // mixed plans: the synthesis contraction on the tensor cores (legendre_tc.cu)
   int tc_syn = 0;
-  int syn_two = 0;  // its items are up to two tiles (spin 0, one or two maps)
+  int syn_two = 0;  // its items, where it is on, are up to two tiles (spin 0, one or two maps)
   // mixed plans: the analysis contraction on the tensor cores (legendre_tc_ana.cu;
   // tiles of kAnaThreads ring pairs, one per thread)
   int tc_ana = 0;
@@ -289,6 +291,11 @@ cudaError_t launch_leg_tc_batch(int spin, int nj, bool two, const void *targs, c
                                 cudaStream_t st);
 bool tc_supported(int spin, int njobs_pad);
 bool tc_syn_two_tiles(const sht_plan_s *P, int64_t tiles);  // its items are up to two of the tiles
+inline bool syn_two_on(const sht_plan_s *P) { return P->tc_syn && P->syn_two; }
+inline const int2 *syn_items(const sht_plan_s *P, int polar) {
+  return syn_two_on(P) ? P->d_syn_two[polar] : P->d_syn_items[polar];
+}
+inline int nsyn_items(const sht_plan_s *P, int polar) { return syn_two_on(P) ? P->nsyn_two[polar] : P->nsyn_items[polar]; }
 float tc_lambda_bound(int lmax);
 // tensor-core analysis (legendre_tc_ana.cu): mixargs with its analysis work list set
 cudaError_t launch_leg_tc_ana(const sht_plan_s *P, const void *mixargs, int n, cudaStream_t st);
