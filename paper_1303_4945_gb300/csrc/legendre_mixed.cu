@@ -16,7 +16,7 @@
 // are scaled down every 8 steps; values at scale 0 and -1 are accumulated (the
 // latter times 2^-104), anything smaller is negligible.  A mixed plan hands the
 // items of small m near the poles to the FP64 kernels (sht_plan_s::fp64_m_below).
-#include "mixed_common.cuh"
+#include "dual.cuh"
 
 namespace sht {
 
@@ -640,6 +640,212 @@ __device__ __forceinline__ void mix_ana_body(const MixArgs &a, const int4 item) 
     }
   }
 }
+// ---------------------------------------------------------------------------
+// Spin 0, two ring pairs per thread: the same tiles, chunks and slots with the packed
+// FP32 instructions of dual.cuh -- the two pairs' recursions as two lanes, the real and
+// imaginary sums of a product as two lanes, and of a warp's 32 columns two at a time in
+// the reduction, whose slot table holds high and low words in planes of their own (so
+// that two columns' words load as a pair) -- and one CTA barrier per two chunks, after
+// which warps 0 and 1 add one chunk each.
+// Bound by the FP32 pipe (a packed instruction holds it twice as long) and by warps
+// waiting for one another at the barrier (1.7 stalls per issue each, 68% issue at 24 warps
+// per SM).  One map, lmax 4095 22.7 -> 21.6 ms (packed lanes 22.6, one barrier per two
+// chunks 21.9, the products' multiplies scalar again, without the moves that doubled an
+// operand, 21.6); HEALPix 1535 1.89 -> 1.78 ms; lmax 511 147 -> 133 us.  4, 5, 7 or 8 CTAs
+// per SM instead of six were slower (24.0, 23.8, 23.0, 22.8 against 22.7 before).
+// ---------------------------------------------------------------------------
+template <int NJ>
+__device__ __forceinline__ void mix_ana_pair_body(const MixArgs &a, const int4 item) {
+  constexpr int V = 2 * NJ, LC = 32 / V, TH = kAnaThreads, NP = 2;
+  constexpr int ROW = TH + 2;  // 16 rows' pairs of words fall into different banks
+  static_assert(LC % 2 == 0 && ROW % 2 == 0, "two degrees at a time; pairs of words");
+  __shared__ __align__(8) float sloth[32][ROW], slotl[32][ROW];
+  __shared__ f2 quart[2][2][TH / 32][32];  // by parity of the chunk pair, chunk
+  __shared__ int tstart[2][TH / 32];     // per tile (parity): the warps' earliest join degree
+  const int mi = item.x, ng = item.z & 255;
+  const int m = a.mval[mi], l0 = m, lmax = a.lmax, nl = lmax - l0 + 1;
+  const float4 *__restrict__ cf = a.coef32 + (a.coef_off[mi] - l0);
+  double *const outp = a.part + a.part_off[mi] + (int64_t)(item.z >> 8) * nl * V;
+  const int tid = threadIdx.x;
+
+#pragma unroll 1
+  for (int gi = 0; gi < ng; ++gi) {
+    const int tile = item.y + gi;
+    Dual<false> rec;
+    rec.p = rec.q = d2{both(0.f), both(0.f)};
+    int sc[NP] = {0, 0}, lj[NP];
+    // G_N + G_S and G_N - G_S of each pair: high and low words, (re, im) as lanes
+    float2 gh[NP][NJ][2], gl[NP][NJ][2];
+    double xd[NP];
+    bool near = false;
+#pragma unroll
+    for (int k = 0; k < NP; ++k) {
+      const int p = tile * (TH * NP) + tid + k * TH;
+      const bool valid = p < a.npairs;
+      const PairDev pd = a.pairs[valid ? p : 0];
+      xd[k] = pd.x;
+      near = near || (valid && 1.0 - pd.x < 0.5 * kPolarTheta * kPolarTheta);
+      lj[k] = valid ? __float_as_int(__ldg(a.join + ((size_t)mi * a.npairs + p) * 3 + 2).z) : lmax + 1;
+#pragma unroll
+      for (int j = 0; j < NJ; ++j) {
+        double2 gn = make_double2(0, 0), gs = make_double2(0, 0);
+        if (valid) {
+          const double2 *gp = a.phase + (((size_t)j * a.nm + mi) * a.npairs + p) * 2;
+          gn = gp[0];
+          if (pd.south) gs = gp[1];
+        }
+        const f2 er = f2_of(gn.x + gs.x), ei = f2_of(gn.y + gs.y);
+        const f2 orr = f2_of(gn.x - gs.x), oi = f2_of(gn.y - gs.y);
+        gh[k][j][0] = make_float2(er.h, ei.h);
+        gl[k][j][0] = make_float2(er.l, ei.l);
+        gh[k][j][1] = make_float2(orr.h, oi.h);
+        gl[k][j][1] = make_float2(orr.l, oi.l);
+      }
+    }
+    const int jmin = min(lj[0], lj[1]);
+    const bool polar = __any_sync(0xffffffffu, near);
+#pragma unroll
+    for (int k = 0; k < NP; ++k) rec.x[k] = node_of(xd[k], polar);
+
+    // the tile's earliest join block; the first tile zeroes the slot's degrees before it
+    {
+      const int wmin = __reduce_min_sync(0xffffffffu, jmin);
+      if ((tid & 31) == 0) tstart[gi & 1][tid >> 5] = wmin;
+    }
+    __syncthreads();
+    int lstart = tstart[gi & 1][0];
+#pragma unroll
+    for (int w = 1; w < TH / 32; ++w) lstart = min(lstart, tstart[gi & 1][w]);
+    if (gi == 0)
+      for (int i = tid; i < (min(lstart, lmax + 1) - l0) * V; i += TH) outp[i] = 0.0;
+
+    float2 wf = both(1.f);  // the lanes' accumulation weights
+    // degree l into row q of the chunk (past lmax lmax's coefficients stand in: finite
+    // values, never stored); ODD: the sums over G_N - G_S
+    auto step = [&](const StepMode mode, int l, int q, const int odd, const bool act) __attribute__((always_inline)) {
+      const float4 cc = __ldg(cf + (l <= lmax ? l : lmax));
+      float2 h = rec.p.h, lo = rec.p.l;
+      if (!act) {
+        h = mul2(h, wf);
+        lo = mul2(lo, wf);
+      }
+#pragma unroll
+      for (int j = 0; j < NJ; ++j) {
+        // each pair's exact product (one multiply, three FMAs a part), then their sum
+        const float2 A = gh[0][j][odd], a1 = gl[0][j][odd], B = gh[1][j][odd], b1 = gl[1][j][odd];
+        const float2 p = make_float2(__fmul_rn(h.x, A.x), __fmul_rn(h.x, A.y));
+        const float2 r = make_float2(__fmul_rn(h.y, B.x), __fmul_rn(h.y, B.y));
+        float2 e, f;
+        e.x = __fmaf_rn(lo.x, A.x, __fmaf_rn(h.x, a1.x, __fmaf_rn(h.x, A.x, -p.x)));
+        e.y = __fmaf_rn(lo.x, A.y, __fmaf_rn(h.x, a1.y, __fmaf_rn(h.x, A.y, -p.y)));
+        f.x = __fmaf_rn(lo.y, B.x, __fmaf_rn(h.y, b1.x, __fmaf_rn(h.y, B.x, -r.x)));
+        f.y = __fmaf_rn(lo.y, B.y, __fmaf_rn(h.y, b1.y, __fmaf_rn(h.y, B.y, -r.y)));
+        const d2 t = two_sum(p, r);
+        const float2 tl = add2(e, add2(t.l, f));
+        sloth[q * V + 2 * j][tid] = t.h.x;
+        sloth[q * V + 2 * j + 1][tid] = t.h.y;
+        slotl[q * V + 2 * j][tid] = tl.x;
+        slotl[q * V + 2 * j + 1][tid] = tl.y;
+      }
+      rec.step(mode, cc);
+    };
+    auto skip = [&](const StepMode mode, int l, int q) __attribute__((always_inline)) {  // no terms
+#pragma unroll
+      for (int v = 0; v < V; ++v) sloth[q * V + v][tid] = slotl[q * V + v][tid] = 0.f;
+      rec.step(mode, __ldg(cf + (l <= lmax ? l : lmax)));
+    };
+
+    int since = 0;         // steps since the last exponent check
+    bool settled = false;  // every lane's values at scale 0: they stay there (warp-uniform)
+    int cb = 0;            // parity of the chunk pair: the quart buffer
+    for (int lb2 = lstart; lb2 <= lmax; lb2 += 2 * LC) {
+      // the slot entry that this lane adds to (warps 0 and 1: one chunk each), from the
+      // previous tiles: read early, added at the end
+      const int ch = tid >> 5, ll = lb2 + ch * LC + (tid & 31) / V;
+      const bool mine = ch < 2 && ll <= lmax;
+      double *const o = outp + (int64_t)(lb2 + ch * LC - l0) * V + (tid & 31);
+      const double prev = (gi > 0 && mine) ? *o : 0.0;
+#pragma unroll 1
+      for (int c2 = 0; c2 < 2; ++c2) {
+        const int lb = lb2 + c2 * LC;
+        bool joins = false;
+#pragma unroll
+        for (int k = 0; k < NP; ++k)
+          if (lj[k] == lb) {
+            const int p = tile * (TH * NP) + tid + k * TH;
+            const JoinRec r = ld_join(a.join + ((size_t)mi * a.npairs + p) * 3, polar);
+            rec.start(k, r.lpc, r.lpp, 1.f);
+            sc[k] = r.scp;
+            joins = true;
+          }
+        if (joins) wf = make_float2(scale_weight(sc[0]), scale_weight(sc[1]));
+        if (__any_sync(0xffffffffu, joins)) settled = false;
+        // a warp none of whose lanes has joined skips this chunk's steps
+        const bool wlive = lb <= lmax && __any_sync(0xffffffffu, jmin <= lb);
+        auto chunk = [&](const StepMode mode) __attribute__((always_inline)) {
+#pragma unroll 1
+          for (int q = 0; q < LC; q += 2) {
+            const int l = lb + q;
+            if (l > lmax) break;
+            if (!settled) settled = __all_sync(0xffffffffu, sc[0] == 0 && sc[1] == 0);
+            if (settled) {
+              step(mode, l, q, 0, true);
+              step(mode, l + 1, q + 1, 1, true);
+            } else {
+              if (__all_sync(0xffffffffu, negligible(lane0(rec.p), sc[0]) && negligible(lane1(rec.p), sc[1]))) {
+                skip(mode, l, q);
+                skip(mode, l + 1, q + 1);
+              } else {
+                step(mode, l, q, 0, false);
+                step(mode, l + 1, q + 1, 1, false);
+              }
+              since += 2;
+              if (since >= 8) {
+                rec.rescale(sc[0], sc[1]);
+                wf = make_float2(scale_weight(sc[0]), scale_weight(sc[1]));
+                since = 0;
+              }
+            }
+          }
+        };
+        if (wlive) {
+          if (polar) chunk(kPolar);
+          else chunk(kCareful);
+        }
+        // a warp's slot columns are written and read by that warp only: warp-level sync
+        __syncwarp();
+        // each warp sums its own 32 columns of its lane's row
+        const int sl = tid & 31, part = tid >> 5;
+        f2 t = {0.f, 0.f};
+        if (wlive) {
+          const float2 *rh = reinterpret_cast<const float2 *>(&sloth[sl][part * 32]);
+          const float2 *rl = reinterpret_cast<const float2 *>(&slotl[sl][part * 32]);
+          d2 c = {rh[0], rl[0]};
+#pragma unroll
+          for (int i = 1; i < 16; ++i) {
+            const d2 u = two_sum(c.h, rh[i]);
+            c = {u.h, add2(add2(c.l, rl[i]), u.l)};
+          }
+          t = f2_add_lazy(lane0(c), lane1(c));
+        }
+        quart[cb][c2][part][sl] = t;
+        __syncwarp();
+      }
+      // one barrier per two chunks: quart is double-buffered, so warps 0 and 1 read these
+      // partials while the others fill the other buffer, and they have read them before
+      // they reach the next barrier, after which this buffer is written again
+      __syncthreads();
+      if (ch < 2) {
+        f2 t = quart[cb][ch][0][tid & 31];
+#pragma unroll
+        for (int w = 1; w < TH / 32; ++w) t = f2_add(t, quart[cb][ch][w][tid & 31]);
+        if (mine) *o = prev + f2_val(t);
+      }
+      cb ^= 1;
+    }
+  }
+}
+
 // one-job shapes of up to two pairs a thread are held to 80 registers: six CTAs
 // per SM instead of five (their shared slot table allows six); measured at one
 // E/B pair, lmax 4095: 84.1 ms against 85.0 (two pairs) and 84.0 against 86.8 (one)
@@ -649,14 +855,20 @@ constexpr int mix_ana_min_blocks() {
 }
 template <int NJ, int PPT, bool SPIN>
 __global__ void __launch_bounds__(kAnaThreads, (mix_ana_min_blocks<NJ, PPT, SPIN>())) mix_ana(MixArgs a) {
-  mix_ana_body<NJ, PPT, SPIN>(a, a.ana_items[blockIdx.x]);
+  if constexpr (!SPIN && PPT == 2)
+    mix_ana_pair_body<NJ>(a, a.ana_items[blockIdx.x]);
+  else
+    mix_ana_body<NJ, PPT, SPIN>(a, a.ana_items[blockIdx.x]);
 }
 template <int NJ, int PPT, bool SPIN>
 __global__ void __launch_bounds__(kAnaThreads, (mix_ana_min_blocks<NJ, PPT, SPIN>())) mix_ana_batch(const MixArgs *__restrict__ args,
     const int4 *__restrict__ items) {
   const int4 it = items[blockIdx.x];
   const MixArgs &a = args[it.w];
-  mix_ana_body<NJ, PPT, SPIN>(a, make_int4(it.x, it.y, it.z, 0));
+  if constexpr (!SPIN && PPT == 2)
+    mix_ana_pair_body<NJ>(a, make_int4(it.x, it.y, it.z, 0));
+  else
+    mix_ana_body<NJ, PPT, SPIN>(a, make_int4(it.x, it.y, it.z, 0));
 }
 
 // ---------------------------------------------------------------------------

@@ -124,3 +124,24 @@ def test_analysis_keeps_nan(sht, bad, ncomp, tca):
         assert not torch.isfinite(torch.view_as_real(alm[0])[lmax + 1:]).any()
         assert not torch.isfinite(alm[0][: lmax + 1].real).any()
         assert all(torch.isfinite(torch.view_as_real(a)).all() for a in alm[1:])
+
+
+@pytest.mark.parametrize("nlat,lmax", [(1, 0), (2, 1), (31, 33), (254, 47), (257, 64), (511, 300), (514, 65), (770, 515), (700, 2100)])
+@pytest.mark.parametrize("ncomp", [1, 2])
+def test_analysis_of_two_pairs_a_thread(sht, nlat, lmax, ncomp):
+    """Rings around whole tiles of 256 pairs, last chunks of every length class, FP64
+    columns (lmax >= 2000), no polar cut, added outputs."""
+    geom = sht.sht_geom_gauss(nlat, 64)
+    lay = sht.sht_alm_create(lmax, lmax)
+    mixed = sht.sht_plan_create(geom, lay, 0, ncomp, sht.SHT_MIXED)
+    mixed.set_tiling(2)
+    ref = sht.sht_plan_create(geom, lay, 0, ncomp, sht.SHT_FP64)
+    g = torch.Generator(device="cuda").manual_seed(512)
+    maps = [torch.randn(geom.npix, dtype=torch.float64, device="cuda", generator=g) for _ in range(ncomp)]
+    got, want = ([torch.ones(lay.size(), dtype=torch.complex128, device="cuda") for _ in range(ncomp)] for _ in range(2))
+    for flags in (0, sht.SHT_NO_POLAR_OPT, sht.SHT_ADD_OUTPUT):
+        for type_ in (sht.SHT_ANALYSIS, sht.SHT_ADJOINT_SYNTHESIS):
+            sht.sht_execute(mixed, type_, got, maps, flags)
+            sht.sht_execute(ref, type_, want, maps, flags)
+            for x, y in zip(got, want):
+                assert rel(x, y) <= MIX_L2
