@@ -355,6 +355,7 @@ __global__ void __launch_bounds__(kSynTile) mix_syn_spin_batch(const MixArgs *__
 template <int NJ, int PPT, bool SPIN>
 __device__ __forceinline__ void mix_ana_body(const MixArgs &a, const int4 item) {
   constexpr int V = (SPIN ? 4 : 2) * NJ, LC = 32 / V;
+  constexpr bool OUT = PPT >= 2;  // the polar steps (step_spin)
   static_assert(V * LC == 32, "32 slots per chunk");
   __shared__ f2 slot[32][kAnaThreads + 1];
   __shared__ f2 quart[2][kAnaThreads / 32][32];  // by chunk parity
@@ -383,14 +384,14 @@ __device__ __forceinline__ void mix_ana_body(const MixArgs &a, const int4 item) 
     f2 g[PPT][NJ][SPIN ? 4 : 2][2];
     int jmin = lmax + 1;
     double xd[PPT];
-    bool near = false;
+    bool near[PPT];
   #pragma unroll
     for (int k = 0; k < PPT; ++k) {
       const int p = tile * (kAnaThreads * PPT) + tid + k * kAnaThreads;
       const bool valid = p < a.npairs;
       const PairDev pd = a.pairs[valid ? p : 0];
       xd[k] = pd.x;
-      near = near || (valid && 1.0 - pd.x < 0.5 * kPolarTheta * kPolarTheta);
+      near[k] = valid && 1.0 - pd.x < 0.5 * kPolarTheta * kPolarTheta;
       lj[k] = valid ? __float_as_int(__ldg(a.join + ((size_t)mi * a.npairs + p) * 3 + 2).z) : lmax + 1;
       jmin = min(jmin, lj[k]);
       lpc[k] = lmc[k] = lpp[k] = lmp[k] = f2{0.f, 0.f};
@@ -432,9 +433,14 @@ __device__ __forceinline__ void mix_ana_body(const MixArgs &a, const int4 item) 
       }
     }
 
-    const bool polar = __any_sync(0xffffffffu, near);
+    // which of the warp's pairs run the difference form: of a tile's pairs the first
+    // 128 at most hold the rings that need it, and a CTA waits for its slowest warp
+    unsigned polar = 0u;
   #pragma unroll
-    for (int k = 0; k < PPT; ++k) x[k] = node_of(xd[k], polar);
+    for (int k = 0; k < PPT; ++k) {
+      if (__any_sync(0xffffffffu, near[k])) polar |= 1u << k;
+      x[k] = node_of(xd[k], (polar >> k) & 1u);
+    }
 
     // the tile starts at its pairs' earliest join block; the first tile of the group
     // zeroes the slot's degrees before it (the others leave their sums there)
@@ -472,7 +478,7 @@ __device__ __forceinline__ void mix_ana_body(const MixArgs &a, const int4 item) 
               acc_mul(c[2 * j + 1], wp, gi.h, gi.l);
             }
           }
-          step_s0(cc, x[k], pol, lpc[k], lpp[k]);
+          step_s0<OUT>(cc, x[k], OUT ? (polar >> k) & 1u : pol, lpc[k], lpp[k]);
         } else {
           const f2 wm = act ? lmc[k] : weight(lmc[k], scm[k]);
           const f2 sp = odd ? neg(wp) : wp, sm = odd ? neg(wm) : wm;
@@ -495,7 +501,7 @@ __device__ __forceinline__ void mix_ana_body(const MixArgs &a, const int4 item) 
             acc_mul(c[4 * j + 2], sp, g[k][j][3][0].h, g[k][j][3][0].l);
             acc_mul(c[4 * j + 3], sp, g[k][j][3][1].h, g[k][j][3][1].l);
           }
-          step_spin(cc, x[k], pol, lpc[k], lpp[k], lmc[k], lmp[k]);
+          step_spin<OUT>(cc, x[k], OUT ? (polar >> k) & 1u : pol, lpc[k], lpp[k], lmc[k], lmp[k]);
         }
       }
     };
@@ -523,8 +529,9 @@ __device__ __forceinline__ void mix_ana_body(const MixArgs &a, const int4 item) 
       const Coef32 cc = ld_coef32(cf + (l <= lmax ? l : lmax));
   #pragma unroll
       for (int k = 0; k < PPT; ++k) {
-        if (!SPIN) step_s0(cc, x[k], pol, lpc[k], lpp[k]);
-        else step_spin(cc, x[k], pol, lpc[k], lpp[k], lmc[k], lmp[k]);
+        const bool pk = OUT ? (polar >> k) & 1u : pol;
+        if (!SPIN) step_s0<OUT>(cc, x[k], pk, lpc[k], lpp[k]);
+        else step_spin<OUT>(cc, x[k], pk, lpc[k], lpp[k], lmc[k], lmp[k]);
       }
     };
     auto mode = [&]() {  // 0: all terms at scale 0, 2: all negligible, 1: weighted
@@ -548,7 +555,7 @@ __device__ __forceinline__ void mix_ana_body(const MixArgs &a, const int4 item) 
       for (int k = 0; k < PPT; ++k)
         if (lj[k] == lb) {
           const int p = tile * (kAnaThreads * PPT) + tid + k * kAnaThreads;
-          const JoinRec r = ld_join(a.join + ((size_t)mi * a.npairs + p) * 3, polar);
+          const JoinRec r = ld_join(a.join + ((size_t)mi * a.npairs + p) * 3, (polar >> k) & 1u);
           lpc[k] = r.lpc;
           lpp[k] = r.lpp;
           lmc[k] = r.lmc;
@@ -609,7 +616,8 @@ __device__ __forceinline__ void mix_ana_body(const MixArgs &a, const int4 item) 
         }
       };
       if (wlive) {
-        if (polar) chunk(true);
+        if (OUT) chunk(false);
+        else if (polar) chunk(true);
         else chunk(false);
       }
       // a warp's slot columns are written and read by that warp only: warp-level sync

@@ -175,21 +175,44 @@ __device__ __forceinline__ void step_polar(f2 a, f2 b, const f3 &y, f2 &p, f2 &d
   p = f2_add(p, d);
 }
 // one step of the +s / -s recursions (spin 0: the +s one with b = 0); polar: see above.
-// The kernels pass a constant, chosen around their loops: a test per step cost 7 - 10%.
+// Small shapes pass a constant, chosen around their loops (a test per step cost them 7 -
+// 10%); OUT: large ones test per step and call the difference form out of line, as a
+// second copy of their loops (or the form inlined) overflows the instruction cache
+// (analysis of two spin-2 pairs at two ring pairs a thread, lmax 1023: 5.5 ms with two
+// copies, 3.9 inlined, kOutNote called).
+struct PolarState {
+  f2 p, d;
+};
+static __device__ __noinline__ PolarState step_polar_out(f2 a, f2 b, float yh, float ym, f2 p, f2 d) {
+  step_polar(a, b, f3{yh, ym, 0.f}, p, d);
+  return {p, d};
+}
+template <bool OUT>
+__device__ __forceinline__ void step_polar_at(f2 a, f2 b, const f3 &y, f2 &p, f2 &d) {
+  if (OUT) {
+    const PolarState r = step_polar_out(a, b, y.h, y.m, p, d);
+    p = r.p;
+    d = r.d;
+  } else {
+    step_polar(a, b, y, p, d);
+  }
+}
+template <bool OUT = false>
 __device__ __forceinline__ void step_s0(const Coef32 &c, const f3 &x, bool polar, f2 &lc, f2 &lp) {
   if (polar) {
-    step_polar(c.a, f2{0.f, 0.f}, x, lc, lp);
+    step_polar_at<OUT>(c.a, f2{0.f, 0.f}, x, lc, lp);
     return;
   }
   const f2 n = mul_sub(mul(c.a, x), lc, lp);
   lp = lc;
   lc = n;
 }
+template <bool OUT = false>
 __device__ __forceinline__ void step_spin(const Coef32 &c, const f3 &x, bool polar, f2 &lpc, f2 &lpp, f2 &lmc,
                                           f2 &lmp) {
   if (polar) {
-    step_polar(c.a, c.b, x, lpc, lpp);
-    step_polar(c.a, neg(c.b), x, lmc, lmp);
+    step_polar_at<OUT>(c.a, c.b, x, lpc, lpp);
+    step_polar_at<OUT>(c.a, neg(c.b), x, lmc, lmp);
     return;
   }
   const f2 t = mul(c.a, x);

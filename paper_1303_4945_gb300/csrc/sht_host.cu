@@ -877,15 +877,18 @@ static int upload(sht_plan_s *P, const std::vector<T> &h, T **d) {
 }
 
 // Tilings of the analysis Legendre kernels (ring pairs per thread) built for a
-// spin class and padded job count; the first is the default.  One spin-0 map: two pairs a
-// thread in the mixed form (lmax 4095 22.6 ms against 24.7 at four, lmax 1535 on HEALPix
-// 1.89 against 2.53: four spill), four in FP64.
+// spin class and padded job count; the first is the default.  In the mixed form the
+// difference form of the warps next to a pole weighs more the more pairs a thread has
+// (their CTA waits for them): spin 0 two pairs a thread, packed (lmax 1023, one map 0.50 ms,
+// two 0.76, against four's figures in mix_ana_body), spin s one (one E/B pair 1.29 ms against
+// 1.77 at two, two 2.31 against 3.38).
 static std::vector<int> ana_ppt_candidates(int spin, int nj, int precision) {
   if (spin == 0) {
     if (nj == 1) return precision == SHT_MIXED ? std::vector<int>{2, 4, 8} : std::vector<int>{4, 8, 2};
-    if (nj == 2) return {4, 2};
+    if (nj == 2) return precision == SHT_MIXED ? std::vector<int>{2, 4} : std::vector<int>{4, 2};
     return {2};
   }
+  if (precision == SHT_MIXED && nj <= 2) return nj == 1 ? std::vector<int>{1, 2, 4} : std::vector<int>{1, 2};
   if (nj == 1) return {2, 4, 1};
   if (nj == 2) return {2, 1};
   return {2};
@@ -1090,12 +1093,14 @@ static int build_ana_lists(sht_plan_s *P, int ppt) {
   }
   P->ana_ppt = ppt;
   // What the call that allocates nothing counts against its area: of the FP64 form the
-  // FP64 kernel's tiling, of one spin-0 map in the mixed form four pairs a thread until a
-  // tiling is chosen, whichever tiles run
+  // FP64 kernel's tiling, of one or two jobs in the mixed form four pairs a thread (spin 0)
+  // or two until a tiling is chosen, whichever tiles run
   P->part_limit = need;
   if (P->tc64_ana) P->part_limit = ana_part_need(P, kAnaThreads * ppt, 1);
-  else if (mixed && P->spin == 0 && P->njobs_pad == 1 && !P->tc_ana && !P->tiling_chosen)
-    P->part_limit = ana_part_need(P, kAnaThreads * 4, ana_group(P, kAnaThreads * 4, 1));
+  else if (mixed && P->njobs_pad <= 2 && !P->tc_ana && !P->tiling_chosen) {
+    const int ta = kAnaThreads * (P->spin ? 2 : 4);
+    P->part_limit = ana_part_need(P, ta, ana_group(P, ta, 1));
+  }
   return SHT_OK;
 }
 
