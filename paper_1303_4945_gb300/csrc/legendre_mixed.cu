@@ -1044,7 +1044,8 @@ cudaError_t launch_leg_mixed_items(const sht_plan_s *P, int stage, int polar, co
       });
     else
       ana_shape_spin(nj, P->ana_ppt, [&](auto sh) {
-        mix_ana<decltype(sh)::nj, decltype(sh)::ppt, true><<<n, kAnaThreads, 0, st>>>(a);
+        if constexpr (decltype(sh)::nj <= 2)
+          mix_ana<decltype(sh)::nj, decltype(sh)::ppt, true><<<n, kAnaThreads, 0, st>>>(a);
       });
   }
   return cudaGetLastError();
@@ -1112,7 +1113,8 @@ cudaError_t launch_leg_mixed_batch(int stage, int spin, int nj, int ppt, const v
       });
     else
       ana_shape_spin(nj, ppt, [&](auto sh) {
-        mix_ana_batch<decltype(sh)::nj, decltype(sh)::ppt, true><<<n, kAnaThreads, 0, st>>>(a, items);
+        if constexpr (decltype(sh)::nj <= 2)
+          mix_ana_batch<decltype(sh)::nj, decltype(sh)::ppt, true><<<n, kAnaThreads, 0, st>>>(a, items);
       });
   }
   return cudaGetLastError();

@@ -95,6 +95,7 @@ struct AnaShape {
   static constexpr int WARPS = TH / 32;
   static constexpr int NP = SPIN ? 1 : 2;                // ring pairs per thread
   static constexpr bool QUAD = NJ == 4;
+  static constexpr bool GROUPED = QUAD || (SPIN && NJ == 2);  // runs plans of more jobs NJ at a time
   static constexpr int TILE = QUAD ? 2 * kTile : kTile;  // ring pairs per tile of the work list
   static constexpr int TILES = NP * TH / TILE;           // tiles walked at a time
   static constexpr int NACC = NJ == 1 ? 4 : 2;           // accumulators
@@ -204,7 +205,7 @@ __device__ __forceinline__ void split6(float2 h, float2 l, float2 (&d)[kDig]) {
 // G_N - G_S, the two lanes two neighbouring pairs.
 // ---------------------------------------------------------------------------
 template <int NJ, bool SPIN>
-__device__ __forceinline__ void tc_ana_body(const TcArgs &ta, const int4 item, const int j0, unsigned char *tca_smem) {
+__device__ __forceinline__ void tc_ana_body(const TcArgs &ta, const int4 item_, const int j0, unsigned char *tca_smem) {
   using S = tca::AnaShape<NJ, SPIN>;
   constexpr int NSET = S::NSET, NC = S::NC, kDig = tca::kDig, TH = S::TH, NP = S::NP;
   constexpr int NACC = S::NACC, GROUPS = S::GROUPS, LAG = S::LAG;
@@ -214,7 +215,10 @@ __device__ __forceinline__ void tc_ana_body(const TcArgs &ta, const int4 item, c
   __shared__ int tstart[S::WARPS];
   __shared__ volatile int stop;
   const MixArgs &a = ta.m;
-  const int V = S::QUAD ? 2 * a.nj : S::V;  // the plan's partial sums per degree; the CTA's jobs from j0 on
+  // the work list's tiles in tiles of this kernel (plans of more than two jobs: 256 pairs)
+  const int tmul = S::GROUPED && !S::QUAD && a.nj > NJ ? 2 : 1;
+  const int4 item = make_int4(item_.x, item_.y * tmul, ((item_.z >> 8) << 8) | ((item_.z & 255) * tmul), 0);
+  const int V = S::GROUPED ? (SPIN ? 4 : 2) * a.nj : S::V;  // the plan's partial sums per degree; the CTA's jobs from j0 on
   // the warp's number from a shuffle: the compiler sees it uniform, and so the MMAs'
   // descriptors, which then live in uniform registers
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
@@ -320,8 +324,8 @@ __device__ __forceinline__ void tc_ana_body(const TcArgs &ta, const int4 item, c
           gv[t][4 * j + 2] = gn.x - gs.x;
           gv[t][4 * j + 3] = gn.y - gs.y;
         } else {
-          const double2 *gq = a.phase + (((size_t)(2 * j) * a.nm + mi) * a.npairs + p) * 2;
-          const double2 *gu = a.phase + (((size_t)(2 * j + 1) * a.nm + mi) * a.npairs + p) * 2;
+          const double2 *gq = a.phase + (((size_t)(2 * (j0 + j)) * a.nm + mi) * a.npairs + p) * 2;
+          const double2 *gu = a.phase + (((size_t)(2 * (j0 + j) + 1) * a.nm + mi) * a.npairs + p) * 2;
           const double2 qn = gq[0], un = gu[0];
           const double2 qs = south ? gq[1] : make_double2(0.0, 0.0), us = south ? gu[1] : make_double2(0.0, 0.0);
           // W+_N, W-_N, W+_S', W-_S' (re, im)
@@ -390,7 +394,7 @@ __device__ __forceinline__ void tc_ana_body(const TcArgs &ta, const int4 item, c
       for (int i = tid; i < (min(lstart, lmax + 1) - l0) * S::V; i += TH) {
         const int v = i % S::V;
         const bool nan = bad && tca::not_finite(vmax[SPIN ? v : 4 * (v >> 1) + (v & 1)]);
-        if (gi == 0 || nan) outp[(int64_t)(i / S::V) * V + (S::QUAD ? 2 * j0 : 0) + v] = nan ? CUDART_NAN : 0.0;
+        if (gi == 0 || nan) outp[(int64_t)(i / S::V) * V + (SPIN ? 4 : 2) * j0 + v] = nan ? CUDART_NAN : 0.0;
       }
     // v_c of the column that this lane sums (epi_sum, epi_quad)
     const int vcol = S::QUAD ? 4 * (warp & 3) + ((lane >> 2) & 3) : (S::CPW == 1 ? (warp & 3) : 2 * (warp & 3) + ((lane >> 3) & 1));
@@ -535,7 +539,7 @@ __device__ __forceinline__ void tc_ana_body(const TcArgs &ta, const int4 item, c
       if (!oact || l > lmax) return nullptr;
       if (SPIN) {
         neg = cc >= 2 && (odeg & 1);  // T2 = s (s T2)
-        return outp + (int64_t)(l - l0) * V + 4 * j + cc;
+        return outp + (int64_t)(l - l0) * V + 4 * (j0 + j) + cc;
       }
       // spin 0: the even-l columns at even l - l0, the odd ones at odd
       return (cc >> 1) == (odeg & 1) ? outp + (int64_t)(l - l0) * V + 2 * j + (cc & 1) : nullptr;
@@ -755,7 +759,8 @@ template <int NJ, bool SPIN>
 __global__ void __launch_bounds__((tca::AnaShape<NJ, SPIN>::TH), (tca::AnaShape<NJ, SPIN>::MINB))
     tc_ana(TcArgs ta, int groups) {
   extern __shared__ __align__(128) unsigned char tca_smem[];
-  const int g = NJ == 4 ? blockIdx.x % groups : 0, i = NJ == 4 ? blockIdx.x / groups : blockIdx.x;
+  constexpr bool G = tca::AnaShape<NJ, SPIN>::GROUPED;
+  const int g = G ? blockIdx.x % groups : 0, i = G ? blockIdx.x / groups : blockIdx.x;
   tc_ana_body<NJ, SPIN>(ta, ta.m.ana_items[i], NJ * g, tca_smem);
 }
 
@@ -764,8 +769,9 @@ template <int NJ, bool SPIN>
 __global__ void __launch_bounds__((tca::AnaShape<NJ, SPIN>::TH), (tca::AnaShape<NJ, SPIN>::MINB))
     tc_ana_batch(const TcArgs *__restrict__ args, const int4 *__restrict__ items, int groups) {
   extern __shared__ __align__(128) unsigned char tca_smem[];
-  const int g = NJ == 4 ? blockIdx.x % groups : 0;
-  const int4 it = items[NJ == 4 ? blockIdx.x / groups : blockIdx.x];
+  constexpr bool G = tca::AnaShape<NJ, SPIN>::GROUPED;
+  const int g = G ? blockIdx.x % groups : 0;
+  const int4 it = items[G ? blockIdx.x / groups : blockIdx.x];
   tc_ana_body<NJ, SPIN>(args[it.w], make_int4(it.x, it.y, it.z, 0), NJ * g, tca_smem);
 }
 
@@ -800,7 +806,7 @@ bool tc_ana_supported(int spin, int njobs_pad) {
 // maps, lmax 31: 22 / 107 us, 2047: 20.2 / 65.7 ms), which has no instance for them.  Error
 // against the FP64 form: lmax 31 2.3e-14 to 2.4e-14 (that contraction 2.1e-14 to 2.4e-14),
 // 255 8.4e-14 (8.4e-14), 511 1.0e-13 (1.2e-13), 2047 3.7e-13 (3.7e-13).
-bool tc_ana_quad(const sht_plan_s *P) { return P->precision == SHT_MIXED && P->spin == 0 && P->njobs_pad >= 4; }
+bool tc_ana_quad(const sht_plan_s *P) { return P->precision == SHT_MIXED && P->njobs_pad >= 4; }
 
 int tc_ana_tiles(int spin, int njobs_pad) {
   if (spin == 0) return njobs_pad == 1 ? tca::AnaShape<1, false>::TILES : tca::AnaShape<2, false>::TILES;
@@ -822,7 +828,6 @@ bool tca_shape(int spin, int nj, F &&f) {
     else f(AnaLaunch<4, false>());
     return true;
   }
-  if (nj > 2) return false;
   if (nj == 1) f(AnaLaunch<1, true>());
   else f(AnaLaunch<2, true>());
   return true;

@@ -145,3 +145,23 @@ def test_analysis_of_two_pairs_a_thread(sht, nlat, lmax, ncomp):
             sht.sht_execute(ref, type_, want, maps, flags)
             for x, y in zip(got, want):
                 assert rel(x, y) <= MIX_L2
+
+
+@pytest.mark.parametrize("nlat,lmax,ncomp", [(2, 2, 4), (31, 33, 3), (257, 260, 5), (513, 518, 4), (700, 2100, 3), (254, 100, 8)])
+def test_spin_analysis_of_more_than_two_jobs(sht, nlat, lmax, ncomp):
+    """Two E/B pairs at a time on the tensor cores, over tiles of 256 ring pairs."""
+    geom = sht.sht_geom_gauss(nlat, 64)
+    lay = sht.sht_alm_create(lmax, lmax)
+    mixed = sht.sht_plan_create(geom, lay, 2, ncomp, sht.SHT_MIXED)
+    ref = sht.sht_plan_create(geom, lay, 2, ncomp, sht.SHT_FP64)
+    n = 2 * ncomp
+    g = torch.Generator(device="cuda").manual_seed(37)
+    maps = [torch.randn(geom.npix, dtype=torch.float64, device="cuda", generator=g) for _ in range(n)]
+    got, want = ([torch.ones(lay.size(), dtype=torch.complex128, device="cuda") for _ in range(n)] for _ in range(2))
+    for flags in (0, sht.SHT_NO_POLAR_OPT, sht.SHT_ADD_OUTPUT):
+        for type_ in (sht.SHT_ANALYSIS, sht.SHT_ADJOINT_SYNTHESIS):
+            sht.sht_execute(mixed, type_, got, maps, flags)
+            sht.sht_execute(ref, type_, want, maps, flags)
+            assert mixed.device_status() == 0
+            for x, y in zip(got, want):
+                assert rel(x, y) <= MIX_L2
