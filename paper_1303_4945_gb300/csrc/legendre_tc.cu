@@ -64,7 +64,6 @@ constexpr int kLamDigits = 3;       // bf16 digits of Lambda (plus an FP32 remai
 constexpr int kAlmDigits = 6;       // bf16 digits of the a_lm columns
 constexpr int kLevels = 6;          // TMEM levels read: digit products with i + j <= 5
 constexpr int kATile = kRows * kK * 2;  // bytes of one 128 x 16 bf16 tile
-constexpr int kPack = 8;            // degrees of digits held in registers before a 16-byte shared-memory store
 // the warp issuing the MMAs (an elected lane): the last, whose threads neither load
 // the staged rows nor build B (threads 0-63 at one E/B pair), so that the warps
 // reach the K-step's barrier together (152.4 -> 151.8 ms per headline pair)
@@ -83,6 +82,10 @@ constexpr int kIssuerWarp = 3;
 template <int NJ, bool SPIN, bool TWO>
 struct Shape {
   static constexpr bool DUAL = TWO;
+  // degrees of digits held in registers before a shared-memory store: eight, but four
+  // where the remainder sums of four E/B pairs make the unrolled code of three step
+  // forms outgrow the instruction cache (lmax 511 546 us at eight, 387 at four; 1023 2.37, 2.05 ms)
+  static constexpr int PACK = SPIN && NJ >= 4 ? 4 : 8;
   static constexpr int NP = DUAL ? 2 : 1;         // ring pairs per thread
   static constexpr int NL = SPIN || DUAL ? 2 : 1; // A sets
   static constexpr int NB = SPIN ? 2 : 1;         // B stacks
@@ -351,19 +354,19 @@ __device__ __forceinline__ void tc_syn_body(const TcArgs &ta, const int2 item, u
       rec.start(0, lc, lp, 1.f);
     }
   };
-  // kPack degrees from rows (lb - l0 even): digits (quanta 2^-7, 2^-15, 2^-23) packed
+  // PACK degrees from rows (lb - l0 even): digits (quanta 2^-7, 2^-15, 2^-23) packed
   // per pair of degrees into pk[set][digit][q / 2], remainders contracted into racc,
   // recursion advanced.  Unless every lane is at scale 0 (kFast; a polar warp tests
   // too) the values take their weights, and every second degree the warp votes: if
   // every lane's values are negligible for the next two steps (as in the double-float
   // kernels) the digits are zero and only the recursion runs.
   auto part = [&](const StepMode mode, const float4 *rows,
-                  uint32_t (&pk)[NL][tc::kLamDigits][tc::kPack / 2]) __attribute__((always_inline)) {
+                  uint32_t (&pk)[NL][tc::kLamDigits][S::PACK / 2]) __attribute__((always_inline)) {
     constexpr float s0 = 98304.0f, s1 = s0 * 0x1p-8f, s2 = s0 * 0x1p-16f;  // 1.5 * 2^23 * quantum
     float2 dlo[tc::kLamDigits];
     bool dead = false;
 #pragma unroll
-    for (int q = 0; q < tc::kPack; ++q) {
+    for (int q = 0; q < S::PACK; ++q) {
       // past lmax the staged rows are zero: the recursion runs on zero coefficients
       // (values of one degree's size, alternating) and meets zero a_lm, so those degrees
       // add nothing and need no test
@@ -440,15 +443,18 @@ __device__ __forceinline__ void tc_syn_body(const TcArgs &ta, const int2 item, u
     wf = make_float2(scale_weight(sc0), scale_weight(sc1));
     settled = __all_sync(0xffffffffu, sc0 == 0 && sc1 == 0);
   };
-  // this thread's digits of degrees q0 .. q0 + kPack - 1 of the K-step into the A tiles
-  auto store_a = [&](int q0, const uint32_t (&pk)[NL][tc::kLamDigits][tc::kPack / 2]) {
+  // this thread's digits of degrees q0 .. q0 + PACK - 1 of the K-step into the A tiles
+  auto store_a = [&](int q0, const uint32_t (&pk)[NL][tc::kLamDigits][S::PACK / 2]) {
 #pragma unroll
     for (int t = 0; t < NL; ++t)
 #pragma unroll
       for (int i = 0; i < tc::kLamDigits; ++i) {
         unsigned char *dst = Abuf + (t * tc::kLamDigits + i) * tc::kATile + (tid / 8) * 256 + (q0 / 8) * 128 +
                              (tid % 8) * 16 + (q0 % 8) * 2;
-        *reinterpret_cast<uint4 *>(dst) = make_uint4(pk[t][i][0], pk[t][i][1], pk[t][i][2], pk[t][i][3]);
+        if constexpr (S::PACK == 8)
+          *reinterpret_cast<uint4 *>(dst) = make_uint4(pk[t][i][0], pk[t][i][1], pk[t][i][2], pk[t][i][3]);
+        else
+          *reinterpret_cast<uint2 *>(dst) = make_uint2(pk[t][i][0], pk[t][i][1]);
       }
   };
 
@@ -543,8 +549,8 @@ __device__ __forceinline__ void tc_syn_body(const TcArgs &ta, const int2 item, u
     if (ks + 1 < nks) prefetch(ks + 1);  // its latency hides behind this K-step's work
     bool fail = false;
 #pragma unroll 1
-    for (int q0 = 0; q0 < tc::kK; q0 += tc::kPack) {
-      uint32_t pk[NL][tc::kLamDigits][tc::kPack / 2];
+    for (int q0 = 0; q0 < tc::kK; q0 += S::PACK) {
+      uint32_t pk[NL][tc::kLamDigits][S::PACK / 2];
       if (wlive) {
         if (polar) part(kPolar, rows + q0 * S::ROW, pk);
         else if (settled && lb >= lfast) part(kFast, rows + q0 * S::ROW, pk);
@@ -555,9 +561,9 @@ __device__ __forceinline__ void tc_syn_body(const TcArgs &ta, const int2 item, u
 #pragma unroll
           for (int i = 0; i < tc::kLamDigits; ++i)
 #pragma unroll
-            for (int q = 0; q < tc::kPack / 2; ++q) pk[t][i][q] = 0u;
+            for (int q = 0; q < S::PACK / 2; ++q) pk[t][i][q] = 0u;
       }
-      rescale();  // after every eight degrees
+      if ((q0 + S::PACK) % 8 == 0) rescale();  // after every eight degrees
       // the previous K-step's MMAs read the A and B tiles: wait for them before
       // the first write (they have long finished by now)
       if (q0 == 0 && ncommit > nwaited) {

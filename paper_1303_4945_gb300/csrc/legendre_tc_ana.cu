@@ -801,6 +801,9 @@ bool tc_ana_supported(int spin, int njobs_pad) {
   return njobs_pad <= 2;
 }
 
+// Spin s, more than two E/B pairs, two at a time: four pairs, lmax 31 20 us against 54 for
+// the double-float contraction, 511 0.41 ms against 1.11, 2047 18.6 against 41.6; eight, lmax
+// 1023 5.1 against 15.1.
 // Spin 0, more than two maps: faster than the double-float contraction at every size
 // (four maps, lmax 31: 22.5 us against 24.4; 255: 74 / 112; 2047: 4.99 / 10.35 ms; sixteen
 // maps, lmax 31: 22 / 107 us, 2047: 20.2 / 65.7 ms), which has no instance for them.  Error

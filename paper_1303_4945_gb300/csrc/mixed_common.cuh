@@ -179,7 +179,7 @@ __device__ __forceinline__ void step_polar(f2 a, f2 b, const f3 &y, f2 &p, f2 &d
 // 10%); OUT: large ones test per step and call the difference form out of line, as a
 // second copy of their loops (or the form inlined) overflows the instruction cache
 // (analysis of two spin-2 pairs at two ring pairs a thread, lmax 1023: 5.5 ms with two
-// copies, 3.9 inlined, kOutNote called).
+// copies, 3.9 inlined, 3.4 called, 3.2 called for the pairs that need it only).
 struct PolarState {
   f2 p, d;
 };

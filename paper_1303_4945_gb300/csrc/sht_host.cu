@@ -880,8 +880,8 @@ static int upload(sht_plan_s *P, const std::vector<T> &h, T **d) {
 // spin class and padded job count; the first is the default.  In the mixed form the
 // difference form of the warps next to a pole weighs more the more pairs a thread has
 // (their CTA waits for them): spin 0 two pairs a thread, packed (lmax 1023, one map 0.50 ms,
-// two 0.76, against four's figures in mix_ana_body), spin s one (one E/B pair 1.29 ms against
-// 1.77 at two, two 2.31 against 3.38).
+// two 0.76, against 0.9 and 1.11 at four), spin s one (one E/B pair 1.29 ms against 1.74 at
+// two, two 2.31 against 3.18).
 static std::vector<int> ana_ppt_candidates(int spin, int nj, int precision) {
   if (spin == 0) {
     if (nj == 1) return precision == SHT_MIXED ? std::vector<int>{2, 4, 8} : std::vector<int>{4, 8, 2};
