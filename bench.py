@@ -363,10 +363,10 @@ MEASURED_TRAFFIC = {
     # one launch at the headline size (spin 2, GL 4096 x 8191, lmax 4095), single-pass
     # dram__bytes_read.sum + dram__bytes_write.sum (the pair's traffic capture under profiles/);
     # sha256 over the kernel file and its headers (_kernel_digest)
-    "mixed:legendre_analysis:tc": {"bytes": 4001973504 + 2131988992,
-                                   "sha256": "8992b7456376424874dc34ab13698b6e8fdf662921ba8387a1bf6a9a3598a047"},
-    "mixed:legendre_synthesis": {"bytes": 822240512 + 333381376,
-                                 "sha256": "27f6f176d8deecc2e9d79217b9e50f084adec901dcffa36f46880253b4aae717"},
+    "mixed:legendre_analysis:tc": {"bytes": 883405824 + 435014912,
+                                   "sha256": "56b9b6d13b0ca098eb4b9030f5867c119bb221215b012fc14b9bc63f969b6c69"},
+    "mixed:legendre_synthesis": {"bytes": 687071232 + 330579968,
+                                 "sha256": "35df1c03f561150b8de275f568d25b7b33690e7f5c74a0efe27c451b3ac2d7d4"},
 }
 
 
@@ -444,7 +444,9 @@ def roofline_for(stages, plan, spin, precision, peaks, steps, ncomp=1):
                "peak_source": ("FP64 pipe, measured on this GPU by sht_measure_pipe_peaks (FMA = 2 flops)"
                                if measured else
                                "FP64 pipe derived: 152 SMs x 2 DFMA lanes/clk x 2 flops x sm_max clock"),
-               "peak_derived": derived}
+               "peak_derived": derived,
+               "note": "from lmax ~200 on the contraction runs on the tensor cores in exact 8-bit digits: the FP64 pipe "
+                       "carries the recursions only (10 of 26 flops at spin s), so frac can exceed 1"}
     else:
         tc_syn = name == "legendre_synthesis" and bool(getattr(plan, "tensor_cores", False))
         tc_ana = name == "legendre_analysis" and bool(getattr(plan, "tensor_core_analysis", False))
@@ -464,7 +466,8 @@ def roofline_for(stages, plan, spin, precision, peaks, steps, ncomp=1):
                "issue_frac_note": ("the contraction runs on the tensor cores: the double-float operation count "
                                    "does not apply" if tc else
                                    "double-float FP32-pipe operations issued per second over the FP32 issue rate "
-                                   "(emulation work included; not the method's work)"),
+                                   "(emulation work included; not the method's work; counted with the "
+                                   "three-coefficient recursion, 16 (spin) or 4 more than are issued)"),
                "tensor_cores": tc,
                "fp32_ops_per_triple": None if tc else f32_ops_per_triple(spin, ncomp),
                "fp64_equivalent_tflops": achieved, "fp64_pipe_tflops": fp64_pipe}
@@ -1031,14 +1034,16 @@ def main():
                          "roofline": roofline_for(stages, plan, SPIN, form_kind, peaks, args.steps),
                          "stage_rooflines": stage_rooflines(stages, plan, SPIN, form_kind, peaks, args.steps),
                          "synthesis_contraction": "tensor cores (tcgen05, exact bf16 digit split)" if tc
-                         else ("FP64" if prec == sht.SHT_FP64 else "double-float FP32"),
+                         else ("FP64, or exact 8-bit digits on the tensor cores by size" if prec == sht.SHT_FP64
+                               else "double-float FP32"),
                          "triples": plan.triples(0), "workspace_bytes": plan.workspace(),
                          "setup": {"plan_create_ms": 1e3 * (t1 - t0), "autotune_ms": 1e3 * (t2 - t1),
                                    "workspace_over_data": plan.workspace() / data_bytes},
                          "fp64_columns": plan.fp64_columns if prec == sht.SHT_MIXED else 0,
                          "analysis_contraction": ("tensor cores (tcgen05, exact bf16 digit split)"
                                                   if prec == sht.SHT_MIXED and plan.tensor_core_analysis
-                                                  else ("FP64" if prec == sht.SHT_FP64 else "double-float FP32")),
+                                                  else ("FP64, or exact 8-bit digits on the tensor cores by size"
+                                                        if prec == sht.SHT_FP64 else "double-float FP32")),
                          "tiling": {"analysis_pairs_per_thread": plan.tiling()[0],
                                     "tensor_core_analysis": prec == sht.SHT_MIXED and plan.tensor_core_analysis,
                                     "autotune_ms_per_candidate": {str(k): v for k, v in tune.items()}}}

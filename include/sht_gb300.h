@@ -67,7 +67,7 @@ extern "C" {
 #define SHT_ECP_FEJER2 1 /* theta_n = n pi / (nlat + 1),  n = 1..nlat */
 #define SHT_ECP_CC 2     /* theta_n = n pi / (nlat - 1),  n = 0..nlat-1 (Clenshaw-Curtis) */
 
-#define SHT_FP64 0  /* recursion and accumulation in IEEE double */
+#define SHT_FP64 0  /* recursion in IEEE double; accumulation too, or (larger sizes) of exact digit products on the tensor cores, to the same errors */
 #define SHT_MIXED 1 /* recursion, accumulation and (by default) ring FFTs in compensated FP32 pairs; FP64 kept for tables and start values */
 
 #define SHT_SYNTHESIS 0         /* a_lm -> map, Eq. syn_used */
@@ -241,7 +241,9 @@ SHT_API void sht_plan_destroy(sht_plan_t plan);
  * walks (more pairs amortise the per-degree reduction across the CTA, fewer
  * leave room for more resident warps) -- is chosen per plan by measurement.
  * A plan offers the tilings its kernels are built for (1 to 3 values,
- * depending on spin class and ncomp); the first is the default.
+ * depending on spin class, ncomp and form); the first is the default.  An FP64 plan
+ * that contracts on the tensor cores takes one of the FP64 kernel's tilings, and
+ * that kernel, when it is set.
  *
  * sht_plan_get_tiling writes the current pairs per thread and, when the
  * pointers are not NULL, the number of candidates and the candidates (at most
@@ -275,9 +277,9 @@ SHT_API int sht_plan_autotune(sht_plan_t plan, void *cuda_stream, float *ms_per_
  * (12 at lmax 2047, 24 at 4095, 48 at 8191), 0 below: every ring's own error
  * stays near or below 5e-11 (spin-2 synthesis against the FP64 form, ring by
  * ring; the rings nearest the poles need the most columns), and the FP64 items
- * stay hidden beside the mixed kernels.  The plan keeps FP64 coefficients (32
- * bytes per (m, l)) and, at spin s, a P = E+iB, M = E-iB table (16 bytes per (m,
- * l) and array) only for the columns below the bound.  sht_plan_set_fp64_columns
+ * stay hidden beside the mixed kernels.  The plan keeps FP64 coefficients (16
+ * bytes per (m, l)) and a table of scaled a_lm (at spin s P = E+iB, M = E-iB; 16
+ * bytes per (m, l) and array) only for the columns below the bound.  sht_plan_set_fp64_columns
  * changes it (any m_below >= 0; it rebuilds the work lists and, for a higher
  * bound, reallocates those tables, which synchronises the device);
  * sht_plan_get_fp64_columns reads it.
@@ -318,8 +320,8 @@ SHT_API int sht_plan_get_fft_precision(sht_plan_t plan, int *precision);
  * SHT_DERIV_SYNTHESIS through sht_execute and sht_execute_noalloc, and is a
  * mixed plan's default for every supported shape except a single spin-0 map,
  * where the double-float contraction is faster (measured on GB300 at lmax 4095:
- * spin 2 one E/B pair 54.3 ms against 62.7, spin 0 eight maps 69.9 against 103.7,
- * spin 0 one map 26.3 against 22.2).  sht_plan_set_tensor_cores(plan, 1 or 0)
+ * spin 2 one E/B pair 38.7 ms against 57.6, spin 0 eight maps 59.2 against 102.3; one
+ * spin-0 map 18.7 against 20.4, but lmax 511 137 us against 106).  sht_plan_set_tensor_cores(plan, 1 or 0)
  * selects it or the double-float contraction; sht_plan_get_tensor_cores reads the
  * setting.  A batch runs each plan with the setting it had when the batch was
  * made (the setting cannot change while a batch refers to the plan).  Errors: SHT_ERR_INVALID_ARG (NULL, an
@@ -345,13 +347,15 @@ SHT_API int sht_plan_device_status(sht_plan_t plan, int *status);
  * the ring pair's phase values times u_p are split into six bf16 digits on a
  * grid per tile and column; the digit products are summed over the tile's pairs
  * in FP32 accumulators where no rounding can occur, and the levels are added in
- * double-float.  Shapes: ncomp <= 2 (SHT_ERR_UNSUPPORTED otherwise); tiles of
- * one pair per thread (the call sets that tiling).  It serves SHT_ANALYSIS and
+ * double-float.  Plans of ncomp >= 3 always run it, four spin-0 maps or two E/B
+ * pairs at a time, on their one tiling (lmax 2047, four maps 5.0 ms against 10.4 for
+ * the double-float analysis, four pairs 18.6 against 41.6).  The setting is of ncomp <= 2 (SHT_ERR_UNSUPPORTED
+ * otherwise), with tiles of 128 pairs (the call sets that tiling).  It serves SHT_ANALYSIS and
  * SHT_ADJOINT_SYNTHESIS through sht_execute, sht_execute_noalloc and the stage
  * call, and in a batch made while the plan has it set.  sht_plan_autotune selects it
- * where it is measured faster (GB300, lmax 4095: spin 2 one E/B pair 73.8 ms
- * against 76.5 for the double-float analysis, two pairs 100.7 against 134.1;
- * spin 0 one map 45.7 against 25.2); sht_plan_set_tensor_core_analysis(plan, 1
+ * where it is measured faster (GB300, lmax 2047: spin 2 one E/B pair 7.2 ms
+ * against 9.1 for the double-float analysis; lmax 4095, spin 0 one map 27.2 against
+ * 21.5); sht_plan_set_tensor_core_analysis(plan, 1
  * or 0)
  * sets it, sht_plan_get_tensor_core_analysis reads it.  Its waits are bounded
  * like the synthesis kernel's (status word bit 0).  Errors: SHT_ERR_INVALID_ARG
@@ -464,7 +468,8 @@ SHT_API int sht_execute_rings(sht_plan_t plan, int type, double *phase, double *
  * working memory (the phase array, the analysis partial sums and the converted
  * a_lm tables) comes from a fixed 64 MiB area compiled into the library, and
  * the call allocates nothing, on the device or the host.  What the plan
- * allocated when it was made is still used: its read-only tables and, for
+ * allocated when it was made is still used: its read-only tables, the scaled
+ * spin-0 a_lm of FP64 kernels, partial sums larger than the rest of the area and, for
  * rings longer than 14336 points, its FFT scratch slots.  Every GPU that
  * loads the library holds the area until the process exits.  Limit:
  * transforms whose working memory exceeds 64 MiB (about nmaps * nm * npairs *
