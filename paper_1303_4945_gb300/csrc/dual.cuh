@@ -113,7 +113,7 @@ __device__ __forceinline__ float scale_weight(int sc) { return sc == 0 ? 1.f : (
 
 // the degree from which on |a x| >= |b| for every lane of the warp: |b| <= a |s| / (l + 1)
 // as m <= l (a margin of 1% covers the roundings); lmax + 1 if a ring lies on the
-// equator or south of it
+// equator
 __device__ __forceinline__ int fast_from(int as, float x, bool valid, int lmax) {
   const float need = valid ? (x > 0.f ? 1.01f * (float)as / x : 1e9f) : 0.f;
   const unsigned w = __reduce_max_sync(0xffffffffu, __float_as_uint(need));  // need >= 0

@@ -527,15 +527,16 @@ struct PhaseWalk {
 
 // The term of coefficient m for one ring pair, conj?(cN e^{i m phiN}) + i conj?(cS e^{i m phiS})
 // (conj_ for the m < 0 half of the sum), in the engine's arithmetic; pn, ps are the
-// phases e^{i m phi} of rings with phi0 != 0 (ph_n, ph_s).  F below the first pair
-// the Legendre stage processed for this m is zero.
+// phases e^{i m phi} of rings with phi0 != 0 (ph_n, ph_s); slot: the phase slot of the
+// pair's first ring (1: a lone southern ring).  F below the first pair the Legendre stage
+// processed for this m is zero.
 template <class N>
-__device__ __forceinline__ typename N::C synth_term(const FftArgs &a, int j, int p, int m, bool south, bool conj_,
-                                                    bool ph_n, bool ph_s, typename N::C pn, typename N::C ps) {
+__device__ __forceinline__ typename N::C synth_term(const FftArgs &a, int j, int p, int slot, int m, bool south,
+                                                    bool conj_, bool ph_n, bool ph_s, typename N::C pn, typename N::C ps) {
   using C = typename N::C;
   const int mi = a.minv[m];
   if (mi < 0 || p < a.syn_first[mi]) return N::zero();
-  const double2 *f = a.phase + (((size_t)j * a.nm + mi) * a.npairs + p) * 2;
+  const double2 *f = a.phase + (((size_t)j * a.nm + mi) * a.npairs + p) * 2 + slot;
   C z = N::of(f[0]);
   if (ph_n) z = N::mul(z, pn);
   if (conj_) z = N::conj(z);
@@ -554,14 +555,14 @@ __device__ __forceinline__ typename N::C synth_term(const FftArgs &a, int j, int
 // the term m = k + N i has phase e^{i k phi} (e^{i N phi})^i, the conjugate term
 // m = N (i + 1) - k has e^{-i k phi} (e^{i N phi})^(i + 1).
 template <class N>
-__device__ typename N::C spectrum_at(const FftArgs &a, int j, int p, int k, int Nr, bool south, bool ph_n, bool ph_s,
+__device__ typename N::C spectrum_at(const FftArgs &a, int j, int p, int slot, int k, int Nr, bool south, bool ph_n, bool ph_s,
                                      typename N::C en, typename N::C es, typename N::C bn, typename N::C bs) {
   using C = typename N::C;
   const int mc = k == 0 ? Nr : Nr - k;  // first m of the conjugate terms
   C z = N::zero();
   bool first = true;
   auto add = [&](int m, bool cj, C pn, C ps) {
-    const C t = synth_term<N>(a, j, p, m, south, cj, ph_n, ph_s, pn, ps);
+    const C t = synth_term<N>(a, j, p, slot, m, south, cj, ph_n, ph_s, pn, ps);
     z = first ? t : N::add(z, t);
     first = false;
   };
@@ -594,6 +595,7 @@ __device__ __forceinline__ void fft_syn_kernel_body(Ring ring, const FftArgs &a,
   const int2 rr = a.pair_rings[p];
   const RingDev rn = a.rings[rr.x];
   const bool south = rr.y >= 0;
+  const int slot = rr.y == kLoneSouth;  // the phase slot of ring rr.x
   const RingDev rs = a.rings[south ? rr.y : rr.x];
   const int Nphi = fp.n;
   const bool ph_n = rn.phi0 != 0.0, ph_s = south && rs.phi0 != 0.0;
@@ -612,7 +614,7 @@ __device__ __forceinline__ void fft_syn_kernel_body(Ring ring, const FftArgs &a,
   }
   const C *chirp = N::chirp(fp);
   for (int k = threadIdx.x; k < Nphi; k += blockDim.x) {
-    const C z = N::conj(spectrum_at<N>(a, j, p, k, Nphi, south, ph_n, ph_s, phn.e, phs.e, bn, bs));
+    const C z = N::conj(spectrum_at<N>(a, j, p, slot, k, Nphi, south, ph_n, ph_s, phn.e, phs.e, bn, bs));
     if (fp.kind == 0) {
       buf[k] = z;
     } else if (fp.kind == 1) {
@@ -675,6 +677,7 @@ __device__ __forceinline__ void fft_ana_kernel_body(Ring ring, const FftArgs &a,
   const int2 rr = a.pair_rings[p];
   const RingDev rn = a.rings[rr.x];
   const bool south = rr.y >= 0;
+  const int slot = rr.y == kLoneSouth;  // the phase slot of ring rr.x
   const RingDev rs = a.rings[south ? rr.y : rr.x];
   const int Nphi = fp.n;
   const double *mp = ptrs[j];
@@ -725,8 +728,8 @@ __device__ __forceinline__ void fft_ana_kernel_body(Ring ring, const FftArgs &a,
     const double2 gn = N::val(pn);
     const double2 gs = south ? N::val(ps) : make_double2(0.0, 0.0);
     double2 *g = a.phase + (((size_t)j * a.nm + mi) * a.npairs + p) * 2;
-    g[0] = gn;
-    g[1] = gs;
+    g[slot] = gn;
+    g[1 - slot] = gs;
   }
 }
 template <class N>

@@ -271,7 +271,8 @@ struct AnaShape64 {
 // ---------------------------------------------------------------------------
 // The bound 2^lexp on |p_l| per (m, ring pair), once per plan, from a plain FP32 walk of
 // the recursion in difference form (step_polar in mixed_common.cuh: relative errors
-// well inside the margin of 1/16 next to the poles too); not below 2^-30.  A thread
+// well inside the margin of 1/16 next to the poles too, as cos(theta) >= 0 in every
+// pair: 1 - cos(theta) keeps its digits there); not below 2^-30.  A thread
 // walks kBoundPairs pairs, which share the conversions of the coefficients.
 // ---------------------------------------------------------------------------
 constexpr int kBoundPairs = 8;

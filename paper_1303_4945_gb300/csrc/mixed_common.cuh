@@ -147,7 +147,7 @@ __device__ __forceinline__ Coef32 ld_coef32(const float4 *p) {
   const float4 u = __ldg(p);
   return {{u.x, u.y}, {u.z, u.w}};
 }
-// Warps holding a ring within kPolarTheta of the north pole run the recursion in
+// Warps holding a ring within kPolarTheta of a pole (cos theta >= 0 in every pair) run the recursion in
 // difference form, d_{l+1} = d_l + (u - 2) p_l, p_{l+1} = p_l + d_{l+1} (d_l = p_l -
 // p_{l-1}), with u - 2 = (a - 2) - a (1 - cos theta) + b.  There u is close to 2 and
 // a rounding of u p_l - p_{l-1} of relative size 2^-48 grows by ~1/theta over the

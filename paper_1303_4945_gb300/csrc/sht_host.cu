@@ -903,7 +903,8 @@ static std::vector<int> ana_ppt_candidates(int spin, int nj, int precision) {
 // lmax 2047, 24 at 4095, 48 at 8191) keep every ring near or below 5e-11 in
 // spin-2 synthesis (measured against the FP64 form ring by ring), and their
 // FP64 items stay hidden on the side stream.  Below lmax 2000 the rings' errors
-// are below 3e-11 without them, and the items would no longer be hidden.
+// are below 5e-11 without them (lmax 1535, rings 0.0015 - 0.0065 rad from either pole,
+// m <= 40: 4.6e-11 at spin 0, 3.9e-11 at spin 2), and the items would no longer be hidden.
 static int default_fp64_columns(int lmax) { return lmax < 2000 ? 0 : lmax / 170; }
 
 // Entries of the coefficient table that the columns m < m_below occupy, as a
@@ -1132,16 +1133,21 @@ static int plan_build(sht_plan_s *P, const sht_geom_s *g) {
     P->pair_pole[p] = std::min(th, (double)kPiL - th);
     long double t = th;
     PairDev &d = pd[p];
-    d.x = cos(th);
+    // a southern ring without its mirror image is the south half of a pair whose north
+    // half has no ring: the kernels see cos(theta) >= 0 only, so their forms and bounds for
+    // the rings next to a pole hold at both
+    const bool lone_south = P->pair_s[p] < 0 && cos(th) < 0.0;
+    d.x = lone_south ? -cos(th) : cos(th);
     long double sn = sinl(t), tn = tanl(0.5L * t);
     long double l1 = (sn > 0) ? log2l(sn) : 0.0L, l2 = (tn > 0) ? log2l(tn) : 0.0L;
+    if (lone_south) l2 = -l2;
     d.l1_hi = (double)l1;
     d.l1_lo = (double)(l1 - (long double)d.l1_hi);
     d.l2_hi = (double)l2;
     d.l2_lo = (double)(l2 - (long double)d.l2_hi);
     d.pole = (th == 0.0 || th == M_PI) ? 1 : 0;
-    d.south = P->pair_s[p] >= 0;
-    pr[p] = make_int2(P->pair_n[p], P->pair_s[p]);
+    d.south = P->pair_s[p] >= 0 || lone_south;
+    pr[p] = make_int2(P->pair_n[p], lone_south ? kLoneSouth : P->pair_s[p]);
   }
   if ((rc = upload(P, pd, &P->d_pairs)) != SHT_OK) return rc;
   if ((rc = upload(P, pr, &P->d_pair_rings)) != SHT_OK) return rc;

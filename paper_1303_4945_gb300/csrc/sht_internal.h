@@ -48,14 +48,18 @@ constexpr double kScaleUp = 0x1p+300;     // rescale when |lambda| exceeds this
 constexpr double kScaleFactor = 0x1p-600;
 
 struct PairDev {
-  double x;        // cos(theta) of the ring in the north slot (libm cos of the given theta)
+  double x;        // cos(theta) >= 0 of the north slot (libm cos of the given theta; of a lone southern ring its mirror image's)
   double l1_hi;    // log2(sin theta), double-double
   double l1_lo;
-  double l2_hi;    // log2(tan(theta/2)), double-double
+  double l2_hi;    // log2(tan(theta/2)) of the north slot, double-double
   double l2_lo;
   int pole;        // 1 if theta == 0 exactly (sin theta == 0)
-  int south;       // 1 if the pair has a mirrored southern ring
+  int south;       // 1 if the pair has a southern ring
 };
+
+// Ring indices of a pair (pair_rings): (north, south), (north, -1) without a southern
+// ring, or (south, kLoneSouth) without a northern one.  The phase slots are [north, south].
+constexpr int kLoneSouth = -2;
 
 // Per-ring data for the FFT stage.
 struct RingDev {

@@ -28,7 +28,7 @@ __global__ void phase_pack(int nmaps, int nm, int npairs, int nrings, const int2
   const bool cut = syn_first && p < syn_first[i];
   const double2 *src = in + (((size_t)c * nm + i) * npairs + p) * 2;
   double2 *dst = out + ((size_t)c * nm + i) * nrings;
-  dst[r.x] = cut ? make_double2(0.0, 0.0) : src[0];
+  dst[r.x] = cut ? make_double2(0.0, 0.0) : src[r.y == kLoneSouth];
   if (r.y >= 0) dst[r.y] = cut ? make_double2(0.0, 0.0) : src[1];
 }
 
@@ -41,8 +41,9 @@ __global__ void phase_unpack(int nmaps, int nm, int npairs, int nrings, const in
   const int2 r = pair_rings[p];
   const double2 *src = in + ((size_t)c * nm + i) * nrings;
   double2 *dst = out + (((size_t)c * nm + i) * npairs + p) * 2;
-  dst[0] = src[r.x];
-  dst[1] = r.y >= 0 ? src[r.y] : make_double2(0.0, 0.0);
+  const int first = r.y == kLoneSouth;  // the slot of ring r.x
+  dst[first] = src[r.x];
+  dst[1 - first] = r.y >= 0 ? src[r.y] : make_double2(0.0, 0.0);
 }
 
 int check_common(const sht_plan_s *P, int type, int flags, int allowed) {
