@@ -927,14 +927,36 @@ static bool lo_item(const sht_plan_s *P, int mi, int p0, int p1) {
   return false;
 }
 
+// Device arrays of a new set of work lists: freed again unless every one of them could
+// be made (done), so that a plan keeps its old lists when a change fails.
+struct FreshLists {
+  std::vector<void *> made;
+  int64_t bytes = 0;
+  template <class T>
+  int put(const std::vector<T> &h, T **d) {
+    *d = nullptr;
+    CUDA_TRY(cudaMalloc((void **)d, std::max<size_t>(1, h.size() * sizeof(T))));
+    made.push_back(*d);
+    bytes += h.size() * sizeof(T);
+    if (!h.empty()) CUDA_TRY(cudaMemcpy(*d, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice));
+    return SHT_OK;
+  }
+  template <class T>
+  int put_items(const std::vector<std::pair<int64_t, T>> &list, T **d) {
+    std::vector<T> v;
+    for (auto &e : list) v.push_back(e.second);
+    return put(v, d);
+  }
+  void done() { made.clear(); }
+  ~FreshLists() {
+    for (void *p : made) cudaFree(p);
+  }
+};
+
 template <class T>
-static int upload_list(sht_plan_s *P, const std::vector<std::pair<int64_t, T>> &list, T **d, int *n) {
-  std::vector<T> v;
-  for (auto &e : list) v.push_back(e.second);
-  if (*d) cudaFree(*d);
-  *d = nullptr;
-  *n = (int)v.size();
-  return upload(P, v, d);
+static void replace_array(T **held, T *fresh) {
+  if (*held) cudaFree(*held);
+  *held = fresh;
 }
 
 // Synthesis work lists: per polar variant the cost-sorted (m, first pair)
@@ -946,9 +968,14 @@ static int build_syn_lists(sht_plan_s *P) {
   int64_t ntile = 0;  // of the polar-cut variant
   for (int i = 0; i < P->nm; ++i)
     if (P->lmax >= std::max(P->mval[i], as)) ntile += (P->npairs + kSynTile - 1) / kSynTile - P->first_pair[i] / kSynTile;
-  P->syn_two = tc_syn_two_tiles(P, ntile);
+  const int syn_two = tc_syn_two_tiles(P, ntile);
+  std::vector<std::pair<int64_t, int2>> lists[2][3];  // syn, two, lo
+  int2 *d[2][3];
+  int *dfirst[2];
+  int64_t triples[2];
+  FreshLists fresh;
   for (int polar = 0; polar < 2; ++polar) {
-    std::vector<std::pair<int64_t, int2>> syn, two, lo;
+    auto &syn = lists[polar][0], &two = lists[polar][1], &lo = lists[polar][2];
     std::vector<int> sfirst(P->nm);
     int64_t trip = 0;
     for (int i = 0; i < P->nm; ++i) {
@@ -966,26 +993,36 @@ static int build_syn_lists(sht_plan_s *P) {
         (lo_item(P, i, p, p + kSynTile) ? lo : syn)
             .push_back({(int64_t)nl * std::min(kSynTile, P->npairs - p), make_int2(i, p)});
       // the same tiles for the kernel that takes two neighbours where both are its own
-      for (int p = sf; P->syn_two && p < P->npairs; p += kSynTile) {
+      for (int p = sf; syn_two && p < P->npairs; p += kSynTile) {
         if (lo_item(P, i, p, p + kSynTile)) continue;
         const bool pair = p + kSynTile < P->npairs && !lo_item(P, i, p + kSynTile, p + 2 * kSynTile);
         two.push_back({(int64_t)nl * std::min((pair ? 2 : 1) * kSynTile, P->npairs - p), make_int2(i, pair ? p | kSynTwoTiles : p)});
         if (pair) p += kSynTile;
       }
     }
-    P->triples[polar] = trip;
-    std::stable_sort(syn.begin(), syn.end(), [](auto &a, auto &b) { return a.first > b.first; });
-    std::stable_sort(two.begin(), two.end(), [](auto &a, auto &b) { return a.first > b.first; });
-    std::stable_sort(lo.begin(), lo.end(), [](auto &a, auto &b) { return a.first > b.first; });
-    P->syn_list[polar] = syn;
-    P->syn_list_two[polar] = two;
-    P->syn_list_lo[polar] = lo;
-    if ((rc = upload_list(P, syn, &P->d_syn_items[polar], &P->nsyn_items[polar])) != SHT_OK) return rc;
-    if ((rc = upload_list(P, two, &P->d_syn_two[polar], &P->nsyn_two[polar])) != SHT_OK) return rc;
-    if ((rc = upload_list(P, lo, &P->d_syn_lo[polar], &P->nsyn_lo[polar])) != SHT_OK) return rc;
-    if (P->d_syn_first[polar]) cudaFree(P->d_syn_first[polar]);
-    P->d_syn_first[polar] = nullptr;
-    if ((rc = upload(P, sfirst, &P->d_syn_first[polar])) != SHT_OK) return rc;
+    triples[polar] = trip;
+    for (int k = 0; k < 3; ++k) {
+      std::stable_sort(lists[polar][k].begin(), lists[polar][k].end(), [](auto &a, auto &b) { return a.first > b.first; });
+      if ((rc = fresh.put_items(lists[polar][k], &d[polar][k])) != SHT_OK) return rc;
+    }
+    if ((rc = fresh.put(sfirst, &dfirst[polar])) != SHT_OK) return rc;
+  }
+  fresh.done();
+  P->workspace += fresh.bytes - P->syn_list_bytes;
+  P->syn_list_bytes = fresh.bytes;
+  P->syn_two = syn_two;
+  for (int polar = 0; polar < 2; ++polar) {
+    P->triples[polar] = triples[polar];
+    P->syn_list[polar].swap(lists[polar][0]);
+    P->syn_list_two[polar].swap(lists[polar][1]);
+    P->syn_list_lo[polar].swap(lists[polar][2]);
+    P->nsyn_items[polar] = (int)P->syn_list[polar].size();
+    P->nsyn_two[polar] = (int)P->syn_list_two[polar].size();
+    P->nsyn_lo[polar] = (int)P->syn_list_lo[polar].size();
+    replace_array(&P->d_syn_items[polar], d[polar][0]);
+    replace_array(&P->d_syn_two[polar], d[polar][1]);
+    replace_array(&P->d_syn_lo[polar], d[polar][2]);
+    replace_array(&P->d_syn_first[polar], dfirst[polar]);
   }
   return SHT_OK;
 }
@@ -1049,8 +1086,14 @@ static int build_ana_lists(sht_plan_s *P, int ppt) {
                                : 1;
   const int group = mixed || P->tc64_ana ? ana_group(P, TA, nt) : 1;
   int64_t need = 0;
+  std::vector<std::pair<int64_t, int4>> lists[2][2];  // ana, lo
+  int4 *d[2][2];
+  int64_t *doff[2];
+  int *dslot[2];
+  double *dpart = nullptr;
+  FreshLists fresh;
   for (int polar = 0; polar < 2; ++polar) {
-    std::vector<std::pair<int64_t, int4>> ana, lo;
+    auto &ana = lists[polar][0], &lo = lists[polar][1];
     std::vector<int64_t> poff(P->nm);
     std::vector<int> nslot(P->nm, 0);
     int64_t off = 0;
@@ -1071,26 +1114,32 @@ static int build_ana_lists(sht_plan_s *P, int ppt) {
       nslot[i] = slot;
       off += (int64_t)slot * nl * V;
     }
-    std::stable_sort(ana.begin(), ana.end(), [](auto &a, auto &b) { return a.first > b.first; });
-    std::stable_sort(lo.begin(), lo.end(), [](auto &a, auto &b) { return a.first > b.first; });
-    if (P->d_ana_part_off[polar]) cudaFree(P->d_ana_part_off[polar]);
-    if (P->d_ana_nslot[polar]) cudaFree(P->d_ana_nslot[polar]);
-    P->d_ana_part_off[polar] = nullptr;
-    P->d_ana_nslot[polar] = nullptr;
-    P->ana_list[polar] = ana;
-    P->ana_list_lo[polar] = lo;
-    if ((rc = upload_list(P, ana, &P->d_ana_items[polar], &P->nana_items[polar])) != SHT_OK) return rc;
-    if ((rc = upload_list(P, lo, &P->d_ana_lo[polar], &P->nana_lo[polar])) != SHT_OK) return rc;
-    if ((rc = upload(P, poff, &P->d_ana_part_off[polar])) != SHT_OK) return rc;
-    if ((rc = upload(P, nslot, &P->d_ana_nslot[polar])) != SHT_OK) return rc;
+    for (int k = 0; k < 2; ++k) {
+      std::stable_sort(lists[polar][k].begin(), lists[polar][k].end(), [](auto &a, auto &b) { return a.first > b.first; });
+      if ((rc = fresh.put_items(lists[polar][k], &d[polar][k])) != SHT_OK) return rc;
+    }
+    if ((rc = fresh.put(poff, &doff[polar])) != SHT_OK) return rc;
+    if ((rc = fresh.put(nslot, &dslot[polar])) != SHT_OK) return rc;
     need = std::max(need, off);
   }
   if (need != P->part_doubles || !P->d_part) {  // sized for the current tiling
-    if (P->d_part) cudaFree(P->d_part);
-    P->d_part = nullptr;
+    CUDA_TRY(cudaMalloc(&dpart, std::max<int64_t>(1, need) * sizeof(double)));
+    replace_array(&P->d_part, dpart);
     P->workspace += (need - P->part_doubles) * (int64_t)sizeof(double);
     P->part_doubles = need;
-    CUDA_TRY(cudaMalloc(&P->d_part, std::max<int64_t>(1, P->part_doubles) * sizeof(double)));
+  }
+  fresh.done();
+  P->workspace += fresh.bytes - P->ana_list_bytes;
+  P->ana_list_bytes = fresh.bytes;
+  for (int polar = 0; polar < 2; ++polar) {
+    P->ana_list[polar].swap(lists[polar][0]);
+    P->ana_list_lo[polar].swap(lists[polar][1]);
+    P->nana_items[polar] = (int)P->ana_list[polar].size();
+    P->nana_lo[polar] = (int)P->ana_list_lo[polar].size();
+    replace_array(&P->d_ana_items[polar], d[polar][0]);
+    replace_array(&P->d_ana_lo[polar], d[polar][1]);
+    replace_array(&P->d_ana_part_off[polar], doff[polar]);
+    replace_array(&P->d_ana_nslot[polar], dslot[polar]);
   }
   P->ana_ppt = ppt;
   // What the call that allocates nothing counts against its area: of the FP64 form the
@@ -1430,9 +1479,14 @@ extern "C" int sht_plan_set_fp64_columns(sht_plan_t P, int m_below) {
     }
   }
   if (rc == SHT_OK) {
+    const int old = P->fp64_m_below;
     P->fp64_m_below = m_below;
     rc = build_syn_lists(P);
     if (rc == SHT_OK) rc = build_ana_lists(P, P->ana_ppt);
+    if (rc != SHT_OK) {  // each direction's lists are whole: the synthesis' follow the old bound again
+      P->fp64_m_below = old;
+      build_syn_lists(P);
+    }
   }
   if (cur != P->device) cudaSetDevice(cur);
   return rc;

@@ -151,6 +151,7 @@ struct sht_plan_s {
   double2 *d_phase = nullptr;              // F / G workspace
   double *d_part = nullptr;                // analysis partials
   int64_t part_doubles = 0;
+  int64_t syn_list_bytes = 0, ana_list_bytes = 0;  // of the work lists, in workspace
   int64_t part_limit = 0;  // of them, what sht_execute_noalloc counts (sht_host.cu)
   int tiling_chosen = 0;   // a call chose the analysis tiling
 
