@@ -1539,7 +1539,12 @@ extern "C" int sht_plan_set_tensor_core_analysis(sht_plan_t P, int on) {
     if (rc != SHT_OK) P->tc_ana = 0;
     return rc;
   }
-  P->tc_ana = on ? 1 : 0;
+  if (!on && P->tc_ana) {  // the double-float kernels' items: no whole passes of two tiles
+    P->tc_ana = 0;
+    const int rc = retile(P, P->ana_ppt);
+    if (rc != SHT_OK) P->tc_ana = 1;
+    return rc;
+  }
   return SHT_OK;
 }
 
@@ -1577,6 +1582,7 @@ extern "C" int sht_plan_autotune(sht_plan_t P, void *stream, float *ms_per_candi
   if (cur != P->device) CUDA_TRY(cudaSetDevice(P->device));
   cudaStream_t st = (cudaStream_t)stream;
   const auto cands = ana_ppt_candidates(P->spin, P->njobs_pad, P->precision);
+  const int old_ppt = P->ana_ppt, old_tc = P->tc_ana, old_tc64 = P->tc64_ana, old_chosen = P->tiling_chosen;
   P->tiling_chosen = 1;
   // the analysis kernels read the phase array: give it defined contents
   const size_t nph = (size_t)P->nmaps_pad * P->nm * P->npairs * 2;
@@ -1628,8 +1634,16 @@ extern "C" int sht_plan_autotune(sht_plan_t P, void *stream, float *ms_per_candi
       best_tc = tc ? 1 : 0;
     }
   }
+  // (also where the last candidate had the same tiling: the tensor-core analysis' items
+  // are whole passes of two tiles)
   P->tc_ana = best_tc;
-  if (rc == SHT_OK && e == cudaSuccess && P->ana_ppt != best) rc = build_ana_lists(P, best);
+  if (rc == SHT_OK && e == cudaSuccess) rc = build_ana_lists(P, best);
+  if (rc != SHT_OK || e != cudaSuccess) {  // back to the setting before
+    P->tc_ana = old_tc;
+    P->tc64_ana = old_tc64;
+    P->tiling_chosen = old_chosen;
+    build_ana_lists(P, old_ppt);
+  }
   for (auto x : ev)
     if (x) cudaEventDestroy(x);
   if (cur != P->device) cudaSetDevice(cur);

@@ -38,3 +38,25 @@ def test_workspace_follows_the_lists(sht, precision):
         plan.fp64_columns = 3
         plan.fp64_columns = 9
         assert plan.workspace() == nine
+@pytest.mark.parametrize("spin,ncomp", [(2, 1), (2, 2)])
+def test_lists_follow_the_kernel(sht, spin, ncomp):
+    """292 rings are two tiles of 128 pairs: one item of the tensor-core analysis, two of
+    the double-float one."""
+    partials = {}
+    for how in ("tiling", "switch", "autotune"):
+        plan = make(sht, 144, 292, spin, ncomp, sht.SHT_MIXED)
+        base = plan.workspace()
+        if how == "tiling":
+            plan.set_tiling(2)
+            plan.set_tiling(1)
+        elif how == "switch":
+            plan.tensor_core_analysis = True
+            plan.tensor_core_analysis = False
+        else:
+            plan.autotune(torch.cuda.current_stream())
+            if plan.tensor_core_analysis:
+                plan.tensor_core_analysis = False
+            plan.set_tiling(1)
+        assert plan.tiling()[0] == 1 and not plan.tensor_core_analysis
+        partials[how] = plan.workspace() - base
+    assert partials["switch"] == partials["tiling"] == partials["autotune"]
