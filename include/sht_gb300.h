@@ -241,14 +241,16 @@ SHT_API void sht_plan_destroy(sht_plan_t plan);
  * walks (more pairs amortise the per-degree reduction across the CTA, fewer
  * leave room for more resident warps) -- is chosen per plan by measurement.
  * A plan offers the tilings its kernels are built for (1 to 3 values,
- * depending on spin class, ncomp and form); the first is the default.  An FP64 plan
- * that contracts on the tensor cores takes one of the FP64 kernel's tilings, and
- * that kernel, when it is set.
+ * depending on spin class, ncomp and form); the first is the default.  The tilings
+ * of an FP64 plan are its IEEE contraction's.  A plan that can contract on the tensor
+ * cores does so at its default tiling; another one selects the IEEE contraction with
+ * it, the default's value returns, and sht_plan_autotune times both.
  *
  * sht_plan_get_tiling writes the current pairs per thread and, when the
  * pointers are not NULL, the number of candidates and the candidates (at most
  * 4).  sht_plan_set_tiling selects a candidate (SHT_ERR_UNSUPPORTED for any
- * other value, and for any value but 1 while the tensor-core analysis is on).
+ * other value, and for any value but 1 while the tensor-core analysis is on); the
+ * current one is accepted and changes no kernel.  A call that fails changes nothing.
  * sht_plan_autotune runs the plan's analysis Legendre kernel once untimed and
  * twice timed per candidate on cuda_stream -- the tilings with the double-float
  * analysis and, for a mixed plan of a shape the tensor-core analysis supports,

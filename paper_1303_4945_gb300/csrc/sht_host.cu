@@ -1165,7 +1165,7 @@ static int build_ana_lists(sht_plan_s *P, int ppt) {
 static void tc64_choose(sht_plan_s *P) {
   const int n = P->nmaps_pad;  // arrays per side
   P->tc64_syn = tc64_syn_supported(P->spin, P->njobs_pad) && P->lmax >= (n == 1 ? 224 : (n == 2 ? 192 : 48));
-  P->tc64_ana = tc64_ana_supported(P->spin, P->njobs_pad) && P->lmax >= (n == 1 ? 208 : 24);
+  P->tc64_ana = P->tc64_able = tc64_ana_supported(P->spin, P->njobs_pad) && P->lmax >= (n == 1 ? 208 : 24);
 }
 
 static int plan_build(sht_plan_s *P, const sht_geom_s *g) {
@@ -1416,18 +1416,27 @@ extern "C" int sht_plan_set_tiling(sht_plan_t P, int pairs_per_thread) {
   if (std::find(c.begin(), c.end(), pairs_per_thread) == c.end())
     return fail(SHT_ERR_UNSUPPORTED, "no analysis kernel with %d ring pairs per thread for this plan",
                 pairs_per_thread);
-  if (pairs_per_thread == P->ana_ppt && !P->tc64_ana) {
-    if (!P->batch_refs) {
+  if (pairs_per_thread == P->ana_ppt) {  // nothing changes (an FP64 plan keeps its kernel)
+    if (!P->batch_refs && P->precision == SHT_MIXED) {
       P->tiling_chosen = 1;
       P->part_limit = P->part_doubles;
     }
     return SHT_OK;
   }
-  if (!P->batch_refs) P->tiling_chosen = 1;
-  if (P->tc64_ana && !P->batch_refs) P->tc64_ana = 0;  // a tiling asked for is one of the FP64 kernel
   if (P->tc_ana)
     return fail(SHT_ERR_UNSUPPORTED, "the tensor-core analysis takes one ring pair per thread");
-  return retile(P, pairs_per_thread);
+  // an FP64 plan contracts on the tensor cores, where it can, at its default tiling only
+  const int old_tc64 = P->tc64_ana, old_chosen = P->tiling_chosen;
+  if (!P->batch_refs) {
+    P->tc64_ana = P->tc64_able && pairs_per_thread == c[0];
+    P->tiling_chosen = 1;
+  }
+  const int rc = retile(P, pairs_per_thread);
+  if (rc != SHT_OK) {
+    P->tc64_ana = old_tc64;
+    P->tiling_chosen = old_chosen;
+  }
+  return rc;
 }
 
 extern "C" int sht_plan_get_tiling(sht_plan_t P, int *pairs_per_thread, int *ncandidates, int *candidates) {
@@ -1598,7 +1607,7 @@ extern "C" int sht_plan_autotune(sht_plan_t P, void *stream, float *ms_per_candi
   const size_t ncand = cands.size() + (tc_cand ? 1 : 0);
   int best_tc = P->tc_ana;
   // an FP64 plan's tensor-core analysis is timed too, last, without a time of its own
-  const bool t64 = P->precision == SHT_FP64 && P->tc64_ana;
+  const bool t64 = P->tc64_able != 0;
   const size_t ncand64 = ncand + (t64 ? 1 : 0);
   P->tc64_ana = 0;
   if (ms_per_candidate)

@@ -187,6 +187,7 @@ struct sht_plan_s {
   // sizes where they are faster (tc64_choose in sht_host.cu); d_lexp: per (m index, pair)
   // the exponent of a power of two bounding the recursion's values
   int tc64_syn = 0, tc64_ana = 0;
+  int tc64_able = 0;  // the analysis can: at the default tiling, where autotuning did not find another faster
   signed char *d_lexp = nullptr;
   int *d_err = nullptr;      // device status word written by kernels with bounded waits
   float4 *d_join = nullptr;  // mixed plans: join record per (m index, pair), 3 float4 each
