@@ -962,7 +962,7 @@ __device__ __forceinline__ void tc64_ana_body(const LegArgs &a, const int4 item,
       epi_sum(o, neg, prev);
     }
   }
-  if (!ok && tid == 0) atomicOr(a.err, 1);
+  if (!ok && lane == 0) atomicOr(a.err, 1);  // each warp its own (see legendre_tc_ana.cu)
   if (nmine > nmine_done) tc::bar_wait(&mine[warp], (uint32_t)(nmine - 1) & 1u);
   tc::fence_before();
   __syncthreads();

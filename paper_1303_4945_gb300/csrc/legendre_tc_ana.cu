@@ -744,9 +744,10 @@ __device__ __forceinline__ void tc_ana_body(const TcArgs &ta, const int4 item_, 
     }
   }
 
-  // leave: flag a wait that gave up, let this warp's products in flight finish
-  // (bounded), release TMEM
-  if (!ok && tid == 0) atomicOr(ta.err, 1);
+  // leave: flag a wait that gave up (each warp its own: the two groups wait for different
+  // accumulators, and after the last tile no barrier tells the others), let this warp's
+  // products in flight finish (bounded), release TMEM
+  if (!ok && lane == 0) atomicOr(ta.err, 1);
   if (nmine > nmine_done) tc::bar_wait(&mine[warp], (uint32_t)(nmine - 1) & 1u);
   tc::fence_before();
   __syncthreads();
