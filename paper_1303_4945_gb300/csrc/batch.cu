@@ -32,6 +32,7 @@ struct Group {
   int precision = 0, spin = 0, nj = 1, ppt = 2;
   bool tc = false;                   // mixed plans whose synthesis runs on the tensor cores
   bool two = false;                  // tensor-core synthesis items of up to two tiles
+  int pf = 0;                        // mixed plans: where the synthesis keeps the difference form
   bool tca = false;                  // mixed plans whose analysis runs on the tensor cores
   void *d_targs[2] = {nullptr, nullptr};  // per polar: their TcArgs records (tensor-core kernels)
   std::vector<int> plans;            // batch indices; item.w is the position in this list
@@ -130,7 +131,7 @@ int build(sht_batch_s *B) {
     Group *g = nullptr;
     for (auto &c : B->groups)
       if (c.precision == precision && c.spin == spin_class && c.nj == P->njobs_pad && c.ppt == P->ana_ppt &&
-          c.tc == tc && c.tca == tca && c.two == two)
+          c.tc == tc && c.tca == tca && c.two == two && c.pf == P->polar_form)
         g = &c;
     if (!g) {
       B->groups.emplace_back();
@@ -142,6 +143,7 @@ int build(sht_batch_s *B) {
       g->tc = tc;
       g->tca = tca;
       g->two = two;
+      g->pf = P->polar_form;
     }
     g->plans.push_back(k);
     g->lo.push_back(lo ? 1 : 0);
@@ -335,7 +337,7 @@ extern "C" int sht_batch_execute(sht_batch_t B, int type, double *const *const *
         else if (stage == 1 && g.tca)
           r = launch_leg_tc_ana_batch(g.spin, g.nj, g.d_targs[polar], items, ni, s);
         else
-          r = mixed_groups ? launch_leg_mixed_batch(stage, g.spin, g.nj, g.ppt, g.d_args[polar], items, ni, s)
+          r = mixed_groups ? launch_leg_mixed_batch(stage, g.spin, g.nj, g.ppt, g.pf, g.d_args[polar], items, ni, s)
                            : launch_leg_fp64_batch(stage, g.spin, g.nj, g.ppt, g.d_args[polar], items, ni, s);
       }
       return r;

@@ -57,12 +57,31 @@ struct Dual {
 
   __device__ __forceinline__ void step(StepMode mode, const float4 &c) {
     const f2 a = {c.x, c.y}, b = {c.z, c.w};
-    if (mode == kPolar) {
-      f2 p0 = lane0(p), q0 = lane0(q), p1 = lane1(p), q1 = lane1(q);
-      step_polar(a, b, x[0], p0, q0);
-      step_polar(a, neg(b), x[SPIN ? 0 : 1], p1, q1);
-      p = {make_float2(p0.h, p1.h), make_float2(p0.l, p1.l)};
-      q = {make_float2(q0.h, q1.h), make_float2(q0.l, q1.l)};
+    if (mode == kPolar) {  // step_polar of both lanes, every lane rounded as there
+      const f3 &y0 = x[0], &y1 = x[SPIN ? 0 : 1];
+      auto lane_of = [&](const f3 &y) {  // (a - 2) - a y as a pair (spin s: the same for both lanes)
+        const float m = __fmul_rn(a.h, y.h);
+        float e = __fmaf_rn(a.h, y.h, -m);
+        e = __fmaf_rn(a.h, y.m, e);
+        e = __fmaf_rn(a.l, y.h, e);
+        const f2 t = two_sum(__fsub_rn(a.h, 2.0f), -m);
+        return f2{t.h, __fadd_rn(__fsub_rn(a.l, e), t.l)};
+      };
+      const f2 t0 = lane_of(y0), t1 = SPIN ? t0 : lane_of(y1);
+      d2 v = {make_float2(t0.h, t1.h), make_float2(t0.l, t1.l)};
+      if (SPIN) {
+        const d2 t = two_sum(v.h, make_float2(b.h, -b.h));
+        v = {t.h, add2(add2(v.l, t.l), make_float2(b.l, -b.l))};
+      }
+      v = fast_two_sum(v.h, v.l);
+      const float2 m = mul2(v.h, p.h);
+      float2 e;
+      e.x = __fmaf_rn(v.l.x, p.h.x, __fmaf_rn(v.h.x, p.l.x, __fmaf_rn(v.h.x, p.h.x, -m.x)));
+      e.y = __fmaf_rn(v.l.y, p.h.y, __fmaf_rn(v.h.y, p.l.y, __fmaf_rn(v.h.y, p.h.y, -m.y)));
+      const d2 s = two_sum(m, q.h);
+      q = fast_two_sum(s.h, add2(add2(e, q.l), s.l));
+      const d2 r = two_sum(p.h, q.h);
+      p = fast_two_sum(r.h, add2(add2(p.l, q.l), r.l));
       return;
     }
     d2 u;

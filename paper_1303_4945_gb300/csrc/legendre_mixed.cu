@@ -16,6 +16,8 @@
 // are scaled down every 8 steps; values at scale 0 and -1 are accumulated (the
 // latter times 2^-104), anything smaller is negligible.  A mixed plan hands the
 // items of small m near the poles to the FP64 kernels (sht_plan_s::fp64_m_below).
+#include <type_traits>
+
 #include "dual.cuh"
 
 namespace sht {
@@ -78,7 +80,7 @@ __global__ void alm_to_f2(int lmax, int spin, int nm, int narr, int astride, con
 // further: the double-float step is ~170 instructions, and longer unrolled
 // bodies stalled the issue on instruction fetch.
 // ---------------------------------------------------------------------------
-template <int NJ>
+template <int NJ, PolarForm PF>
 __device__ __forceinline__ void mix_syn_s0_body(const MixArgs &a, const int2 item) {
   const int mi = item.x;
   const int p = item.y + threadIdx.x;
@@ -88,13 +90,13 @@ __device__ __forceinline__ void mix_syn_s0_body(const MixArgs &a, const int2 ite
   const int64_t co = a.coef_off[mi] - l0;
   const float4 *__restrict__ cf = a.coef32 + co;
   const PairDev pd = a.pairs[valid ? p : 0];
-  const bool polar = polar_warp(pd.x, valid);
-  const f3 x = node_of(pd.x, polar);
   // zero until the pair joins at its join record's block (no terms, a recursion of zeros)
   f2 lc = {0.f, 0.f}, lp = {0.f, 0.f};
   int scale = 0;
   const float4 *jrec = a.join + ((size_t)mi * a.npairs + (valid ? p : 0)) * 3;
   const int lj = valid ? __float_as_int(__ldg(jrec + 2).z) : lmax + 1;
+  const bool polar = PF == kPolarAll || (PF == kPolarCopy && __any_sync(0xffffffffu, near_pole(pd.x, valid)));
+  const f3 x = node_of(pd.x, polar);
   f2 acc[2][NJ][2];
 #pragma unroll
   for (int q = 0; q < 2; ++q)
@@ -164,8 +166,8 @@ __device__ __forceinline__ void mix_syn_s0_body(const MixArgs &a, const int2 ite
     }
     if (l <= lmax) step(pol, l, 0, true);
   };
-  if (polar) walk(true);
-  else walk(false);
+  if (PF == kPolarAll || (PF == kPolarCopy && polar)) walk(true);
+  if (PF == kPolarNone || (PF == kPolarCopy && !polar)) walk(false);
   if (!valid) return;
 #pragma unroll
   for (int j = 0; j < NJ; ++j) {
@@ -178,22 +180,22 @@ __device__ __forceinline__ void mix_syn_s0_body(const MixArgs &a, const int2 ite
     o[1] = fs;
   }
 }
-template <int NJ>
+template <int NJ, PolarForm PF = kPolarCopy>
 __global__ void __launch_bounds__(kSynTile) mix_syn_s0(MixArgs a) {
-  mix_syn_s0_body<NJ>(a, a.syn_items[blockIdx.x]);
+  mix_syn_s0_body<NJ, PF>(a, a.syn_items[blockIdx.x]);
 }
-template <int NJ>
+template <int NJ, PolarForm PF = kPolarCopy>
 __global__ void __launch_bounds__(kSynTile) mix_syn_s0_batch(const MixArgs *__restrict__ args,
     const int4 *__restrict__ items) {
   const int4 it = items[blockIdx.x];
   const MixArgs &a = args[it.w];
-  mix_syn_s0_body<NJ>(a, make_int2(it.x, it.y));
+  mix_syn_s0_body<NJ, PF>(a, make_int2(it.x, it.y));
 }
 
 // ---------------------------------------------------------------------------
 // synthesis, spin s: separate +s / -s recursions (see legendre_fp64.cu)
 // ---------------------------------------------------------------------------
-template <int NJ>
+template <int NJ, PolarForm PF>
 __device__ __forceinline__ void mix_syn_spin_body(const MixArgs &a, const int2 item) {
   const int mi = item.x;
   const int p = item.y + threadIdx.x;
@@ -204,13 +206,13 @@ __device__ __forceinline__ void mix_syn_spin_body(const MixArgs &a, const int2 i
   const int64_t co = a.coef_off[mi] - l0;
   const float4 *__restrict__ cf = a.coef32 + co;
   const PairDev pd = a.pairs[valid ? p : 0];
-  const bool polar = polar_warp(pd.x, valid);
-  const f3 x = node_of(pd.x, polar);
   // zero until the pair joins at its join record's block (no terms, a recursion of zeros)
   f2 lpc = {0.f, 0.f}, lmc = {0.f, 0.f}, lpp = {0.f, 0.f}, lmp = {0.f, 0.f};
   int scp = 0, scm = 0;
   const float4 *jrec = a.join + ((size_t)mi * a.npairs + (valid ? p : 0)) * 3;
   const int lj = valid ? __float_as_int(__ldg(jrec + 2).z) : lmax + 1;
+  const bool polar = PF == kPolarAll || (PF == kPolarCopy && __any_sync(0xffffffffu, near_pole(pd.x, valid)));
+  const f3 x = node_of(pd.x, polar);
   // N1 = sum P l+, N2 = sum M l-, S3 = sum (-1)^(l-l0) P l-, S4 = sum (-1)^(l-l0) M l+
   f2 r[NJ][4][2];
 #pragma unroll
@@ -297,8 +299,8 @@ __device__ __forceinline__ void mix_syn_spin_body(const MixArgs &a, const int2 i
     }
     if (l <= lmax) step(pol, l, 0, true);
   };
-  if (polar) walk(true);
-  else walk(false);
+  if (PF == kPolarAll || (PF == kPolarCopy && polar)) walk(true);
+  if (PF == kPolarNone || (PF == kPolarCopy && !polar)) walk(false);
   if (!valid) return;
 
   const double sig = (as & 1) ? -1.0 : 1.0;
@@ -326,16 +328,16 @@ __device__ __forceinline__ void mix_syn_spin_body(const MixArgs &a, const int2 i
     ou[1] = us;
   }
 }
-template <int NJ>
+template <int NJ, PolarForm PF = kPolarCopy>
 __global__ void __launch_bounds__(kSynTile) mix_syn_spin(MixArgs a) {
-  mix_syn_spin_body<NJ>(a, a.syn_items[blockIdx.x]);
+  mix_syn_spin_body<NJ, PF>(a, a.syn_items[blockIdx.x]);
 }
-template <int NJ>
+template <int NJ, PolarForm PF = kPolarCopy>
 __global__ void __launch_bounds__(kSynTile) mix_syn_spin_batch(const MixArgs *__restrict__ args,
     const int4 *__restrict__ items) {
   const int4 it = items[blockIdx.x];
   const MixArgs &a = args[it.w];
-  mix_syn_spin_body<NJ>(a, make_int2(it.x, it.y));
+  mix_syn_spin_body<NJ, PF>(a, make_int2(it.x, it.y));
 }
 
 // ---------------------------------------------------------------------------
@@ -391,8 +393,8 @@ __device__ __forceinline__ void mix_ana_body(const MixArgs &a, const int4 item) 
       const bool valid = p < a.npairs;
       const PairDev pd = a.pairs[valid ? p : 0];
       xd[k] = pd.x;
-      near[k] = valid && 1.0 - pd.x < 0.5 * kPolarTheta * kPolarTheta;
       lj[k] = valid ? __float_as_int(__ldg(a.join + ((size_t)mi * a.npairs + p) * 3 + 2).z) : lmax + 1;
+      near[k] = near_pole(pd.x, valid);
       jmin = min(jmin, lj[k]);
       lpc[k] = lmc[k] = lpp[k] = lmp[k] = f2{0.f, 0.f};
       scp[k] = scm[k] = 0;
@@ -692,8 +694,8 @@ __device__ __forceinline__ void mix_ana_pair_body(const MixArgs &a, const int4 i
       const bool valid = p < a.npairs;
       const PairDev pd = a.pairs[valid ? p : 0];
       xd[k] = pd.x;
-      near = near || (valid && 1.0 - pd.x < 0.5 * kPolarTheta * kPolarTheta);
       lj[k] = valid ? __float_as_int(__ldg(a.join + ((size_t)mi * a.npairs + p) * 3 + 2).z) : lmax + 1;
+      near = near || near_pole(pd.x, valid);
 #pragma unroll
       for (int j = 0; j < NJ; ++j) {
         double2 gn = make_double2(0, 0), gs = make_double2(0, 0);
@@ -1007,6 +1009,25 @@ cudaError_t launch_join_records(const sht_plan_s *P, cudaStream_t st) {
   return cudaGetLastError();
 }
 
+// Where the synthesis of sixteen maps or eight E/B pairs keeps the difference form.  Two
+// copies of these loops in one kernel overflow the instruction cache, and the polar warp's
+// CTA, the longest, waits for instructions (513 Clenshaw-Curtis rings, lmax 255, sixteen
+// maps: 708 us in two copies, 416 with the form in every warp, which also has the
+// smaller errors: lmax 1023 6.6e-13 -> 4.7e-13).  A step of it costs 5% more, so plans
+// without such rings keep the plain form (256 Gauss-Legendre rings 221 us, 241), and from
+// lmax 1200 on, where the other CTAs cover the wait, two copies are as fast or faster
+// (eight pairs, lmax 1535: HEALPix 43.8 ms against 46.1, Clenshaw-Curtis 50.0, 49.5).
+int mix_polar_form(const sht_plan_s *P, bool polar_rings) {
+  if (P->precision != SHT_MIXED || P->njobs_pad < (P->spin ? 8 : 16)) return kPolarCopy;
+  return !polar_rings ? kPolarNone : (P->lmax < 1200 ? kPolarAll : kPolarCopy);
+}
+template <class F>
+static void polar_shape(int pf, F &&f) {
+  if (pf == kPolarAll) f(std::integral_constant<PolarForm, kPolarAll>{});
+  else if (pf == kPolarNone) f(std::integral_constant<PolarForm, kPolarNone>{});
+  else f(std::integral_constant<PolarForm, kPolarCopy>{});
+}
+
 // Legendre stage over an explicit work list (stage 0: synthesis items int2, 1:
 // analysis items int4); no a_lm conversion (launch_alm_prepare_mixed does it)
 cudaError_t launch_leg_mixed_items(const sht_plan_s *P, int stage, int polar, const void *items, int n,
@@ -1023,14 +1044,18 @@ cudaError_t launch_leg_mixed_items(const sht_plan_s *P, int stage, int polar, co
         case 2: mix_syn_s0<2><<<n, kSynTile, 0, st>>>(a); break;
         case 4: mix_syn_s0<4><<<n, kSynTile, 0, st>>>(a); break;
         case 8: mix_syn_s0<8><<<n, kSynTile, 0, st>>>(a); break;
-        default: mix_syn_s0<16><<<n, kSynTile, 0, st>>>(a); break;
+        default:
+          polar_shape(P->polar_form, [&](auto f) { mix_syn_s0<16, f.value><<<n, kSynTile, 0, st>>>(a); });
+          break;
       }
     } else {
       switch (nj) {
         case 1: mix_syn_spin<1><<<n, kSynTile, 0, st>>>(a); break;
         case 2: mix_syn_spin<2><<<n, kSynTile, 0, st>>>(a); break;
         case 4: mix_syn_spin<4><<<n, kSynTile, 0, st>>>(a); break;
-        default: mix_syn_spin<8><<<n, kSynTile, 0, st>>>(a); break;
+        default:
+          polar_shape(P->polar_form, [&](auto f) { mix_syn_spin<8, f.value><<<n, kSynTile, 0, st>>>(a); });
+          break;
       }
     }
   } else {
@@ -1083,7 +1108,7 @@ cudaError_t launch_alm_prepare_mixed(const sht_plan_s *P, const DevPtrs &alm, cu
   return cudaGetLastError();
 }
 
-cudaError_t launch_leg_mixed_batch(int stage, int spin, int nj, int ppt, const void *args, const int4 *items,
+cudaError_t launch_leg_mixed_batch(int stage, int spin, int nj, int ppt, int pf, const void *args, const int4 *items,
                                    int n, cudaStream_t st) {
   if (n == 0) return cudaSuccess;
   const MixArgs *a = static_cast<const MixArgs *>(args);
@@ -1094,14 +1119,18 @@ cudaError_t launch_leg_mixed_batch(int stage, int spin, int nj, int ppt, const v
         case 2: mix_syn_s0_batch<2><<<n, kSynTile, 0, st>>>(a, items); break;
         case 4: mix_syn_s0_batch<4><<<n, kSynTile, 0, st>>>(a, items); break;
         case 8: mix_syn_s0_batch<8><<<n, kSynTile, 0, st>>>(a, items); break;
-        default: mix_syn_s0_batch<16><<<n, kSynTile, 0, st>>>(a, items); break;
+        default:
+          polar_shape(pf, [&](auto f) { mix_syn_s0_batch<16, f.value><<<n, kSynTile, 0, st>>>(a, items); });
+          break;
       }
     } else {
       switch (nj) {
         case 1: mix_syn_spin_batch<1><<<n, kSynTile, 0, st>>>(a, items); break;
         case 2: mix_syn_spin_batch<2><<<n, kSynTile, 0, st>>>(a, items); break;
         case 4: mix_syn_spin_batch<4><<<n, kSynTile, 0, st>>>(a, items); break;
-        default: mix_syn_spin_batch<8><<<n, kSynTile, 0, st>>>(a, items); break;
+        default:
+          polar_shape(pf, [&](auto f) { mix_syn_spin_batch<8, f.value><<<n, kSynTile, 0, st>>>(a, items); });
+          break;
       }
     }
   } else {

@@ -327,7 +327,7 @@ __device__ __forceinline__ void tc_syn_body(const TcArgs &ta, const int2 item, u
 #pragma unroll
   for (int t = 0; t < NP; ++t) {
     xd[t] = a.pairs[valid[t] ? pr[t] : 0].x;
-    near = near || (valid[t] && 1.0 - xd[t] < 0.5 * kPolarTheta * kPolarTheta);
+    near = near || near_pole(xd[t], valid[t]);
   }
   const bool polar = __any_sync(0xffffffffu, near);
   Dual<!S::DUAL> rec;

@@ -414,7 +414,7 @@ __device__ __forceinline__ void tc_ana_body(const TcArgs &ta, const int4 item_, 
 #pragma unroll
     for (int t = 0; t < NP; ++t) {
       xd[t] = valid[t] ? a.pairs[pr[t]].x : 0.0;
-      near = near || (valid[t] && 1.0 - xd[t] < 0.5 * kPolarTheta * kPolarTheta);
+      near = near || near_pole(xd[t], valid[t]);
     }
     const bool polar = __any_sync(0xffffffffu, near);
 #pragma unroll

@@ -155,9 +155,8 @@ __device__ __forceinline__ Coef32 ld_coef32(const float4 *p) {
 // d.  Errors of lambda at lmax 1535, theta 0.0015 - 0.0065, m <= 4: 9e-12 against
 // 5e-11.  A step takes about twice the operations, in the first warp or two of each
 // m's pairs only.  x holds 1 - cos theta (two floats) and lp the difference there.
-constexpr double kPolarTheta = 0.005;
-__device__ __forceinline__ bool polar_warp(double x, bool valid) {
-  return __any_sync(0xffffffffu, valid && 1.0 - x < 0.5 * kPolarTheta * kPolarTheta);
+__device__ __forceinline__ bool near_pole(double x, bool valid) {
+  return valid && 1.0 - x < 0.5 * kPolarTheta * kPolarTheta;
 }
 __device__ __forceinline__ f3 node_of(double x, bool polar) {
   const f3 r = f3_of(polar ? 1.0 - x : x);

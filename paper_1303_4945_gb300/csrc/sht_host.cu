@@ -1198,6 +1198,8 @@ static int plan_build(sht_plan_s *P, const sht_geom_s *g) {
     d.south = P->pair_s[p] >= 0 || lone_south;
     pr[p] = make_int2(P->pair_n[p], lone_south ? kLoneSouth : P->pair_s[p]);
   }
+  // (pairs run from the poles on; the kernels compare cosines)
+  P->polar_form = mix_polar_form(P, P->npairs > 0 && P->pair_pole[0] < 1.01 * kPolarTheta);
   if ((rc = upload(P, pd, &P->d_pairs)) != SHT_OK) return rc;
   if ((rc = upload(P, pr, &P->d_pair_rings)) != SHT_OK) return rc;
   std::vector<RingDev> rd(g->nrings);

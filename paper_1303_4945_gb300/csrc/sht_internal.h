@@ -36,6 +36,10 @@ constexpr int kFftMinBlocks = 512 / kFftThreads;  // launch bound: at most 128 r
 // longest in-place transform: the ring buffer (16 bytes a point) must fit the
 // opt-in shared memory of one CTA (227 KB on sm_103a)
 constexpr int kFftMaxLen = 14336;
+constexpr double kPolarTheta = 0.005;  // rad: the mixed form's difference form (mixed_common.cuh) nearer a pole
+// which warps of a mixed synthesis run it: those with such a ring, in a second copy of the
+// loops; all; none (mix_polar_form)
+enum PolarForm { kPolarCopy, kPolarAll, kPolarNone };
 constexpr double kFp64PolarCap = 0.05;  // rad; see sht_plan_s::fp64_m_below
 // longest transform at all: longer rings run from a global scratch slot per CTA
 // (1 MiB each), which stays in L2
@@ -175,6 +179,7 @@ struct sht_plan_s {
   // the small-m recursion is non-oscillatory for l < ~1/theta and amplifies its
   // per-step rounding by a power of l
   int fp64_m_below = 0;
+  int polar_form = 0;  // PolarForm of the double-float synthesis
   bool fft_df = false;  // ring FFTs in double-float (mixed plans, by default)
   // mixed plans: the synthesis contraction on the tensor cores (legendre_tc.cu)
   int tc_syn = 0;
@@ -341,8 +346,9 @@ cudaError_t launch_alm_prepare_mixed(const sht_plan_s *P, const DevPtrs &alm, cu
 // stage 0: synthesis, 1: analysis
 cudaError_t launch_leg_fp64_batch(int stage, int spin, int nj, int ppt, const void *args, const int4 *items,
                                   int n, cudaStream_t st);
-cudaError_t launch_leg_mixed_batch(int stage, int spin, int nj, int ppt, const void *args, const int4 *items,
+cudaError_t launch_leg_mixed_batch(int stage, int spin, int nj, int ppt, int pf, const void *args, const int4 *items,
                                    int n, cudaStream_t st);
+int mix_polar_form(const sht_plan_s *P, bool polar_rings);
 cudaError_t launch_fft_batch(int stage, bool df, const void *args, const int4 *items, int n, int threads, int smem,
                              const PtrTable &tbl, cudaStream_t st);
 }  // namespace sht
