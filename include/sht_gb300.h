@@ -67,7 +67,11 @@ extern "C" {
 #define SHT_ECP_FEJER2 1 /* theta_n = n pi / (nlat + 1),  n = 1..nlat */
 #define SHT_ECP_CC 2     /* theta_n = n pi / (nlat - 1),  n = 0..nlat-1 (Clenshaw-Curtis) */
 
-#define SHT_FP64 0  /* recursion in IEEE double; accumulation too, or (larger sizes) of exact digit products on the tensor cores, to the same errors */
+/* recursion in IEEE double; accumulation too, or, at larger sizes, of fixed-point digits on
+ * the tensor cores: operands rounded to 2^-54 of the largest of their column (an m's a_lm, an
+ * m's rings), used where what meets at one result lies within 2^14 of one another, so that
+ * this stays below the recursion's own error; other columns are accumulated in IEEE double */
+#define SHT_FP64 0
 #define SHT_MIXED 1 /* recursion, accumulation and (by default) ring FFTs in compensated FP32 pairs; FP64 kept for tables and start values */
 
 #define SHT_SYNTHESIS 0         /* a_lm -> map, Eq. syn_used */

@@ -330,15 +330,16 @@ extern "C" int sht_batch_execute(sht_batch_t B, int type, double *const *const *
         if ((g.precision == SHT_MIXED) != mixed_groups || r != cudaSuccess) continue;
         const int4 *items = stage ? g.d_ana[polar] : g.d_syn[polar];
         const int ni = stage ? g.nana[polar] : g.nsyn[polar];
-        if (!mixed_groups && (stage ? g.tca : g.tc))
-          r = launch_leg_tc64_batch(stage, g.spin, g.nj, g.d_args[polar], items, ni, s);
-        else if (stage == 0 && g.tc)
+        if (!mixed_groups) {
+          r = (stage ? g.tca : g.tc) ? launch_leg_tc64_batch(stage, g.spin, g.nj, g.d_args[polar], items, ni, s)
+                                     : launch_leg_fp64_batch(stage, g.spin, g.nj, g.ppt, g.d_args[polar], items, ni, s);
+        } else if (stage == 0 && g.tc) {
           r = launch_leg_tc_batch(g.spin, g.nj, g.two, g.d_targs[polar], items, ni, s);
-        else if (stage == 1 && g.tca)
+        } else if (stage == 1 && g.tca) {
           r = launch_leg_tc_ana_batch(g.spin, g.nj, g.d_targs[polar], items, ni, s);
-        else
-          r = mixed_groups ? launch_leg_mixed_batch(stage, g.spin, g.nj, g.ppt, g.pf, g.d_args[polar], items, ni, s)
-                           : launch_leg_fp64_batch(stage, g.spin, g.nj, g.ppt, g.d_args[polar], items, ni, s);
+        } else {
+          r = launch_leg_mixed_batch(stage, g.spin, g.nj, g.ppt, g.pf, g.d_args[polar], items, ni, s);
+        }
       }
       return r;
     };

@@ -10,10 +10,10 @@
 // kernels (legendre_tc.cu, legendre_tc_ana.cu; the structure of both is theirs):
 //
 //  * Lambda / u_p, u_p = 2^lexp a bound on the pair's values (bound_kernel, once per
-//    plan), is rounded to a multiple of 2^-56 and cut into seven 8-bit digits in
+//    plan), is rounded to a multiple of 2^-55 and cut into seven 8-bit digits in
 //    [-128, 127]: the bytes of its two's complement form after 0x80 is added to each.
-//    An IEEE double of Lambda's typical size, a quarter of the bound, is itself rounded
-//    to 2^-55 of it.
+//    An IEEE double of Lambda's typical size, a quarter of the bound, is itself a multiple
+//    of 2^-55 of it.
 //  * The other operand (a_lm per column and 256-degree window; G_m times u_p per column
 //    and tile) is scaled by a power of two of its largest value (in FP64, so the full
 //    exponent range passes) and cut the same way.
@@ -21,9 +21,17 @@
 //    most 2^23 units a product sum of 512 entries, each level's sums added in pairs of
 //    at most 2^24 or by exact two-sums), levels 4 to 6 (2^-32 and below) are added in
 //    FP32, rounding below 2^-56 of the bound; higher levels are dropped.  The sums are
-//    added up in FP64.  An FP64 dot product rounds every product and sum instead: the
-//    errors against 64-bit references are the same or smaller.
-//  * A column holding an infinity or NaN gives NaN.
+//    added up in FP64.
+//
+// An IEEE sum loses 2^-53 of each term, these operands 2^-54 of the largest input of a
+// column.  Where the inputs that meet at one result lie within 2^10 of one another that
+// stays below the error of Lambda itself, and the errors against 64-bit references are the
+// same (below).  Where they do not (a spectrum falling steeply over degrees a ring hardly
+// sees, one ring far brighter than the rest, a geometry without the equator, infinities
+// and NaN, the ends of the exponent range), the CTA runs the IEEE sums (leg64_ieee.cuh):
+// alm_to_pm decides for a synthesis' columns, tc64_ana_body for an analysis' items.  (As
+// kernels of their own behind these, over the same items, they cost 4 us a call when
+// nothing needed them, and a column of two E/B pairs at lmax 511 alone 0.3 ms.)
 //
 // Every wait is bounded (see legendre_tc_ana.cu).
 //
@@ -37,7 +45,7 @@
 // 5.8e-14 / 1.0e-13).  Analysis CTAs of 256 threads with four accumulators (as in the mixed
 // form): 1.52 and 1.44 ms on the first two, but 429 against 280 us at lmax 511, spin 0.
 #include "dual.cuh"
-#include "leg64.cuh"
+#include "leg64_ieee.cuh"
 #include "tcgen05.cuh"
 
 namespace sht {
@@ -241,7 +249,6 @@ struct AnaShape64 {
   static constexpr int NP = SPIN ? 1 : 2;
   static constexpr int TILES = NP * TH / kTile;
   static constexpr int NACC = 2;
-  static constexpr int GROUPS = WARPS / 4;
   static constexpr int LAG = 1;
   static constexpr int NC = 4 * NJ;
   static constexpr int CPW = NC / 4;
@@ -261,7 +268,7 @@ struct AnaShape64 {
   static constexpr int V = (SPIN ? 4 : 2) * NJ;
   static constexpr int MINB = NJ == 1 ? 4 : 2;
   static_assert(kColRows * NC <= kM && CPW <= 2, "columns within the MMA's rows");
-  static_assert(LAG % GROUPS == 0 && LAG < NACC, "a group reads the blocks it holds the turn of");
+  static_assert(WARPS == 4 && LAG < NACC, "every warp reads a quarter of every block");
   static_assert((KG - 1) * A_LBO + 7 * A_SBO + 128 <= A_BYTES + B_BYTES, "A operand inside shared memory");
   static_assert(MINB * (SMEM_LAUNCH + 2048) <= 228 * 1024, "CTAs per SM");
 };
@@ -272,12 +279,12 @@ struct AnaShape64 {
 // The bound 2^lexp on |p_l| per (m, ring pair), once per plan, from a plain FP32 walk of
 // the recursion in difference form (step_polar in mixed_common.cuh: relative errors
 // well inside the margin of 1/16 next to the poles too, as cos(theta) >= 0 in every
-// pair: 1 - cos(theta) keeps its digits there); not below 2^-30.  A thread
+// pair: 1 - cos(theta) keeps its digits there); not below 2^-90.  A thread
 // walks kBoundPairs pairs, which share the conversions of the coefficients.
 // ---------------------------------------------------------------------------
 constexpr int kBoundPairs = 8;
 template <bool SPIN>
-__global__ void __launch_bounds__(128) bound_kernel(LegArgs a, signed char *__restrict__ out) {
+__global__ void __launch_bounds__(128) bound_kernel(LegArgs a, signed char *__restrict__ out, unsigned char *__restrict__ geo) {
   const int mi = blockIdx.y, pb = blockIdx.x * 128 * kBoundPairs + threadIdx.x;
   if (pb >= a.npairs) return;
   const int m = a.mval[mi];
@@ -285,6 +292,7 @@ __global__ void __launch_bounds__(128) bound_kernel(LegArgs a, signed char *__re
   const int l0 = m > as ? m : as, lmax = a.lmax;
   const double2 *__restrict__ cf = a.coef + (a.coef_off[mi] - l0);
   float vmax[kBoundPairs];
+  int elow = 4096;  // of the equator-most pair: the exponent of the smaller start value
 #pragma unroll
   for (int k = 0; k < kBoundPairs; ++k) vmax[k] = 0.f;
 #pragma unroll 1
@@ -304,6 +312,7 @@ __global__ void __launch_bounds__(128) bound_kernel(LegArgs a, signed char *__re
         sc[k] = (e + 32) >= 0 ? (e + 32) / 64 : -((-(e + 32) + 63) / 64);
         p[k] = (float)ldexp(mant, e - 64 * sc[k]);
       }
+      if (pb + 128 * k == a.npairs - 1) elow = min(elow, mant != 0.0 ? ilogb(mant) + e : -4096);
       d[k] = p[k];
       w[k] = sc[k] == 0 ? 1.f : (sc[k] == -1 ? 0x1p-64f : 0.f);
     }
@@ -329,13 +338,15 @@ __global__ void __launch_bounds__(128) bound_kernel(LegArgs a, signed char *__re
 #pragma unroll
   for (int k = 0; k < kBoundPairs; ++k) {
     if (pb + 128 * k >= a.npairs) break;
-    int e = -30;
+    int e = -90;
     if (vmax[k] > 0.f) {
       int ev;
       frexpf(vmax[k] * 1.0625f, &ev);
       e = max(e, min(ev, 100));
     }
     out[(size_t)mi * a.npairs + pb + 128 * k] = (signed char)e;
+    // every degree's sum has terms of about its largest bound if this pair starts near it
+    if (pb + 128 * k == a.npairs - 1) geo[mi] = elow >= e - 6;
   }
 }
 
@@ -504,7 +515,7 @@ __device__ __forceinline__ void tc64_syn_body(const LegArgs &a, const int2 item,
         const double t = level_sum(L(0), L(1), L(2), 0.f, L(3), 0.f, lo);
         const int e = em[value_of(c0 + c)];
         double &acc = accs[(c0 + c) * kRows + tid];
-        acc += e == 2047 ? __longlong_as_double(0x7ff8000000000000ll) : scale_pow2(t, e - 1021 - 14);
+        acc += scale_pow2(t, e - 1021 - 14);
       }
     }
   };
@@ -625,17 +636,18 @@ __device__ __forceinline__ void tc64_syn_body(const LegArgs &a, const int2 item,
 
 // ---------------------------------------------------------------------------
 // analysis (K entries, columns and pipeline as in legendre_tc_ana.cu; the partial
-// sums, as in legendre_fp64.cu, in items that walk a group of tiles into one slot)
+// sums, as in legendre_fp64.cu, in items that walk a group of tiles into one slot); false
+// if the item is left to the IEEE sums
 // ---------------------------------------------------------------------------
 template <int NJ, bool SPIN>
-__device__ __forceinline__ void tc64_ana_body(const LegArgs &a, const int4 item, unsigned char *smem) {
+__device__ __forceinline__ bool tc64_ana_body(const LegArgs &a, const int4 item, unsigned char *smem) {
   using namespace t64;
   using S = AnaShape64<NJ, SPIN>;
   constexpr int NC = S::NC, V = S::V, TH = S::TH, NP = S::NP;
-  constexpr int NACC = S::NACC, GROUPS = S::GROUPS, LAG = S::LAG;
+  constexpr int NACC = S::NACC, LAG = S::LAG;
   __shared__ __align__(8) uint64_t full[NACC], freeb[NACC], mine[S::WARPS];
   __shared__ uint32_t tslot;
-  __shared__ int vmax[NC];
+  __shared__ int vmax[NC], eqmax[NC];
   __shared__ int tstart[S::WARPS];
   __shared__ volatile int stop;
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
@@ -681,6 +693,75 @@ __device__ __forceinline__ void tc64_ana_body(const LegArgs &a, const int4 item,
   const uint64_t bdesc0 = tc::mat_desc(tc::smem_u32(Bbuf), kKStride, S::B_SBO);
   constexpr uint32_t idesc = tc::instr_desc(kM, kN, true);
 
+  // the K entries of pair p (spin: both of its lanes; spin 0: lane t) for every column
+  auto load_pair = [&](int p, int t, double (&gv)[2][NC]) __attribute__((always_inline)) {
+    const bool south = a.pairs[p].south;
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) {
+      if (!SPIN) {
+        const double2 *gp = a.phase + (((size_t)j * a.nm + mi) * a.npairs + p) * 2;
+        const double2 gn = gp[0], gs = south ? gp[1] : make_double2(0.0, 0.0);
+        gv[t][4 * j + 0] = gn.x + gs.x;
+        gv[t][4 * j + 1] = gn.y + gs.y;
+        gv[t][4 * j + 2] = gn.x - gs.x;
+        gv[t][4 * j + 3] = gn.y - gs.y;
+      } else {
+        const double2 *gq = a.phase + (((size_t)(2 * j) * a.nm + mi) * a.npairs + p) * 2;
+        const double2 *gu = a.phase + (((size_t)(2 * j + 1) * a.nm + mi) * a.npairs + p) * 2;
+        const double2 qn = gq[0], un = gu[0];
+        const double2 qs = south ? gq[1] : make_double2(0.0, 0.0), us = south ? gu[1] : make_double2(0.0, 0.0);
+        gv[0][4 * j + 0] = qn.x - un.y;          // T1: l+ W+_N
+        gv[0][4 * j + 1] = qn.y + un.x;
+        gv[0][4 * j + 2] = sg0 * (qs.x + us.y);  // s T2: l+ W-_S'
+        gv[0][4 * j + 3] = sg0 * (qs.y - us.x);
+        gv[1][4 * j + 0] = sg0 * (qs.x - us.y);  // T1: s l- W+_S'
+        gv[1][4 * j + 1] = sg0 * (qs.y + us.x);
+        gv[1][4 * j + 2] = qn.x + un.y;          // s T2: s l- W-_N
+        gv[1][4 * j + 3] = qn.y - un.x;
+      }
+    }
+  };
+  // The size of column c's largest entry in gv, |G u_p|, as an exponent field (scaled by
+  // 2^200, so that u_p keeps it positive; infinities and NaN: 4000)
+  auto size_of = [&](const double (&gv)[2][NC], const int (&lexp)[NP], int c) __attribute__((always_inline)) {
+    int mx = 0;
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+      const int e = size_field(gv[t][c]);
+      if (e > 0) mx = max(mx, e == 2047 ? 4000 : e + 200 + lexp[SPIN ? 0 : t]);
+    }
+    return mx;
+  };
+
+  // Whether the item's values range too far for fixed point (it then returns false): at degree l
+  // the sum comes from the pairs between some latitude and the equator, below l0's from the
+  // ones next to it, and the others' Lambda falls away exponentially; so no pair's |G u_p|
+  // may exceed 2^kWideRange times the largest of the 32 next to the equator (columns of
+  // zeros there are zero).  One warp finds those; each pass compares its own.
+  if (warp == 0) {
+    const int p = a.npairs - 1 - lane;
+    int mx[NC];
+    {
+      double gv[2][NC];
+      int lexp[NP];
+#pragma unroll
+      for (int t = 0; t < 2; ++t)
+#pragma unroll
+        for (int c = 0; c < NC; ++c) gv[t][c] = 0.0;
+#pragma unroll
+      for (int t = 0; t < NP; ++t) lexp[t] = p >= 0 ? a.lexp[(size_t)mi * a.npairs + p] : 0;
+      if (p >= 0) load_pair(p, 0, gv);
+#pragma unroll
+      for (int c = 0; c < NC; ++c) mx[c] = size_of(gv, lexp, c);
+    }
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      const int e = __reduce_max_sync(0xffffffffu, mx[c]);
+      if (lane == 0) eqmax[c] = e;
+    }
+  }
+  bool wide = false;
+
   int ib = 0;
   int nmine = 0, nmine_done = 0;
   bool ok = true;
@@ -695,7 +776,7 @@ __device__ __forceinline__ void tc64_ana_body(const LegArgs &a, const int4 item,
   };
 
 #pragma unroll 1
-  for (int gi = 0; gi < ng; gi += S::TILES) {
+  for (int gi = 0; gi < ng && !wide; gi += S::TILES) {
     int pr[NP], lexp[NP];
     bool valid[NP];
     double gv[2][NC];
@@ -708,33 +789,7 @@ __device__ __forceinline__ void tc64_ana_body(const LegArgs &a, const int4 item,
       pr[t] = (item.y + gi) * kTile + NP * tid + t;
       valid[t] = pr[t] < min(a.npairs, (item.y + ng) * kTile);
       lexp[t] = valid[t] ? a.lexp[(size_t)mi * a.npairs + pr[t]] : 0;
-      if (!valid[t]) continue;
-      const int p = pr[t];
-      const bool south = a.pairs[p].south;
-#pragma unroll
-      for (int j = 0; j < NJ; ++j) {
-        if (!SPIN) {
-          const double2 *gp = a.phase + (((size_t)j * a.nm + mi) * a.npairs + p) * 2;
-          const double2 gn = gp[0], gs = south ? gp[1] : make_double2(0.0, 0.0);
-          gv[t][4 * j + 0] = gn.x + gs.x;
-          gv[t][4 * j + 1] = gn.y + gs.y;
-          gv[t][4 * j + 2] = gn.x - gs.x;
-          gv[t][4 * j + 3] = gn.y - gs.y;
-        } else {
-          const double2 *gq = a.phase + (((size_t)(2 * j) * a.nm + mi) * a.npairs + p) * 2;
-          const double2 *gu = a.phase + (((size_t)(2 * j + 1) * a.nm + mi) * a.npairs + p) * 2;
-          const double2 qn = gq[0], un = gu[0];
-          const double2 qs = south ? gq[1] : make_double2(0.0, 0.0), us = south ? gu[1] : make_double2(0.0, 0.0);
-          gv[0][4 * j + 0] = qn.x - un.y;          // T1: l+ W+_N
-          gv[0][4 * j + 1] = qn.y + un.x;
-          gv[0][4 * j + 2] = sg0 * (qs.x + us.y);  // s T2: l+ W-_S'
-          gv[0][4 * j + 3] = sg0 * (qs.y - us.x);
-          gv[1][4 * j + 0] = sg0 * (qs.x - us.y);  // T1: s l- W+_S'
-          gv[1][4 * j + 1] = sg0 * (qs.y + us.x);
-          gv[1][4 * j + 2] = qn.x + un.y;          // s T2: s l- W-_N
-          gv[1][4 * j + 3] = qn.y - un.x;
-        }
-      }
+      if (valid[t]) load_pair(pr[t], t, gv);
     }
     // the recursions up to the warp's first block with a value at scale 0
     Rec<SPIN, false> rec;
@@ -756,17 +811,15 @@ __device__ __forceinline__ void tc64_ana_body(const LegArgs &a, const int4 item,
     if (lane == 0) tstart[warp] = lw;
     __syncthreads();
 #pragma unroll
-    for (int c = 0; c < NC; ++c) {  // column bounds over the tile: exponent fields of |G u_p| (2200: not finite)
-      int mx = 0;
-#pragma unroll
-      for (int t = 0; t < 2; ++t) {
-        const int e = exp_field(gv[t][c]);
-        if (e > 0) mx = max(mx, e == 2047 ? 4000 : e + 200 + lexp[SPIN ? 0 : t]);
-      }
-      mx = __reduce_max_sync(0xffffffffu, mx);
+    for (int c = 0; c < NC; ++c) {  // column bounds over the tile
+      const int mx = __reduce_max_sync(0xffffffffu, size_of(gv, lexp, c));
       if (lane == 0) atomicMax(&vmax[c], mx);
     }
     __syncthreads();
+#pragma unroll
+    for (int c = 0; c < NC; ++c)
+      wide = wide || (vmax[c] > 0 && (vmax[c] > eqmax[c] + kWideRange || vmax[c] < kFieldMin + 200 || vmax[c] >= kFieldMax + 200));
+    if (wide) break;  // the same for every thread; no product is in flight here
     int lstart = tstart[0];
 #pragma unroll
     for (int w = 1; w < S::WARPS; ++w) lstart = min(lstart, tstart[w]);
@@ -775,7 +828,7 @@ __device__ __forceinline__ void tc64_ana_body(const LegArgs &a, const int4 item,
 #pragma unroll
       for (int t = 0; t < 2; ++t) {
         // |G u_p 2^(1221 - vmax)| < 1/2
-        const uint64_t f = fix64(vmax[c] >= 4000 ? 0.0 : scale_pow2(gv[t][c], lexp[SPIN ? 0 : t] + 1221 - vmax[c]));
+        const uint64_t f = fix64(scale_pow2(gv[t][c], lexp[SPIN ? 0 : t] + 1221 - vmax[c]));
         unsigned char *dst = Abuf + S::a_at(c, 0, t * (TH / 8) + tid / 8) + (tid % 8) * 2;
 #pragma unroll
         for (int j = 0; j < kDig; ++j) *reinterpret_cast<uint16_t *>(dst + j * 16) = tc::bf16_of(digit(f, j));
@@ -893,7 +946,7 @@ __device__ __forceinline__ void tc64_ana_body(const LegArgs &a, const int4 item,
       if (o) {
         const double t = level_sum(D(0, 0), __fadd_rn(D(1, 0), D(0, 1)), __fadd_rn(D(2, 0), D(1, 1)), D(0, 2),
                                    __fadd_rn(D(3, 0), D(2, 1)), __fadd_rn(D(1, 2), D(0, 3)), lo);
-        const double val = vm >= 4000 ? __longlong_as_double(0x7ff8000000000000ll) : scale_pow2(t, vm - 1221 - 14);
+        const double val = scale_pow2(t, vm - 1221 - 14);
         *o = prev + (neg ? -val : val);
       }
       __syncwarp();
@@ -904,7 +957,7 @@ __device__ __forceinline__ void tc64_ana_body(const LegArgs &a, const int4 item,
 #pragma unroll 1
     for (; lb <= lmax; lb += kBlk, ++ib) {
       const int xb = ib % NACC;
-      const bool turn = ib - LAG >= ib0 && (GROUPS == 1 || (ib & 1) == (warp >> 2));
+      const bool turn = ib - LAG >= ib0;
       bool neg_prev = false;
       double *const o_prev = turn ? out_at(lb - LAG * kBlk, neg_prev) : nullptr;
       double prev = 0.0;
@@ -953,7 +1006,6 @@ __device__ __forceinline__ void tc64_ana_body(const LegArgs &a, const int4 item,
     if (!ok) continue;
 #pragma unroll 1
     for (int k = ib - LAG > ib0 ? ib - LAG : ib0; k < ib; ++k) {
-      if (GROUPS > 1 && (k & 1) != (warp >> 2)) continue;
       bool neg;
       double *o = out_at(lb - (ib - k) * kBlk, neg);
       const double prev = (o && gi > 0) ? *o : 0.0;
@@ -968,34 +1020,52 @@ __device__ __forceinline__ void tc64_ana_body(const LegArgs &a, const int4 item,
   __syncthreads();
   tc::fence_after();
   if (warp == 0) tc::tmem_dealloc(tbase, S::TCOLS);
+  return !wide;
 }
 
 // ---------------------------------------------------------------------------
 // kernels and launchers (plans, and batches: item.w selects the plan's record)
 // ---------------------------------------------------------------------------
 template <int NJ, bool SPIN>
+__device__ __forceinline__ void tc64_syn_item(const LegArgs &a, const int2 item, unsigned char *smem) {
+  if (!a.wide_syn[item.x]) tc64_syn_body<NJ, SPIN>(a, item, smem);
+  else if constexpr (SPIN) leg_syn_spin_body<NJ>(a, item);
+  else leg_syn_s0_body<NJ>(a, item);
+}
+template <int NJ, bool SPIN>
+__device__ __forceinline__ void tc64_ana_item(const LegArgs &a, const int4 item, unsigned char *smem) {
+  if (a.geo[item.x] && tc64_ana_body<NJ, SPIN>(a, item, smem)) return;
+  __syncthreads();
+  double (*const red)[32] = reinterpret_cast<double (*)[32]>(smem);
+#pragma unroll 1
+  for (int gi = 0; gi < (item.z & 255); ++gi) {  // tile after tile into the item's slot
+    if constexpr (SPIN) leg_ana_spin_body<NJ, 1>(a, item, gi, red);
+    else leg_ana_s0_body<NJ, 1>(a, item, gi, red);
+  }
+}
+template <int NJ, bool SPIN>
 __global__ void __launch_bounds__(t64::kRows, (t64::Shape<NJ, SPIN>::MINB)) tc64_syn(LegArgs a) {
   extern __shared__ __align__(128) unsigned char tc64_smem[];
-  tc64_syn_body<NJ, SPIN>(a, a.syn_items[blockIdx.x], tc64_smem);
+  tc64_syn_item<NJ, SPIN>(a, a.syn_items[blockIdx.x], tc64_smem);
 }
 template <int NJ, bool SPIN>
 __global__ void __launch_bounds__(t64::kRows, (t64::Shape<NJ, SPIN>::MINB))
     tc64_syn_batch(const LegArgs *__restrict__ args, const int4 *__restrict__ items) {
   extern __shared__ __align__(128) unsigned char tc64_smem[];
   const int4 it = items[blockIdx.x];
-  tc64_syn_body<NJ, SPIN>(args[it.w], make_int2(it.x, it.y), tc64_smem);
+  tc64_syn_item<NJ, SPIN>(args[it.w], make_int2(it.x, it.y), tc64_smem);
 }
 template <int NJ, bool SPIN>
 __global__ void __launch_bounds__((t64::AnaShape64<NJ, SPIN>::TH), (t64::AnaShape64<NJ, SPIN>::MINB)) tc64_ana(LegArgs a) {
   extern __shared__ __align__(128) unsigned char tc64_smem[];
-  tc64_ana_body<NJ, SPIN>(a, a.ana_items[blockIdx.x], tc64_smem);
+  tc64_ana_item<NJ, SPIN>(a, a.ana_items[blockIdx.x], tc64_smem);
 }
 template <int NJ, bool SPIN>
 __global__ void __launch_bounds__((t64::AnaShape64<NJ, SPIN>::TH), (t64::AnaShape64<NJ, SPIN>::MINB))
     tc64_ana_batch(const LegArgs *__restrict__ args, const int4 *__restrict__ items) {
   extern __shared__ __align__(128) unsigned char tc64_smem[];
   const int4 it = items[blockIdx.x];
-  tc64_ana_body<NJ, SPIN>(args[it.w], make_int4(it.x, it.y, it.z, 0), tc64_smem);
+  tc64_ana_item<NJ, SPIN>(args[it.w], make_int4(it.x, it.y, it.z, 0), tc64_smem);
 }
 
 // f.template operator()<NJ, SPIN>() for the shapes the kernels are built for
@@ -1112,8 +1182,8 @@ cudaError_t launch_bounds64(const sht_plan_s *P, cudaStream_t st) {
   LegArgs a;
   leg_fp64_fill_args(P, 1, &a);
   const dim3 grid((P->npairs + 128 * kBoundPairs - 1) / (128 * kBoundPairs), P->nm);
-  if (P->spin) bound_kernel<true><<<grid, 128, 0, st>>>(a, P->d_lexp);
-  else bound_kernel<false><<<grid, 128, 0, st>>>(a, P->d_lexp);
+  if (P->spin) bound_kernel<true><<<grid, 128, 0, st>>>(a, P->d_lexp, P->d_geo);
+  else bound_kernel<false><<<grid, 128, 0, st>>>(a, P->d_lexp, P->d_geo);
   return cudaGetLastError();
 }
 

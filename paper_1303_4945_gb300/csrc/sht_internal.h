@@ -194,6 +194,10 @@ struct sht_plan_s {
   int tc64_syn = 0, tc64_ana = 0;
   int tc64_able = 0;  // the analysis can: at the default tiling, where autotuning did not find another faster
   signed char *d_lexp = nullptr;
+  // per m index: whether the geometry allows the analysis; a byte per job, what of a
+  // synthesis runs in IEEE double instead (LegArgs in leg64.cuh)
+  unsigned char *d_geo = nullptr;
+  unsigned *d_wide_syn = nullptr;
   int *d_err = nullptr;      // device status word written by kernels with bounded waits
   float4 *d_join = nullptr;  // mixed plans: join record per (m index, pair), 3 float4 each
   int64_t triples_joined = 0;  // steps from each kept pair's join block on (polar cut applied)
