@@ -17,7 +17,7 @@ SRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT, "libsht_gb300.so")
 UNITS = ["sht_host.cu", "tables.cu", "legendre_fp64.cu", "legendre_tc64.cu", "legendre_mixed.cu", "legendre_tc.cu", "legendre_tc_ana.cu", "fft.cu", "noalloc.cu", "stages.cu", "batch.cu", "peaks.cu"]
-HEADERS = ["sht_internal.h", "sht_device.cuh", "leg64.cuh", "leg64_ieee.cuh", "df.cuh", "mixed_common.cuh", "dual.cuh", "tcgen05.cuh"]
+HEADERS = ["sht_internal.h", "sht_device.cuh", "leg64.cuh", "leg64_ieee.cuh", "df.cuh", "mixed_common.cuh", "mix_ana.cuh", "dual.cuh", "tcgen05.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden",
          "-I", os.path.join(ROOT, "include")]

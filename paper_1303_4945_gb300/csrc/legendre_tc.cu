@@ -754,6 +754,7 @@ void leg_tc_fill_args(const sht_plan_s *P, int polar, void *out) {
   TcArgs ta;
   leg_mixed_fill_args(P, polar, &ta.m);
   ta.err = P->d_err;
+  ta.force = P->quad_off;
   memcpy(out, &ta, sizeof(ta));
 }
 
@@ -773,6 +774,7 @@ cudaError_t launch_leg_tc_syn(const sht_plan_s *P, const void *mixargs, int n, c
   TcArgs ta;
   memcpy(&ta.m, mixargs, sizeof(MixArgs));
   ta.err = P->d_err;
+  ta.force = P->quad_off;
   const bool ok = syn_shape(P->spin, P->njobs_pad, P->syn_two != 0, [&](auto sh) {
     using H = decltype(sh);
     tc_syn<H::nj, H::spin, H::two><<<n, tc::kRows, H::smem, st>>>(ta);

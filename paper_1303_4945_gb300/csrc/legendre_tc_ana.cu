@@ -54,6 +54,7 @@
 #include <math_constants.h>
 
 #include "dual.cuh"
+#include "mix_ana.cuh"
 #include "tcgen05.cuh"
 
 namespace sht {
@@ -205,13 +206,14 @@ __device__ __forceinline__ void split6(float2 h, float2 l, float2 (&d)[kDig]) {
 // G_N - G_S, the two lanes two neighbouring pairs.
 // ---------------------------------------------------------------------------
 template <int NJ, bool SPIN>
-__device__ __forceinline__ void tc_ana_body(const TcArgs &ta, const int4 item_, const int j0, unsigned char *tca_smem) {
+__device__ __forceinline__ bool tc_ana_body(const TcArgs &ta, const int4 item_, const int j0, unsigned char *tca_smem) {
   using S = tca::AnaShape<NJ, SPIN>;
   constexpr int NSET = S::NSET, NC = S::NC, kDig = tca::kDig, TH = S::TH, NP = S::NP;
   constexpr int NACC = S::NACC, GROUPS = S::GROUPS, LAG = S::LAG;
   __shared__ __align__(8) uint64_t full[NACC], freeb[NACC], mine[S::WARPS];
   __shared__ uint32_t tslot;
-  __shared__ unsigned vmax[NC];
+  __shared__ unsigned vmax[NC], eqmax[NC];
+  __shared__ int eqok;
   __shared__ int tstart[S::WARPS];
   __shared__ volatile int stop;
   const MixArgs &a = ta.m;
@@ -267,6 +269,84 @@ __device__ __forceinline__ void tc_ana_body(const TcArgs &ta, const int4 item_, 
   const uint64_t bdesc0 = tc::mat_desc(tc::smem_u32(Bbuf), S::KSTRIDE, S::B_SBO);
   constexpr uint32_t idesc = tc::instr_desc(S::M, tca::kN, true);
 
+  // the K entries of pair p (spin: both of its lanes; spin 0: lane t) for every column
+  auto load_pair = [&](int p, int t, double (&gv)[NSET][NC]) __attribute__((always_inline)) {
+    const bool south = a.pairs[p].south;
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) {
+      if (!SPIN) {
+        const double2 *gp = a.phase + (((size_t)(j0 + j) * a.nm + mi) * a.npairs + p) * 2;
+        const double2 gn = gp[0], gs = south ? gp[1] : make_double2(0.0, 0.0);
+        gv[t][4 * j + 0] = gn.x + gs.x;
+        gv[t][4 * j + 1] = gn.y + gs.y;
+        gv[t][4 * j + 2] = gn.x - gs.x;
+        gv[t][4 * j + 3] = gn.y - gs.y;
+      } else {
+        const double2 *gq = a.phase + (((size_t)(2 * (j0 + j)) * a.nm + mi) * a.npairs + p) * 2;
+        const double2 *gu = a.phase + (((size_t)(2 * (j0 + j) + 1) * a.nm + mi) * a.npairs + p) * 2;
+        const double2 qn = gq[0], un = gu[0];
+        const double2 qs = south ? gq[1] : make_double2(0.0, 0.0), us = south ? gu[1] : make_double2(0.0, 0.0);
+        // W+_N, W-_N, W+_S', W-_S' (re, im)
+        const double wpn_r = qn.x - un.y, wpn_i = qn.y + un.x;
+        const double wmn_r = qn.x + un.y, wmn_i = qn.y - un.x;
+        const double wps_r = sg0 * (qs.x - us.y), wps_i = sg0 * (qs.y + us.x);
+        const double wms_r = sg0 * (qs.x + us.y), wms_i = sg0 * (qs.y - us.x);
+        gv[0][4 * j + 0] = wpn_r;  // T1: l+ W+_N
+        gv[0][4 * j + 1] = wpn_i;
+        gv[0][4 * j + 2] = wms_r;  // s T2: l+ W-_S'
+        gv[0][4 * j + 3] = wms_i;
+        gv[1][4 * j + 0] = wps_r;  // T1: s l- W+_S'
+        gv[1][4 * j + 1] = wps_i;
+        gv[1][4 * j + 2] = wmn_r;  // s T2: s l- W-_N
+        gv[1][4 * j + 3] = wmn_i;
+      }
+    }
+  };
+  // Plans that always run this kernel (more than two jobs): whether the item's values range too far for
+  // the digits, which lose 2^-50 of a column's largest |G'| where the double-float sums lose
+  // 2^-46 of each term; the item is then left to those (false).  At degree l the sum comes
+  // from the pairs between some latitude and the equator (l0: next to it), the others' Lambda
+  // falls away exponentially, so no |G'| may exceed 2^kWideRange times the largest of the 32
+  // pairs next to the equator, and the last of them has to start near its bound at l0.
+  // (White maps without ring weights range over u_p, 2^5 at lmax 2047, and their extremes.)
+  constexpr int kWideRange = 8;
+  bool wide = false;
+  const bool guard = S::QUAD || (S::GROUPED && a.nj > NJ);
+  if (guard && warp == 0) {
+    const int p = a.npairs - 1 - lane;
+    unsigned mx[NC];
+    {
+      double gv[NSET][NC];
+#pragma unroll
+      for (int t = 0; t < NSET; ++t)
+#pragma unroll
+        for (int c = 0; c < NC; ++c) gv[t][c] = 0.0;
+      JoinRec r = {};
+      if (p >= 0) {
+        r = ld_join(a.join + ((size_t)mi * a.npairs + p) * 3);
+        load_pair(p, 0, gv);
+      }
+      if (lane == 0) {
+        const float low = SPIN ? fminf(fabsf(r.lpc.h), fabsf(r.lmc.h)) : fabsf(r.lpc.h);
+        eqok = r.lj == l0 && r.scp == 0 && (!SPIN || r.scm == 0) && low >= ldexpf(1.f, r.lexp - 6);
+      }
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
+        mx[c] = 0u;
+#pragma unroll
+        for (int t = 0; t < (SPIN ? 2 : 1); ++t) {
+          const unsigned hi = (unsigned)__double2hiint(gv[t][c]) & 0x7fffffffu;
+          if (p >= 0 && r.lj <= lmax && hi > 0u) mx[c] = max(mx[c], tca::not_finite(hi) ? 0x7ff00000u : tca::add_exp(hi, r.lexp));
+        }
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      const unsigned e = __reduce_max_sync(0xffffffffu, mx[c]);
+      if (lane == 0) eqmax[c] = e;
+    }
+  }
+
   int ib = 0;                    // blocks walked by the CTA over all its tiles: accumulator ib % NACC
   int nmine = 0, nmine_done = 0;  // this warp's commits to mine[warp], and those waited for
   bool ok = true;
@@ -310,40 +390,8 @@ __device__ __forceinline__ void tc_ana_body(const TcArgs &ta, const int4 item_, 
 #pragma unroll
       for (int c = 0; c < NC; ++c) gv[t][c] = 0.0;
 #pragma unroll
-    for (int t = 0; t < NP; ++t) {
-      if (!valid[t]) continue;
-      const int p = pr[t];
-      const bool south = a.pairs[p].south;
-#pragma unroll
-      for (int j = 0; j < NJ; ++j) {
-        if (!SPIN) {
-          const double2 *gp = a.phase + (((size_t)(j0 + j) * a.nm + mi) * a.npairs + p) * 2;
-          const double2 gn = gp[0], gs = south ? gp[1] : make_double2(0.0, 0.0);
-          gv[t][4 * j + 0] = gn.x + gs.x;
-          gv[t][4 * j + 1] = gn.y + gs.y;
-          gv[t][4 * j + 2] = gn.x - gs.x;
-          gv[t][4 * j + 3] = gn.y - gs.y;
-        } else {
-          const double2 *gq = a.phase + (((size_t)(2 * (j0 + j)) * a.nm + mi) * a.npairs + p) * 2;
-          const double2 *gu = a.phase + (((size_t)(2 * (j0 + j) + 1) * a.nm + mi) * a.npairs + p) * 2;
-          const double2 qn = gq[0], un = gu[0];
-          const double2 qs = south ? gq[1] : make_double2(0.0, 0.0), us = south ? gu[1] : make_double2(0.0, 0.0);
-          // W+_N, W-_N, W+_S', W-_S' (re, im)
-          const double wpn_r = qn.x - un.y, wpn_i = qn.y + un.x;
-          const double wmn_r = qn.x + un.y, wmn_i = qn.y - un.x;
-          const double wps_r = sg0 * (qs.x - us.y), wps_i = sg0 * (qs.y + us.x);
-          const double wms_r = sg0 * (qs.x + us.y), wms_i = sg0 * (qs.y - us.x);
-          gv[0][4 * j + 0] = wpn_r;  // T1: l+ W+_N
-          gv[0][4 * j + 1] = wpn_i;
-          gv[0][4 * j + 2] = wms_r;  // s T2: l+ W-_S'
-          gv[0][4 * j + 3] = wms_i;
-          gv[1][4 * j + 0] = wps_r;  // T1: s l- W+_S'
-          gv[1][4 * j + 1] = wps_i;
-          gv[1][4 * j + 2] = wmn_r;  // s T2: s l- W-_N
-          gv[1][4 * j + 3] = wmn_i;
-        }
-      }
-    }
+    for (int t = 0; t < NP; ++t)
+      if (valid[t]) load_pair(pr[t], t, gv);
     __syncthreads();  // the previous tile's products are complete (its last accumulator was read)
     if (stop) {       // read after a barrier: the same for every warp
       ok = false;
@@ -368,6 +416,14 @@ __device__ __forceinline__ void tc_ana_body(const TcArgs &ta, const int4 item_, 
       if (lane == 0) atomicMax(&vmax[c], w);
     }
     __syncthreads();
+    if (guard) {
+      wide = !eqok || ta.force;
+#pragma unroll
+      for (int c = 0; c < NC; ++c)  // (a column that is not finite: below)
+        wide = wide || (vmax[c] > 0u && !tca::not_finite(vmax[c]) && !tca::not_finite(eqmax[c]) &&
+                        (vmax[c] >> 20) > (eqmax[c] >> 20) + kWideRange);
+      if (wide) break;  // the same for every thread; no product is in flight here
+    }
     int lstart = tstart[0];
 #pragma unroll
     for (int w = 1; w < S::WARPS; ++w) lstart = min(lstart, tstart[w]);
@@ -753,6 +809,18 @@ __device__ __forceinline__ void tc_ana_body(const TcArgs &ta, const int4 item_, 
   __syncthreads();
   tc::fence_after();
   if (warp == 0) tc::tmem_dealloc(tbase, S::TCOLS);
+  return !wide;
+}
+
+template <int NJ, bool SPIN>
+__device__ __forceinline__ void tc_ana_item(const TcArgs &ta, const int4 item, const int j0, unsigned char *smem) {
+  using S = tca::AnaShape<NJ, SPIN>;
+  if (tc_ana_body<NJ, SPIN>(ta, item, j0, smem)) return;
+  if constexpr (S::GROUPED) {  // the item's tiles of 256 pairs in double-float
+    static_assert(sizeof(MixAnaShared) <= S::SMEM, "its table in the digits' shared memory");
+    __syncthreads();
+    mix_ana_body<NJ, 2, SPIN>(ta.m, item, *reinterpret_cast<MixAnaShared *>(smem), j0, (SPIN ? 4 : 2) * ta.m.nj, true);
+  }
 }
 
 // a plan of more than four jobs: consecutive CTAs take its groups of four
@@ -762,7 +830,7 @@ __global__ void __launch_bounds__((tca::AnaShape<NJ, SPIN>::TH), (tca::AnaShape<
   extern __shared__ __align__(128) unsigned char tca_smem[];
   constexpr bool G = tca::AnaShape<NJ, SPIN>::GROUPED;
   const int g = G ? blockIdx.x % groups : 0, i = G ? blockIdx.x / groups : blockIdx.x;
-  tc_ana_body<NJ, SPIN>(ta, ta.m.ana_items[i], NJ * g, tca_smem);
+  tc_ana_item<NJ, SPIN>(ta, ta.m.ana_items[i], NJ * g, tca_smem);
 }
 
 // batches: item (mi, first tile, slot << 8 | tiles, record); the record holds the plan's arguments
@@ -773,7 +841,7 @@ __global__ void __launch_bounds__((tca::AnaShape<NJ, SPIN>::TH), (tca::AnaShape<
   constexpr bool G = tca::AnaShape<NJ, SPIN>::GROUPED;
   const int g = G ? blockIdx.x % groups : 0;
   const int4 it = items[G ? blockIdx.x / groups : blockIdx.x];
-  tc_ana_body<NJ, SPIN>(args[it.w], make_int4(it.x, it.y, it.z, 0), NJ * g, tca_smem);
+  tc_ana_item<NJ, SPIN>(args[it.w], make_int4(it.x, it.y, it.z, 0), NJ * g, tca_smem);
 }
 
 template <int NJ, bool SPIN>
@@ -854,6 +922,7 @@ cudaError_t launch_leg_tc_ana(const sht_plan_s *P, const void *mixargs, int n, c
   TcArgs ta;
   memcpy(&ta.m, mixargs, sizeof(MixArgs));
   ta.err = P->d_err;
+  ta.force = P->quad_off;
   const bool ok = tca_shape(P->spin, P->njobs_pad, [&](auto sh) {
     using H = decltype(sh);
     const int groups = P->njobs_pad / H::nj;

@@ -187,6 +187,7 @@ struct sht_plan_s {
   // mixed plans: the analysis contraction on the tensor cores (legendre_tc_ana.cu;
   // tiles of kAnaThreads ring pairs, one per thread)
   int tc_ana = 0;
+  int quad_off = 0;  // plans of more than two jobs: the caller asked for the double-float analysis
   float tc_lam_bound = 0.f;  // power of two bounding |Lambda_lm| for lmax
   // FP64 plans: the contractions on the tensor cores (legendre_tc64.cu), for shapes and
   // sizes where they are faster (tc64_choose in sht_host.cu); d_lexp: per (m index, pair)

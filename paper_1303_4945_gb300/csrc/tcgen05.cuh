@@ -170,6 +170,7 @@ __device__ __forceinline__ float pow2_above(float x) {
 struct TcArgs {
   MixArgs m;        // tables, work items and phase array of the mixed form
   int *err;         // device status word: bit 0 set when a bounded wait gave up
+  int force;        // analysis of more than two jobs: every item in double-float
 };
 
 }  // namespace sht
