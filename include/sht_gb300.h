@@ -328,13 +328,16 @@ SHT_API int sht_plan_get_fft_precision(sht_plan_t plan, int *precision);
  * where the double-float contraction is faster (measured on GB300 at lmax 4095:
  * spin 2 one E/B pair 38.7 ms against 57.6, spin 0 eight maps 59.2 against 102.3; one
  * spin-0 map 18.7 against 20.4, but lmax 511 137 us against 106).  sht_plan_set_tensor_cores(plan, 1 or 0)
- * selects it or the double-float contraction; sht_plan_get_tensor_cores reads the
- * setting.  A batch runs each plan with the setting it had when the batch was
- * made (the setting cannot change while a batch refers to the plan).  Errors: SHT_ERR_INVALID_ARG (NULL, an
- * FP64 plan, a plan in a batch), SHT_ERR_UNSUPPORTED.
+ * selects it or the double-float contraction; sht_plan_get_tensor_cores reads
+ * whether the plan's synthesis contracts on the tensor cores.  An FP64 plan chooses by
+ * size when it is made (fixed-point digits, see SHT_FP64; columns that they do not hold
+ * run in IEEE double): it takes 0, which keeps every column in IEEE double for good, and
+ * refuses 1.  A batch runs each plan with the setting it had when the batch was
+ * made (the setting cannot change while a batch refers to the plan).  Errors: SHT_ERR_INVALID_ARG (NULL, 1
+ * for an FP64 plan, a plan in a batch), SHT_ERR_UNSUPPORTED.
  *
- * The tensor-core kernel waits on its own matrix products with a bounded number
- * of tries; if a wait gives up it stops, records bit 0 in the plan's device
+ * The tensor-core kernels (of both forms) wait on their own matrix products with a bounded number
+ * of tries; if a wait gives up its CTA stops, records bit 0 in the plan's device
  * status word and leaves its outputs undefined.  sht_plan_device_status
  * synchronises the device, writes the word to *status, clears it and returns
  * SHT_ERR_TIMEOUT if it was set (SHT_OK otherwise).
@@ -353,19 +356,23 @@ SHT_API int sht_plan_device_status(sht_plan_t plan, int *status);
  * the ring pair's phase values times u_p are split into six bf16 digits on a
  * grid per tile and column; the digit products are summed over the tile's pairs
  * in FP32 accumulators where no rounding can occur, and the levels are added in
- * double-float.  Plans of ncomp >= 3 always run it, four spin-0 maps or two E/B
- * pairs at a time, on their one tiling (lmax 2047, four maps 5.0 ms against 10.4 for
- * the double-float analysis, four pairs 18.6 against 41.6).  The setting is of ncomp <= 2 (SHT_ERR_UNSUPPORTED
- * otherwise), with tiles of 128 pairs (the call sets that tiling).  It serves SHT_ANALYSIS and
+ * double-float.  What it loses is relative to a tile's brightest ring (2^-50), where the
+ * double-float sums keep 2^-46 of each term.  Plans of ncomp >= 3 run it from the start, four
+ * spin-0 maps or two E/B pairs at a time, on their one tiling (lmax 2047, four maps 5.0 ms
+ * against 10.4 for the double-float analysis, four pairs 18.6 against 41.6), with items
+ * whose rings range too far in double-float; 0 puts all of their items there for good, 1 is
+ * refused (SHT_ERR_UNSUPPORTED).  For ncomp <= 2 it is a setting, with tiles of 128 pairs (the
+ * call sets that tiling).  An FP64 plan takes 0, as for the synthesis above (at its current
+ * tiling), and refuses 1.  It serves SHT_ANALYSIS and
  * SHT_ADJOINT_SYNTHESIS through sht_execute, sht_execute_noalloc and the stage
  * call, and in a batch made while the plan has it set.  sht_plan_autotune selects it
  * where it is measured faster (GB300, lmax 2047: spin 2 one E/B pair 7.2 ms
  * against 9.1 for the double-float analysis; lmax 4095, spin 0 one map 27.2 against
- * 21.5); sht_plan_set_tensor_core_analysis(plan, 1
- * or 0)
- * sets it, sht_plan_get_tensor_core_analysis reads it.  Its waits are bounded
+ * 21.5); sht_plan_set_tensor_core_analysis(plan, 1 or 0) sets it, and
+ * sht_plan_get_tensor_core_analysis reads whether the plan's analysis contracts on the
+ * tensor cores.  Its waits are bounded
  * like the synthesis kernel's (status word bit 0).  Errors: SHT_ERR_INVALID_ARG
- * (NULL, an FP64 plan, a plan in a batch), SHT_ERR_UNSUPPORTED, and those of
+ * (NULL, 1 for an FP64 plan, a plan in a batch), SHT_ERR_UNSUPPORTED, and those of
  * sht_plan_set_tiling.
  */
 SHT_API int sht_plan_set_tensor_core_analysis(sht_plan_t plan, int on);

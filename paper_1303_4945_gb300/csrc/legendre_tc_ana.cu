@@ -417,7 +417,7 @@ __device__ __forceinline__ bool tc_ana_body(const TcArgs &ta, const int4 item_, 
     }
     __syncthreads();
     if (guard) {
-      wide = !eqok || ta.force;
+      wide = !eqok;
 #pragma unroll
       for (int c = 0; c < NC; ++c)  // (a column that is not finite: below)
         wide = wide || (vmax[c] > 0u && !tca::not_finite(vmax[c]) && !tca::not_finite(eqmax[c]) &&
@@ -815,7 +815,8 @@ __device__ __forceinline__ bool tc_ana_body(const TcArgs &ta, const int4 item_, 
 template <int NJ, bool SPIN>
 __device__ __forceinline__ void tc_ana_item(const TcArgs &ta, const int4 item, const int j0, unsigned char *smem) {
   using S = tca::AnaShape<NJ, SPIN>;
-  if (tc_ana_body<NJ, SPIN>(ta, item, j0, smem)) return;
+  const bool off = S::GROUPED && ta.force;
+  if (!off && tc_ana_body<NJ, SPIN>(ta, item, j0, smem)) return;
   if constexpr (S::GROUPED) {  // the item's tiles of 256 pairs in double-float
     static_assert(sizeof(MixAnaShared) <= S::SMEM, "its table in the digits' shared memory");
     __syncthreads();

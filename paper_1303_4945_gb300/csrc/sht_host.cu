@@ -1531,22 +1531,37 @@ extern "C" int sht_plan_get_fft_precision(sht_plan_t P, int *precision) {
 
 extern "C" int sht_plan_set_tensor_cores(sht_plan_t P, int on) {
   if (!P) return fail(SHT_ERR_INVALID_ARG, "plan is NULL");
-  if (on && P->precision != SHT_MIXED) return fail(SHT_ERR_INVALID_ARG, "FP64 plans have no tensor-core form");
+  if (on && P->precision != SHT_MIXED)
+    return fail(SHT_ERR_INVALID_ARG, "FP64 plans choose their contraction by size when they are made; 0 keeps the IEEE one");
   if (on && !tc_supported(P->spin, P->njobs_pad))
     return fail(SHT_ERR_UNSUPPORTED, "tensor-core synthesis holds at most 32 columns (spin 0: ncomp <= 8, spin: ncomp <= 4)");
   if (P->batch_refs)
     return fail(SHT_ERR_INVALID_ARG, "the plan belongs to %d batch(es); destroy them first", P->batch_refs);
-  P->tc_syn = on ? 1 : 0;
+  if (P->precision == SHT_FP64) P->tc64_syn = 0;
+  else P->tc_syn = on ? 1 : 0;
   return SHT_OK;
 }
 
 extern "C" int sht_plan_set_tensor_core_analysis(sht_plan_t P, int on) {
   if (!P) return fail(SHT_ERR_INVALID_ARG, "plan is NULL");
-  if (on && P->precision != SHT_MIXED) return fail(SHT_ERR_INVALID_ARG, "FP64 plans have no tensor-core form");
+  if (on && P->precision != SHT_MIXED)
+    return fail(SHT_ERR_INVALID_ARG, "FP64 plans choose their contraction by size when they are made; 0 keeps the IEEE one");
   if (on && !tc_ana_supported(P->spin, P->njobs_pad))
-    return fail(SHT_ERR_UNSUPPORTED, "tensor-core analysis holds at most two jobs (ncomp <= 2)");
+    return fail(SHT_ERR_UNSUPPORTED, "the tensor-core analysis is set for ncomp <= 2; plans of more have it from the start, until 0 is set");
   if (P->batch_refs)
     return fail(SHT_ERR_INVALID_ARG, "the plan belongs to %d batch(es); destroy them first", P->batch_refs);
+  if (P->precision == SHT_FP64) {
+    const int old = P->tc64_ana;
+    P->tc64_ana = 0;
+    const int rc = old ? retile(P, P->ana_ppt) : SHT_OK;
+    if (rc == SHT_OK) P->tc64_able = 0;
+    else P->tc64_ana = old;
+    return rc;
+  }
+  if (tc_ana_quad(P)) {
+    P->quad_off = 1;
+    return SHT_OK;
+  }
   if (on && !P->tc_ana) {  // its tiles: one ring pair per thread
     P->tc_ana = 1;
     const int rc = retile(P, 1);
@@ -1564,13 +1579,13 @@ extern "C" int sht_plan_set_tensor_core_analysis(sht_plan_t P, int on) {
 
 extern "C" int sht_plan_get_tensor_core_analysis(sht_plan_t P, int *on) {
   if (!P || !on) return fail(SHT_ERR_INVALID_ARG, "NULL argument");
-  *on = P->tc_ana;
+  *on = P->precision == SHT_FP64 ? P->tc64_ana : (tc_ana_quad(P) ? !P->quad_off : P->tc_ana);
   return SHT_OK;
 }
 
 extern "C" int sht_plan_get_tensor_cores(sht_plan_t P, int *on) {
   if (!P || !on) return fail(SHT_ERR_INVALID_ARG, "NULL argument");
-  *on = P->tc_syn;
+  *on = P->precision == SHT_FP64 ? P->tc64_syn : P->tc_syn;
   return SHT_OK;
 }
 

@@ -258,7 +258,7 @@ class Plan(_Handle):
 
     @property
     def tensor_cores(self):
-        """Mixed plans: True when the synthesis contraction runs on the tensor cores."""
+        """True when the synthesis contraction runs on the tensor cores (FP64 plans take False only)."""
         n = ctypes.c_int()
         _check(_lib.sht_plan_get_tensor_cores(self._h, ctypes.byref(n)), "sht_plan_get_tensor_cores")
         return bool(n.value)
@@ -269,7 +269,8 @@ class Plan(_Handle):
 
     @property
     def tensor_core_analysis(self):
-        """Mixed plans: True when the analysis contraction runs on the tensor cores."""
+        """True when the analysis contraction runs on the tensor cores (FP64 plans and mixed ones
+        of ncomp >= 3 take False only)."""
         n = ctypes.c_int()
         _check(_lib.sht_plan_get_tensor_core_analysis(self._h, ctypes.byref(n)), "sht_plan_get_tensor_core_analysis")
         return bool(n.value)

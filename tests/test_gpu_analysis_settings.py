@@ -102,3 +102,63 @@ def test_a_refused_tiling_changes_nothing(sht):
     m = [torch.zeros(plan.geom.npix, dtype=torch.float64, device="cuda")]
     a = [torch.zeros(plan.alm.size(), dtype=torch.complex128, device="cuda")]
     sht.sht_execute_noalloc(plan, sht.SHT_ANALYSIS, a, m)
+
+
+def analysis(sht, plan, maps):
+    out = [torch.full((plan.alm.size(),), complex(float("nan")), dtype=torch.complex128, device="cuda") for _ in maps]
+    sht.sht_execute(plan, sht.SHT_ANALYSIS, out, maps)
+    assert plan.device_status() == 0
+    return out
+
+
+def close(x, y, tol):
+    return float(torch.linalg.vector_norm(x - y)) <= tol * float(torch.linalg.vector_norm(y))
+
+
+# three or more jobs: one and several tiles of 256 pairs, padded jobs, several groups
+@pytest.mark.parametrize("spin,ncomp,nlat", [(0, 3, 31), (0, 16, 300), (2, 3, 520), (-1, 8, 300)])
+def test_double_float_on_request(sht, spin, ncomp, nlat):
+    """Plans of more than two jobs contract their analysis on the tensor cores and say so;
+    0 takes every item to double-float."""
+    geom, lay = sht.sht_geom_gauss(nlat, 64), sht.sht_alm_create(299, 299)
+    plan, ref = (sht.sht_plan_create(geom, lay, spin, ncomp, sht.SHT_MIXED) for _ in range(2))
+    g = torch.Generator(device="cuda").manual_seed(nlat)
+    maps = [torch.randn(geom.npix, dtype=torch.float64, device="cuda", generator=g) for _ in range(plan.narrays)]
+    assert plan.tensor_core_analysis
+    a = analysis(sht, plan, maps)
+    plan.tensor_core_analysis = False
+    assert not plan.tensor_core_analysis and ref.tensor_core_analysis
+    b = analysis(sht, plan, maps)
+    assert any(not torch.equal(x, y) for x, y in zip(a, b))
+    assert all(close(x, y, 1e-10) for x, y in zip(a, b))
+    with pytest.raises(sht.ShtError):
+        plan.tensor_core_analysis = True
+
+
+@pytest.mark.parametrize("spin,ncomp", [(0, 1), (0, 2), (2, 1)])
+def test_ieee_on_request(sht, spin, ncomp):
+    """An FP64 plan says which contraction it has; 0 keeps the IEEE one, for both directions."""
+    plan = make(sht, 300, 302, spin, ncomp, sht.SHT_FP64)
+    small = make(sht, 20, 22, spin, ncomp, sht.SHT_FP64)
+    assert plan.tensor_cores and plan.tensor_core_analysis
+    assert not small.tensor_cores and not small.tensor_core_analysis
+    g = torch.Generator(device="cuda").manual_seed(spin)
+    alm = [torch.randn(plan.alm.size(), dtype=torch.complex128, device="cuda", generator=g) for _ in range(plan.narrays)]
+    maps = [[torch.empty(plan.geom.npix, dtype=torch.float64, device="cuda") for _ in alm] for _ in range(2)]
+    sht.sht_execute(plan, sht.SHT_SYNTHESIS, alm, maps[0])
+    a = analysis(sht, plan, maps[0])
+    plan.tensor_cores = False
+    plan.tensor_core_analysis = False
+    assert not plan.tensor_cores and not plan.tensor_core_analysis
+    sht.sht_execute(plan, sht.SHT_SYNTHESIS, alm, maps[1])
+    b = analysis(sht, plan, maps[0])
+    for x, y in zip(maps[0] + a, maps[1] + b):
+        assert not torch.equal(x, y) and close(x, y, 1e-12)
+    plan.set_tiling(plan.tiling()[1][1])  # (for good: no tiling and no timing returns to the tensor cores)
+    plan.set_tiling(plan.tiling()[1][0])
+    plan.autotune(torch.cuda.current_stream())
+    assert not plan.tensor_core_analysis
+    for on in ("tensor_cores", "tensor_core_analysis"):
+        with pytest.raises(sht.ShtError) as e:
+            setattr(plan, on, True)
+        assert e.value.code == sht.SHT_ERR_INVALID_ARG
