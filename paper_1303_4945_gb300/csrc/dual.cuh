@@ -45,43 +45,77 @@ __device__ __forceinline__ d2 mul_sub(const d2 &u, const d2 &p, const d2 &q) {
 // two-sum); kCareful: any order; kPolar: the difference form of a polar warp.
 enum StepMode { kFast, kCareful, kPolar };
 
+// step_polar of mixed_common.cuh in both lanes, every lane rounded as there (spin s: one
+// ring, +b and -b; spin 0: two rings)
+struct DualState {
+  d2 p, q;
+};
+template <bool SPIN>
+__device__ __forceinline__ DualState dual_polar_step(float4 c, f3 y0, f3 y1, d2 p, d2 q) {
+  const f2 a = {c.x, c.y}, b = {c.z, c.w};
+  auto lane_of = [&](const f3 &y) {  // (a - 2) - a y as a pair (spin s: the same for both lanes)
+    const float m = __fmul_rn(a.h, y.h);
+    float e = __fmaf_rn(a.h, y.h, -m);
+    e = __fmaf_rn(a.h, y.m, e);
+    e = __fmaf_rn(a.l, y.h, e);
+    const f2 t = two_sum(__fsub_rn(a.h, 2.0f), -m);
+    return f2{t.h, __fadd_rn(__fsub_rn(a.l, e), t.l)};
+  };
+  const f2 t0 = lane_of(y0), t1 = SPIN ? t0 : lane_of(y1);
+  d2 v = {make_float2(t0.h, t1.h), make_float2(t0.l, t1.l)};
+  if (SPIN) {
+    const d2 t = two_sum(v.h, make_float2(b.h, -b.h));
+    v = {t.h, add2(add2(v.l, t.l), make_float2(b.l, -b.l))};
+  }
+  v = fast_two_sum(v.h, v.l);
+  const float2 m = mul2(v.h, p.h);
+  float2 e;
+  e.x = __fmaf_rn(v.l.x, p.h.x, __fmaf_rn(v.h.x, p.l.x, __fmaf_rn(v.h.x, p.h.x, -m.x)));
+  e.y = __fmaf_rn(v.l.y, p.h.y, __fmaf_rn(v.h.y, p.l.y, __fmaf_rn(v.h.y, p.h.y, -m.y)));
+  const d2 s = two_sum(m, q.h);
+  q = fast_two_sum(s.h, add2(add2(e, q.l), s.l));
+  const d2 r = two_sum(p.h, q.h);
+  p = fast_two_sum(r.h, add2(add2(p.l, q.l), r.l));
+  return {p, q};
+}
+template <bool SPIN>
+static __device__ __noinline__ DualState dual_polar_step_out(float4 c, f3 y0, f3 y1, d2 p, d2 q) {
+  return dual_polar_step<SPIN>(c, y0, y1, p, q);
+}
+
 // The recursions of one thread.  SPIN: lane 0 runs lambda(+s), lane 1 (-1)^(l - l0)
 // lambda(-s), whose recursion is p_{l+1} = (b - a x) p_l - p_{l-1}: the sign the spin
 // columns need (in a polar warp lane 1 runs lambda(-s) itself, and d2 q holds the
 // differences).  Spin 0: lane t runs ring pair t.  x: cos theta, or 1 - cos theta
 // in a polar warp.
-template <bool SPIN>
+//
+// PS: a polar warp's step.  Packed in both lanes, in line; called, where unrolled into a
+// kernel's degrees it takes registers and instruction cache from the warps that never run
+// it (tensor-core synthesis of two E/B pairs, lmax 127 on 257 Clenshaw-Curtis rings: scalar 66
+// us, packed 57, called 53; the analysis of one at lmax 2047: 7.20 ms, 7.11, 7.20); or two
+// scalar steps, where the registers are held to 80 (double-float analysis of one map, lmax
+// 2047: 3.03 ms, packed 3.09, called 3.11).
+enum PolarStep { kScalar, kPacked, kCalled };
+template <bool SPIN, PolarStep PS>
 struct Dual {
   d2 p, q;  // current and previous values
   f3 x[SPIN ? 1 : 2];
 
   __device__ __forceinline__ void step(StepMode mode, const float4 &c) {
     const f2 a = {c.x, c.y}, b = {c.z, c.w};
-    if (mode == kPolar) {  // step_polar of both lanes, every lane rounded as there
+    if (mode == kPolar) {
       const f3 &y0 = x[0], &y1 = x[SPIN ? 0 : 1];
-      auto lane_of = [&](const f3 &y) {  // (a - 2) - a y as a pair (spin s: the same for both lanes)
-        const float m = __fmul_rn(a.h, y.h);
-        float e = __fmaf_rn(a.h, y.h, -m);
-        e = __fmaf_rn(a.h, y.m, e);
-        e = __fmaf_rn(a.l, y.h, e);
-        const f2 t = two_sum(__fsub_rn(a.h, 2.0f), -m);
-        return f2{t.h, __fadd_rn(__fsub_rn(a.l, e), t.l)};
-      };
-      const f2 t0 = lane_of(y0), t1 = SPIN ? t0 : lane_of(y1);
-      d2 v = {make_float2(t0.h, t1.h), make_float2(t0.l, t1.l)};
-      if (SPIN) {
-        const d2 t = two_sum(v.h, make_float2(b.h, -b.h));
-        v = {t.h, add2(add2(v.l, t.l), make_float2(b.l, -b.l))};
+      if (PS == kScalar) {
+        f2 p0 = lane0(p), q0 = lane0(q), p1 = lane1(p), q1 = lane1(q);
+        step_polar(a, b, y0, p0, q0);
+        step_polar(a, neg(b), y1, p1, q1);
+        p = {make_float2(p0.h, p1.h), make_float2(p0.l, p1.l)};
+        q = {make_float2(q0.h, q1.h), make_float2(q0.l, q1.l)};
+      } else {
+        const DualState n = PS == kCalled ? dual_polar_step_out<SPIN>(c, y0, y1, p, q) : dual_polar_step<SPIN>(c, y0, y1, p, q);
+        p = n.p;
+        q = n.q;
       }
-      v = fast_two_sum(v.h, v.l);
-      const float2 m = mul2(v.h, p.h);
-      float2 e;
-      e.x = __fmaf_rn(v.l.x, p.h.x, __fmaf_rn(v.h.x, p.l.x, __fmaf_rn(v.h.x, p.h.x, -m.x)));
-      e.y = __fmaf_rn(v.l.y, p.h.y, __fmaf_rn(v.h.y, p.l.y, __fmaf_rn(v.h.y, p.h.y, -m.y)));
-      const d2 s = two_sum(m, q.h);
-      q = fast_two_sum(s.h, add2(add2(e, q.l), s.l));
-      const d2 r = two_sum(p.h, q.h);
-      p = fast_two_sum(r.h, add2(add2(p.l, q.l), r.l));
       return;
     }
     d2 u;

@@ -372,7 +372,7 @@ __device__ __forceinline__ void mix_ana_pair_body(const MixArgs &a, const int4 i
 #pragma unroll 1
   for (int gi = 0; gi < ng; ++gi) {
     const int tile = item.y + gi;
-    Dual<false> rec;
+    Dual<false, kScalar> rec;
     rec.p = rec.q = d2{both(0.f), both(0.f)};
     int sc[NP] = {0, 0}, lj[NP];
     // G_N + G_S and G_N - G_S of each pair: high and low words, (re, im) as lanes

@@ -330,7 +330,7 @@ __device__ __forceinline__ void tc_syn_body(const TcArgs &ta, const int2 item, u
     near = near || near_pole(xd[t], valid[t]);
   }
   const bool polar = __any_sync(0xffffffffu, near);
-  Dual<!S::DUAL> rec;
+  Dual<!S::DUAL, S::DUAL ? kPacked : kCalled> rec;
   rec.p = rec.q = d2{both(0.f), both(0.f)};
 #pragma unroll
   for (int t = 0; t < NP; ++t) rec.x[t] = node_of(xd[t], polar);

@@ -328,7 +328,7 @@ __device__ __forceinline__ bool tc_ana_body(const TcArgs &ta, const int4 item_, 
       }
       if (lane == 0) {
         const float low = SPIN ? fminf(fabsf(r.lpc.h), fabsf(r.lmc.h)) : fabsf(r.lpc.h);
-        eqok = r.lj == l0 && r.scp == 0 && (!SPIN || r.scm == 0) && low >= ldexpf(1.f, r.lexp - 6);
+        eqok = !ta.force && r.lj == l0 && r.scp == 0 && (!SPIN || r.scm == 0) && low >= ldexpf(1.f, r.lexp - 6);
       }
 #pragma unroll
       for (int c = 0; c < NC; ++c) {
@@ -462,7 +462,7 @@ __device__ __forceinline__ bool tc_ana_body(const TcArgs &ta, const int4 item_, 
 
     // the walk over the tile's blocks of 8 degrees (from its pairs' earliest join):
     // the recursions run on Lambda / u_p
-    Dual<SPIN> rec;
+    Dual<SPIN, kPacked> rec;
     rec.p = rec.q = d2{both(0.f), both(0.f)};
     int sc0 = 0, sc1 = 0;
     double xd[NP];
@@ -815,8 +815,7 @@ __device__ __forceinline__ bool tc_ana_body(const TcArgs &ta, const int4 item_, 
 template <int NJ, bool SPIN>
 __device__ __forceinline__ void tc_ana_item(const TcArgs &ta, const int4 item, const int j0, unsigned char *smem) {
   using S = tca::AnaShape<NJ, SPIN>;
-  const bool off = S::GROUPED && ta.force;
-  if (!off && tc_ana_body<NJ, SPIN>(ta, item, j0, smem)) return;
+  if (tc_ana_body<NJ, SPIN>(ta, item, j0, smem)) return;
   if constexpr (S::GROUPED) {  // the item's tiles of 256 pairs in double-float
     static_assert(sizeof(MixAnaShared) <= S::SMEM, "its table in the digits' shared memory");
     __syncthreads();
