@@ -206,12 +206,12 @@ int build(sht_batch_s *B) {
     const sht_plan_s *P = B->plans[k];
     FftGroup *g = nullptr;
     for (auto &c : B->fft)
-      if (c.df == P->fft_df && c.threads == P->fft_threads) g = &c;
+      if (c.df == P->fft_df && c.threads == P->fft_batch_threads) g = &c;
     if (!g) {
       B->fft.emplace_back();
       g = &B->fft.back();
       g->df = P->fft_df;
-      g->threads = P->fft_threads;
+      g->threads = P->fft_batch_threads;
     }
     g->smem = std::max(g->smem, P->fft_smem);
     for (int p = 0; p < P->npairs; ++p)

@@ -776,9 +776,15 @@ __global__ void __launch_bounds__(kFftThreads) fft_ana_kernel_global(FftArgs a, 
 // points (Rader 613) 133 / 114 / 88; 1024 FP64 384 / 308 / 295; 2047 FP64 881 / 764 / 769; 2048
 // (HEALPix Nside 512) 667 / 581 / 690; 4095, eight maps 4306 / 3655 / 3967; 6006 1027 / 1004 /
 // 1479.
-int fft_cta_threads(int len) {
-  if (len <= 1024) return kFftThreads / 4;
-  return 2 * (len * (int)sizeof(double2) + 2048) <= 227 * 1024 ? kFftThreads / 2 : kFftThreads;
+// Where a call has too few rings for that (rings: its ring pairs times maps, per SM) a ring
+// takes the threads itself.  At most one per SM (us, mixed form, 512 / 256 / 128 threads): 96
+// points 30 / 29 / 27; 512 32 / 30 / 35; 613 56 / 60 / 80; 1000 41 / 42 / 53; 2048 51 / 59 / 84;
+// 4095 84 / 110 / 160.  Two: 96 points 47 / 31 / 29; 512 53 / 36 / 38; 1000 68 / 49 / 59.
+int fft_cta_threads(int len, double rings) {
+  const int t = len <= 1024 ? kFftThreads / 4 : (2 * (len * (int)sizeof(double2) + 2048) <= 227 * 1024 ? kFftThreads / 2 : kFftThreads);
+  if (rings > 2.0 || len <= 128) return t;
+  if (rings <= 1.0) return len <= 600 ? kFftThreads / 2 : kFftThreads;
+  return std::max(t, kFftThreads / 2);
 }
 
 static FftArgs make_fft_args(const sht_plan_s *P, const DevPtrs &map, int polar) {

@@ -1345,7 +1345,8 @@ static int plan_build(sht_plan_s *P, const sht_geom_s *g) {
   if ((rc = upload(P, pf, &P->d_pair_fft)) != SHT_OK) return rc;
   if (maxlen <= kFftMaxLen) {
     P->fft_smem = maxlen * (int)sizeof(double2);
-    P->fft_threads = fft_cta_threads(maxlen);
+    P->fft_threads = fft_cta_threads(maxlen, (double)P->npairs * P->nmaps / P->sms);
+    P->fft_batch_threads = fft_cta_threads(maxlen, 1e9);  // (with the other plans' rings)
   } else {  // rings beyond shared memory: one L2-resident scratch slot per SM (one CTA each)
     int sms = 0;
     CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, P->device));

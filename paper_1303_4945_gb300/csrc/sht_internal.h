@@ -222,7 +222,7 @@ struct sht_plan_s {
   int nfft = 0;
   int *d_pair_fft = nullptr;  // per pair: plan index
   int fft_smem = 0;           // bytes of dynamic shared memory for the FFT kernels
-  int fft_threads = sht::kFftThreads;  // their CTA size (fft_cta_threads)
+  int fft_threads = sht::kFftThreads, fft_batch_threads = sht::kFftThreads;  // their CTA size (fft_cta_threads): own calls, batches
   std::vector<int> pair_len;  // per pair: the longer ring length (FFT cost)
   double2 *d_fft_scratch = nullptr;  // rings beyond kFftMaxLen: one slot of fft_slot_len points per CTA
   int fft_slots = 0, fft_slot_len = 0;
@@ -328,7 +328,7 @@ cudaError_t launch_fft_syn(const sht_plan_s *P, const DevPtrs &map, int polar, i
 cudaError_t launch_fft_ana(const sht_plan_s *P, const DevPtrs &map, int weighted, cudaStream_t st, int p0 = 0,
                            int p1 = -1);
 // threads per CTA for rings of up to len points (at most kFftMaxLen)
-int fft_cta_threads(int len);
+int fft_cta_threads(int len, double rings);
 // lets every FFT kernel use the device's opt-in shared memory (once per device, at plan time:
 // the limit is one value per kernel and process, so it is only ever raised, never per call)
 cudaError_t fft_prepare_device(int device);
