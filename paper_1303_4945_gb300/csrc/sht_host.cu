@@ -1162,9 +1162,16 @@ static int build_ana_lists(sht_plan_s *P, int ppt) {
 // 1194; two 127 70 -> 74, 191 114 -> 108, 767 2250 -> 1080; four 31 41 -> 39, 63 41 -> 37,
 // 767 3569 -> 1324; analysis, one 191 117 -> 119, 255 164 -> 158, 1023 2350 -> 1560; two
 // 31 36 -> 30, 767 3826 -> 1228; four 31 53 -> 31, 767 6277 -> 1506.
+// One array's synthesis needs a warp of ring pairs per SM quarter too: with fewer (few rings
+// or few m) a CTA's own chain of degrees is what counts, and the IEEE one is shorter (lmax
+// 1023, 300 rings, 41 m, whole call 243 us against 280; lmax 255, 40 rings, all m 129, 142).
 static void tc64_choose(sht_plan_s *P) {
   const int n = P->nmaps_pad;  // arrays per side
-  P->tc64_syn = tc64_syn_supported(P->spin, P->njobs_pad) && P->lmax >= (n == 1 ? 224 : (n == 2 ? 192 : 48));
+  int64_t warps = 0;
+  for (int i = 0; i < P->nm; ++i)
+    if (P->lmax >= std::max(P->mval[i], abs(P->spin))) warps += (P->npairs + 31) / 32;
+  P->tc64_syn = tc64_syn_supported(P->spin, P->njobs_pad) && P->lmax >= (n == 1 ? 224 : (n == 2 ? 192 : 48)) &&
+                (n > 1 || warps >= 4 * P->sms);
   P->tc64_ana = P->tc64_able = tc64_ana_supported(P->spin, P->njobs_pad) && P->lmax >= (n == 1 ? 208 : 24);
 }
 

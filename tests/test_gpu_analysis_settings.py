@@ -162,3 +162,20 @@ def test_ieee_on_request(sht, spin, ncomp):
         with pytest.raises(sht.ShtError) as e:
             setattr(plan, on, True)
         assert e.value.code == sht.SHT_ERR_INVALID_ARG
+
+
+def test_fp64_synthesis_of_few_columns_or_rings(sht):
+    """One array's synthesis goes to the tensor cores where its columns' warps of ring pairs
+    reach one per SM quarter; results are the IEEE sums' either way."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    for lmax, nlat, mmax, on in ((255, 256, 255, 1024 >= 4 * sms), (255, 40, 255, 256 >= 4 * sms), (1023, 300, 40, 205 >= 4 * sms), (1023, 300, 1023, 5120 >= 4 * sms)):
+        geom = sht.sht_geom_gauss(nlat, 2 * mmax + 2)
+        plan = sht.sht_plan_create(geom, sht.sht_alm_create(lmax, mmax), 0, 1, sht.SHT_FP64)
+        assert plan.tensor_cores == on
+        g = torch.Generator(device="cuda").manual_seed(nlat)
+        alm = [torch.randn(plan.alm.size(), dtype=torch.complex128, device="cuda", generator=g)]
+        maps = [torch.empty(geom.npix, dtype=torch.float64, device="cuda") for _ in range(2)]
+        sht.sht_execute(plan, sht.SHT_SYNTHESIS, alm, maps[:1])
+        plan.tensor_cores = False
+        sht.sht_execute(plan, sht.SHT_SYNTHESIS, alm, maps[1:])
+        assert close(maps[0], maps[1], 1e-12)
