@@ -19,15 +19,32 @@ struct LegArgs {
   const int4 *ana_items;
   const int64_t *part_off;
   double *part;
-  // tensor-core form (legendre_tc64.cu): 2^lexp bounds |p_l| of (m index, pair); geo[m index]:
-  // the equator-most ring reaches that from the first degree on
+  // tensor-core form (legendre_tc64.cu): 2^lexp bounds |p_l| of (m index, pair); ref[m index]:
+  // the pair whose value at the first degree is nearest to its bound (RefPair)
   const signed char *lexp;
-  const unsigned char *geo;
+  const unsigned long long *ref;
   // per m index, a byte per job: the columns of a synthesis that its fixed-point operands
   // do not hold to an IEEE sum's accuracy
   const unsigned *wide_syn;
   int *err;  // device status word (bounded waits)
 };
+
+// An m's reference pair, as one number that orders: from the top 1 for the pair next to the
+// equator where all its values at the first degree lie within 2^-kRefNear of the bound (the
+// equator serves then), the exponent of the largest value over the bound plus 2^16, the
+// pair, and a bit for each value (+s, -s) that near to the bound.
+constexpr int kRefNear = 6;
+__device__ __forceinline__ unsigned long long ref_key(bool equator, int exponent, int pair, int lanes) {
+  return ((unsigned long long)(equator ? 1u : 0u) << 63) | ((unsigned long long)(unsigned)(max(exponent, -60000) + 65536) << 36) |
+         ((unsigned long long)(unsigned)pair << 2) | (unsigned)lanes;
+}
+struct RefPair {
+  int pair, lanes;
+  bool near;  // no pair is near its bound where not
+};
+__device__ __forceinline__ RefPair ref_of(unsigned long long k) {
+  return {(int)((k >> 2) & 0x3ffffffffull), (int)(k & 3u), (int)((k >> 36) & 0x7ffffffu) - 65536 >= -kRefNear};
+}
 
 // The tensor-core form rounds a column's inputs to 2^-54 of the largest and Lambda to 2^-56
 // of its bound, so what a term loses is relative to the largest of its column.  kWideRange

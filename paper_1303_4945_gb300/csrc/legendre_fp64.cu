@@ -147,8 +147,9 @@ __global__ void ana_reduce(int lmax, int spin, int nm, int njobs_pad, int ncomp,
 // column's values range too far for it.  On a ring where only the degrees from some l on
 // have Lambda near its bound (below, it falls away exponentially) the result comes from
 // those alone, so of every four neighbouring degrees, and of the last two, one has to lie
-// within 2^kWideRange of the largest of the column.  Spectra like 1/(l + 1) do from m = 8
-// on; a column of zeros does; a band limit below lmax or an infinity does not.
+// within 2^kWideRange of the largest of the column.  Spectra like 1/(l + 1) do (lmax 1023: a
+// factor of some 2^10 in a column, and 2^2 to 2^3 of chance); a column of zeros does; a band
+// limit below lmax or an infinity does not.
 constexpr int kPmThreads = 256;
 __global__ void __launch_bounds__(kPmThreads)
     alm_to_pm(int lmax, int spin, int nm, int astride, const int *__restrict__ mval, const int64_t *__restrict__ mstart,
@@ -249,7 +250,7 @@ static LegArgs make_args(const sht_plan_s *P, int polar, bool lo = false) {
   a.part_off = P->d_ana_part_off[polar];
   a.part = P->d_part;
   a.lexp = P->d_lexp;
-  a.geo = P->d_geo;
+  a.ref = P->d_ref;
   a.wide_syn = P->d_wide_syn;
   a.err = P->d_err;
   return a;

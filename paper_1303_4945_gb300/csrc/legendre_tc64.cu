@@ -17,10 +17,12 @@
 //  * The other operand (a_lm per column and 256-degree window; G_m times u_p per column
 //    and tile) is scaled by a power of two of its largest value (in FP64, so the full
 //    exponent range passes) and cut the same way.
-//  * Products of digits i and j belong to level i + j.  The levels 0 to 3 are exact (at
-//    most 2^23 units a product sum of 512 entries, each level's sums added in pairs of
-//    at most 2^24 or by exact two-sums), levels 4 to 6 (2^-32 and below) are added in
-//    FP32, rounding below 2^-56 of the bound; higher levels are dropped.  The sums are
+//  * Products of digits i and j belong to level i + j.  The levels 0 to 2 are exact whatever
+//    the digits (sums of at most 2^24 units over 512 entries), and level 3 but for inputs
+//    whose digits are all near their ends at once (the synthesis sums its four products in
+//    one accumulator, 1.5 2^24 units at worst; beyond 2^24 its last bit, 2^-38 of sums above
+//    2^-14); levels 4 to 6 (2^-32 and below) are added in FP32, rounding below 2^-56 of the
+//    bound; higher levels are dropped.  Level sums meet in exact two-sums and are
 //    added up in FP64.
 //
 // An IEEE sum loses 2^-53 of each term, these operands 2^-54 of the largest input of a
@@ -284,7 +286,7 @@ struct AnaShape64 {
 // ---------------------------------------------------------------------------
 constexpr int kBoundPairs = 8;
 template <bool SPIN>
-__global__ void __launch_bounds__(128) bound_kernel(LegArgs a, signed char *__restrict__ out, unsigned char *__restrict__ geo) {
+__global__ void __launch_bounds__(128) bound_kernel(LegArgs a, signed char *__restrict__ out, unsigned long long *__restrict__ ref) {
   const int mi = blockIdx.y, pb = blockIdx.x * 128 * kBoundPairs + threadIdx.x;
   if (pb >= a.npairs) return;
   const int m = a.mval[mi];
@@ -292,9 +294,12 @@ __global__ void __launch_bounds__(128) bound_kernel(LegArgs a, signed char *__re
   const int l0 = m > as ? m : as, lmax = a.lmax;
   const double2 *__restrict__ cf = a.coef + (a.coef_off[mi] - l0);
   float vmax[kBoundPairs];
-  int elow = 4096;  // of the equator-most pair: the exponent of the smaller start value
+  int e0[kBoundPairs], e1[kBoundPairs];  // the exponents of the values at the first degree
 #pragma unroll
-  for (int k = 0; k < kBoundPairs; ++k) vmax[k] = 0.f;
+  for (int k = 0; k < kBoundPairs; ++k) {
+    vmax[k] = 0.f;
+    e1[k] = -70000;
+  }
 #pragma unroll 1
   for (int t = 0; t < (SPIN ? 2 : 1); ++t) {
     float p[kBoundPairs], d[kBoundPairs], y[kBoundPairs], w[kBoundPairs];  // values p 2^(64 sc), w their weight
@@ -312,7 +317,7 @@ __global__ void __launch_bounds__(128) bound_kernel(LegArgs a, signed char *__re
         sc[k] = (e + 32) >= 0 ? (e + 32) / 64 : -((-(e + 32) + 63) / 64);
         p[k] = (float)ldexp(mant, e - 64 * sc[k]);
       }
-      if (pb + 128 * k == a.npairs - 1) elow = min(elow, mant != 0.0 ? ilogb(mant) + e : -4096);
+      (t ? e1[k] : e0[k]) = mant != 0.0 ? ilogb(mant) + e : -70000;
       d[k] = p[k];
       w[k] = sc[k] == 0 ? 1.f : (sc[k] == -1 ? 0x1p-64f : 0.f);
     }
@@ -335,6 +340,7 @@ __global__ void __launch_bounds__(128) bound_kernel(LegArgs a, signed char *__re
 #pragma unroll
     for (int k = 0; k < kBoundPairs; ++k) vmax[k] = fmaxf(vmax[k], fabsf(p[k]) * w[k]);
   }
+  unsigned long long best = 0;
 #pragma unroll
   for (int k = 0; k < kBoundPairs; ++k) {
     if (pb + 128 * k >= a.npairs) break;
@@ -345,9 +351,12 @@ __global__ void __launch_bounds__(128) bound_kernel(LegArgs a, signed char *__re
       e = max(e, min(ev, 100));
     }
     out[(size_t)mi * a.npairs + pb + 128 * k] = (signed char)e;
-    // every degree's sum has terms of about its largest bound if this pair starts near it
-    if (pb + 128 * k == a.npairs - 1) geo[mi] = elow >= e - 6;
+    const int d0 = e0[k] - e, d1 = SPIN ? e1[k] - e : d0, lanes = (d0 >= -kRefNear ? 1 : 0) | (d1 >= -kRefNear ? 2 : 0);
+    const int p = pb + 128 * k;
+    const unsigned long long key = ref_key(p == a.npairs - 1 && lanes == 3, max(d0, d1), p, lanes);
+    best = key > best ? key : best;
   }
+  atomicMax(ref + mi, best);
 }
 
 // ---------------------------------------------------------------------------
@@ -723,23 +732,26 @@ __device__ __forceinline__ bool tc64_ana_body(const LegArgs &a, const int4 item,
   };
   // The size of column c's largest entry in gv, |G u_p|, as an exponent field (scaled by
   // 2^200, so that u_p keeps it positive; infinities and NaN: 4000)
-  auto size_of = [&](const double (&gv)[2][NC], const int (&lexp)[NP], int c) __attribute__((always_inline)) {
+  auto size_of = [&](const double (&gv)[2][NC], const int (&lexp)[NP], int c, int lanes) __attribute__((always_inline)) {
     int mx = 0;
 #pragma unroll
     for (int t = 0; t < 2; ++t) {
       const int e = size_field(gv[t][c]);
-      if (e > 0) mx = max(mx, e == 2047 ? 4000 : e + 200 + lexp[SPIN ? 0 : t]);
+      if (e > 0 && (lanes >> t & 1)) mx = max(mx, e == 2047 ? 4000 : e + 200 + lexp[SPIN ? 0 : t]);
     }
     return mx;
   };
 
-  // Whether the item's values range too far for fixed point (it then returns false): at degree l
-  // the sum comes from the pairs between some latitude and the equator, below l0's from the
-  // ones next to it, and the others' Lambda falls away exponentially; so no pair's |G u_p|
-  // may exceed 2^kWideRange times the largest of the 32 next to the equator (columns of
-  // zeros there are zero).  One warp finds those; each pass compares its own.
+  // Whether the item's values range too far for fixed point (it then returns false): at every
+  // degree the sum comes from the pairs between two latitudes, which close in on the
+  // reference pair towards the first degree (next to the equator, but for m about |s| > 5),
+  // and the others' Lambda falls away exponentially; so no pair's |G u_p| may exceed
+  // 2^kWideRange times the largest of the 32 about that pair (of the values +s, -s that are
+  // near their bound there; columns of zeros there are zero).  One warp finds those; each
+  // pass compares its own.
   if (warp == 0) {
-    const int p = a.npairs - 1 - lane;
+    const RefPair rp = ref_of(a.ref[mi]);
+    const int p = max(min(rp.pair + 15, a.npairs - 1) - lane, -1);
     int mx[NC];
     {
       double gv[2][NC];
@@ -752,7 +764,7 @@ __device__ __forceinline__ bool tc64_ana_body(const LegArgs &a, const int4 item,
       for (int t = 0; t < NP; ++t) lexp[t] = p >= 0 ? a.lexp[(size_t)mi * a.npairs + p] : 0;
       if (p >= 0) load_pair(p, 0, gv);
 #pragma unroll
-      for (int c = 0; c < NC; ++c) mx[c] = size_of(gv, lexp, c);
+      for (int c = 0; c < NC; ++c) mx[c] = size_of(gv, lexp, c, SPIN ? rp.lanes : 3);
     }
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
@@ -812,7 +824,7 @@ __device__ __forceinline__ bool tc64_ana_body(const LegArgs &a, const int4 item,
     __syncthreads();
 #pragma unroll
     for (int c = 0; c < NC; ++c) {  // column bounds over the tile
-      const int mx = __reduce_max_sync(0xffffffffu, size_of(gv, lexp, c));
+      const int mx = __reduce_max_sync(0xffffffffu, size_of(gv, lexp, c, 3));
       if (lane == 0) atomicMax(&vmax[c], mx);
     }
     __syncthreads();
@@ -1034,7 +1046,7 @@ __device__ __forceinline__ void tc64_syn_item(const LegArgs &a, const int2 item,
 }
 template <int NJ, bool SPIN>
 __device__ __forceinline__ void tc64_ana_item(const LegArgs &a, const int4 item, unsigned char *smem) {
-  if (a.geo[item.x] && tc64_ana_body<NJ, SPIN>(a, item, smem)) return;
+  if (ref_of(a.ref[item.x]).near && tc64_ana_body<NJ, SPIN>(a, item, smem)) return;
   __syncthreads();
   double (*const red)[32] = reinterpret_cast<double (*)[32]>(smem);
 #pragma unroll 1
@@ -1182,8 +1194,8 @@ cudaError_t launch_bounds64(const sht_plan_s *P, cudaStream_t st) {
   LegArgs a;
   leg_fp64_fill_args(P, 1, &a);
   const dim3 grid((P->npairs + 128 * kBoundPairs - 1) / (128 * kBoundPairs), P->nm);
-  if (P->spin) bound_kernel<true><<<grid, 128, 0, st>>>(a, P->d_lexp, P->d_geo);
-  else bound_kernel<false><<<grid, 128, 0, st>>>(a, P->d_lexp, P->d_geo);
+  if (P->spin) bound_kernel<true><<<grid, 128, 0, st>>>(a, P->d_lexp, P->d_ref);
+  else bound_kernel<false><<<grid, 128, 0, st>>>(a, P->d_lexp, P->d_ref);
   return cudaGetLastError();
 }
 

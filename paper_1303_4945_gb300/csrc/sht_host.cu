@@ -841,7 +841,7 @@ static void free_plan(sht_plan_s *P) {
   cudaGetDevice(&cur);
   cudaSetDevice(P->device);
   void *ptrs[] = {P->d_pairs, P->d_pair_rings, P->d_rings, P->d_mval, P->d_mstart, P->d_coef_off,
-                  P->d_coef, P->d_alpha, P->d_lexp, P->d_geo, P->d_wide_syn, P->d_coef32, P->d_alm32, P->d_pm64, P->d_mpre, P->d_minv, P->d_phase, P->d_part, P->d_fft,
+                  P->d_coef, P->d_alpha, P->d_lexp, P->d_ref, P->d_wide_syn, P->d_coef32, P->d_alm32, P->d_pm64, P->d_mpre, P->d_minv, P->d_phase, P->d_part, P->d_fft,
                   P->d_pair_fft, P->d_fft_scratch, P->d_err, P->d_join};
   for (void *p : ptrs)
     if (p) cudaFree(p);
@@ -1277,10 +1277,11 @@ static int plan_build(sht_plan_s *P, const sht_geom_s *g) {
       CUDA_TRY(tc64_prepare_device());
       const size_t bytes = (size_t)P->nm * P->npairs;
       CUDA_TRY(cudaMalloc(&P->d_lexp, bytes));
-      CUDA_TRY(cudaMalloc(&P->d_geo, P->nm));
+      CUDA_TRY(cudaMalloc(&P->d_ref, P->nm * sizeof(unsigned long long)));
+      CUDA_TRY(cudaMemset(P->d_ref, 0, P->nm * sizeof(unsigned long long)));
       CUDA_TRY(cudaMalloc(&P->d_wide_syn, P->nm * sizeof(unsigned)));
       CUDA_TRY(cudaMemset(P->d_wide_syn, 0, P->nm * sizeof(unsigned)));  // (the bytes of jobs it has not)
-      P->workspace += bytes + P->nm * (1 + sizeof(unsigned));
+      P->workspace += bytes + P->nm * (sizeof(unsigned long long) + sizeof(unsigned));
       CUDA_TRY(launch_bounds64(P, 0));
     }
   }

@@ -195,9 +195,9 @@ struct sht_plan_s {
   int tc64_syn = 0, tc64_ana = 0;
   int tc64_able = 0;  // the analysis can: at the default tiling, where autotuning did not find another faster
   signed char *d_lexp = nullptr;
-  // per m index: whether the geometry allows the analysis; a byte per job, what of a
-  // synthesis runs in IEEE double instead (LegArgs in leg64.cuh)
-  unsigned char *d_geo = nullptr;
+  // per m index: the reference pair of an analysis (RefPair in leg64.cuh); a byte per job,
+  // what of a synthesis runs in IEEE double instead
+  unsigned long long *d_ref = nullptr;
   unsigned *d_wide_syn = nullptr;
   int *d_err = nullptr;      // device status word written by kernels with bounded waits
   float4 *d_join = nullptr;  // mixed plans: join record per (m index, pair), 3 float4 each

@@ -121,7 +121,7 @@ def bright_ring(geom, rng, spin):
 
 
 @pytest.mark.parametrize("how", ["plain", "batch", "noalloc", "graph"])
-@pytest.mark.parametrize("spin", [0, 2])
+@pytest.mark.parametrize("spin", [0, 2, 9, 37])
 def test_analysis_beside_a_bright_ring(sht, spin, how):
     """The coefficients that a ring 10^10 times as bright as the rest does not reach."""
     geom = sht.sht_geom_gauss(NLAT, 2 * LMAX + 1)
