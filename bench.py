@@ -363,18 +363,18 @@ MEASURED_TRAFFIC = {
     # one launch at the headline size (spin 2, GL 4096 x 8191, lmax 4095), single-pass
     # dram__bytes_read.sum + dram__bytes_write.sum (the pair's traffic capture under profiles/);
     # sha256 over the kernel file and its headers (_kernel_digest)
-    "mixed:legendre_analysis:tc": {"bytes": 883405824 + 435014912,
-                                   "sha256": "56b9b6d13b0ca098eb4b9030f5867c119bb221215b012fc14b9bc63f969b6c69"},
-    "mixed:legendre_synthesis": {"bytes": 687071232 + 330579968,
-                                 "sha256": "35df1c03f561150b8de275f568d25b7b33690e7f5c74a0efe27c451b3ac2d7d4"},
+    "mixed:legendre_analysis:tc": {"bytes": 881962752 + 434122496,
+                                   "sha256": "d81b2b4e14ee5277c0f28d0140910ff81c57be9582f7ce6a1bc8eaabab10824f"},
+    "mixed:legendre_synthesis": {"bytes": 686050304 + 330387456,
+                                 "sha256": "7e282f2674934bae05b8e247ae63697855e0491c963c0435d1d451f5a2ca2b7d"},
 }
 
 
-KERNEL_HEADERS = {"legendre_fp64.cu": ("sht_device.cuh",),
-                  "legendre_mixed.cu": ("df.cuh", "sht_device.cuh", "mixed_common.cuh", "sht_internal.h"),
+KERNEL_HEADERS = {"legendre_fp64.cu": ("sht_device.cuh", "leg64.cuh", "leg64_ieee.cuh"),
+                  "legendre_mixed.cu": ("df.cuh", "sht_device.cuh", "mixed_common.cuh", "dual.cuh", "mix_ana.cuh", "sht_internal.h"),
                   "legendre_tc.cu": ("df.cuh", "sht_device.cuh", "mixed_common.cuh", "dual.cuh", "tcgen05.cuh"),
-                  "legendre_tc_ana.cu": ("df.cuh", "sht_device.cuh", "mixed_common.cuh", "dual.cuh", "tcgen05.cuh",
-                                         "sht_internal.h")}
+                  "legendre_tc_ana.cu": ("df.cuh", "sht_device.cuh", "mixed_common.cuh", "dual.cuh", "mix_ana.cuh",
+                                         "tcgen05.cuh", "sht_internal.h")}
 
 
 def _kernel_digest(kernel_file):
