@@ -779,7 +779,9 @@ __global__ void __launch_bounds__(kFftThreads) fft_ana_kernel_global(FftArgs a, 
 // Where a call has too few rings for that (rings: its ring pairs times maps, per SM) a ring
 // takes the threads itself.  At most one per SM (us, mixed form, 512 / 256 / 128 threads): 96
 // points 30 / 29 / 27; 512 32 / 30 / 35; 613 56 / 60 / 80; 1000 41 / 42 / 53; 2048 51 / 59 / 84;
-// 4095 84 / 110 / 160.  Two: 96 points 47 / 31 / 29; 512 53 / 36 / 38; 1000 68 / 49 / 59.
+// 4095 84 / 110 / 160.  Two: 96 points 47 / 31 / 29; 512 53 / 36 / 38; 1000 68 / 49 / 59.  (Equal
+// rings: HEALPix grids, with a few long and many short ones, keep the rule by length, Nside 81
+// Jacobi analysis 654 us, 721 with this.)
 int fft_cta_threads(int len, double rings) {
   const int t = len <= 1024 ? kFftThreads / 4 : (2 * (len * (int)sizeof(double2) + 2048) <= 227 * 1024 ? kFftThreads / 2 : kFftThreads);
   if (rings > 2.0 || len <= 128) return t;

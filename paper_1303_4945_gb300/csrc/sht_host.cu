@@ -1353,8 +1353,9 @@ static int plan_build(sht_plan_s *P, const sht_geom_s *g) {
   if ((rc = upload(P, pf, &P->d_pair_fft)) != SHT_OK) return rc;
   if (maxlen <= kFftMaxLen) {
     P->fft_smem = maxlen * (int)sizeof(double2);
-    P->fft_threads = fft_cta_threads(maxlen, (double)P->npairs * P->nmaps / P->sms);
-    P->fft_batch_threads = fft_cta_threads(maxlen, 1e9);  // (with the other plans' rings)
+    // by the rings too where they are equal and alone (in a batch they run with other plans')
+    P->fft_batch_threads = fft_cta_threads(maxlen, 1e9);
+    P->fft_threads = P->nfft == 1 ? fft_cta_threads(maxlen, (double)P->npairs * P->nmaps / P->sms) : P->fft_batch_threads;
   } else {  // rings beyond shared memory: one L2-resident scratch slot per SM (one CTA each)
     int sms = 0;
     CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, P->device));
